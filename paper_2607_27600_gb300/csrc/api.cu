@@ -21,6 +21,7 @@
 
 #include "attn.cuh"
 #include "compact.cuh"
+#include "fewrow.cuh"
 #include "gemm.cuh"
 #include "gemv.cuh"
 #include "keyattn.cuh"
@@ -154,6 +155,17 @@ bool tmap_rows(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, u
   return make_tmap(m, base, 2, dims, strides, box);
 }
 
+// A rotated projection's weights [heads * dh][K] as the few-row kernel loads
+// them (fewrow.cuh): [heads][dh / 32][2][16][K], the middle dimension the two
+// halves of a head, so that a tile's rows come in rotate-half pairs 16 apart.
+bool tmap_pairs(CUtensorMap *m, const void *base, uint64_t n, uint64_t k, int dh) {
+  const uint64_t row = k * 2;
+  const uint64_t dims[5] = {k, 16, 2, (uint64_t)dh / 32, n / dh};
+  const uint64_t strides[4] = {row, row * (dh / 2), row * 16, row * dh};
+  const uint32_t box[5] = {64, 16, 2, (uint32_t)dh / 32, (uint32_t)(128 / dh)};
+  return make_tmap(m, base, 5, dims, strides, box);
+}
+
 // ---------------------------------------------------------------------------
 // checks
 // ---------------------------------------------------------------------------
@@ -233,14 +245,11 @@ bool kv_format_ok(const cc_model_cfg *c, const cc_kv_cache *kv) {
 }
 
 struct ScoreWs {
-  size_t xn, q, o, h, act, part, ztgt, hpart, sspart, flags, total;
+  size_t xn, q, o, h, act, part, ztgt, hpart, sspart, total;
   int n_vtiles;
   int n_htiles;   // column tiles of a d-column projection (at most d / 128): partials of
                   // the fused logit head (logit mode) and of the post-attention RMSNorm
 };
-
-// Per-tile progress flags of split-K GEMMs (at most one wave of tiles split).
-constexpr int kSplitFlags = 1024;
 
 // With CC_SCORE_PRECISE either pass carries the GEMM activations
 // (normalised inputs, attention output, SwiGLU output) and the queries as
@@ -266,7 +275,6 @@ ScoreWs score_layout(const cc_model_cfg *c, int batch, int cap, cc_score_mode mo
     w.hpart = take(R * w.n_htiles * 8);
   }
   w.sspart = take(R * w.n_htiles * 4);
-  w.flags = take(kSplitFlags * 4);
   w.total = off;
   return w;
 }
@@ -323,6 +331,8 @@ struct Gemm {
   CUtensorMap a, b, b2, b3;
   GemmParams p;
   uint64_t rows_est;   // rows visited at most (tile-count estimate on the host)
+  FewPlan few;         // few.nb > 0: a launch of few rows (fewrow.cuh)
+  bool one_group;      // few: one row group
 };
 
 // One GEMM over the cache rows: A [R][K] (bf16 workspace) x W [N][K]^T.
@@ -331,18 +341,14 @@ struct Gemm {
 // every slot of the batch).
 cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, const void *W2, int N,
                      int batch, int cap, const int32_t *seq_len, unsigned *status,
-                     bool a_split = false, uint64_t rows_hint = 0) {
+                     bool a_split = false, uint64_t rows_hint = 0, int few_tiles = 0) {
   const uint64_t R = (uint64_t)batch * cap;
   const uint64_t R_est = rows_hint ? rows_hint : R;
   int bn = gemm_block_n(epi);
-  // narrow problems (less than one wave of 256-column tiles): 128-column
-  // tiles double the tiles that share the SMs
-  // (a residual GEMM long enough for two K splits keeps wide tiles and splits
-  // K instead: plan_k_splits, measured faster for the down projection)
-  const int nk_total = ((K + 63) / 64) * (a_split ? 2 : 1);
+  // narrow problems (less than one wave of 256-column tiles) that stay on this
+  // kernel: 128-column tiles double the tiles that share the SMs
   const bool narrowable = epi == EPI_F32 || epi == EPI_QROPE || epi == EPI_RESID_BF16 ||
-                          ((epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT) && nk_total < 128) ||
-                          epi == EPI_BF16;
+                          epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT || epi == EPI_BF16;
   DevState *dev_info = nullptr;
   const bool have_dev = dev_state(&dev_info);
   // CTA pairs: for launches of two waves or more of 128 x 256 tiles (a pair
@@ -357,10 +363,26 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
                     (pair_mode == 2 ||
                      (pair_mode == 1 && ((R_est + 127) / 128) * (uint64_t)((N + bn - 1) / bn) >=
                                             2 * (uint64_t)dev_info->sms));
-  if (!tmap_rows(&g.a, A, R, a_split ? 2 * K : K, 128)) return tmap_fail();
-  if (!tmap_rows(&g.b, W, N, K, epi == EPI_SWIGLU || pair ? 128 : bn)) return tmap_fail();
+  // launches below two waves of tiles: few.nb rows per group on the N side,
+  // the K range over a cluster's CTAs (CC_GEMM_PAIRS keeps them on this kernel)
+  g.few = FewPlan{};
+  g.one_group = false;
+  const uint64_t per_seq = rows_hint ? (rows_hint + batch - 1) / batch : (uint64_t)cap;
+  // (a batch of sequences with a few rows each would read every weight tile
+  // once per sequence's group: 16 one-row groups 5.5 ms against 4.25 ms)
+  if (have_dev && !pair && !pairs_env && epi != EPI_F32 && epi != EPI_LSE &&
+      (batch == 1 || per_seq >= 16)) {
+    g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
+                     batch, (long long)per_seq, dev_info->sms);
+    g.one_group = batch == 1 && per_seq <= (uint64_t)g.few.nb;
+    bn = kFewTileCols;
+  }
+  const bool few = g.few.nb > 0;
+  const uint32_t b_box = few || epi == EPI_SWIGLU || pair ? 128 : (uint32_t)bn;
+  if (!tmap_rows(&g.a, A, R, a_split ? 2 * K : K, few ? (uint32_t)g.few.nb : 128)) return tmap_fail();
+  if (!tmap_rows(&g.b, W, N, K, b_box)) return tmap_fail();
   if (epi == EPI_SWIGLU) {
-    if (!tmap_rows(&g.b2, W2, N, K, 128)) return tmap_fail();
+    if (!tmap_rows(&g.b2, W2, N, K, b_box)) return tmap_fail();
   } else {
     g.b2 = g.b;
   }
@@ -372,7 +394,8 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   g.p.N = N;
   g.p.K = K;
   g.p.block_n = epi == EPI_SWIGLU ? 256 : bn;
-  g.p.n_tiles = (N + bn - 1) / bn;
+  g.p.n_tiles = few ? g.few.n_tiles : (N + bn - 1) / bn;
+  g.p.kv_cap = cap;
   g.p.status = status;
   g.p.a_split = a_split ? 1 : 0;
   // Tile order for L2 reuse: keep a slab of one operand resident (evict-last;
@@ -425,15 +448,17 @@ cc_status gemm_setup_qkv(Gemm &g, const void *xn, const cc_model_cfg *c,
                          const cc_layer_weights &lw, int batch, int cap, const int32_t *seq_len,
                          unsigned *status, uint64_t rows_hint) {
   const int d = c->d_model, qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
+  const int fq = (qd + 127) / 128, fk = (kvd + 127) / 128;   // column tiles of a few-row launch
   cc_status s = gemm_setup(g, EPI_QKV, xn, d, lw.wq, nullptr, qd + 2 * kvd, batch, cap, seq_len,
-                           status, false, rows_hint);
+                           status, false, rows_hint, fq + 2 * fk);
   if (s != CC_OK) return s;
-  const uint32_t box = g.p.pair ? 128 : 256;   // a pair's CTAs load half a tile each
-  if (!tmap_rows(&g.b, lw.wq, qd, d, box) || !tmap_rows(&g.b2, lw.wk, kvd, d, box) ||
-      !tmap_rows(&g.b3, lw.wv, kvd, d, box))
-    return tmap_fail();
-  g.p.n_q_tiles = qd / 256;
-  g.p.n_k_tiles = kvd / 256;
+  const bool few = g.few.nb > 0;
+  const uint32_t box = few || g.p.pair ? 128 : 256;   // a pair's CTAs load half a tile each
+  const bool q_ok = few ? tmap_pairs(&g.b, lw.wq, qd, d, c->head_dim) : tmap_rows(&g.b, lw.wq, qd, d, box);
+  const bool k_ok = few ? tmap_pairs(&g.b2, lw.wk, kvd, d, c->head_dim) : tmap_rows(&g.b2, lw.wk, kvd, d, box);
+  if (!q_ok || !k_ok || !tmap_rows(&g.b3, lw.wv, kvd, d, box)) return tmap_fail();
+  g.p.n_q_tiles = few ? fq : qd / 256;
+  g.p.n_k_tiles = few ? fk : kvd / 256;
   g.p.ldo = qd;
   g.p.ldo_kv = kvd;
   g.p.bias = reinterpret_cast<const __nv_bfloat16 *>(lw.bq);
@@ -444,35 +469,19 @@ cc_status gemm_setup_qkv(Gemm &g, const void *xn, const cc_model_cfg *c,
   return CC_OK;
 }
 
-// K splits for a residual GEMM with less than one wave of output tiles
-// (short caches): each split is a work item; splits add into the fp32
-// residual in order (flags in the caller's workspace, tagged per launch).
-void plan_k_splits(Gemm &g, int epi, int sms, unsigned *flags) {
-  g.p.k_splits = 1;
-  if ((epi != EPI_RESID_F32 && epi != EPI_RESID_LOGIT) || !flags || g.p.pair) return;
-  const uint64_t tiles = ((g.rows_est + 127) / 128) * (uint64_t)g.p.n_tiles;
-  const int nk_total = ((g.p.K + 63) / 64) * (g.p.a_split ? 2 : 1);
-  if (tiles == 0 || tiles >= (uint64_t)sms || tiles > (uint64_t)kSplitFlags) return;
-  // >= 64 k-blocks (K >= 4096) per split: shorter splits lose more to the
-  // ordered epilogues than they gain (measured on Qwen2.5 O projections)
-  int splits = std::min<int>((int)(sms / tiles), std::min(8, nk_total / 64));
-  if (splits < 2) return;
-  static std::atomic<unsigned> epoch{0};
-  g.p.k_splits = splits;
-  g.p.split_flags = flags;
-  g.p.epoch = (epoch.fetch_add(1) % (1u << 27)) + 1;   // flags hold epoch * 16 + split
-}
-
-// Zeroes the split-K flags of a workspace once per call (a fresh workspace
-// may hold any bits; later launches tag their values with new epochs).
-cc_status clear_split_flags(unsigned *flags, cudaStream_t st) {
-  CC_TRY(cudaMemsetAsync(flags, 0, kSplitFlags * 4, st));
+// The weights' map of a rotated projection once head_dim is known (gemm_setup
+// maps plain rows).
+cc_status rope_weights(Gemm &g, const void *w, int n, int k, int head_dim) {
+  if (g.few.nb && !tmap_pairs(&g.b, w, n, k, head_dim)) return tmap_fail();
   return CC_OK;
 }
 
 cc_status run_gemm(Gemm &g, int epi, int kind, int sms, cudaStream_t st) {
   TimedScope t(kind, st);
-  CC_TRY(launch_gemm(epi, g.a, g.b, g.b2, g.b3, g.p, sms, st));
+  if (g.few.nb)
+    CC_TRY(launch_few(epi, g.a, g.b, g.b2, g.b3, g.p, g.few, g.one_group, sms, st));
+  else
+    CC_TRY(launch_gemm(epi, g.a, g.b, g.b2, g.b3, g.p, sms, st));
   return CC_OK;
 }
 
@@ -784,9 +793,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   void *xn = wsb + L.s.xn, *q = wsb + L.s.q, *o = wsb + L.s.o, *act = wsb + L.s.act;
   float *h = reinterpret_cast<float *>(wsb + L.s.h);
   int32_t *lo = reinterpret_cast<int32_t *>(wsb + L.lo), *hi = reinterpret_cast<int32_t *>(wsb + L.hi);
-  unsigned *flags = reinterpret_cast<unsigned *>(wsb + L.s.flags);
   unsigned *status = dev->status;
-  if ((s = clear_split_flags(flags, st)) != CC_OK) return s;
   const uint64_t used = (uint64_t)batch * max_count;   // rows the GEMMs visit at most
   AttnPartials parts;
   parts.o = reinterpret_cast<float *>(wsb + L.part_o);
@@ -867,7 +874,10 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
         g.p.k_qscale = 1.f / kvf.k_scale;
         g.p.v_qscale = 1.f / kvf.v_scale;
       }
-      if (pj.epi == EPI_QROPE) rope_turns(c, g.p.turns);
+      if (pj.epi == EPI_QROPE) {
+        rope_turns(c, g.p.turns);
+        if ((s = rope_weights(g, pj.w, pj.n, d, c->head_dim)) != CC_OK) return s;
+      }
       if ((s = run_gemm(g, pj.epi, pj.kind, dev->sms, st)) != CC_OK) return s;
     }
     // o = attention of the chunk rows over the memory and the chunk (causal)
@@ -903,7 +913,6 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     go.p.norm_gain = reinterpret_cast<const __nv_bfloat16 *>(lw.mlp_norm);
     go.p.ld_norm = d;
     go.p.ss_part = ss_part;
-    plan_k_splits(go, EPI_RESID_F32, dev->sms, flags);
     if ((s = run_gemm(go, EPI_RESID_F32, CC_KERNEL_GEMM_OPROJ, dev->sms, st)) != CC_OK) return s;
     Gemm gu;
     if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, batch, cap, hi, status,
@@ -924,7 +933,6 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     gd.p.row_lo = lo;
     gd.p.out = h;
     gd.p.ldo = d;
-    plan_k_splits(gd, EPI_RESID_F32, dev->sms, flags);
     if ((s = run_gemm(gd, EPI_RESID_F32, CC_KERNEL_GEMM_DOWN, dev->sms, st)) != CC_OK) return s;
   }
   {
@@ -1009,8 +1017,6 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
   // keys always run to the sequence end
   const int32_t *sl = rng_hi ? rng_hi : kv->seq_len;
   unsigned *status = dev->status;
-  unsigned *flags = reinterpret_cast<unsigned *>(wsb + L.flags);
-  if ((s = clear_split_flags(flags, st)) != CC_OK) return s;
   int n_htiles = 0;   // column tiles of the fused head's partials
 
   if (full) {
@@ -1056,6 +1062,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     gq.p.bias = reinterpret_cast<const __nv_bfloat16 *>(lw.bq);
     gq.p.head_dim = c->head_dim;
     rope_turns(c, gq.p.turns);
+    if ((s = rope_weights(gq, lw.wq, qd, d, c->head_dim)) != CC_OK) return s;
     if ((s = run_gemm(gq, EPI_QROPE, CC_KERNEL_GEMM_QROPE, dev->sms, st)) != CC_OK) return s;
     // O = counter-causal attention
     CC_TRY(wait_kv_ready(kv, l, l + 1, st));
@@ -1086,7 +1093,6 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     go.p.norm_split = split ? 1 : 0;
     go.p.ss_part = ss_part;
     go.p.ab_f16 = go.p.out_f16 = f16 ? 1 : 0;
-    plan_k_splits(go, epi_o, dev->sms, flags);
     if ((s = run_gemm(go, epi_o, CC_KERNEL_GEMM_OPROJ, dev->sms, st)) != CC_OK) return s;
     // act = silu(xn Wg^T / rms(h)) * (xn Wu^T / rms(h))
     Gemm gu;
@@ -1131,7 +1137,6 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
       gd.p.ss_part = ss_part;
       ss_tiles = gd.p.n_tiles;
     }
-    plan_k_splits(gd, epi_d, dev->sms, flags);
     if ((s = run_gemm(gd, epi_d, CC_KERNEL_GEMM_DOWN, dev->sms, st)) != CC_OK) return s;
   }
   // head

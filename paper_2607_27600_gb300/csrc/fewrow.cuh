@@ -1,0 +1,33 @@
+// fewrow.cuh -- interface of the GEMM for launches of few rows (short
+// caches, small chunks, decode batches): gemm.cuh's products with the weight
+// rows on the tensor cores' M side.
+#pragma once
+#include "gemm.cuh"
+
+namespace cc {
+
+constexpr int kFewMaxSplit = 8;   // K splits = CTAs of a cluster (the portable cluster size)
+
+// How a launch is cut: row groups of nb activation rows (the N of a product),
+// column tiles of 128 columns, and the K range of each tile over `split` CTAs
+// of a cluster.
+struct FewPlan {
+  int nb, split;
+  int n_tiles;     // column tiles (EPI_QKV: those of Q, K and V, each rounded up)
+  double cycles;   // estimated SM cycles
+};
+
+constexpr int kFewTileCols = 128;   // output columns of a tile
+// The plan for `groups(nb)` row groups: seqs sequences of at most rows_per_seq rows each.
+FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
+                 int sms);
+// a: A rows x K, box 64 x plan.nb; b (b2, b3): weights N x K, box 64 x 128, and
+// for rotated projections (EPI_QROPE's b, EPI_QKV's b and b2) the 5-D view
+// [heads][head_dim / 32][2][16][K], box {64, 16, 2, head_dim / 32, 128 / head_dim}.
+// one_group: the launch has one row group (known on the host), so the first
+// weight tiles are fetched before the previous kernel has finished.
+cudaError_t launch_few(int epi, const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
+                       const CUtensorMap &b3, const GemmParams &p, const FewPlan &plan,
+                       bool one_group, int sms, cudaStream_t stream);
+
+}  // namespace cc

@@ -311,16 +311,16 @@ CC_DEV void logit_partials(const GemmParams &p, uint32_t tacc, int grow, bool va
 }
 
 // fp32 outputs (EPI_F32, EPI_RESID_*), through the staging tile: out = acc
-// (+ bf16 resid, or += for RESID_F32); with norm_out (last K split) also
+// (+ bf16 resid, or += for RESID_F32); with norm_out also
 // bf16(out * norm_gain) (and the lo part; fp16 instead with out_f16) and the
 // tile's partial sum of out^2.
 template <int EPI, int TBN>
 CC_DEV void f32_epilogue(const GemmParams &p, uint32_t tacc, int grow, bool valid, int nt,
-                         int tile_n0, bool last, float *stage) {
+                         int tile_n0, float *stage) {
   const int lane = threadIdx.x & 31, cq = (lane & 7) * 4;
   const int nv = __popc(__ballot_sync(0xFFFFFFFFu, valid));
   const int grow0 = __shfl_sync(0xFFFFFFFFu, grow, 0);
-  const bool nrm = (EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32) && p.norm_out && last;
+  const bool nrm = (EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32) && p.norm_out;
   float ss[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) ss[i] = 0.f;
@@ -350,7 +350,7 @@ CC_DEV void f32_epilogue(const GemmParams &p, uint32_t tacc, int grow, bool vali
         const uint2 h = *reinterpret_cast<const uint2 *>(
             reinterpret_cast<const __nv_bfloat16 *>(p.resid) + row * p.ld_resid + col + cq);
         a[i].x += bf16_lo(h.x); a[i].y += bf16_hi(h.x); a[i].z += bf16_lo(h.y); a[i].w += bf16_hi(h.y);
-      } else if constexpr (EPI == EPI_RESID_F32 || EPI == EPI_RESID_LOGIT) {
+      } else if constexpr (EPI == EPI_RESID_F32) {
         const float4 h = *reinterpret_cast<const float4 *>(
             reinterpret_cast<const float *>(p.out) + row * p.ldo + col + cq);
         a[i].x += h.x; a[i].y += h.y; a[i].z += h.z; a[i].w += h.w;
@@ -395,16 +395,11 @@ CC_DEV void f32_epilogue(const GemmParams &p, uint32_t tacc, int grow, bool vali
 
 template <int EPI, int TBN>
 CC_DEV void epilogue_tile(const GemmParams &p, uint32_t tacc, int grow, bool valid, int nt,
-                          int tile_n0, bool last, float *stage) {
+                          int tile_n0, float *stage) {
   if constexpr (EPI == EPI_RESID_LOGIT) {
-    if (last) {
-      logit_partials<TBN>(p, tacc, grow, valid, nt, tile_n0, stage);
-      return;
-    }
-  }
-  if constexpr (EPI == EPI_F32 || EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32 ||
-                EPI == EPI_RESID_LOGIT) {
-    f32_epilogue<EPI, TBN>(p, tacc, grow, valid, nt, tile_n0, last, stage);
+    logit_partials<TBN>(p, tacc, grow, valid, nt, tile_n0, stage);
+  } else if constexpr (EPI == EPI_F32 || EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32) {
+    f32_epilogue<EPI, TBN>(p, tacc, grow, valid, nt, tile_n0, stage);
   } else if constexpr (EPI == EPI_QROPE) {   // kv_fp8: the K rows of an e4m3 cache
     const long long orow = p.kv_dest ? cache_row(p, grow, valid) : grow;
     const bool hm = p.kv_dest && p.pg.head_major;
@@ -567,7 +562,7 @@ CC_DEV void tile_coords(const GemmParams &p, int t, int num_m, int &m, int &n) {
 // epilogue warps release an accumulator by arriving on CTA 0's barrier.
 // (A relay thread in CTA 1 that waited for its own stage barrier and then
 // arrived on CTA 0's measured 3.4x slower on the gate/up shape: the
-// hand-over latency sat on every stage.)  K splits run on single CTAs only.
+// hand-over latency sat on every stage.)
 template <int EPI, int TBN, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -598,7 +593,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   int *prefix = reinterpret_cast<int *>(smem + ring_bytes(PAIR) + 256);
   float *stage_all = reinterpret_cast<float *>(smem + ring_bytes(PAIR) + 256 + kPrefixBytes);
-  __shared__ int split_ok;   // K splits: the previous split of the tile has published
 
   // a pair kernel launched without its cluster of two has no partner for
   // the pair instructions: every CTA reports it and leaves before any
@@ -641,11 +635,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int total = num_mu * p.n_tiles;
   const int nk = (p.K + BK - 1) / BK;           // k-blocks of one operand pass
   const int nk_total = p.a_split ? 2 * nk : nk;  // split A: the hi pass, then the lo pass
-  // Work item = (tile, K split): the splits of a tile are consecutive items.
-  const int S = (!PAIR && (EPI == EPI_RESID_F32 || EPI == EPI_RESID_LOGIT) && p.k_splits > 1)
-                    ? p.k_splits
-                    : 1;
-  const int total_items = total * S;
   const int unit0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int n_units = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   // row tile of this CTA in row unit u (-1: past the last tile, the second
@@ -665,8 +654,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int item = unit0; ok && item < total_items; item += n_units) {
-        const int tile = item / S, split = item - tile * S;
+      for (int tile = unit0; ok && tile < total; tile += n_units) {
         int mu, nt;
         tile_coords(p, tile, num_mu, mu, nt);
         const int mt = row_tile(mu);
@@ -675,11 +663,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int b = find_seq(prefix, p.batch, mt);
           row0 = b * p.cap + (p.row_lo ? p.row_lo[b] : 0) + (mt - prefix[b]) * BM;
         }
-        const int kb0 = split * nk_total / S, kb1 = (split + 1) * nk_total / S;
         // a pair's second row tile exists (CTA 0 counts its A bytes)
         const bool a1 = PAIR && 2 * mu + 1 < num_m;
-        for (int kbs = kb0; kbs < kb1; kbs += KB2) {
-          const int nb = min(KB2, kb1 - kbs);
+        for (int kbs = 0; kbs < nk_total; kbs += KB2) {
+          const int nb = min(KB2, nk_total - kbs);
           if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status))) break;
           if (!PAIR) mbar_arrive_expect_tx(&full[stage], nb * (A_BYTES + TB_BYTES));
           else if (rank == 0) mbar_arrive_expect_tx(&full[stage], nb * ((a1 ? 2 : 1) * A_BYTES + TB_BYTES));
@@ -727,14 +714,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t b_desc0 = make_sdesc_sw128(smem_u32(sB), 16, 1024);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
-      for (int item = unit0; item < total_items; item += n_units) {
-        const int split = item % S;
-        const int kb0 = split * nk_total / S, kb1 = (split + 1) * nk_total / S;
+      for (int tile = unit0; tile < total; tile += n_units) {
         if (!mbar_wait<PAIR>(&tempty[acc], acc_phase ^ 1, abort_flag, p.status)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * TBN;
-        for (int kbs = kb0; kbs < kb1; kbs += KB2) {
-          const int nb = min(KB2, kb1 - kbs);
+        for (int kbs = 0; kbs < nk_total; kbs += KB2) {
+          const int nb = min(KB2, nk_total - kbs);
           if (!mbar_wait<PAIR>(&full[stage], phase, abort_flag, p.status)) goto mma_done;
           tc_fence_after();
           for (int j = 0; j < nb; ++j) {
@@ -745,7 +730,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t bd = b_desc0 + (uint64_t)(slot * (SB >> 4));
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k) {
-              const uint32_t accum = (kb != kb0 || k != 0) ? 1u : 0u;
+              const uint32_t accum = (kb != 0 || k != 0) ? 1u : 0u;
               if constexpr (PAIR) umma_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, accum);
               else umma_ss(d_tmem, ad + 2 * k, bd + 2 * k, idesc, accum);
             }
@@ -765,8 +750,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = q * 32 + lane;   // accumulator row of this thread
     int acc = 0;
     uint32_t acc_phase = 0;
-    for (int item = unit0; item < total_items; item += n_units) {
-      const int tile = item / S, split = item - tile * S;
+    for (int tile = unit0; tile < total; tile += n_units) {
       int mu, nt;
       tile_coords(p, tile, num_mu, mu, nt);
       const int mt = row_tile(mu);
@@ -781,28 +765,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, p.status)) break;
       tc_fence_after();
       const uint32_t tacc = tmem_base + acc * TBN + (uint32_t(q * 32) << 16);
-      // K splits add into out in split order (deterministic sums): split s
-      // waits until split s-1 of the tile has published epoch * 16 + s.
-      // Split s-1 is a lower work item, and every CTA takes its items in
-      // increasing order, so the wait always ends (bounded all the same).
-      bool add = mt >= 0;
-      if (S > 1) {
-        if (warp == 2 && lane == 0)
-          split_ok = split == 0 || wait_value(&p.split_flags[tile], p.epoch * 16u + split, p.status);
-        named_barrier_sync(1, 128);
-        add = split_ok != 0;   // a wait that gave up (status set) skips this split's add
-      }
-      if (add)
-        epilogue_tile<EPI, TBN>(p, tacc, grow, valid, nt, nt * TBN, split == S - 1,
-                                stage_all + q * 32 * kStageLd);
+      if (mt >= 0)
+        epilogue_tile<EPI, TBN>(p, tacc, grow, valid, nt, nt * TBN, stage_all + q * 32 * kStageLd);
       tc_fence_before();
-      if (S > 1) {
-        named_barrier_sync(1, 128);
-        if (warp == 2 && lane == 0) {
-          __threadfence();
-          st_release_u32(&p.split_flags[tile], p.epoch * 16u + split + 1);
-        }
-      }
       __syncwarp();
       if (lane == 0) {
         if (PAIR && rank == 1) mbar_arrive_cluster(cluster_addr(&tempty[acc], 0));

@@ -63,7 +63,7 @@ struct GemmParams {
                            // (B kept in L2, A streamed per group); 1 = groups of `group`
                            // row tiles stay resident (A kept, B streamed per group)
   int group;
-  int pair;                // run as CTA pairs (256-column tiles, k_splits 1): the B tensor
+  int pair;                // run as CTA pairs (256-column tiles): the B tensor
                            // maps' boxes are 128 rows (each CTA loads half of a tile);
                            // raster 1 groups count pairs of row tiles
   int out_split;           // EPI_SWIGLU, EPI_QROPE (not into the cache): out rows are
@@ -72,12 +72,6 @@ struct GemmParams {
   int out_f16;             // the activations written for the next product (EPI_SWIGLU and
                            // EPI_QROPE out, norm_out) are fp16 (not with the splits); a
                            // value above 65504 in magnitude sets CC_ERR_RANGE in status
-  int k_splits;            // EPI_RESID_F32 / EPI_RESID_LOGIT only: K range split over
-                           // k_splits work items per tile (< one wave of tiles); the splits
-                           // add into out in order (EPI_RESID_LOGIT: the last one takes the
-                           // partials instead)
-  unsigned *split_flags;   // [tiles] (k_splits > 1): per-tile progress, epoch * 16 + split
-  unsigned epoch;          // per-launch tag (>= 1) of split_flags values
   int n_q_tiles, n_k_tiles;   // EPI_QKV: column tiles of Q and of K (V has n_k_tiles too)
   void *out_k, *out_v;        // EPI_QKV: bf16 [rows][ldo_kv] destinations of K and V
   int ldo_kv;
@@ -85,6 +79,9 @@ struct GemmParams {
   int kv_dest;                // EPI_QROPE / EPI_BF16: the output is K / V cache rows (paged
                               // through pg; EPI_QKV: always for its K and V parts)
   KvLayout pg;                // paged K/V (pg.table nullptr: row b * cap + i)
+  int kv_cap;                 // slots per sequence of the cache
+  const int32_t *rowmap;      // nullptr: row r is cache slot b * cap + i itself; else packed
+                              // rows, rowmap[r] = b * kv_cap + i (< 0: no row)
   int kv_fp8;                 // EPI_QKV: K and V destinations are e4m3 (one byte each);
                               // EPI_QROPE / EPI_BF16: the destination is e4m3 K / V
   float k_qscale, v_qscale;   // kv_fp8: 1 / the K and V scales (code = rne(value * qscale))
