@@ -1549,7 +1549,7 @@ def main():
     ap.add_argument("--kv-fp8", action="store_true",
                     help="store the cache's K/V as e4m3 codes with per-layer scales")
     ap.add_argument("--batch", type=int, default=1,
-                    help="--decode: sequences decoded together (1-4 take the GEMV path)")
+                    help="--decode: sequences decoded together")
     ap.add_argument("--head-major", action="store_true",
                     help="keep the refresh bench's K/V head-major ([B, Hkv, cap, dh])")
     ap.add_argument("--paged", type=int, default=0, metavar="SLOTS",

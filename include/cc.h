@@ -353,9 +353,8 @@ size_t cc_append_workspace_size(const cc_model_cfg *cfg, int32_t batch, int32_t 
  * next_tokens[b] = argmax of the logits (the lowest id on ties; -1 for a
  * sequence that could not append: full cache, reported on the device) and,
  * if next_logit is non-NULL, its logit.  Needs everything cc_append_chunk
- * needs plus final_norm and lm_head.  Each sequence's row is its own GEMM row
- * tile: one sequence reads the weights once per step, a batch of B reads
- * them B times (decode batching across sequences is not fused). */
+ * needs plus final_norm and lm_head.  The sequences' rows are packed into one
+ * product: every weight is read once per step. */
 size_t cc_decode_workspace_size(const cc_model_cfg *cfg, int32_t batch, int32_t cap);
 cc_status cc_decode_step(const cc_model_cfg *cfg, const cc_model_weights *w,
                          const cc_kv_cache *cache, const int32_t *tokens_in,

@@ -23,7 +23,6 @@
 #include "compact.cuh"
 #include "fewrow.cuh"
 #include "gemm.cuh"
-#include "gemv.cuh"
 #include "keyattn.cuh"
 #include "rowops.cuh"
 #include "select.cuh"
@@ -330,20 +329,16 @@ cc_status device_fail() {
 struct Gemm {
   CUtensorMap a, b, b2, b3;
   GemmParams p;
-  uint64_t rows_est;   // rows visited at most (tile-count estimate on the host)
   FewPlan few;         // few.nb > 0: a launch of few rows (fewrow.cuh)
   bool one_group;      // few: one row group
 };
 
 // One GEMM over the cache rows: A [R][K] (bf16 workspace) x W [N][K]^T.
 // a_split: A rows are [hi | lo] (2K values) and the product is hi W^T + lo W^T.
-// rows_hint: rows the GEMM visits at most (the traffic model's A size; 0 =
-// every slot of the batch).
 cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, const void *W2, int N,
                      int batch, int cap, const int32_t *seq_len, unsigned *status,
-                     bool a_split = false, uint64_t rows_hint = 0, int few_tiles = 0) {
+                     bool a_split = false, int few_tiles = 0) {
   const uint64_t R = (uint64_t)batch * cap;
-  const uint64_t R_est = rows_hint ? rows_hint : R;
   int bn = gemm_block_n(epi);
   // narrow problems (less than one wave of 256-column tiles) that stay on this
   // kernel: 128-column tiles double the tiles that share the SMs
@@ -357,24 +352,20 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   const char *pairs_env = getenv("CC_GEMM_PAIRS");
   const int pair_mode = !pairs_env ? 1 : pairs_env[0] == '0' ? 0 : pairs_env[0] == '2' ? 2 : 1;
   if (narrowable && have_dev && pair_mode != 2 &&
-      ((R_est + 127) / 128) * (uint64_t)((N + 255) / 256) < (uint64_t)dev_info->sms)
+      ((R + 127) / 128) * (uint64_t)((N + 255) / 256) < (uint64_t)dev_info->sms)
     bn = 128;
   const bool pair = have_dev && epi != EPI_ARGMAX && (epi == EPI_SWIGLU || bn == 256) &&
                     (pair_mode == 2 ||
-                     (pair_mode == 1 && ((R_est + 127) / 128) * (uint64_t)((N + bn - 1) / bn) >=
+                     (pair_mode == 1 && ((R + 127) / 128) * (uint64_t)((N + bn - 1) / bn) >=
                                             2 * (uint64_t)dev_info->sms));
   // launches below two waves of tiles: few.nb rows per group on the N side,
   // the K range over a cluster's CTAs (CC_GEMM_PAIRS keeps them on this kernel)
   g.few = FewPlan{};
   g.one_group = false;
-  const uint64_t per_seq = rows_hint ? (rows_hint + batch - 1) / batch : (uint64_t)cap;
-  // (a batch of sequences with a few rows each would read every weight tile
-  // once per sequence's group: 16 one-row groups 5.5 ms against 4.25 ms)
-  if (have_dev && !pair && !pairs_env && epi != EPI_F32 && epi != EPI_LSE &&
-      (batch == 1 || per_seq >= 16)) {
+  if (have_dev && !pair && !pairs_env && epi != EPI_F32 && epi != EPI_LSE) {
     g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
-                     batch, (long long)per_seq, dev_info->sms);
-    g.one_group = batch == 1 && per_seq <= (uint64_t)g.few.nb;
+                     batch, cap, dev_info->sms);
+    g.one_group = batch == 1 && cap <= g.few.nb;
     bn = kFewTileCols;
   }
   const bool few = g.few.nb > 0;
@@ -408,7 +399,6 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   // even where a count of whole-slab re-reads favoured the latter by up to
   // 16 %.  The activation-resident order is taken only when that count is
   // below 0.8x (an LM head whose weight is far larger than L2).
-  const uint64_t R_used = R_est;
   // The slab budget: 40 MB, or 60 MB for an fp32-output GEMM whose streamed
   // activations outweigh its output (the down projection: each group of
   // resident weight tiles re-reads the activations).  Measured at the Llama-3-8B 16k launches (DRAM bytes read
@@ -418,14 +408,13 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   // 2.3 / 2.8 / 5.1 GB.
   const bool f32_out = epi == EPI_F32 || epi == EPI_RESID_BF16 || epi == EPI_RESID_F32 ||
                        epi == EPI_RESID_LOGIT;
-  const double act_bytes = (double)R_used * K * (a_split ? 2.0 : 1.0) * 2;
-  const double out_bytes = (double)R_used * N * (f32_out ? 4.0 : 2.0);
+  const double act_bytes = (double)R * K * (a_split ? 2.0 : 1.0) * 2;
+  const double out_bytes = (double)R * N * (f32_out ? 4.0 : 2.0);
   const double budget = (f32_out && act_bytes > out_bytes ? 60.0 : 40.0) * (1 << 20);
-  g.rows_est = R_used;
-  const int num_m = (int)((R_used + 127) / 128), num_n = g.p.n_tiles;
+  const int num_m = (int)((R + 127) / 128), num_n = g.p.n_tiles;
   const double k_a = (a_split ? 2.0 : 1.0) * K;
   const int b_rows = epi == EPI_SWIGLU ? 256 : bn;   // weight rows of one column tile
-  const double a_bytes = (double)R_used * k_a * 2, b_bytes = (double)num_n * b_rows * K * 2;
+  const double a_bytes = (double)R * k_a * 2, b_bytes = (double)num_n * b_rows * K * 2;
   const double a_slab = 128.0 * k_a * 2, b_slab = (double)b_rows * K * 2;
   const int gn = (int)std::max(1.0, std::min((double)num_n, floor(budget / b_slab)));
   const int gm = (int)std::max(1.0, std::min((double)num_m, floor(budget / a_slab)));
@@ -446,11 +435,11 @@ bool qkv_fusable(const cc_model_cfg *c) {
 
 cc_status gemm_setup_qkv(Gemm &g, const void *xn, const cc_model_cfg *c,
                          const cc_layer_weights &lw, int batch, int cap, const int32_t *seq_len,
-                         unsigned *status, uint64_t rows_hint) {
+                         unsigned *status) {
   const int d = c->d_model, qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
   const int fq = (qd + 127) / 128, fk = (kvd + 127) / 128;   // column tiles of a few-row launch
   cc_status s = gemm_setup(g, EPI_QKV, xn, d, lw.wq, nullptr, qd + 2 * kvd, batch, cap, seq_len,
-                           status, false, rows_hint, fq + 2 * fk);
+                           status, false, fq + 2 * fk);
   if (s != CC_OK) return s;
   const bool few = g.few.nb > 0;
   const uint32_t box = few || g.p.pair ? 128 : 256;   // a pair's CTAs load half a tile each
@@ -528,7 +517,7 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
                         KvFmt kvf = KvFmt(), bool q_split = false,
                         const int32_t *range_lo = nullptr, const int32_t *range_hi = nullptr,
                         void *kv_scratch = nullptr, size_t kv_scratch_bytes = 0,
-                        bool f16 = false) {
+                        bool f16 = false, const int32_t *pbase = nullptr, int packed_rows = 0) {
   const int G = c->n_q_heads / c->n_kv_heads, dh = c->head_dim;
   const int P = attn_positions_per_unit(G);
   const uint64_t R = (uint64_t)batch * cap;
@@ -566,7 +555,7 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
   {
     // q_split: rows [hi heads | lo heads], the map spans both (lo at head Hq + t)
     const uint64_t qh = (uint64_t)c->n_q_heads * (q_split ? 2 : 1);
-    const uint64_t dims[3] = {(uint64_t)dh, qh, R};
+    const uint64_t dims[3] = {(uint64_t)dh, qh, pbase ? (uint64_t)packed_rows : R};
     const uint64_t strides[2] = {(uint64_t)dh * 2, qh * dh * 2};
     const uint32_t box[3] = {64, (uint32_t)G, (uint32_t)P};
     if (!make_tmap(&tq, q, 3, dims, strides, box)) return tmap_fail();
@@ -612,6 +601,7 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
   // counter-causal row range [range_lo, range_hi) (cc_score_rows); causal: row_lo
   p.row_lo = row_lo ? row_lo : range_lo;
   p.row_hi = row_lo ? nullptr : range_hi;
+  p.pbase = pbase;
   p.q_span = row_lo ? q_span : cap;
   const long long units = attn_units(p);
   if (decode) {   // one query row per sequence: the decode kernel
@@ -639,24 +629,30 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
 // inference cycle, pre-fill: chunk append over the memory
 // ---------------------------------------------------------------------------
 struct AppendWs {
-  ScoreWs s;          // xn, q, o, h, act rows b*cap + slot (the chunk's rows only are used)
-  size_t lo, hi, part_o, part_ml, total;   // part_*: key-split partials of the attention
+  ScoreWs s;          // xn, q, o, h, act: the appended slots as packed rows
+  size_t lo, hi, pbase, ptotal, rowmap;   // AppendRows
+  size_t part_o, part_ml, total;          // part_*: key-split partials of the attention
 };
 
 AppendWs append_layout(const cc_model_cfg *c, int batch, int cap) {
   AppendWs w{};
   w.s = score_layout(c, batch, cap, CC_SCORE_LOGIT, false);
   size_t off = w.s.total;
-  w.lo = off;
-  off = align256(off + (size_t)batch * 4);
-  w.hi = off;
-  off = align256(off + (size_t)batch * 4);
-  w.part_o = off;
-  off = align256(off + (size_t)kAttnMaxSplitSlots * 256 * c->head_dim * 4);
-  w.part_ml = off;
-  off = align256(off + (size_t)kAttnMaxSplitSlots * 256 * 8);
+  auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
+  w.lo = take((size_t)batch * 4);
+  w.hi = take((size_t)batch * 4);
+  w.pbase = take((size_t)batch * 4);
+  w.ptotal = take(4);
+  w.rowmap = take((size_t)batch * cap * 4);
+  w.part_o = take((size_t)kAttnMaxSplitSlots * 256 * c->head_dim * 4);
+  w.part_ml = take((size_t)kAttnMaxSplitSlots * 256 * 8);
   w.total = off;
   return w;
+}
+
+AppendRows append_rows(const AppendWs &L, uint8_t *ws) {
+  auto at = [&](size_t o) { return reinterpret_cast<int32_t *>(ws + o); };
+  return {at(L.lo), at(L.hi), at(L.pbase), at(L.ptotal), at(L.rowmap)};
 }
 
 // The tile attention over an e4m3 cache, or with fp16 operands, reads a
@@ -700,244 +696,156 @@ cc_status check_append_args(const cc_model_cfg *c, const cc_model_weights *w,
   return CC_OK;
 }
 
-// Decode-sized appends (one row per sequence, at most kGemvMaxRows
-// sequences) run the layer products as weight-streaming GEMVs with the
-// RMSNorms fused in: the tile GEMM would cover the weights with a few dozen
-// CTAs for a single row.  Shared memory bounds the staged rows (K of every
-// product, with the largest warp-partial buffer a plan can need).
-bool gemv_decode_ok(const cc_model_cfg *c, int batch, int max_count) {
-  if (max_count != 1 || batch < 1 || batch > kGemvMaxRows) return false;
-  if (c->n_kv_heads * c->head_dim < 16 || c->vocab < 16) return false;   // 16 output rows at least
-  const int ks[3] = {c->d_model, c->n_q_heads * c->head_dim, c->d_ff};
-  for (int K : ks) {
-    if (K < kGemvBoxK) return false;   // boxes no wider than the weights
-    GemvParams p{};
-    p.batch = batch;
-    p.K = K;
-    p.n_seg = 0;
-    if (K % 8 || !gemv_plan(p, 1)) return false;
-  }
-  return true;
-}
-
-// One GEMV launch: up to three weight matrices (segments) over the same rows.
-struct GemvCall {
-  GemvLaunch l{};
-  const void *w[kGemvMaxSegs][2] = {};
-  void add(const void *w0, const void *w1, const void *bias, void *out, int ldo, int n, int epi) {
-    GemvSeg &sg = l.p.seg[l.p.n_seg];
-    sg = GemvSeg{};
-    sg.bias = reinterpret_cast<const __nv_bfloat16 *>(bias);
-    sg.out = out;
-    sg.ldo = ldo;
-    sg.N = n;
-    sg.epi = epi;
-    w[l.p.n_seg][0] = w0;
-    w[l.p.n_seg][1] = w1;
-    ++l.p.n_seg;
-  }
-};
-
-GemvCall gemv_call(const cc_model_cfg *c, const cc_kv_cache *kv, const int32_t *lo,
-                   const int32_t *hi, unsigned *status, const void *x, int ldx, int K,
-                   const void *norm_gain) {
-  GemvCall g;
-  GemvParams &p = g.l.p;
-  p.batch = kv->batch;
-  p.cap = kv->cap;
-  p.row_lo = lo;
-  p.row_hi = hi;
-  p.pos = kv->pos;
-  p.head_dim = c->head_dim;
-  p.eps = c->rms_eps;
-  p.status = status;
-  p.x = x;
-  p.ldx = ldx;
-  p.K = K;
-  p.norm_gain = reinterpret_cast<const __nv_bfloat16 *>(norm_gain);
-  rope_turns(c, p.turns);
-  return g;
-}
-
-cc_status run_gemv(GemvCall &g, int kind, int sms, cudaStream_t st) {
-  GemvParams &p = g.l.p;
-  if (!gemv_plan(p, sms)) return CC_ERR_UNSUPPORTED;
-  for (int s = 0; s < p.n_seg; ++s) {
-    const uint64_t dims[2] = {(uint64_t)p.K, (uint64_t)p.seg[s].N};
-    const uint64_t strides[1] = {(uint64_t)p.K * 2};
-    const uint32_t box[2] = {(uint32_t)kGemvBoxK, 8};
-    for (int j = 0; j < 2; ++j)
-      if (g.w[s][j] && !make_tmap(&g.l.w[s][j], g.w[s][j], 2, dims, strides, box,
-                                  CU_TENSOR_MAP_SWIZZLE_NONE))
-        return tmap_fail();
-  }
-  TimedScope t(kind, st);
-  CC_TRY(launch_gemv(g.l, st));
-  return CC_OK;
-}
-
+// Appends a chunk (or a decode step's token) per sequence through every layer.
+// The workspace rows are the appended slots packed (AppendRows), so a batch
+// of sequences with a few rows each reads every weight once.  final_gain
+// (decode): the last layer also writes h * final_gain and its sums of squares
+// (*ss_tiles column tiles) for the LM head, and seq_len is left to the caller.
 cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_kv_cache *kv,
                      const int32_t *tokens_in, const int32_t *pos_in, const int32_t *count,
-                     int max_count, void *ws, size_t ws_bytes, void *stream) {
+                     int max_count, void *ws, size_t ws_bytes, void *stream,
+                     const void *final_gain = nullptr, int *ss_tiles_out = nullptr) {
   cc_status s = check_append_args(c, w, kv, tokens_in, count, max_count, ws, ws_bytes);
   if (s != CC_OK) return s;
   if (max_count == 0) return CC_OK;
   DevState *dev;
   if (!dev_state(&dev)) return device_fail();
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int batch = kv->batch, cap = kv->cap, rows = batch * cap;
+  const int batch = kv->batch, cap = kv->cap;
   const int d = c->d_model, qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
   const int f = c->d_ff;
   const AppendWs L = append_layout(c, batch, cap);
   uint8_t *wsb = reinterpret_cast<uint8_t *>(ws);
   void *xn = wsb + L.s.xn, *q = wsb + L.s.q, *o = wsb + L.s.o, *act = wsb + L.s.act;
   float *h = reinterpret_cast<float *>(wsb + L.s.h);
-  int32_t *lo = reinterpret_cast<int32_t *>(wsb + L.lo), *hi = reinterpret_cast<int32_t *>(wsb + L.hi);
+  float *ss_part = reinterpret_cast<float *>(wsb + L.s.sspart);
+  const AppendRows rows = append_rows(L, wsb);
+  const int32_t *total = rows.total;
   unsigned *status = dev->status;
-  const uint64_t used = (uint64_t)batch * max_count;   // rows the GEMMs visit at most
+  const int max_rows = (int)std::min((uint64_t)batch * max_count, (uint64_t)batch * cap);
   AttnPartials parts;
   parts.o = reinterpret_cast<float *>(wsb + L.part_o);
   parts.ml = reinterpret_cast<float2 *>(wsb + L.part_ml);
-  const bool use_gemv = gemv_decode_ok(c, batch, max_count);
 
   {
     TimedScope t(CC_KERNEL_APPEND, st);
     CC_TRY(launch_append_prepare(kv->seq_len, count, tokens_in, pos_in, max_count, kv->tokens,
-                                 kv->pos, lo, hi, batch, cap, status, st));
+                                 kv->pos, rows, batch, cap, status, st));
   }
+  // xn = h * g (unnormalised) and the sums of h^2 of each layer's attention
+  // norm come from the kernel that wrote h: the embedding, then the down
+  // projections; the projections scale their rows by 1 / rms(h)
+  int ss_tiles = 1;
   {
     TimedScope t(CC_KERNEL_EMBED, st);
-    CC_TRY(launch_embed(w->embed, kv->tokens, h, d, c->vocab, hi, cap, rows, status, st, lo,
-                        max_count));
+    CC_TRY(launch_append_embed(w->embed, kv->tokens, rows, max_rows, w->layers[0].attn_norm, h, xn,
+                               ss_part, d, c->vocab, status, st));
   }
+  auto scaled = [&](Gemm &g) {   // unnormalised A rows
+    g.p.row_ss = ss_part;
+    g.p.n_ss = ss_tiles;
+    g.p.ss_d = d;
+    g.p.eps = c->rms_eps;
+  };
+  // residual add, with the next norm's gain (or null) fused as in the scoring pass
+  auto resid = [&](const void *a, int k, const void *wm, const void *gain, int kind) -> cc_status {
+    Gemm g;
+    cc_status r = gemm_setup(g, EPI_RESID_F32, a, k, wm, nullptr, d, 1, max_rows, total, status);
+    if (r != CC_OK) return r;
+    g.p.out = h;
+    g.p.ldo = d;
+    if (gain) {
+      g.p.norm_out = reinterpret_cast<__nv_bfloat16 *>(xn);
+      g.p.norm_gain = reinterpret_cast<const __nv_bfloat16 *>(gain);
+      g.p.ld_norm = d;
+      g.p.ss_part = ss_part;
+      ss_tiles = g.p.n_tiles;
+    }
+    return run_gemm(g, EPI_RESID_F32, kind, dev->sms, st);
+  };
   for (int l = 0; l < c->n_layers; ++l) {
     const cc_layer_weights &lw = w->layers[l];
     const KvFmt kvf = kv_fmt(c, kv, l);   // e4m3 cache: K/V rows written as codes of value / scale
     CC_TRY(wait_kv_ready(kv, l, l + 1, st));
     if (l == c->n_layers - 1 && kv->h_last) {   // H^(L-1), recorded for the fast approximation
       TimedScope t(CC_KERNEL_APPEND, st);
-      CC_TRY(launch_store_bf16(h, kv->h_last, d, hi, lo, cap, rows, st, max_count));
-    }
-    if (use_gemv) {   // RMSNorm fused; q, k and v in one launch
-      GemvCall g = gemv_call(c, kv, lo, hi, status, h, d, d, lw.attn_norm);
-      g.add(lw.wq, nullptr, lw.bq, q, qd, qd, GEMV_ROPE);
-      g.add(lw.wk, nullptr, lw.bk, kv->k[l], kvd, kvd, GEMV_ROPE);
-      g.add(lw.wv, nullptr, lw.bv, kv->v[l], kvd, kvd, GEMV_BF16);
-      for (int j = 1; j < 3; ++j) {   // K and V into the cache (e4m3 codes; paged rows)
-        g.l.p.seg[j].fp8 = kvf.fp8 ? 1 : 0;
-        g.l.p.seg[j].qscale = 1.f / (j == 1 ? kvf.k_scale : kvf.v_scale);
-        g.l.p.seg[j].kv_dest = 1;
-      }
-      g.l.p.pg = kvf.pg;
-      if ((s = run_gemv(g, CC_KERNEL_GEMM_QKV, dev->sms, st)) != CC_OK) return s;
-    } else {
-      TimedScope t(CC_KERNEL_RMSNORM, st);
-      CC_TRY(launch_rmsnorm(h, true, lw.attn_norm, xn, d, c->rms_eps, hi, cap, rows, false, st, lo,
-                            max_count));
+      CC_TRY(launch_store_bf16(h, kv->h_last, d, rows, max_rows, st));
     }
     // q = RoPE(xn Wq^T + bq) into the workspace; k = RoPE(xn Wk^T + bk) and
     // v = xn Wv^T + bv straight into the cache slots of the chunk
-    if (!use_gemv && qkv_fusable(c)) {   // one GEMM over [Wq; Wk; Wv]
+    if (qkv_fusable(c)) {   // one GEMM over [Wq; Wk; Wv]
       Gemm g;
-      if ((s = gemm_setup_qkv(g, xn, c, lw, batch, cap, hi, status, used)) != CC_OK) return s;
-      g.p.row_lo = lo;
+      if ((s = gemm_setup_qkv(g, xn, c, lw, 1, max_rows, total, status)) != CC_OK) return s;
+      scaled(g);
       g.p.out = q;
       g.p.out_k = kv->k[l];
       g.p.out_v = kv->v[l];
       g.p.pos = kv->pos;
+      g.p.rowmap = rows.rowmap;
+      g.p.kv_cap = cap;
       g.p.kv_fp8 = kvf.fp8 ? 1 : 0;
       g.p.k_qscale = 1.f / kvf.k_scale;
       g.p.v_qscale = 1.f / kvf.v_scale;
       g.p.pg = kvf.pg;
       if ((s = run_gemm(g, EPI_QKV, CC_KERNEL_GEMM_QKV, dev->sms, st)) != CC_OK) return s;
-    }
-    struct Proj { const void *w, *bias; void *out; int n, epi, kind; };
-    const Proj projs[3] = {{lw.wq, lw.bq, q, qd, EPI_QROPE, CC_KERNEL_GEMM_QROPE},
-                           {lw.wk, lw.bk, kv->k[l], kvd, EPI_QROPE, CC_KERNEL_GEMM_KV},
-                           {lw.wv, lw.bv, kv->v[l], kvd, EPI_BF16, CC_KERNEL_GEMM_KV}};
-    for (const Proj &pj : projs) {
-      if (use_gemv || qkv_fusable(c)) break;
-      Gemm g;
-      if ((s = gemm_setup(g, pj.epi, xn, d, pj.w, nullptr, pj.n, batch, cap, hi, status, false,
-                          used)) != CC_OK)
-        return s;
-      g.p.row_lo = lo;
-      g.p.out = pj.out;
-      g.p.ldo = pj.n;
-      g.p.pos = kv->pos;
-      g.p.bias = reinterpret_cast<const __nv_bfloat16 *>(pj.bias);
-      g.p.head_dim = c->head_dim;
-      if (pj.kind == CC_KERNEL_GEMM_KV) {   // K or V rows into the cache
-        g.p.kv_dest = 1;
-        g.p.pg = kvf.pg;
-        g.p.kv_fp8 = kvf.fp8 ? 1 : 0;
-        g.p.k_qscale = 1.f / kvf.k_scale;
-        g.p.v_qscale = 1.f / kvf.v_scale;
+    } else {
+      struct Proj { const void *w, *bias; void *out; int n, epi, kind; };
+      const Proj projs[3] = {{lw.wq, lw.bq, q, qd, EPI_QROPE, CC_KERNEL_GEMM_QROPE},
+                             {lw.wk, lw.bk, kv->k[l], kvd, EPI_QROPE, CC_KERNEL_GEMM_KV},
+                             {lw.wv, lw.bv, kv->v[l], kvd, EPI_BF16, CC_KERNEL_GEMM_KV}};
+      for (const Proj &pj : projs) {
+        Gemm g;
+        if ((s = gemm_setup(g, pj.epi, xn, d, pj.w, nullptr, pj.n, 1, max_rows, total, status)) !=
+            CC_OK)
+          return s;
+        scaled(g);
+        g.p.out = pj.out;
+        g.p.ldo = pj.n;
+        g.p.pos = kv->pos;
+        g.p.rowmap = rows.rowmap;
+        g.p.kv_cap = cap;
+        g.p.bias = reinterpret_cast<const __nv_bfloat16 *>(pj.bias);
+        g.p.head_dim = c->head_dim;
+        if (pj.kind == CC_KERNEL_GEMM_KV) {   // K or V rows into the cache
+          g.p.kv_dest = 1;
+          g.p.pg = kvf.pg;
+          g.p.kv_fp8 = kvf.fp8 ? 1 : 0;
+          g.p.k_qscale = 1.f / kvf.k_scale;
+          g.p.v_qscale = 1.f / kvf.v_scale;
+        }
+        if (pj.epi == EPI_QROPE) {
+          rope_turns(c, g.p.turns);
+          if ((s = rope_weights(g, pj.w, pj.n, d, c->head_dim)) != CC_OK) return s;
+        }
+        if ((s = run_gemm(g, pj.epi, pj.kind, dev->sms, st)) != CC_OK) return s;
       }
-      if (pj.epi == EPI_QROPE) {
-        rope_turns(c, g.p.turns);
-        if ((s = rope_weights(g, pj.w, pj.n, d, c->head_dim)) != CC_OK) return s;
-      }
-      if ((s = run_gemm(g, pj.epi, pj.kind, dev->sms, st)) != CC_OK) return s;
     }
     // o = attention of the chunk rows over the memory and the chunk (causal)
     // (act is free until the MLP: an e4m3 layer's bf16 copy for the tile attention)
-    if ((s = run_attention(c, q, kv->k[l], kv->v[l], o, hi, batch, cap, status, st, false, lo,
-                           max_count, &parts, dev->sms, kvf, false, nullptr, nullptr, act,
-                           (size_t)batch * cap * c->d_ff * 2)) != CC_OK)
+    if ((s = run_attention(c, q, kv->k[l], kv->v[l], o, rows.hi, batch, cap, status, st, false,
+                           rows.lo, max_count, &parts, dev->sms, kvf, false, nullptr, nullptr, act,
+                           (size_t)batch * cap * c->d_ff * 2, false, rows.pbase, max_rows)) != CC_OK)
       return s;
-    // h += o Wo^T; xn = RMSNorm(h); act = SwiGLU; h += act Wd^T
-    if (use_gemv) {
-      GemvCall go = gemv_call(c, kv, lo, hi, status, o, qd, qd, nullptr);
-      go.add(lw.wo, nullptr, nullptr, h, d, d, GEMV_RESID_F32);
-      if ((s = run_gemv(go, CC_KERNEL_GEMM_OPROJ, dev->sms, st)) != CC_OK) return s;
-      GemvCall gu = gemv_call(c, kv, lo, hi, status, h, d, d, lw.mlp_norm);
-      gu.add(lw.w_gate, lw.w_up, nullptr, act, f, f, GEMV_SWIGLU);
-      if ((s = run_gemv(gu, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
-      GemvCall gd = gemv_call(c, kv, lo, hi, status, act, f, f, nullptr);
-      gd.add(lw.w_down, nullptr, nullptr, h, d, d, GEMV_RESID_F32);
-      if ((s = run_gemv(gd, CC_KERNEL_GEMM_DOWN, dev->sms, st)) != CC_OK) return s;
-      continue;
-    }
-    Gemm go;
-    if ((s = gemm_setup(go, EPI_RESID_F32, o, qd, lw.wo, nullptr, d, batch, cap, hi, status,
-                        false, used)) != CC_OK)
-      return s;
-    go.p.row_lo = lo;
-    go.p.out = h;
-    go.p.ldo = d;
-    // the post-attention RMSNorm fused across the O and gate/up epilogues
-    // (as in the scoring pass)
-    float *ss_part = reinterpret_cast<float *>(wsb + L.s.sspart);
-    go.p.norm_out = reinterpret_cast<__nv_bfloat16 *>(xn);
-    go.p.norm_gain = reinterpret_cast<const __nv_bfloat16 *>(lw.mlp_norm);
-    go.p.ld_norm = d;
-    go.p.ss_part = ss_part;
-    if ((s = run_gemm(go, EPI_RESID_F32, CC_KERNEL_GEMM_OPROJ, dev->sms, st)) != CC_OK) return s;
+    // h += o Wo^T; act = SwiGLU(RMSNorm(h)); h += act Wd^T
+    if ((s = resid(o, qd, lw.wo, lw.mlp_norm, CC_KERNEL_GEMM_OPROJ)) != CC_OK) return s;
     Gemm gu;
-    if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, batch, cap, hi, status,
-                        false, used)) != CC_OK)
+    if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, 1, max_rows, total, status)) !=
+        CC_OK)
       return s;
-    gu.p.row_lo = lo;
+    scaled(gu);
     gu.p.out = act;
     gu.p.ldo = f;
-    gu.p.row_ss = ss_part;
-    gu.p.n_ss = go.p.n_tiles;
-    gu.p.ss_d = d;
-    gu.p.eps = c->rms_eps;
     if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
-    Gemm gd;
-    if ((s = gemm_setup(gd, EPI_RESID_F32, act, f, lw.w_down, nullptr, d, batch, cap, hi, status,
-                        false, used)) != CC_OK)
-      return s;
-    gd.p.row_lo = lo;
-    gd.p.out = h;
-    gd.p.ldo = d;
-    if ((s = run_gemm(gd, EPI_RESID_F32, CC_KERNEL_GEMM_DOWN, dev->sms, st)) != CC_OK) return s;
+    const void *next_gain = l + 1 < c->n_layers ? w->layers[l + 1].attn_norm : final_gain;
+    if ((s = resid(act, f, lw.w_down, next_gain, CC_KERNEL_GEMM_DOWN)) != CC_OK) return s;
+  }
+  if (final_gain) {
+    *ss_tiles_out = ss_tiles;
+    return CC_OK;
   }
   {
     TimedScope t(CC_KERNEL_APPEND, st);
-    CC_TRY(launch_append_finish(kv->seq_len, hi, batch, st));
+    CC_TRY(launch_append_finish(kv->seq_len, rows.hi, batch, st));
   }
   return CC_OK;
 }
@@ -1039,7 +947,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     if (ss_tiles == 0) {
       TimedScope t(CC_KERNEL_RMSNORM, st);
       CC_TRY(launch_rmsnorm(first_from_bf16 ? kv->h_last : (const void *)h, !first_from_bf16,
-                            lw.attn_norm, xn, d, c->rms_eps, sl, cap, rows, split, st, rng_lo, 0,
+                            lw.attn_norm, xn, d, c->rms_eps, sl, cap, rows, split, st, rng_lo,
                             f16, status));
     }
     // Q = RoPE(xn Wq^T)
@@ -1377,17 +1285,14 @@ cc_status cc_score_h2o(const cc_kv_cache *kv, int32_t recent, float *scores, voi
 }
 
 // ---- decode step (greedy): append one token each, LM head, argmax -------------
-constexpr int kDecodeMinParts = 1024;   // argmax pairs per sequence the workspace holds at least
-
 size_t decode_part_offset(const cc_model_cfg *c, int batch, int cap) {
   return align256(append_layout(c, batch, cap).total);
 }
 
 size_t cc_decode_workspace_size(const cc_model_cfg *cfg, int32_t batch, int32_t cap) {
   if (check_cfg(cfg) != CC_OK || batch < 1 || cap < 1) return 0;
-  // (max, column) pairs per sequence: one per LM-head column tile of either
-  // width, or one per CTA of the weight-streaming LM head
-  const size_t n_tiles = std::max<size_t>(((size_t)cfg->vocab + 127) / 128, kDecodeMinParts);
+  // (max, column) pairs per sequence: one per LM-head column tile of either width
+  const size_t n_tiles = ((size_t)cfg->vocab + 127) / 128;
   return decode_part_offset(cfg, batch, cap) + align256((size_t)batch * n_tiles * 8);
 }
 
@@ -1400,7 +1305,9 @@ cc_status cc_decode_step(const cc_model_cfg *cfg, const cc_model_weights *w,
   if (!aligned16(w->final_norm) || !aligned16(w->lm_head)) return CC_ERR_INVALID_ARG;
   if (!ws || ws_bytes < cc_decode_workspace_size(cfg, cache->batch, cache->cap))
     return CC_ERR_WORKSPACE;
-  cc_status s = run_append(cfg, w, cache, tokens_in, nullptr, nullptr, 1, ws, ws_bytes, stream);
+  int ss_tiles = 0;
+  cc_status s = run_append(cfg, w, cache, tokens_in, nullptr, nullptr, 1, ws, ws_bytes, stream,
+                           w->final_norm, &ss_tiles);
   if (s != CC_OK) return s;
   DevState *dev;
   if (!dev_state(&dev)) return device_fail();
@@ -1408,37 +1315,22 @@ cc_status cc_decode_step(const cc_model_cfg *cfg, const cc_model_weights *w,
   const int batch = cache->batch, cap = cache->cap, d = cfg->d_model;
   const AppendWs L = append_layout(cfg, batch, cap);
   uint8_t *wsb = reinterpret_cast<uint8_t *>(ws);
-  void *xn = wsb + L.s.xn;
-  float *h = reinterpret_cast<float *>(wsb + L.s.h);
-  int32_t *lo = reinterpret_cast<int32_t *>(wsb + L.lo), *hi = reinterpret_cast<int32_t *>(wsb + L.hi);
+  const AppendRows rows = append_rows(L, wsb);
   float2 *part = reinterpret_cast<float2 *>(wsb + decode_part_offset(cfg, batch, cap));
-  if (gemv_decode_ok(cfg, batch, 1) && dev->sms <= kDecodeMinParts) {
-    // final norm fused; one (max, first column) pair per CTA
-    GemvCall g = gemv_call(cfg, cache, lo, hi, dev->status, h, d, d, w->final_norm);
-    g.add(w->lm_head, nullptr, nullptr, nullptr, 0, cfg->vocab, GEMV_ARGMAX);
-    g.l.p.part = part;
-    if ((s = run_gemv(g, CC_KERNEL_GEMM_LMHEAD, dev->sms, st)) != CC_OK) return s;
-    TimedScope t(CC_KERNEL_APPEND, st);
-    CC_TRY(launch_argmax_combine(part, g.l.p.part_ld, lo, hi, batch, next_tokens, next_logit, st));
-    return CC_OK;
-  }
-  {
-    TimedScope t(CC_KERNEL_RMSNORM, st);
-    CC_TRY(launch_rmsnorm(h, true, w->final_norm, xn, d, cfg->rms_eps, hi, cap, batch * cap, false,
-                          st, lo, 1));
-  }
   Gemm g;
-  if ((s = gemm_setup(g, EPI_ARGMAX, xn, d, w->lm_head, nullptr, cfg->vocab, batch, cap, hi,
-                      dev->status, false, (uint64_t)batch)) != CC_OK)
+  if ((s = gemm_setup(g, EPI_ARGMAX, wsb + L.s.xn, d, w->lm_head, nullptr, cfg->vocab, 1, batch,
+                      rows.total, dev->status)) != CC_OK)
     return s;
-  g.p.row_lo = lo;
+  g.p.row_ss = reinterpret_cast<float *>(wsb + L.s.sspart);   // the final norm
+  g.p.n_ss = ss_tiles;
+  g.p.ss_d = d;
+  g.p.eps = cfg->rms_eps;
   g.p.out = part;
   g.p.ldo = g.p.n_tiles;
   if ((s = run_gemm(g, EPI_ARGMAX, CC_KERNEL_GEMM_LMHEAD, dev->sms, st)) != CC_OK) return s;
-  {
-    TimedScope t(CC_KERNEL_APPEND, st);
-    CC_TRY(launch_argmax_combine(part, g.p.n_tiles, lo, hi, batch, next_tokens, next_logit, st));
-  }
+  TimedScope t(CC_KERNEL_APPEND, st);
+  CC_TRY(launch_argmax_combine(part, g.p.n_tiles, rows, batch, cache->seq_len, next_tokens,
+                               next_logit, st));
   return CC_OK;
 }
 

@@ -113,6 +113,7 @@ CC_DEV uint32_t e4m3x2_to_f16x2(uint32_t two) {
 // the sequence end.
 struct UnitInfo {
   int b, g, n, q_lo, p0, p_last;
+  int row0;   // workspace row of slot 0 (query and output rows)
   bool bad, valid;
 };
 CC_DEV UnitInfo decode_unit(const AttnParams &p, int unit_id, bool causal) {
@@ -133,6 +134,7 @@ CC_DEV UnitInfo decode_unit(const AttnParams &p, int unit_id, bool causal) {
   // query rows end: the sequence end, or a counter-causal row range's end
   const int q_hi = (!causal && p.row_hi) ? p.row_hi[u.b] : u.n;
   u.bad = u.n < 0 || u.n > p.cap || u.q_lo < 0 || u.q_lo > q_hi || q_hi > u.n;
+  u.row0 = p.pbase ? p.pbase[u.b] - u.q_lo : u.b * p.cap;
   u.p0 = u.q_lo + pb * p.P;
   u.valid = !u.bad && u.p0 < q_hi;
   u.p_last = min(u.p0 + p.P, q_hi) - 1;
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int t0 = CAUSAL ? 0 : (p0 + 1) / BKV;
   const int t1 = CAUSAL ? p_last / BKV : (n - 1) / BKV;
   const int ntiles_unit = t1 - t0 + 1;
-  const size_t row_base = (size_t)b * p.cap;
+  const long long row_base = u.row0;
   // this CTA's share of the unit's key tiles (all of them without splits):
   // local iteration `it` handles tile t_hi - it; the tail tile is t_top
   const int t_top = t1;
@@ -554,7 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool store = row_used && pos <= p_last;
       const float inv = l > 0.f ? p.v_scale / l : 0.f;   // V scale: e4m3 cache (else 1)
       __nv_bfloat16 *dst =
-          p.out + (row_base + (store ? pos : 0)) * p.out_ld + (size_t)(g * G + hl) * DH;
+          p.out + (row_base + (store ? pos : p0)) * p.out_ld + (size_t)(g * G + hl) * DH;
 #pragma unroll 1
       for (int c = 0; c < DH; c += 32) {
         uint32_t o[32];
@@ -647,7 +649,7 @@ __global__ void attn_combine_kernel(const __grid_constant__ AttnParams p) {
   }
   for (; s < S; ++s) o += wgt[s] * p.part_o[(base + (size_t)s * 256) * p.head_dim + d];
   const float v = l > 0.f ? o * p.v_scale / l : 0.f;
-  __nv_bfloat16 *dst = p.out + ((size_t)u.b * p.cap + pos) * p.out_ld +
+  __nv_bfloat16 *dst = p.out + (size_t)(u.row0 + pos) * p.out_ld +
                        (size_t)(u.g * G + hl) * p.head_dim + d;
   if (p.f16) {   // fp16 operand mode: O as fp16 (the same 2 bytes)
     const __half hf = __float2half_rn(v);
@@ -794,7 +796,7 @@ __global__ void __launch_bounds__(kDecThreads) attn_decode_kernel(const __grid_c
   float *sbuf = reinterpret_cast<float *>(smem + L::OFF_S);
   float *pbuf = reinterpret_cast<float *>(smem + L::OFF_P);
   float *fbuf = reinterpret_cast<float *>(smem + L::OFF_F);
-  const size_t row_base = (size_t)u.b * p.cap;
+  const long long row_base = u.row0;
   const int Hkv = p.n_kv_heads;
 
   const uint8_t *kg = reinterpret_cast<const uint8_t *>(p.k);
@@ -837,7 +839,7 @@ __global__ void __launch_bounds__(kDecThreads) attn_decode_kernel(const __grid_c
   for (int i = tid; i < G * DH; i += kDecThreads) {
     const int h = i / DH, d = i - h * DH;
     qs[i] = __bfloat162float(
-        p.q[(row_base + pos) * (size_t)p.n_q_heads * DH + (size_t)(u.g * G + h) * DH + d]);
+        p.q[(size_t)(row_base + pos) * p.n_q_heads * DH + (size_t)(u.g * G + h) * DH + d]);
   }
 
   constexpr int DPT = DH / 32;   // P V: warp h < G owns head h, lane the dims lane*DPT..

@@ -25,6 +25,9 @@ struct AttnParams {
   const int32_t *row_hi;    // counter-causal: null (rows up to seq_len) or device [batch]:
                             // only rows [row_lo, row_hi) are computed, each still attending
                             // every later slot up to seq_len (cc_score_rows)
+  const int32_t *pbase;     // causal: null (query and output rows b * cap + slot) or device
+                            // [batch]: packed rows, slot i of sequence b at row
+                            // pbase[b] + i - row_lo[b]
   int q_span;               // query slots per sequence at most (cap, or the chunk size)
   int kv_splits;            // > 1: each unit's key tiles split over kv_splits CTAs (few units)
   float *part_o;            // kv_splits > 1: [unit][split][256 rows][head_dim] unnormalised O

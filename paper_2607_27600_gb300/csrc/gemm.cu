@@ -57,16 +57,17 @@ static_assert(smem_bytes(false) <= 232448 && smem_bytes(true) <= 232448, "shared
 // bias (optional) is added before the rotation.
 // F8: the destination is an e4m3 cache (one byte per element, the value
 // times qscale = 1 / the layer's scale; pack_e4m3x2).
-// orow: the output row (grow, or the cache row of a paged K destination; < 0: skip)
+// slot: the row's cache slot (its position); orow: the output row (the
+// workspace row, or the cache row of a paged K destination; < 0: skip)
 // Address of output column c of row `orow` (element size EB), or with a
-// head-major cache destination (hm) of head c / head_dim's vector of slot
-// grow % cap (32-column chunks never straddle two heads).
+// head-major cache destination (hm) of head c / head_dim's vector of cache slot
+// `slot` (b * kv_cap + i; 32-column chunks never straddle two heads).
 template <int EB>
 CC_DEV uint8_t *out_at(const GemmParams &p, uint8_t *base, long long orow, int ldo, bool hm,
-                       int grow, int c) {
+                       int slot, int c) {
   if (hm) {
-    const int b = grow / p.cap, i = grow - b * p.cap;
-    return base + ((((size_t)b * p.pg.hkv + c / p.head_dim) * p.cap + i) * p.head_dim +
+    const int b = slot / p.kv_cap, i = slot - b * p.kv_cap;
+    return base + ((((size_t)b * p.pg.hkv + c / p.head_dim) * p.kv_cap + i) * p.head_dim +
                    c % p.head_dim) * EB;
   }
   return base + ((size_t)orow * ldo + c) * EB;
@@ -88,12 +89,12 @@ CC_DEV float row_rms_scale(const GemmParams &p, int grow, bool valid) {
 // rs: scale of the accumulator (before the bias and the rotation).  With
 // p.out_f16 (not F8, lo_off 0) the values are written as fp16.
 template <int TBN, bool F8 = false>
-CC_DEV void rope_store(const GemmParams &p, uint32_t tacc, int grow, long long orow, bool valid,
+CC_DEV void rope_store(const GemmParams &p, uint32_t tacc, int slot, long long orow, bool valid,
                        void *out_base, int ldo, const __nv_bfloat16 *bias, int col0, int n_dest,
                        float qscale = 1.f, bool hm = false, int lo_off = 0, float rs = 1.f) {
   const int half = p.head_dim >> 1;
   valid = valid && orow >= 0;
-  const uint32_t pos = valid ? (uint32_t)p.pos[grow] : 0u;
+  const uint32_t pos = valid ? (uint32_t)p.pos[slot] : 0u;
   uint8_t *base = reinterpret_cast<uint8_t *>(out_base);
 #pragma unroll 1
   for (int hb = 0; hb < TBN; hb += p.head_dim) {
@@ -152,8 +153,8 @@ CC_DEV void rope_store(const GemmParams &p, uint32_t tacc, int grow, long long o
       if constexpr (!F8)
         if (over) set_status(p.status, CC_ERR_RANGE);
       constexpr int EB = F8 ? 1 : 2;
-      uint4 *d1 = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, grow, col));
-      uint4 *d2 = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, grow, col + half));
+      uint4 *d1 = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, slot, col));
+      uint4 *d2 = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, slot, col + half));
 #pragma unroll
       for (int v = 0; v < 2 * EB; ++v) {   // 32 elements: 64 bytes bf16, 32 e4m3
         d1[v] = make_uint4(o1[v * 4], o1[v * 4 + 1], o1[v * 4 + 2], o1[v * 4 + 3]);
@@ -161,9 +162,9 @@ CC_DEV void rope_store(const GemmParams &p, uint32_t tacc, int grow, long long o
       }
       if constexpr (!F8) {
         if (lo_off > 0) {
-          uint4 *e1 = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, grow, col + lo_off));
+          uint4 *e1 = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, slot, col + lo_off));
           uint4 *e2 = reinterpret_cast<uint4 *>(
-              out_at<EB>(p, base, orow, ldo, hm, grow, col + half + lo_off));
+              out_at<EB>(p, base, orow, ldo, hm, slot, col + half + lo_off));
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             e1[v] = make_uint4(l1[v * 4], l1[v * 4 + 1], l1[v * 4 + 2], l1[v * 4 + 3]);
@@ -178,9 +179,9 @@ CC_DEV void rope_store(const GemmParams &p, uint32_t tacc, int grow, long long o
 // Plain bf16 store (+ optional bias) of one accumulator tile row; F8: e4m3
 // codes of (value + bias) * qscale instead.
 template <int TBN, bool F8 = false>
-CC_DEV void plain_store(const GemmParams &p, uint32_t tacc, int grow, long long orow, bool valid,
+CC_DEV void plain_store(const GemmParams &p, uint32_t tacc, int slot, long long orow, bool valid,
                         void *out_base, int ldo, const __nv_bfloat16 *bias, int col0, int n_dest,
-                        float qscale = 1.f, bool hm = false) {
+                        float qscale = 1.f, bool hm = false, float rs = 1.f) {
   constexpr int EB = F8 ? 1 : 2;
   valid = valid && orow >= 0;
   uint8_t *base = reinterpret_cast<uint8_t *>(out_base);
@@ -200,8 +201,8 @@ CC_DEV void plain_store(const GemmParams &p, uint32_t tacc, int grow, long long 
     uint32_t o[16];
 #pragma unroll
     for (int k = 0; k < 32; k += 2) {
-      const float y0 = __uint_as_float(r[k]) + bf16_lo(bb[k / 2]);
-      const float y1 = __uint_as_float(r[k + 1]) + bf16_hi(bb[k / 2]);
+      const float y0 = fmaf(__uint_as_float(r[k]), rs, bf16_lo(bb[k / 2]));
+      const float y1 = fmaf(__uint_as_float(r[k + 1]), rs, bf16_hi(bb[k / 2]));
       if constexpr (F8) {
         const uint32_t e = pack_e4m3x2(y0 * qscale, y1 * qscale);
         if ((k & 2) == 0) o[k / 4] = e;
@@ -210,19 +211,25 @@ CC_DEV void plain_store(const GemmParams &p, uint32_t tacc, int grow, long long 
         o[k / 2] = pack_bf16x2(y0, y1);
       }
     }
-    uint4 *d = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, grow, col));
+    uint4 *d = reinterpret_cast<uint4 *>(out_at<EB>(p, base, orow, ldo, hm, slot, col));
 #pragma unroll
     for (int v = 0; v < 2 * EB; ++v)   // 32 elements: 64 bytes bf16, 32 e4m3
       d[v] = make_uint4(o[v * 4], o[v * 4 + 1], o[v * 4 + 2], o[v * 4 + 3]);
   }
 }
 
-// Cache row of workspace row grow = b * cap + i (paged: through the block
-// table); a bad page is reported and the row skipped (-1).
-CC_DEV long long cache_row(const GemmParams &p, int grow, bool valid) {
-  const int b = grow / p.cap;
-  const long long r = kv_row(p.pg, p.cap, b, grow - b * p.cap);
-  if (r < 0 && valid) set_status(p.status, CC_ERR_DEVICE_ARG);
+// Cache slot b * kv_cap + i of workspace row grow (packed rows: through
+// rowmap; -1: no row).
+CC_DEV int cache_slot(const GemmParams &p, int grow, bool valid) {
+  return valid && p.rowmap ? p.rowmap[grow] : grow;
+}
+// Cache row of a cache slot (paged: through the block table); a bad page is
+// reported and the row skipped (-1).
+CC_DEV long long cache_row(const GemmParams &p, int slot, bool valid) {
+  if (!valid) return -1;
+  const int b = slot / p.kv_cap;
+  const long long r = kv_row(p.pg, p.kv_cap, b, slot - b * p.kv_cap);
+  if (r < 0) set_status(p.status, CC_ERR_DEVICE_ARG);
   return r;
 }
 
@@ -400,42 +407,49 @@ CC_DEV void epilogue_tile(const GemmParams &p, uint32_t tacc, int grow, bool val
     logit_partials<TBN>(p, tacc, grow, valid, nt, tile_n0, stage);
   } else if constexpr (EPI == EPI_F32 || EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32) {
     f32_epilogue<EPI, TBN>(p, tacc, grow, valid, nt, tile_n0, stage);
-  } else if constexpr (EPI == EPI_QROPE) {   // kv_fp8: the K rows of an e4m3 cache
-    const long long orow = p.kv_dest ? cache_row(p, grow, valid) : grow;
-    const bool hm = p.kv_dest && p.pg.head_major;
-    if (p.kv_fp8)
-      rope_store<TBN, true>(p, tacc, grow, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N,
-                            p.k_qscale, hm);
-    else   // with row_ss: the query projection of unnormalised rows (x * gain)
-      rope_store<TBN>(p, tacc, grow, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N, 1.f, hm,
-                      p.out_split ? p.N : 0, row_rms_scale(p, grow, valid));
-  } else if constexpr (EPI == EPI_BF16) {    // kv_fp8: the V rows of an e4m3 cache
-    const long long orow = p.kv_dest ? cache_row(p, grow, valid) : grow;
-    const bool hm = p.kv_dest && p.pg.head_major;
-    if (p.kv_fp8)
-      plain_store<TBN, true>(p, tacc, grow, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N,
-                             p.v_qscale, hm);
-    else
-      plain_store<TBN>(p, tacc, grow, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N, 1.f, hm);
-  } else if constexpr (EPI == EPI_QKV) {
-    // fused projections: column tiles [0, nq) are Q, [nq, nq+nk) K, the rest V (cache rows)
-    const int nq = p.n_q_tiles, nk = p.n_k_tiles;
-    const long long crow = nt < nq ? grow : cache_row(p, grow, valid);
-    const bool hm = p.pg.head_major != 0;   // the K and V parts
-    if (nt < nq)
-      rope_store<TBN>(p, tacc, grow, grow, valid, p.out, p.ldo, p.bias, nt * TBN, nq * TBN);
-    else if (nt < nq + nk && p.kv_fp8)
-      rope_store<TBN, true>(p, tacc, grow, crow, valid, p.out_k, p.ldo_kv, p.bias_k,
-                            (nt - nq) * TBN, nk * TBN, p.k_qscale, hm);
-    else if (nt < nq + nk)
-      rope_store<TBN>(p, tacc, grow, crow, valid, p.out_k, p.ldo_kv, p.bias_k, (nt - nq) * TBN,
-                      nk * TBN, 1.f, hm);
-    else if (p.kv_fp8)
-      plain_store<TBN, true>(p, tacc, grow, crow, valid, p.out_v, p.ldo_kv, p.bias_v,
-                             (nt - nq - nk) * TBN, nk * TBN, p.v_qscale, hm);
-    else
-      plain_store<TBN>(p, tacc, grow, crow, valid, p.out_v, p.ldo_kv, p.bias_v,
-                       (nt - nq - nk) * TBN, nk * TBN, 1.f, hm);
+  } else if constexpr (EPI == EPI_QROPE || EPI == EPI_BF16 || EPI == EPI_QKV) {
+    const int slot = cache_slot(p, grow, valid);
+    valid = valid && slot >= 0;
+    // with row_ss: projections of unnormalised rows (x * gain)
+    const float rs = row_rms_scale(p, grow, valid);
+    if constexpr (EPI == EPI_QROPE) {   // kv_fp8: the K rows of an e4m3 cache
+      const long long orow = p.kv_dest ? cache_row(p, slot, valid) : grow;
+      const bool hm = p.kv_dest && p.pg.head_major;
+      if (p.kv_fp8)
+        rope_store<TBN, true>(p, tacc, slot, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N,
+                              p.k_qscale, hm, 0, rs);
+      else
+        rope_store<TBN>(p, tacc, slot, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N, 1.f, hm,
+                        p.out_split ? p.N : 0, rs);
+    } else if constexpr (EPI == EPI_BF16) {    // kv_fp8: the V rows of an e4m3 cache
+      const long long orow = p.kv_dest ? cache_row(p, slot, valid) : grow;
+      const bool hm = p.kv_dest && p.pg.head_major;
+      if (p.kv_fp8)
+        plain_store<TBN, true>(p, tacc, slot, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N,
+                               p.v_qscale, hm, rs);
+      else
+        plain_store<TBN>(p, tacc, slot, orow, valid, p.out, p.ldo, p.bias, tile_n0, p.N, 1.f, hm, rs);
+    } else {
+      // fused projections: column tiles [0, nq) are Q, [nq, nq+nk) K, the rest V (cache rows)
+      const int nq = p.n_q_tiles, nk = p.n_k_tiles;
+      const long long crow = nt < nq ? grow : cache_row(p, slot, valid);
+      const bool hm = p.pg.head_major != 0;   // the K and V parts
+      if (nt < nq)
+        rope_store<TBN>(p, tacc, slot, grow, valid, p.out, p.ldo, p.bias, nt * TBN, nq * TBN, 1.f,
+                        false, 0, rs);
+      else if (nt < nq + nk && p.kv_fp8)
+        rope_store<TBN, true>(p, tacc, slot, crow, valid, p.out_k, p.ldo_kv, p.bias_k,
+                              (nt - nq) * TBN, nk * TBN, p.k_qscale, hm, 0, rs);
+      else if (nt < nq + nk)
+        rope_store<TBN>(p, tacc, slot, crow, valid, p.out_k, p.ldo_kv, p.bias_k, (nt - nq) * TBN,
+                        nk * TBN, 1.f, hm, 0, rs);
+      else if (p.kv_fp8)
+        plain_store<TBN, true>(p, tacc, slot, crow, valid, p.out_v, p.ldo_kv, p.bias_v,
+                               (nt - nq - nk) * TBN, nk * TBN, p.v_qscale, hm, rs);
+      else
+        plain_store<TBN>(p, tacc, slot, crow, valid, p.out_v, p.ldo_kv, p.bias_v,
+                         (nt - nq - nk) * TBN, nk * TBN, 1.f, hm, rs);
+    }
   } else if constexpr (EPI == EPI_SWIGLU) {
     // columns [0,128) = gate rows nt*128.., [128,256) = up rows nt*128..
     __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(p.out) + (size_t)grow * p.ldo;
@@ -526,8 +540,8 @@ CC_DEV void epilogue_tile(const GemmParams &p, uint32_t tacc, int grow, bool val
       }
     }
     if (valid)
-      reinterpret_cast<float2 *>(p.out)[(size_t)(grow / p.cap) * p.ldo + nt] =
-          make_float2(m, __int_as_float(mi));
+      reinterpret_cast<float2 *>(p.out)[(size_t)grow * p.ldo + nt] =
+          make_float2(m * row_rms_scale(p, grow, valid), __int_as_float(mi));
   }
 }
 

@@ -32,28 +32,12 @@ CC_DEV bool in_score_range(const int32_t *rng_lo, const int32_t *rng_hi, int cap
   return i >= rng_lo[b] && i < rng_hi[b];
 }
 
-// Row ranges of the inference cycle: slots [row_lo[b], seq_len[b]) (row_lo
-// may be null: from slot 0).
+// Rows of the scoring pass: slots [row_lo[b], seq_len[b]) (row_lo may be null:
+// from slot 0).
 CC_DEV bool row_in_range(const int32_t *seq_len, const int32_t *row_lo, int cap, int row) {
   int i, n;
   if (!row_valid(seq_len, cap, row, i, n)) return false;
   return !row_lo || i >= row_lo[row / cap];
-}
-
-// Warp w -> its cache row.  With a span (and row_lo), warps cover only the
-// chunk rows: warp w takes slot row_lo[b] + k of sequence b = w / span,
-// k = w % span; otherwise warp w takes row w of the whole cache.
-CC_DEV bool warp_row(const int32_t *seq_len, const int32_t *row_lo, int cap, int rows, int span,
-                     int w, int &row) {
-  if (span > 0 && row_lo) {
-    const int b = w / span;
-    if (b >= rows / cap) return false;
-    const int i = row_lo[b] + (w - b * span), n = seq_len[b];
-    row = b * cap + i;
-    return i >= 0 && i < n && n <= cap;
-  }
-  row = w;
-  return row < rows && row_in_range(seq_len, row_lo, cap, row);
 }
 
 // 8 bf16 of a uint4 -> float
@@ -132,12 +116,11 @@ CC_DEV void store_norm8(__nv_bfloat16 *o, int d, int e, const float *f, const ui
 template <bool IN_F32>
 __global__ void __launch_bounds__(kWarps * 32)
     rmsnorm_kernel(const void *x, const __nv_bfloat16 *gain, __nv_bfloat16 *out, int d, float eps,
-                   const int32_t *seq_len, const int32_t *row_lo, int cap, int rows, int span,
-                   int split, int f16, unsigned *status) {
+                   const int32_t *seq_len, const int32_t *row_lo, int cap, int rows, int split,
+                   int f16, unsigned *status) {
   const int lane = threadIdx.x & 31;
-  int row;
-  if (!warp_row(seq_len, row_lo, cap, rows, span, blockIdx.x * kWarps + (threadIdx.x >> 5), row))
-    return;
+  const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (row >= rows || !row_in_range(seq_len, row_lo, cap, row)) return;
   const size_t es = IN_F32 ? 4 : 2;
   const void *xr = reinterpret_cast<const uint8_t *>(x) + (size_t)row * d * es;
   const float inv = row_inv_rms<IN_F32>(xr, d, eps, lane);
@@ -166,12 +149,11 @@ __global__ void __launch_bounds__(kWarps * 32)
 // h (fp32) = embed[tokens[row]]
 __global__ void __launch_bounds__(kWarps * 32)
     embed_kernel(const __nv_bfloat16 *embed, const int32_t *tokens, float *h, int d, int vocab,
-                 const int32_t *seq_len, const int32_t *row_lo, int cap, int rows, int span,
+                 const int32_t *seq_len, const int32_t *row_lo, int cap, int rows,
                  unsigned *status) {
   const int lane = threadIdx.x & 31;
-  int row;
-  if (!warp_row(seq_len, row_lo, cap, rows, span, blockIdx.x * kWarps + (threadIdx.x >> 5), row))
-    return;
+  const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (row >= rows || !row_in_range(seq_len, row_lo, cap, row)) return;
   int tok = tokens[row];
   if (tok < 0 || tok >= vocab) {
     if (lane == 0) set_status(status, CC_ERR_DEVICE_ARG);
@@ -187,17 +169,59 @@ __global__ void __launch_bounds__(kWarps * 32)
   }
 }
 
-// out bf16 [row] = h fp32 [row] for the rows in range (H^(L-1) recorded by
-// the inference cycle).
+// The inference cycle's embedding with the first layer's RMSNorm begun, over
+// its packed rows r < *total (one block each): h (fp32) = e, xn (bf16) = e * gain
+// (unnormalised) and ss[r] = sum e^2, where e = embed[token of slot rowmap[r]].
+__global__ void __launch_bounds__(256)
+    append_embed_kernel(const __nv_bfloat16 *embed, const int32_t *tokens, const int32_t *rowmap,
+                        const int32_t *total, const __nv_bfloat16 *gain, float *h,
+                        __nv_bfloat16 *xn, float *ss, int d, int vocab, unsigned *status) {
+  __shared__ float part[8];
+  const int row = blockIdx.x;
+  if (row >= *total) return;
+  int tok = tokens[rowmap[row]];
+  if (tok < 0 || tok >= vocab) {
+    if (threadIdx.x == 0) set_status(status, CC_ERR_DEVICE_ARG);
+    tok = 0;
+  }
+  const __nv_bfloat16 *src = embed + (size_t)tok * d;
+  float acc = 0.f;
+  for (int e = threadIdx.x * 8; e < d; e += 256 * 8) {
+    float f[8], g[8];
+    unpack8(*reinterpret_cast<const uint4 *>(src + e), f);
+    unpack8(*reinterpret_cast<const uint4 *>(gain + e), g);
+    float4 *dst = reinterpret_cast<float4 *>(h + (size_t)row * d + e);
+    dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+    dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+    uint4 v;
+    v.x = pack_bf16x2(f[0] * g[0], f[1] * g[1]);
+    v.y = pack_bf16x2(f[2] * g[2], f[3] * g[3]);
+    v.z = pack_bf16x2(f[4] * g[4], f[5] * g[5]);
+    v.w = pack_bf16x2(f[6] * g[6], f[7] * g[7]);
+    *reinterpret_cast<uint4 *>(xn + (size_t)row * d + e) = v;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc = fmaf(f[k], f[k], acc);
+  }
+  acc = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float t = 0.f;
+    for (int w = 0; w < 8; ++w) t += part[w];
+    ss[row] = t;
+  }
+}
+
+// out bf16 [slot rowmap[r]] = h fp32 [packed row r] for r < *total (H^(L-1)
+// recorded by the inference cycle).
 __global__ void __launch_bounds__(kWarps * 32)
-    store_bf16_kernel(const float *h, __nv_bfloat16 *out, int d, const int32_t *seq_len,
-                      const int32_t *row_lo, int cap, int rows, int span) {
+    store_bf16_kernel(const float *h, __nv_bfloat16 *out, int d, const int32_t *rowmap,
+                      const int32_t *total) {
   const int lane = threadIdx.x & 31;
-  int row;
-  if (!warp_row(seq_len, row_lo, cap, rows, span, blockIdx.x * kWarps + (threadIdx.x >> 5), row))
-    return;
+  const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (row >= *total) return;
   const float *src = h + (size_t)row * d;
-  __nv_bfloat16 *dst = out + (size_t)row * d;
+  __nv_bfloat16 *dst = out + (size_t)rowmap[row] * d;
   for (int e = lane * 8; e < d; e += 256) {
     float f[8];
     load8<true>(src, e, f);
@@ -214,28 +238,47 @@ __global__ void __launch_bounds__(kWarps * 32)
 // its seq_len[b] current ones: row_lo = seq_len, row_hi = seq_len + count;
 // the chunk's tokens and positions (given, or continuing after the last
 // cached position) are written into the cache.  A count outside
-// [0, max_count] or past cap is reported and appends nothing.
+// [0, max_count] or past cap is reported and appends nothing.  The pass's
+// workspace rows are the appended slots packed, sequence after sequence:
+// sequence b's from pbase[b] on, rowmap[r] = b * cap + slot, *total rows.
 __global__ void append_prepare_kernel(const int32_t *seq_len, const int32_t *count,
                                       const int32_t *tok_in, const int32_t *pos_in, int max_count,
-                                      int32_t *tokens, int32_t *pos, int32_t *row_lo,
-                                      int32_t *row_hi, int cap, unsigned *status) {
+                                      int32_t *tokens, int32_t *pos, AppendRows r, int cap,
+                                      unsigned *status) {
+  __shared__ int before[8];
   const int b = blockIdx.x;
+  auto appended = [&](int s) {   // slots sequence s appends; < 0: a bad count or length
+    const int lo = seq_len[s];
+    const int c = count ? count[s] : 1;   // no count array: one token each (a decode step)
+    return lo < 0 || lo > cap || c < 0 || c > max_count || lo + c > cap ? -1 : c;
+  };
+  int base = 0;   // slots the sequences before b append
+  for (int s = threadIdx.x; s < b; s += blockDim.x) base += max(appended(s), 0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xFFFFFFFFu, base, o);
+  if ((threadIdx.x & 31) == 0) before[threadIdx.x >> 5] = base;
+  __syncthreads();
+  base = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) base += before[w];
   const int lo = seq_len[b];
-  int c = count ? count[b] : 1;   // no count array: one token each (a decode step)
-  if (lo < 0 || lo > cap || c < 0 || c > max_count || lo + c > cap) {
+  int c = appended(b);
+  if (c < 0) {
     if (threadIdx.x == 0) set_status(status, CC_ERR_DEVICE_ARG);
     c = 0;   // nothing appended; seq_len is left as it was
   }
   if (threadIdx.x == 0) {
-    row_lo[b] = lo;
-    row_hi[b] = lo + c;
+    r.lo[b] = lo;
+    r.hi[b] = lo + c;
+    r.pbase[b] = base;
+    if (b == (int)gridDim.x - 1) *r.total = base + c;
   }
   if (c == 0) return;
-  const size_t base = (size_t)b * cap;
-  const int next = lo > 0 ? pos[base + lo - 1] + 1 : 0;
+  const size_t slot0 = (size_t)b * cap + lo;
+  const int next = lo > 0 ? pos[slot0 - 1] + 1 : 0;
   for (int i = threadIdx.x; i < c; i += blockDim.x) {
-    tokens[base + lo + i] = tok_in[(size_t)b * max_count + i];
-    pos[base + lo + i] = pos_in ? pos_in[(size_t)b * max_count + i] : next + i;
+    tokens[slot0 + i] = tok_in[(size_t)b * max_count + i];
+    pos[slot0 + i] = pos_in ? pos_in[(size_t)b * max_count + i] : next + i;
+    r.rowmap[base + i] = (int)(slot0 + i);
   }
 }
 
@@ -245,18 +288,17 @@ __global__ void append_finish_kernel(int32_t *seq_len, const int32_t *row_hi, in
 }
 
 // Greedy decoding: the next token of sequence b is the first column of the
-// largest logit over the column tiles' (max, column) pairs; -1 when the
-// sequence appended nothing (row_hi == row_lo).
-__global__ void argmax_combine_kernel(const float2 *part, int n_tiles, const int32_t *row_lo,
-                                      const int32_t *row_hi, int batch, int32_t *next,
-                                      float *best) {
+// largest logit over the column tiles' (max, column) pairs of its row; -1 when
+// the sequence appended nothing.  Also the step's end: seq_len = hi.
+__global__ void argmax_combine_kernel(const float2 *part, int n_tiles, AppendRows r,
+                                      int32_t *seq_len, int32_t *next, float *best) {
   const int b = blockIdx.x;
   const int lane = threadIdx.x;
   float m = -INFINITY;
   int mi = 0x7FFFFFFF;
-  if (row_hi[b] > row_lo[b]) {
+  if (r.hi[b] > r.lo[b]) {
     for (int t = lane; t < n_tiles; t += 32) {
-      const float2 v = part[(size_t)b * n_tiles + t];
+      const float2 v = part[(size_t)r.pbase[b] * n_tiles + t];
       const int idx = __float_as_int(v.y);
       if (idx >= 0 && (v.x > m || (v.x == m && idx < mi))) {
         m = v.x;
@@ -274,6 +316,7 @@ __global__ void argmax_combine_kernel(const float2 *part, int n_tiles, const int
     }
   }
   if (lane == 0) {
+    seq_len[b] = r.hi[b];
     next[b] = mi == 0x7FFFFFFF ? -1 : mi;
     if (best) best[b] = m;
   }
@@ -346,62 +389,67 @@ __global__ void __launch_bounds__(kWarps * 32)
 
 unsigned blocks_for(int rows) { return (unsigned)((rows + kWarps - 1) / kWarps); }
 
-// warps of a row launch: one per cache row, or batch * span with a span
-int warps_for(int rows, int cap, int span, const int32_t *row_lo) {
-  return span > 0 && row_lo ? rows / cap * span : rows;
-}
-
 }  // namespace
 
 cudaError_t launch_rmsnorm(const void *x, bool x_f32, const void *gain, void *out, int d, float eps,
                            const int32_t *seq_len, int cap, int rows, bool split, cudaStream_t st,
-                           const int32_t *row_lo, int span, bool f16, unsigned *status) {
+                           const int32_t *row_lo, bool f16, unsigned *status) {
   if (rows <= 0) return cudaSuccess;
   if (split && f16) return cudaErrorInvalidValue;
   auto *g = reinterpret_cast<const __nv_bfloat16 *>(gain);
   auto *o = reinterpret_cast<__nv_bfloat16 *>(out);
-  const unsigned blocks = blocks_for(warps_for(rows, cap, span, row_lo));
+  const unsigned blocks = blocks_for(rows);
   if (x_f32)
     rmsnorm_kernel<true><<<blocks, kWarps * 32, 0, st>>>(x, g, o, d, eps, seq_len, row_lo, cap, rows,
-                                                          span, split ? 1 : 0, f16 ? 1 : 0, status);
+                                                          split ? 1 : 0, f16 ? 1 : 0, status);
   else
     rmsnorm_kernel<false><<<blocks, kWarps * 32, 0, st>>>(x, g, o, d, eps, seq_len, row_lo, cap,
-                                                           rows, span, split ? 1 : 0, f16 ? 1 : 0,
+                                                           rows, split ? 1 : 0, f16 ? 1 : 0,
                                                            status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_embed(const void *embed, const int32_t *tokens, float *h, int d, int vocab,
                          const int32_t *seq_len, int cap, int rows, unsigned *status,
-                         cudaStream_t st, const int32_t *row_lo, int span) {
+                         cudaStream_t st, const int32_t *row_lo) {
   if (rows <= 0) return cudaSuccess;
-  embed_kernel<<<blocks_for(warps_for(rows, cap, span, row_lo)), kWarps * 32, 0, st>>>(
+  embed_kernel<<<blocks_for(rows), kWarps * 32, 0, st>>>(
       reinterpret_cast<const __nv_bfloat16 *>(embed), tokens, h, d, vocab, seq_len, row_lo, cap,
-      rows, span, status);
+      rows, status);
   return cudaGetLastError();
 }
 
-cudaError_t launch_store_bf16(const float *h, void *out, int d, const int32_t *seq_len,
-                              const int32_t *row_lo, int cap, int rows, cudaStream_t st, int span) {
-  if (rows <= 0) return cudaSuccess;
-  store_bf16_kernel<<<blocks_for(warps_for(rows, cap, span, row_lo)), kWarps * 32, 0, st>>>(
-      h, reinterpret_cast<__nv_bfloat16 *>(out), d, seq_len, row_lo, cap, rows, span);
+cudaError_t launch_append_embed(const void *embed, const int32_t *tokens, const AppendRows &r,
+                                int max_rows, const void *gain, float *h, void *xn, float *ss,
+                                int d, int vocab, unsigned *status, cudaStream_t st) {
+  if (max_rows <= 0) return cudaSuccess;
+  append_embed_kernel<<<max_rows, 256, 0, st>>>(
+      reinterpret_cast<const __nv_bfloat16 *>(embed), tokens, r.rowmap, r.total,
+      reinterpret_cast<const __nv_bfloat16 *>(gain), h, reinterpret_cast<__nv_bfloat16 *>(xn), ss,
+      d, vocab, status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_store_bf16(const float *h, void *out, int d, const AppendRows &r, int max_rows,
+                              cudaStream_t st) {
+  if (max_rows <= 0) return cudaSuccess;
+  store_bf16_kernel<<<blocks_for(max_rows), kWarps * 32, 0, st>>>(
+      h, reinterpret_cast<__nv_bfloat16 *>(out), d, r.rowmap, r.total);
   return cudaGetLastError();
 }
 
 cudaError_t launch_append_prepare(const int32_t *seq_len, const int32_t *count,
                                   const int32_t *tok_in, const int32_t *pos_in, int max_count,
-                                  int32_t *tokens, int32_t *pos, int32_t *row_lo, int32_t *row_hi,
-                                  int batch, int cap, unsigned *status, cudaStream_t st) {
+                                  int32_t *tokens, int32_t *pos, const AppendRows &r, int batch,
+                                  int cap, unsigned *status, cudaStream_t st) {
   append_prepare_kernel<<<batch, 256, 0, st>>>(seq_len, count, tok_in, pos_in, max_count, tokens,
-                                                pos, row_lo, row_hi, cap, status);
+                                                pos, r, cap, status);
   return cudaGetLastError();
 }
 
-cudaError_t launch_argmax_combine(const float2 *part, int n_tiles, const int32_t *row_lo,
-                                  const int32_t *row_hi, int batch, int32_t *next, float *best,
-                                  cudaStream_t st) {
-  argmax_combine_kernel<<<batch, 32, 0, st>>>(part, n_tiles, row_lo, row_hi, batch, next, best);
+cudaError_t launch_argmax_combine(const float2 *part, int n_tiles, const AppendRows &r, int batch,
+                                  int32_t *seq_len, int32_t *next, float *best, cudaStream_t st) {
+  argmax_combine_kernel<<<batch, 32, 0, st>>>(part, n_tiles, r, seq_len, next, best);
   return cudaGetLastError();
 }
 
