@@ -337,7 +337,7 @@ struct Gemm {
 // a_split: A rows are [hi | lo] (2K values) and the product is hi W^T + lo W^T.
 cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, const void *W2, int N,
                      int batch, int cap, const int32_t *seq_len, unsigned *status,
-                     bool a_split = false, int few_tiles = 0) {
+                     bool a_split = false, int few_tiles = 0, int row_pairs = 0) {
   const uint64_t R = (uint64_t)batch * cap;
   int bn = gemm_block_n(epi);
   // narrow problems (less than one wave of 256-column tiles) that stay on this
@@ -354,7 +354,7 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   if (narrowable && have_dev && pair_mode != 2 &&
       ((R + 127) / 128) * (uint64_t)((N + 255) / 256) < (uint64_t)dev_info->sms)
     bn = 128;
-  const bool pair = have_dev && epi != EPI_ARGMAX && (epi == EPI_SWIGLU || bn == 256) &&
+  const bool pair = have_dev && epi != EPI_ARGMAX && row_pairs == 0 && (epi == EPI_SWIGLU || bn == 256) &&
                     (pair_mode == 2 ||
                      (pair_mode == 1 && ((R + 127) / 128) * (uint64_t)((N + bn - 1) / bn) >=
                                             2 * (uint64_t)dev_info->sms));
@@ -364,13 +364,14 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   g.one_group = false;
   if (have_dev && !pair && !pairs_env && epi != EPI_F32 && epi != EPI_LSE) {
     g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
-                     batch, cap, dev_info->sms);
+                     batch, cap, row_pairs, dev_info->sms);
     g.one_group = batch == 1 && cap <= g.few.nb;
     bn = kFewTileCols;
   }
   const bool few = g.few.nb > 0;
   const uint32_t b_box = few || epi == EPI_SWIGLU || pair ? 128 : (uint32_t)bn;
-  if (!tmap_rows(&g.a, A, R, a_split ? 2 * K : K, few ? (uint32_t)g.few.nb : 128)) return tmap_fail();
+  // row pairs: lo rows row_pairs past the hi ones
+  if (!tmap_rows(&g.a, A, row_pairs ? 2 * (uint64_t)row_pairs : R, a_split ? 2 * K : K, few ? (uint32_t)g.few.nb : 128)) return tmap_fail();
   if (!tmap_rows(&g.b, W, N, K, b_box)) return tmap_fail();
   if (epi == EPI_SWIGLU) {
     if (!tmap_rows(&g.b2, W2, N, K, b_box)) return tmap_fail();
@@ -387,6 +388,7 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   g.p.block_n = epi == EPI_SWIGLU ? 256 : bn;
   g.p.n_tiles = few ? g.few.n_tiles : (N + bn - 1) / bn;
   g.p.kv_cap = cap;
+  g.p.row_pairs = few ? row_pairs : 0;
   g.p.status = status;
   g.p.a_split = a_split ? 1 : 0;
   // Tile order for L2 reuse: keep a slab of one operand resident (evict-last;
@@ -435,11 +437,11 @@ bool qkv_fusable(const cc_model_cfg *c) {
 
 cc_status gemm_setup_qkv(Gemm &g, const void *xn, const cc_model_cfg *c,
                          const cc_layer_weights &lw, int batch, int cap, const int32_t *seq_len,
-                         unsigned *status) {
+                         unsigned *status, int row_pairs) {
   const int d = c->d_model, qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
   const int fq = (qd + 127) / 128, fk = (kvd + 127) / 128;   // column tiles of a few-row launch
   cc_status s = gemm_setup(g, EPI_QKV, xn, d, lw.wq, nullptr, qd + 2 * kvd, batch, cap, seq_len,
-                           status, false, fq + 2 * fk);
+                           status, false, fq + 2 * fk, row_pairs);
   if (s != CC_OK) return s;
   const bool few = g.few.nb > 0;
   const uint32_t box = few || g.p.pair ? 128 : 256;   // a pair's CTAs load half a tile each
@@ -496,13 +498,15 @@ int attn_key_splits(long long units, int cap, int sms) {
   return s >= 2 ? (int)s : 1;
 }
 
-// Key splits of the decode attention (one query row per unit): up to one
-// CTA per SM in all, each split at least two chunks of 128 keys.
-int attn_decode_splits(long long units, int cap, int sms) {
-  const long long by_keys = std::max(1LL, ((long long)cap + 255) / 256);
-  const long long s = std::min({std::max(1LL, (long long)sms / units),
-                                std::max(1LL, (long long)kAttnMaxSplitSlots / units), by_keys});
-  return (int)s;
+// Key splits of a decode unit at most: 64 keys each, the partial rows within
+// their buffer, and a few times the CTAs that the even splits need (a longer
+// sequence than four times the average takes longer splits; CTAs past a
+// sequence's end only look up its length).
+int attn_decode_splits(long long units, int cap, int ctas) {
+  const long long by_keys = std::max(1LL, ((long long)cap + 63) / 64);
+  const long long by_rows = std::max(1LL, (long long)kAttnMaxSplitSlots * 256 / kDecMaxG / units);
+  const long long by_ctas = std::max(1LL, 4LL * ctas / units);
+  return (int)std::min({(long long)kDecMaxSplits, by_keys, by_rows, by_ctas});
 }
 
 // out: [R][Hq*dh] bf16, or with split [R][2*Hq*dh] = [hi | lo] per row.
@@ -517,7 +521,8 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
                         KvFmt kvf = KvFmt(), bool q_split = false,
                         const int32_t *range_lo = nullptr, const int32_t *range_hi = nullptr,
                         void *kv_scratch = nullptr, size_t kv_scratch_bytes = 0,
-                        bool f16 = false, const int32_t *pbase = nullptr, int packed_rows = 0) {
+                        bool f16 = false, const int32_t *pbase = nullptr, int packed_rows = 0,
+                        int row_pairs = 0) {
   const int G = c->n_q_heads / c->n_kv_heads, dh = c->head_dim;
   const int P = attn_positions_per_unit(G);
   const uint64_t R = (uint64_t)batch * cap;
@@ -525,10 +530,7 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
   // fp16 operands (q and out fp16): the counter-causal pass with single operands
   if (f16 && (row_lo || split || q_split)) return CC_ERR_UNSUPPORTED;
   // one query row per sequence: the decode kernel, which reads either format
-  const long long units0 = (long long)batch * c->n_kv_heads *
-                           (((row_lo ? q_span : cap) + P - 1) / P);
-  const bool decode = row_lo && q_span == 1 && G <= kDecMaxG && parts && parts->o && parts->ml &&
-                      units0 <= kAttnMaxSplitSlots;
+  const bool decode = row_lo && q_span == 1 && G <= kDecMaxG && parts && parts->o && parts->ml;
   if ((kvf.fp8 || f16) && !decode) {
     // the tile attention over an e4m3 cache, or with fp16 operands: the
     // layer's elements as bf16 or fp16 values (exact) in a slot-major scratch;
@@ -605,10 +607,13 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
   p.q_span = row_lo ? q_span : cap;
   const long long units = attn_units(p);
   if (decode) {   // one query row per sequence: the decode kernel
-    p.kv_splits = attn_decode_splits(units, cap, sms);
+    // as many as are resident, less the part-filled last splits
+    p.dec_ctas = (int)std::max<long long>(sms, 3LL * sms - units / 2);
+    p.kv_splits = attn_decode_splits(units, cap, p.dec_ctas);
     p.part_o = parts->o;
     p.part_ml = parts->ml;
     p.q = reinterpret_cast<const __nv_bfloat16 *>(q);
+    p.q_lo_off = p.out_lo_off = (long long)row_pairs * c->n_q_heads * dh;
     p.k = k;
     p.v = v;
     TimedScope t(CC_KERNEL_ATTN_CAUSAL, st);
@@ -696,6 +701,16 @@ cc_status check_append_args(const cc_model_cfg *c, const cc_model_weights *w,
   return CC_OK;
 }
 
+// A decode step's rows as bf16 pairs in the two halves of a group of the few-row
+// GEMM (GemmParams::row_pairs; 0: single rows): up to 64 sequences, where the
+// weights bound every product, and buffers that hold the lo rows.
+int decode_row_pairs(int batch, int cap) {
+  if (getenv("CC_GEMM_PAIRS")) return 0;   // keeps every product on the tile kernel
+  for (int half = 16; half <= 64; half *= 2)
+    if (batch <= half) return 2LL * half <= (long long)batch * cap ? half : 0;
+  return 0;
+}
+
 // Appends a chunk (or a decode step's token) per sequence through every layer.
 // The workspace rows are the appended slots packed (AppendRows), so a batch
 // of sequences with a few rows each reads every weight once.  final_gain
@@ -723,6 +738,9 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   const int32_t *total = rows.total;
   unsigned *status = dev->status;
   const int max_rows = (int)std::min((uint64_t)batch * max_count, (uint64_t)batch * cap);
+  // (the decode attention, which reads and writes the pairs, takes groups of 8 at most)
+  const int rp = max_count == 1 && c->n_q_heads / c->n_kv_heads <= kDecMaxG
+                     ? decode_row_pairs(batch, cap) : 0;
   AttnPartials parts;
   parts.o = reinterpret_cast<float *>(wsb + L.part_o);
   parts.ml = reinterpret_cast<float2 *>(wsb + L.part_ml);
@@ -739,7 +757,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   {
     TimedScope t(CC_KERNEL_EMBED, st);
     CC_TRY(launch_append_embed(w->embed, kv->tokens, rows, max_rows, w->layers[0].attn_norm, h, xn,
-                               ss_part, d, c->vocab, status, st));
+                               ss_part, d, c->vocab, rp, status, st));
   }
   auto scaled = [&](Gemm &g) {   // unnormalised A rows
     g.p.row_ss = ss_part;
@@ -750,7 +768,8 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   // residual add, with the next norm's gain (or null) fused as in the scoring pass
   auto resid = [&](const void *a, int k, const void *wm, const void *gain, int kind) -> cc_status {
     Gemm g;
-    cc_status r = gemm_setup(g, EPI_RESID_F32, a, k, wm, nullptr, d, 1, max_rows, total, status);
+    cc_status r = gemm_setup(g, EPI_RESID_F32, a, k, wm, nullptr, d, 1, max_rows, total, status,
+                             false, 0, rp);
     if (r != CC_OK) return r;
     g.p.out = h;
     g.p.ldo = d;
@@ -775,7 +794,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     // v = xn Wv^T + bv straight into the cache slots of the chunk
     if (qkv_fusable(c)) {   // one GEMM over [Wq; Wk; Wv]
       Gemm g;
-      if ((s = gemm_setup_qkv(g, xn, c, lw, 1, max_rows, total, status)) != CC_OK) return s;
+      if ((s = gemm_setup_qkv(g, xn, c, lw, 1, max_rows, total, status, rp)) != CC_OK) return s;
       scaled(g);
       g.p.out = q;
       g.p.out_k = kv->k[l];
@@ -795,8 +814,8 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
                              {lw.wv, lw.bv, kv->v[l], kvd, EPI_BF16, CC_KERNEL_GEMM_KV}};
       for (const Proj &pj : projs) {
         Gemm g;
-        if ((s = gemm_setup(g, pj.epi, xn, d, pj.w, nullptr, pj.n, 1, max_rows, total, status)) !=
-            CC_OK)
+        if ((s = gemm_setup(g, pj.epi, xn, d, pj.w, nullptr, pj.n, 1, max_rows, total, status,
+                            false, 0, rp)) != CC_OK)
           return s;
         scaled(g);
         g.p.out = pj.out;
@@ -824,13 +843,13 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     // (act is free until the MLP: an e4m3 layer's bf16 copy for the tile attention)
     if ((s = run_attention(c, q, kv->k[l], kv->v[l], o, rows.hi, batch, cap, status, st, false,
                            rows.lo, max_count, &parts, dev->sms, kvf, false, nullptr, nullptr, act,
-                           (size_t)batch * cap * c->d_ff * 2, false, rows.pbase, max_rows)) != CC_OK)
+                           (size_t)batch * cap * c->d_ff * 2, false, rows.pbase, max_rows, rp)) != CC_OK)
       return s;
     // h += o Wo^T; act = SwiGLU(RMSNorm(h)); h += act Wd^T
     if ((s = resid(o, qd, lw.wo, lw.mlp_norm, CC_KERNEL_GEMM_OPROJ)) != CC_OK) return s;
     Gemm gu;
-    if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, 1, max_rows, total, status)) !=
-        CC_OK)
+    if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, 1, max_rows, total, status,
+                        false, 0, rp)) != CC_OK)
       return s;
     scaled(gu);
     gu.p.out = act;
@@ -1318,8 +1337,9 @@ cc_status cc_decode_step(const cc_model_cfg *cfg, const cc_model_weights *w,
   const AppendRows rows = append_rows(L, wsb);
   float2 *part = reinterpret_cast<float2 *>(wsb + decode_part_offset(cfg, batch, cap));
   Gemm g;
+  const int rp = cfg->n_q_heads / cfg->n_kv_heads <= kDecMaxG ? decode_row_pairs(batch, cap) : 0;
   if ((s = gemm_setup(g, EPI_ARGMAX, wsb + L.s.xn, d, w->lm_head, nullptr, cfg->vocab, 1, batch,
-                      rows.total, dev->status)) != CC_OK)
+                      rows.total, dev->status, false, 0, rp)) != CC_OK)
     return s;
   g.p.row_ss = reinterpret_cast<float *>(wsb + L.s.sspart);   // the final norm
   g.p.n_ss = ss_tiles;

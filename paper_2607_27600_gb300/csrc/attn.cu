@@ -47,6 +47,8 @@
 // TMEM columns: S0 [0,128)  S1 [128,256)  O0 [256,256+DH)  O1 [256+DH, 256+2DH)
 #include "attn.cuh"
 
+#include <type_traits>
+
 namespace cc {
 
 namespace {
@@ -113,7 +115,6 @@ CC_DEV uint32_t e4m3x2_to_f16x2(uint32_t two) {
 // the sequence end.
 struct UnitInfo {
   int b, g, n, q_lo, p0, p_last;
-  int row0;   // workspace row of slot 0 (query and output rows)
   bool bad, valid;
 };
 CC_DEV UnitInfo decode_unit(const AttnParams &p, int unit_id, bool causal) {
@@ -134,11 +135,17 @@ CC_DEV UnitInfo decode_unit(const AttnParams &p, int unit_id, bool causal) {
   // query rows end: the sequence end, or a counter-causal row range's end
   const int q_hi = (!causal && p.row_hi) ? p.row_hi[u.b] : u.n;
   u.bad = u.n < 0 || u.n > p.cap || u.q_lo < 0 || u.q_lo > q_hi || q_hi > u.n;
-  u.row0 = p.pbase ? p.pbase[u.b] - u.q_lo : u.b * p.cap;
   u.p0 = u.q_lo + pb * p.P;
   u.valid = !u.bad && u.p0 < q_hi;
   u.p_last = min(u.p0 + p.P, q_hi) - 1;
   return u;
+}
+
+// Workspace row of slot 0 of the unit's sequence (query and output rows).
+template <bool CAUSAL>
+CC_DEV long long slot0_row(const AttnParams &p, const UnitInfo &u) {
+  if (CAUSAL && p.pbase) return p.pbase[u.b] - u.q_lo;
+  return (long long)u.b * p.cap;
 }
 
 template <int DH, bool CAUSAL, bool SPLIT, bool F16>
@@ -179,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int t0 = CAUSAL ? 0 : (p0 + 1) / BKV;
   const int t1 = CAUSAL ? p_last / BKV : (n - 1) / BKV;
   const int ntiles_unit = t1 - t0 + 1;
-  const long long row_base = u.row0;
+  const size_t row_base = (size_t)slot0_row<CAUSAL>(p, u);   // (modulo 2^64: rows add back)
   // this CTA's share of the unit's key tiles (all of them without splits):
   // local iteration `it` handles tile t_hi - it; the tail tile is t_top
   const int t_top = t1;
@@ -598,20 +605,21 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // Key splits: out = sum_s 2^((m_s - m*) c) O_s / sum_s 2^((m_s - m*) c) l_s
 // per row (m* the largest reference max, c = log2(e)/sqrt(dh)), splits in
-// order; bf16 (and lo) stores as the kernel's own epilogue.  Block = one row
-// of one unit, a thread per head_dim element: the splits' (max, sum) pairs
-// are loaded in parallel and weighted once in shared memory, then every
-// thread sums its element over the splits with eight loads in flight.
-constexpr int kCombineMaxSplits = 256;
+// order; stored as the kernel's own epilogue stores it.  A warp takes one row
+// of one unit, DH / 32 consecutive elements per lane, the loads of eight
+// splits in flight: 256 rows of 32 units over 4 splits (Qwen2.5-7B, a 256-row
+// chunk) took 19 us with a block and a barrier chain per row.
+constexpr int kCombineWarps = 8;
 
-template <bool CAUSAL>
-__global__ void attn_combine_kernel(const __grid_constant__ AttnParams p) {
-  __shared__ float wgt[kCombineMaxSplits];
-  __shared__ float lsum[kCombineMaxSplits];
-  __shared__ float red[4];
+template <int DH, bool CAUSAL>
+__global__ void __launch_bounds__(kCombineWarps * 32)
+    attn_combine_kernel(const __grid_constant__ AttnParams p) {
+  constexpr int DPL = DH / 32;
+  using Vec = std::conditional_t<DPL == 4, float4, float2>;
   pdl_trigger();
   pdl_wait();
-  const int R = blockIdx.x, unit_id = blockIdx.y, d = threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int R = blockIdx.x * kCombineWarps + (threadIdx.x >> 5), unit_id = blockIdx.y;
   const UnitInfo u = decode_unit(p, unit_id, CAUSAL);
   const int G = p.group;
   if (!u.valid || R >= p.P * G) return;
@@ -620,45 +628,45 @@ __global__ void attn_combine_kernel(const __grid_constant__ AttnParams p) {
   const int S = p.kv_splits;
   const float c = p.scale_log2;
   const size_t base = (size_t)unit_id * S * 256 + R;   // split s's row: base + s * 256
-  // reference max over the splits that saw keys
-  float m = -INFINITY;
-  for (int s = d; s < S; s += blockDim.x) {
-    const float2 ml = p.part_ml[base + (size_t)s * 256];
-    wgt[s] = ml.x;
-    lsum[s] = ml.y;
-    if (ml.y > 0.f) m = fmaxf(m, ml.x);
-  }
-  m = warp_max(m);
-  if ((d & 31) == 0) red[d >> 5] = m;
-  __syncthreads();
-  m = red[0];
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-  for (int s = d; s < S; s += blockDim.x)
-    wgt[s] = lsum[s] > 0.f ? exp2f((wgt[s] - m) * c) : 0.f;
-  __syncthreads();
-  float l = 0.f;
-  for (int s = 0; s < S; ++s) l += wgt[s] * lsum[s];
-  float o = 0.f;
-  int s = 0;
-  for (; s + 8 <= S; s += 8) {
-    float v[8];
+  float m = -INFINITY, l = 0.f, o[DPL];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = p.part_o[(base + (size_t)(s + k) * 256) * p.head_dim + d];
+  for (int e = 0; e < DPL; ++e) o[e] = 0.f;
+#pragma unroll 1
+  for (int s0 = 0; s0 < S; s0 += 8) {
+    Vec v[8];
+    float2 ml[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) o += wgt[s + k] * v[k];
+    for (int k = 0; k < 8; ++k) {
+      const size_t row = base + (size_t)min(s0 + k, S - 1) * 256;
+      ml[k] = p.part_ml[row];
+      if (s0 + k >= S) ml[k] = make_float2(-INFINITY, 0.f);
+      v[k] = *reinterpret_cast<const Vec *>(p.part_o + row * DH + lane * DPL);
+    }
+    float mx = m;   // reference max over the splits that saw keys
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (ml[k].y > 0.f) mx = fmaxf(mx, ml[k].x);
+    const float f = l > 0.f ? fast_exp2((m - mx) * c) : 0.f;
+    l *= f;
+#pragma unroll
+    for (int e = 0; e < DPL; ++e) o[e] *= f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      // a split without keys holds no O row (its memory may hold any bits)
+      if (!(ml[k].y > 0.f)) continue;
+      const float w = fast_exp2((ml[k].x - mx) * c);
+      l = fmaf(w, ml[k].y, l);
+#pragma unroll
+      for (int e = 0; e < DPL; ++e) o[e] = fmaf(w, reinterpret_cast<const float *>(&v[k])[e], o[e]);
+    }
+    m = mx;
   }
-  for (; s < S; ++s) o += wgt[s] * p.part_o[(base + (size_t)s * 256) * p.head_dim + d];
-  const float v = l > 0.f ? o * p.v_scale / l : 0.f;
-  __nv_bfloat16 *dst = p.out + (size_t)(u.row0 + pos) * p.out_ld +
-                       (size_t)(u.g * G + hl) * p.head_dim + d;
-  if (p.f16) {   // fp16 operand mode: O as fp16 (the same 2 bytes)
-    const __half hf = __float2half_rn(v);
-    *dst = *reinterpret_cast<const __nv_bfloat16 *>(&hf);
-    return;
-  }
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  *dst = hi;
-  if (p.out_lo > 0) dst[p.out_lo] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  const float inv = l > 0.f ? p.v_scale / l : 0.f;
+  __nv_bfloat16 *dst = p.out + (size_t)(slot0_row<CAUSAL>(p, u) + pos) * p.out_ld +
+                       (size_t)(u.g * G + hl) * DH + lane * DPL;
+#pragma unroll
+  for (int e = 0; e < DPL; e += 2)
+    *reinterpret_cast<uint32_t *>(dst + e) = pack_bf16x2(o[e] * inv, o[e + 1] * inv);
 }
 
 template <int DH, bool CAUSAL, bool SPLIT = false, bool F16 = false>
@@ -698,84 +706,115 @@ cudaError_t launch_dh(const CUtensorMap &q, const CUtensorMap &k, const CUtensor
   if (S > 1) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    attn_combine_kernel<CAUSAL><<<dim3(256, (unsigned)units), DH, 0, stream>>>(pp);
+    if (p.out_lo > 0 || F16) return cudaErrorInvalidValue;   // splits: the append's bf16 rows only
+    return launch_pdl(attn_combine_kernel<DH, CAUSAL>, dim3(256 / kCombineWarps, (unsigned)units),
+                      dim3(kCombineWarps * 32), 0, stream, pp);
   }
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
 // Decode attention: one query row per sequence (q_span == 1), at most
-// kDecMaxG query heads per KV head.  For a single query row the products are
-// a few hundred FMAs per key, so CUDA cores in fp32 suffice and the K/V bytes
-// bound the time: CTA = (unit, key split); chunks of 128 keys are copied to
-// shared memory with cp.async (double-buffered; K rows padded by 16 bytes so
-// the score pass's column reads are conflict-free); per chunk the scores, an
-// online softmax (log2 domain, reference max in raw units as the tile kernel
-// keeps it) and P V; each CTA writes the partial (O, max, sum) rows that
-// attn_combine_kernel merges.
+// kDecMaxG query heads per KV head.  The K/V bytes bound it (16 Llama-3-8B
+// sequences, 35k slots: 144 MB a layer), so CTAs stream chunks of 64 keys
+// through a ring of cp.async stages and the products run on warp-level
+// tensor instructions (m16n8k16, fp32 sums): eight query rows are far too few
+// for a tcgen05 tile, and per key fewer instructions are issued than on CUDA
+// cores.  The 16 rows of a product are the group's heads twice: the hi and
+// the lo parts of fp32 values (hi = bf16(x), lo = bf16(x - hi)), for the
+// queries and for the probabilities alike, so both products carry 16
+// significant bits of them against exact bf16 keys and values.  A thread then
+// holds both parts of its head's scores, which are the operand layout of the
+// second product: no exchange between the two.
+// CTA = 4 warps over one (unit, key split), 16 keys of each chunk per warp, the
+// splits of a batch equally long whatever the sequences' lengths; warps keep
+// their own reference maxima (raised lazily, as the tile kernel does) and meet
+// in shared memory; the splits' partial (O, max, sum) rows are merged by
+// decode_combine_kernel.
+// Measured per layer (ncu) against a CUDA-core kernel that staged 128-key
+// chunks and split each sequence alike: 16 Llama-3-8B sequences 154 us (with
+// its combine) -> 28 us (5.0 TB/s) + 9 us; one Qwen2.5-7B sequence of 8192
+// slots 16.8 us -> 10.8 us, its combine 15.6 -> 5.0 us.  CUDA-core versions of
+// the same plan that kept keys in registers were issue-bound (36 us, 50 us).
 // ---------------------------------------------------------------------------
-constexpr int kDecChunk = 128;
-constexpr int kDecThreads = 256;   // = 2 * kDecChunk: the score pass takes a key and half its dims
+constexpr int kDecWarps = 4;
+constexpr int kDecChunk = 64;      // keys of a stage
+constexpr int kDecStages = 2;      // (three CTAs of 64 KB per SM ahead of two of 96)
 
-// K rows padded so the score pass's column reads are conflict-free: bf16
-// rows +16 bytes (16-byte reads), e4m3 rows +8 bytes (8-byte reads).
-template <int DH, bool FP8>
-struct DecSmem {
-  static constexpr int EB = FP8 ? 1 : 2;   // bytes per cached element
-  static constexpr int K_ROW = DH * EB + (FP8 ? 8 : 16);
-  static constexpr int V_ROW = DH * EB;
-  static constexpr int K_BYTES = kDecChunk * K_ROW;
-  static constexpr int V_BYTES = kDecChunk * V_ROW;
-  static constexpr int BUF = K_BYTES + V_BYTES;
-  static constexpr int OFF_Q = 2 * BUF;                                 // fp32 [G][DH]
-  static constexpr int OFF_S = OFF_Q + kDecMaxG * DH * 4;               // fp32 [2][G][chunk]
-  static constexpr int OFF_P = OFF_S + 2 * kDecMaxG * kDecChunk * 4;    // fp32 [G][chunk]
-  static constexpr int OFF_F = OFF_P + kDecMaxG * kDecChunk * 4;        // fp32 [G]
-  static constexpr int BYTES = OFF_F + kDecMaxG * 4;
-};
-
-CC_DEV void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
-               : "memory");
-}
-CC_DEV void cp_async8(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
+CC_DEV void cp_async16(uint32_t dst, const void *src, bool there) {   // else zeros
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(there ? 16 : 0)
                : "memory");
 }
 CC_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-
-// 8 cached elements -> float: bf16 (16 bytes) or e4m3 codes (8 bytes, via f16)
-template <bool FP8>
-CC_DEV void load8_kv(const uint8_t *src, float *f) {
-  if constexpr (FP8) {
-    const uint2 x = *reinterpret_cast<const uint2 *>(src);
-    const uint32_t h[4] = {e4m3x2_to_f16x2(x.x), e4m3x2_to_f16x2(x.x >> 16),
-                           e4m3x2_to_f16x2(x.y), e4m3x2_to_f16x2(x.y >> 16)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(&h[i]));
-      f[2 * i] = v.x;
-      f[2 * i + 1] = v.y;
-    }
-  } else {
-    const uint4 x = *reinterpret_cast<const uint4 *>(src);
-    f[0] = bf16_lo(x.x); f[1] = bf16_hi(x.x); f[2] = bf16_lo(x.y); f[3] = bf16_hi(x.y);
-    f[4] = bf16_lo(x.z); f[5] = bf16_hi(x.z); f[6] = bf16_lo(x.w); f[7] = bf16_hi(x.w);
-  }
-}
 template <int N>
 CC_DEV void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+CC_DEV void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+CC_DEV void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+CC_DEV void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+template <int DH>
+struct DecSmem {
+  static constexpr int ROW = DH * 2;                      // bytes of a key's bf16 row
+  static constexpr int TILE = kDecChunk * ROW;            // K (or V) of a stage
+  static constexpr int BYTES = kDecStages * 2 * TILE;
+  // 16-byte piece c of row r (swizzled: ldmatrix reads eight rows at one c)
+  CC_DEV static uint32_t at(int r, int c) { return (uint32_t)(r * ROW + ((c ^ (r & 7)) << 4)); }
+  static_assert(kDecWarps * kDecMaxG * DH * 4 <= BYTES, "the warps' partial rows");
+};
+
+// hi + lo products of one sum: an infinite hi stands (an infinite key or value
+// times a lo part of zero is NaN).
+CC_DEV float add_parts(float hi, float lo) { return fabsf(hi) == INFINITY ? hi : hi + lo; }
+
+CC_DEV void store_decode(const AttnParams &p, size_t el, float v) {
+  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+  p.out[el] = hi;
+  if (p.out_lo_off > 0) p.out[el + p.out_lo_off] = __float2bfloat16_rn(v - __bfloat162float(hi));
+}
+
+// Keys of one split of a unit with n_keys keys: the batch's keys over about
+// dec_ctas CTAs (every sequence's splits equally long), but no unit in more
+// than kv_splits of them; whole chunks (which lie in one page).  Every lane
+// calls, all get the same.
+CC_DEV int dec_split_keys(const AttnParams &p, int n_keys) {
+  float total = 0.f;   // (a plan, not a count: fp32 will do)
+  for (int b = threadIdx.x & 31; b < p.batch; b += 32)
+    total += (float)min(max(p.seq_len[b], 0), p.cap);
+  const int even = (int)(warp_sum(total) * (float)p.n_kv_heads / (float)p.dec_ctas);
+  const int keys = max(even, (n_keys + p.kv_splits - 1) / p.kv_splits);
+  return max(1, (keys + kDecChunk - 1) / kDecChunk) * kDecChunk;
+}
 
 template <int DH, bool FP8>
-__global__ void __launch_bounds__(kDecThreads) attn_decode_kernel(const __grid_constant__ AttnParams p) {
-  using L = DecSmem<DH, FP8>;
+__global__ void __launch_bounds__(kDecWarps * 32, 3)
+    attn_decode_kernel(const __grid_constant__ AttnParams p) {
+  using L = DecSmem<DH>;
+  constexpr int KS = DH / 16, NT = DH / 8;   // K steps of Q K^T, column tiles of P V
+  constexpr int PIECES = DH / 8;             // 16-byte bf16 pieces of a row
   extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ float sm[kDecWarps][kDecMaxG], sl[kDecWarps][kDecMaxG];
   pdl_trigger();   // the combine may launch (it waits for this grid before reading)
   pdl_wait();      // q and the new token's K/V come from the projection just before
-  const int S = p.kv_splits;
-  const int unit_id = blockIdx.x / S, split = blockIdx.x - unit_id * S;
+  const int S = p.kv_splits, units = gridDim.x / S;
+  // splits outermost: those past the shorter sequences' ends come last
+  const int split = blockIdx.x / units, unit_id = blockIdx.x - split * units;
   const UnitInfo u = decode_unit(p, unit_id, true);
   if (u.bad) {
     if (threadIdx.x == 0) set_status(p.status, CC_ERR_DEVICE_ARG);
@@ -783,202 +822,280 @@ __global__ void __launch_bounds__(kDecThreads) attn_decode_kernel(const __grid_c
   }
   if (!u.valid) return;
   const int G = p.group, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int pos = u.p0;            // the unit's one query slot
-  const int n_keys = pos + 1;      // causal: keys 0 .. pos
-  const int nch = (n_keys + kDecChunk - 1) / kDecChunk;
-  const int c_lo = split * nch / S, c_hi = (split + 1) * nch / S;
-  const size_t slot = ((size_t)unit_id * S + split) * 256;
-  if (c_lo >= c_hi) {   // nothing for this split: an empty partial
-    if (tid < G) p.part_ml[slot + tid] = make_float2(-INFINITY, 0.f);
-    return;
-  }
-  float *qs = reinterpret_cast<float *>(smem + L::OFF_Q);
-  float *sbuf = reinterpret_cast<float *>(smem + L::OFF_S);
-  float *pbuf = reinterpret_cast<float *>(smem + L::OFF_P);
-  float *fbuf = reinterpret_cast<float *>(smem + L::OFF_F);
-  const long long row_base = u.row0;
-  const int Hkv = p.n_kv_heads;
-
+  const int n_keys = u.p0 + 1;     // causal: keys 0 .. the unit's one query slot
+  const int per = dec_split_keys(p, n_keys);
+  const int k0 = split * per, k1 = min(n_keys, k0 + per);
+  if (k0 >= n_keys) return;        // splits past the last key: the combine skips them
+  const int chunks = (k1 - k0 + kDecChunk - 1) / kDecChunk;
+  const size_t qrow = (size_t)(slot0_row<true>(p, u) + u.p0);
+  const uint32_t sbase = smem_u32(smem);
   const uint8_t *kg = reinterpret_cast<const uint8_t *>(p.k);
   const uint8_t *vg = reinterpret_cast<const uint8_t *>(p.v);
-  auto issue = [&](int c, int buf) {
-    uint8_t *kb = smem + buf * L::BUF, *vb = kb + L::K_BYTES;
-    // K in DH/8 pieces per row (16 bytes bf16, 8 bytes e4m3), V in 16-byte pieces
-    constexpr int KP = DH / 8, KPB = 8 * L::EB, VP = DH * L::EB / 16;
-    // vector index of the chunk's first key (a chunk lies in one page; head-major:
-    // consecutive slots are consecutive vectors, else Hkv apart); -1: bad page
-    const long long cbase = kv_vec(p.pg, p.cap, u.b, u.g, c * kDecChunk);
-    const int vstep = p.pg.head_major ? 1 : Hkv;
-    if (cbase < 0 && tid == 0) set_status(p.status, CC_ERR_DEVICE_ARG);
-    for (int i = tid; i < kDecChunk * KP; i += kDecThreads) {
-      const int r = i / KP, e = i - r * KP;
-      const int j = c * kDecChunk + r;
-      uint8_t *kd = kb + r * L::K_ROW + e * KPB;
-      if (j < n_keys && cbase >= 0) {
-        const uint8_t *src = kg + ((size_t)(cbase + (long long)r * vstep) * DH) * L::EB + e * KPB;
-        if constexpr (FP8) cp_async8(kd, src);
-        else cp_async16(kd, src);
-      } else if constexpr (FP8) {
-        *reinterpret_cast<uint2 *>(kd) = make_uint2(0, 0);
-      } else {
-        *reinterpret_cast<uint4 *>(kd) = make_uint4(0, 0, 0, 0);
+  const int vstep = p.pg.head_major ? 1 : p.n_kv_heads;
+  constexpr int EB = FP8 ? 1 : 2;
+
+  // vector index of a chunk's first key (-1: bad page, its keys are skipped)
+  auto chunk_base = [&](int c) -> long long {
+    return kv_vec(p.pg, p.cap, u.b, u.g, k0 + c * kDecChunk);
+  };
+  auto issue = [&](int c, int st) {   // bf16: chunk c into stage st; past the end: zeros
+    if (c < chunks) {
+      const long long base = chunk_base(c);
+      const int n = base < 0 ? 0 : min(kDecChunk, k1 - (k0 + c * kDecChunk));
+      const uint32_t kd = sbase + st * 2 * L::TILE, vd = kd + L::TILE;
+#pragma unroll
+      for (int i = tid; i < kDecChunk * PIECES; i += kDecWarps * 32) {
+        const int r = i / PIECES, e = i - r * PIECES;
+        const bool there = r < n;
+        const size_t off = there ? (size_t)(base + (long long)r * vstep) * DH * 2 + e * 16 : 0;
+        cp_async16(kd + L::at(r, e), kg + off, there);
+        cp_async16(vd + L::at(r, e), vg + off, there);
       }
-    }
-    for (int i = tid; i < kDecChunk * VP; i += kDecThreads) {
-      const int r = i / VP, e = i - r * VP;
-      const int j = c * kDecChunk + r;
-      uint8_t *vd = vb + r * L::V_ROW + e * 16;
-      if (j < n_keys && cbase >= 0)   // past the last key: zeros (P is 0 there, V must be finite)
-        cp_async16(vd, vg + ((size_t)(cbase + (long long)r * vstep) * DH) * L::EB + e * 16);
-      else
-        *reinterpret_cast<uint4 *>(vd) = make_uint4(0, 0, 0, 0);
     }
     cp_async_commit();
   };
-  issue(c_lo, 0);
-  for (int i = tid; i < G * DH; i += kDecThreads) {
-    const int h = i / DH, d = i - h * DH;
-    qs[i] = __bfloat162float(
-        p.q[(size_t)(row_base + pos) * p.n_q_heads * DH + (size_t)(u.g * G + h) * DH + d]);
-  }
+  // e4m3: chunk c's codes in registers (16 a piece), stored as bf16 later
+  constexpr int FPER = FP8 ? kDecChunk * DH / 16 / (kDecWarps * 32) : 1;
+  uint4 kc[FPER], vc[FPER];
+  auto fetch8 = [&](int c) {
+    if (c >= chunks) return;
+    const long long base = chunk_base(c);
+    const int n = base < 0 ? 0 : min(kDecChunk, k1 - (k0 + c * kDecChunk));
+#pragma unroll
+    for (int x = 0; x < FPER; ++x) {
+      const int i = tid + x * kDecWarps * 32, r = i / (DH / 16), e = i - r * (DH / 16);
+      kc[x] = vc[x] = make_uint4(0, 0, 0, 0);
+      if (r >= n) continue;
+      const size_t off = (size_t)(base + (long long)r * vstep) * DH + e * 16;
+      kc[x] = *reinterpret_cast<const uint4 *>(kg + off);
+      vc[x] = *reinterpret_cast<const uint4 *>(vg + off);
+    }
+  };
+  auto put8 = [&](int st) {
+#pragma unroll
+    for (int x = 0; x < FPER; ++x) {
+      const int i = tid + x * kDecWarps * 32, r = i / (DH / 16), e = i - r * (DH / 16);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const uint4 w = t ? vc[x] : kc[x];
+        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+        uint32_t o[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t h2 = e4m3x2_to_f16x2(ws[j / 2] >> (16 * (j & 1)));
+          const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&h2));
+          o[j] = pack_bf16x2(f.x, f.y);   // exact
+        }
+        uint8_t *d = smem + (st * 2 + t) * L::TILE;
+        *reinterpret_cast<uint4 *>(d + L::at(r, 2 * e)) = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4 *>(d + L::at(r, 2 * e + 1)) = make_uint4(o[4], o[5], o[6], o[7]);
+      }
+    }
+  };
 
-  constexpr int DPT = DH / 32;   // P V: warp h < G owns head h, lane the dims lane*DPT..
-  float m_h = -INFINITY, l_h = 0.f;
-  float o[DPT];
+  if constexpr (FP8) {
+    fetch8(0);
+  } else {
+    for (int c = 0; c < kDecStages - 1; ++c) issue(c, c);
+  }
+  if (chunk_base(0) < 0 && tid == 0) set_status(p.status, CC_ERR_DEVICE_ARG);
+
+  // Q as the first operand: row lane / 4 = the head's hi part, + 8 its lo part
+  const int head = lane >> 2, quad = lane & 3;
+  uint32_t qa[KS][4];
 #pragma unroll
-  for (int i = 0; i < DPT; ++i) o[i] = 0.f;
-  const float c2 = p.scale_log2;
-  for (int c = c_lo; c < c_hi; ++c) {
-    const int buf = (c - c_lo) & 1;
-    if (c + 1 < c_hi) {
-      issue(c + 1, buf ^ 1);
-      cp_async_wait<1>();
+  for (int ks = 0; ks < KS; ++ks) {
+    const __nv_bfloat16 *src =
+        p.q + (qrow * p.n_q_heads + u.g * G + min(head, G - 1)) * DH + ks * 16 + quad * 2;
+    const bool live = head < G, lo = live && p.q_lo_off > 0;
+    qa[ks][0] = live ? *reinterpret_cast<const uint32_t *>(src) : 0u;
+    qa[ks][2] = live ? *reinterpret_cast<const uint32_t *>(src + 8) : 0u;
+    qa[ks][1] = lo ? *reinterpret_cast<const uint32_t *>(src + p.q_lo_off) : 0u;
+    qa[ks][3] = lo ? *reinterpret_cast<const uint32_t *>(src + p.q_lo_off + 8) : 0u;
+  }
+  const float c2 = p.scale_log2, thr = 8.f / c2;
+  float o[NT][4];   // [0..1] the hi part's columns, [2..3] the lo part's
+#pragma unroll
+  for (int t = 0; t < NT; ++t)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[t][k] = 0.f;
+  float m = -INFINITY, l = 0.f;   // of this thread's head (l: this thread's keys only)
+  const int mi = lane >> 3, mr = lane & 7;   // ldmatrix: matrix and row of this lane's address
+#pragma unroll 1
+  for (int c = 0; c < chunks; ++c) {
+    const int st = FP8 ? 0 : c % kDecStages;
+    if constexpr (FP8) {
+      __syncthreads();   // the last chunk is read
+      put8(0);
+      fetch8(c + 1);
     } else {
-      cp_async_wait<0>();
+      issue(c + kDecStages - 1, (c + kDecStages - 1) % kDecStages);
+      cp_async_wait<kDecStages - 1>();
     }
     __syncthreads();
-    const uint8_t *kb = smem + buf * L::BUF, *vb = kb + L::K_BYTES;
-    {   // scores: thread = (key j, half of the dims)
-      const int j = tid & (kDecChunk - 1), half = tid / kDecChunk;
-      const uint8_t *kr = kb + j * L::K_ROW + half * (DH / 2) * L::EB;
-      float sc[kDecMaxG];
+    const uint32_t kt = sbase + st * 2 * L::TILE, vt = kt + L::TILE;
+    float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-      for (int h = 0; h < kDecMaxG; ++h) sc[h] = 0.f;
-#pragma unroll
-      for (int d8 = 0; d8 < DH / 16; ++d8) {
-        float kf[8];
-        load8_kv<FP8>(kr + d8 * 8 * L::EB, kf);
-        const int d0 = half * (DH / 2) + d8 * 8;
-#pragma unroll
-        for (int h = 0; h < kDecMaxG; ++h) {
-          if (h < G) {
-            const float4 qa = *reinterpret_cast<const float4 *>(qs + h * DH + d0);
-            const float4 qb = *reinterpret_cast<const float4 *>(qs + h * DH + d0 + 4);
-            float a = sc[h];
-            a = fmaf(kf[0], qa.x, a); a = fmaf(kf[1], qa.y, a);
-            a = fmaf(kf[2], qa.z, a); a = fmaf(kf[3], qa.w, a);
-            a = fmaf(kf[4], qb.x, a); a = fmaf(kf[5], qb.y, a);
-            a = fmaf(kf[6], qb.z, a); a = fmaf(kf[7], qb.w, a);
-            sc[h] = a;
-          }
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < kDecMaxG; ++h)
-        if (h < G) sbuf[(half * kDecMaxG + h) * kDecChunk + j] = sc[h];
+    for (int ks = 0; ks < KS; ++ks) {   // keys 16 warp .. + 16
+      uint32_t b[4];
+      ldmatrix4(kt + L::at(warp * 16 + (mi >> 1) * 8 + mr, ks * 2 + (mi & 1)), b);
+      mma_16816(s[0], qa[ks], b[0], b[1]);
+      mma_16816(s[1], qa[ks], b[2], b[3]);
     }
-    __syncthreads();
-    if (warp < G) {   // online softmax of head h = warp over the chunk
-      const int h = warp;
-      float sv[kDecChunk / 32];
-      float cm = -INFINITY;
+    // this thread: its head's scores of keys kb + 8 t + {0, 1}
+    const int kb = k0 + c * kDecChunk + warp * 16 + quad * 2;
+    const int end = chunk_base(c) < 0 ? 0 : k1;
+    float x[2][2];
 #pragma unroll
-      for (int q = 0; q < kDecChunk / 32; ++q) {
-        const int j = lane + 32 * q;
-        float v = sbuf[h * kDecChunk + j] + sbuf[(kDecMaxG + h) * kDecChunk + j];
-        if (c * kDecChunk + j >= n_keys) v = -INFINITY;
-        sv[q] = v;
-        cm = fmaxf(cm, v);
-      }
-      cm = warp_max(cm);
-      const float m_new = fmaxf(m_h, cm);
-      const bool any = m_new != -INFINITY;
-      const float factor = any ? fast_exp2((m_h - m_new) * c2) : 1.f;   // 0 when m_h = -inf
-      float ls = 0.f;
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
-      for (int q = 0; q < kDecChunk / 32; ++q) {
-        const float pv = any ? fast_exp2((sv[q] - m_new) * c2) : 0.f;
-        pbuf[h * kDecChunk + lane + 32 * q] = pv;
-        ls += pv;
-      }
-      ls = warp_sum(ls);
-      l_h = l_h * factor + ls;
-      m_h = m_new;
-      if (lane == 0) fbuf[h] = factor;
+      for (int e = 0; e < 2; ++e)
+        x[t][e] = kb + 8 * t + e < end ? add_parts(s[t][e], s[t][2 + e]) : -INFINITY;
+    float mx = fmaxf(fmaxf(x[0][0], x[0][1]), fmaxf(x[1][0], x[1][1]));
+    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
+    if (__any_sync(0xFFFFFFFFu, mx > m + thr)) {   // also -inf -> finite
+      const float m_new = fmaxf(m, mx);
+      const float f = m == -INFINITY ? 0.f : fast_exp2((m - m_new) * c2);
+      m = m_new;
+      l *= f;
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[t][k] *= f;
     }
-    __syncthreads();
-    if (warp < G) {   // O = O * factor + P V
-      const int h = warp;
-      const float f = fbuf[h];
+    uint32_t pa[4];
 #pragma unroll
-      for (int i = 0; i < DPT; ++i) o[i] *= f;
-      const float *ph = pbuf + h * kDecChunk;
-#pragma unroll 4
-      for (int j = 0; j < kDecChunk; ++j) {
-        const float pj = ph[j];
-        const uint8_t *vr = vb + j * L::V_ROW + lane * DPT * L::EB;
-        if constexpr (FP8) {
-#pragma unroll
-          for (int i = 0; i < DPT; i += 2) {
-            const uint32_t hv = e4m3x2_to_f16x2(*reinterpret_cast<const uint16_t *>(vr + i));
-            const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(&hv));
-            o[i] = fmaf(pj, v.x, o[i]);
-            o[i + 1] = fmaf(pj, v.y, o[i + 1]);
-          }
-        } else if constexpr (DPT == 4) {
-          const uint2 v = *reinterpret_cast<const uint2 *>(vr);
-          o[0] = fmaf(pj, bf16_lo(v.x), o[0]);
-          o[1] = fmaf(pj, bf16_hi(v.x), o[1]);
-          o[2] = fmaf(pj, bf16_lo(v.y), o[2]);
-          o[3] = fmaf(pj, bf16_hi(v.y), o[3]);
-        } else {
-          const uint32_t v = *reinterpret_cast<const uint32_t *>(vr);
-          o[0] = fmaf(pj, bf16_lo(v), o[0]);
-          o[1] = fmaf(pj, bf16_hi(v), o[1]);
-        }
-      }
+    for (int t = 0; t < 2; ++t) {
+      const float p0 = x[t][0] == -INFINITY ? 0.f : fast_exp2((x[t][0] - m) * c2);
+      const float p1 = x[t][1] == -INFINITY ? 0.f : fast_exp2((x[t][1] - m) * c2);
+      l += p0 + p1;
+      pa[2 * t] = pack_bf16x2(p0, p1);
+      pa[2 * t + 1] = pack_bf16x2(p0 - bf16_lo(pa[2 * t]), p1 - bf16_hi(pa[2 * t]));
     }
-    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < NT; t += 2) {
+      uint32_t b[4];
+      ldmatrix4_trans(vt + L::at(warp * 16 + (mi & 1) * 8 + mr, t + (mi >> 1)), b);
+      mma_16816(o[t], pa, b[0], b[1]);
+      mma_16816(o[t + 1], pa, b[2], b[3]);
+    }
+    if constexpr (!FP8) __syncthreads();   // the stage may be refilled
   }
-  if (warp < G) {   // partial row R = head warp of the unit's one position
-    float *po = p.part_o + (slot + warp) * DH + lane * DPT;
-#pragma unroll
-    for (int i = 0; i < DPT; ++i) po[i] = o[i];
-    if (lane == 0) p.part_ml[slot + warp] = make_float2(m_h, l_h);
+  // ---- the four warps' partial rows
+  if constexpr (!FP8) cp_async_wait<0>();
+  __syncthreads();
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 1);
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 2);
+  if (quad == 0) {
+    sm[warp][head] = m;
+    sl[warp][head] = l;
   }
+  float *so = reinterpret_cast<float *>(smem);   // [warp][head][DH]
+#pragma unroll
+  for (int t = 0; t < NT; ++t)
+    *reinterpret_cast<float2 *>(so + (warp * kDecMaxG + head) * DH + t * 8 + quad * 2) =
+        make_float2(add_parts(o[t][0], o[t][2]), add_parts(o[t][1], o[t][3]));
+  __syncthreads();
+  const size_t slot = ((size_t)unit_id * S + split) * kDecMaxG;
+  for (int i = tid; i < G * DH; i += kDecWarps * 32) {
+    const int h = i / DH, d = i - h * DH;
+    float mx = -INFINITY, lt = 0.f, ot = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w)
+      if (sl[w][h] > 0.f) mx = fmaxf(mx, sm[w][h]);
+#pragma unroll
+    for (int w = 0; w < kDecWarps; ++w) {   // a warp without keys holds zeros
+      const float f = sl[w][h] > 0.f ? fast_exp2((sm[w][h] - mx) * c2) : 0.f;
+      lt = fmaf(f, sl[w][h], lt);
+      ot = fmaf(f, so[(w * kDecMaxG + h) * DH + d], ot);
+    }
+    if (S == 1) {
+      store_decode(p, qrow * p.out_ld + (size_t)(u.g * G + h) * DH + d,
+                   lt > 0.f ? ot * p.v_scale / lt : 0.f);
+    } else {
+      p.part_o[(slot + h) * DH + d] = ot;
+      if (d == 0) p.part_ml[slot + h] = make_float2(mx, lt);
+    }
+  }
+}
+
+// Merges the splits of one (unit, head): four groups of head_dim threads take
+// every fourth split, all their loads (and the splits' (max, sum) pairs, which
+// every warp weighs for itself) in flight at once; fixed order.
+constexpr int kDecGroups = 4;
+
+template <int DH>
+__global__ void __launch_bounds__(kDecGroups * DH)
+    decode_combine_kernel(const __grid_constant__ AttnParams p) {
+  constexpr int PER = kDecMaxSplits / kDecGroups;
+  __shared__ float part[kDecGroups][DH];
+  pdl_trigger();
+  pdl_wait();
+  const int h = blockIdx.x, unit_id = blockIdx.y, S = p.kv_splits;
+  const int grp = threadIdx.x / DH, d = threadIdx.x - grp * DH, lane = threadIdx.x & 31;
+  const UnitInfo u = decode_unit(p, unit_id, true);
+  if (!u.valid) return;
+  const int n_keys = u.p0 + 1, per = dec_split_keys(p, n_keys);
+  const int used = (n_keys + per - 1) / per;   // <= S
+  const size_t row0 = (size_t)unit_id * S * kDecMaxG + h;   // split s: row0 + s * kDecMaxG
+  float o[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int s = k * kDecGroups + grp;
+    o[k] = s < used ? p.part_o[(row0 + (size_t)s * kDecMaxG) * DH + d] : 0.f;
+  }
+  constexpr int ML = kDecMaxSplits / 32;   // this lane's splits: lane, lane + 32, ...
+  float w[ML], l = 0.f, m = -INFINITY;
+  float2 ml[ML];
+#pragma unroll
+  for (int i = 0; i < ML; ++i) {
+    const int s = lane + 32 * i;
+    ml[i] = s < used ? p.part_ml[row0 + (size_t)s * kDecMaxG] : make_float2(-INFINITY, 0.f);
+    if (ml[i].y > 0.f) m = fmaxf(m, ml[i].x);
+  }
+  m = warp_max(m);
+#pragma unroll
+  for (int i = 0; i < ML; ++i) {
+    w[i] = ml[i].y > 0.f ? fast_exp2((ml[i].x - m) * p.scale_log2) : 0.f;
+    l = fmaf(w[i], ml[i].y, l);
+  }
+  l = warp_sum(l);
+  float acc = 0.f;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {   // splits k * kDecGroups + grp lie in slice k * kDecGroups / 32
+    const int s = k * kDecGroups + grp;
+    acc = fmaf(__shfl_sync(0xFFFFFFFFu, w[k * kDecGroups / 32], s & 31), o[k], acc);
+  }
+  part[grp][d] = acc;
+  __syncthreads();
+  if (grp > 0) return;
+  const float v = ((part[0][d] + part[1][d]) + (part[2][d] + part[3][d])) *
+                  (l > 0.f ? p.v_scale / l : 0.f);
+  store_decode(p, (size_t)(slot0_row<true>(p, u) + u.p0) * p.out_ld + (size_t)(u.g * p.group + h) * DH + d, v);
 }
 
 template <int DH, bool FP8>
 cudaError_t launch_decode_dh(const AttnParams &p, cudaStream_t stream) {
+  const long long units = attn_units(p);
+  if (units <= 0) return cudaSuccess;
+  AttnParams pp = p;
+  pp.streams_per_group = p.batch * p.n_kv_heads;
   static bool attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 64 && !attr_set[dev]) {
     cudaError_t e = cudaFuncSetAttribute(attn_decode_kernel<DH, FP8>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         DecSmem<DH, FP8>::BYTES);
+                                         DecSmem<DH>::BYTES);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
-  const long long units = attn_units(p);
-  if (units <= 0) return cudaSuccess;
-  AttnParams pp = p;
-  pp.streams_per_group = p.batch * p.n_kv_heads;
   cudaError_t e = launch_pdl(attn_decode_kernel<DH, FP8>, dim3((unsigned)(units * pp.kv_splits)),
-                             dim3(kDecThreads), DecSmem<DH, FP8>::BYTES, stream, pp);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(attn_combine_kernel<true>, dim3((unsigned)p.group, (unsigned)units), dim3(DH),
-                    0, stream, pp);
+                             dim3(kDecWarps * 32), DecSmem<DH>::BYTES, stream, pp);
+  if (e != cudaSuccess || pp.kv_splits == 1) return e;
+  return launch_pdl(decode_combine_kernel<DH>, dim3((unsigned)p.group, (unsigned)units),
+                    dim3(kDecGroups * DH), 0, stream, pp);
 }
 
 }  // namespace
@@ -994,6 +1111,7 @@ cudaError_t launch_attention_decode(const AttnParams &p, cudaStream_t stream) {
   if (!p.causal || p.q_span != 1 || p.group > kDecMaxG || p.kv_splits < 1 || !p.q || !p.k ||
       !p.v || !p.part_o || !p.part_ml)
     return cudaErrorInvalidValue;
+  if (p.kv_splits > kDecMaxSplits) return cudaErrorInvalidValue;
   const bool f8 = p.kv_fp8 != 0;
   if (p.head_dim == 128)
     return f8 ? launch_decode_dh<128, true>(p, stream) : launch_decode_dh<128, false>(p, stream);

@@ -32,7 +32,11 @@ struct AttnParams {
   int kv_splits;            // > 1: each unit's key tiles split over kv_splits CTAs (few units)
   float *part_o;            // kv_splits > 1: [unit][split][256 rows][head_dim] unnormalised O
   float2 *part_ml;          // kv_splits > 1: [unit][split][256 rows] (reference max, row sum)
+                            // (the decode kernel: kDecMaxG rows instead of 256)
   const __nv_bfloat16 *q;   // decode kernel: Q [rows][Hq][dh]
+  int dec_ctas;             // decode kernel: CTAs the batch's keys are spread over
+  long long q_lo_off;       // decode kernel: > 0: Q is hi + lo, lo at this element offset
+  long long out_lo_off;     // decode kernel: > 0: also write lo = bf16(o - hi) at this offset
   const void *k, *v;        // decode kernel: cache [rows][Hkv][dh] (bf16, or e4m3 bytes)
   int kv_fp8;               // decode kernel: K/V are e4m3 codes (the tile kernel takes bf16
                             // only: an e4m3 layer arrives as a bf16 copy of its codes); the
@@ -46,6 +50,7 @@ struct AttnParams {
 };
 
 constexpr int kDecMaxG = 8;   // query heads per KV head the decode kernel takes at most
+constexpr int kDecMaxSplits = 128;   // key splits of a decode unit at most
 
 int attn_positions_per_unit(int group);
 // Work units of a launch (before key splits) and the partial-result floats
@@ -57,8 +62,8 @@ constexpr int kAttnPartRowFloats = 256;   // rows of a unit (times head_dim + 2 
 cudaError_t launch_attention(const CUtensorMap &q, const CUtensorMap &k, const CUtensorMap &v,
                              const AttnParams &p, cudaStream_t stream);
 // Causal attention of one query row per sequence (q_span == 1, group <=
-// kDecMaxG): CUDA-core kernel over kv_splits (>= 1) key ranges per unit, then
-// the combine; needs q, k, v, part_o and part_ml.
+// kDecMaxG): CUDA-core kernel over kv_splits (1 .. kDecMaxSplits) key ranges
+// per unit, then (kv_splits > 1) the combine; needs q, k, v, part_o and part_ml.
 cudaError_t launch_attention_decode(const AttnParams &p, cudaStream_t stream);
 
 }  // namespace cc

@@ -23,6 +23,11 @@
 //               both columns of a pair in one warp, 16 lanes apart.
 // What a row needs besides its products (RMSNorm scale, position, cache row)
 // is gathered into shared memory while the products run.
+// A decode step's rows come as bf16 pairs hi + lo (hi = bf16(x),
+// lo = bf16(x - hi)) in two halves of the group: the weights bound such a
+// launch, so the second half of the N side costs nothing and the activations
+// carry 16 significant bits instead of 8 (Qwen2.5-7B and Llama-3-8B, 4 layers:
+// the largest logit's error against 64 bits 2e-3 with single bf16 rows).
 // Without a split two TMEM accumulators let the epilogue of one tile overlap
 // the main loop of the next; with a split the partials take the ring's
 // memory, so the next tile's loads begin when the sums are done.
@@ -215,7 +220,7 @@ CC_DEV LaneCol lane_col(const GemmParams &p, const ProjTile &d, int nt, int q, i
 
 // One value as the next product's operand: bf16 (with lo > 0 also the
 // remainder at that offset) or fp16, a finite overflow reported.
-CC_DEV void store_act(uint16_t *o, float y, bool f16, int lo, bool live, unsigned *status) {
+CC_DEV void store_act(uint16_t *o, float y, bool f16, long long lo, bool live, unsigned *status) {
   uint16_t bits;
   if (f16) {
     if (live && f16_overflow(y)) set_status(status, CC_ERR_RANGE);
@@ -253,7 +258,8 @@ CC_DEV void finish_rows8(const GemmParams &p, const ProjTile &d, const LaneCol &
                          const RowTab &tab, const float (&v)[16], const float (&u)[16], int r0,
                          int n, size_t row0, int lane, bool dry) {
   const bool f16 = p.out_f16 && !(is_proj<EPI> && d.kv);
-  const int lo = p.out_split && !(is_proj<EPI> && d.kv) ? p.N : 0;
+  const long long lo = is_proj<EPI> && d.kv ? 0 : p.row_pairs ? (long long)p.row_pairs * p.ldo
+                                                : p.out_split ? p.N : 0;
   if constexpr (EPI == EPI_SWIGLU) {   // v: gate, u: up
 #pragma unroll
     for (int j = J; j < J + 8; ++j) {
@@ -378,6 +384,8 @@ CC_DEV void finish_block(const GemmParams &p, const ProjTile &d, const LaneCol &
         w[j] = reinterpret_cast<const uint16_t *>(p.head_w)[(size_t)tab.tok[r] * p.N + cc];
     }
     [[maybe_unused]] float z[16];
+    const long long norm_lo = p.row_pairs ? (long long)p.row_pairs * p.ld_norm
+                                          : p.norm_split ? p.N : 0;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const bool live = j < n && lc.ok;
@@ -390,7 +398,7 @@ CC_DEV void finish_block(const GemmParams &p, const ProjTile &d, const LaneCol &
         if (live && !dry) reinterpret_cast<float *>(p.out)[row * p.ldo + lc.c0] = x;
         if (p.norm_out)
           store_act(reinterpret_cast<uint16_t *>(p.norm_out) + row * p.ld_norm + lc.c0, x * lc.gain,
-                    p.out_f16 != 0, p.norm_split ? p.N : 0, live && !dry, p.status);
+                    p.out_f16 != 0, norm_lo, live && !dry, p.status);
       }
       h[j] = live ? x * x : 0.f;
     }
@@ -412,6 +420,16 @@ CC_DEV void bulk_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t ba
           "r"(dst),
       "r"(src), "r"(bytes), "r"(bar)
       : "memory");
+}
+// 16 rows of an accumulator (a row pair's two products added).
+CC_DEV void load_block(uint32_t taddr, int row_pairs, float (&v)[16]) {
+  uint32_t r[16], lo[16];
+  tmem_ld16(taddr, r);
+  if (row_pairs) tmem_ld16(taddr + row_pairs, lo);
+  tmem_ld_wait();
+#pragma unroll
+  for (int j = 0; j < 16; ++j)
+    v[j] = __uint_as_float(r[j]) + (row_pairs ? __uint_as_float(lo[j]) : 0.f);
 }
 CC_DEV uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t a;
@@ -611,7 +629,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int hi = p.seq_len ? p.seq_len[b] : p.cap;
       const int i0 = lo + (g - (one_group ? 0 : prefix[b])) * nb;
       const bool bad = lo < 0 || hi > p.cap;   // reported when the prefix was built
-      const int nv = bad ? 0 : max(0, min(nb, hi - i0));   // valid rows of the group
+      // valid rows of the group
+      const int nv = bad ? 0 : max(0, min(p.row_pairs ? p.row_pairs : nb, hi - i0));
       const size_t row0 = (size_t)b * p.cap + i0;
       // two tables in turn: warps are at most one item apart
       const int par = num_g == 1 ? 0 : (int)(it & 1);
@@ -658,12 +677,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int r0 = grp * kBlock; r0 < nv; r0 += 2 * kBlock) {
 #pragma unroll
             for (int w = 0; w < WT; ++w) {
-              uint32_t r[16];
-              tmem_ld16(tacc + w * acc_cols(nb) + r0, r);
-              tmem_ld_wait();
+              float x[16];
+              load_block(tacc + w * acc_cols(nb) + r0, p.row_pairs, x);
               float *o = reinterpret_cast<float *>(ring) + r0 * ROW + w * BM + c;
 #pragma unroll
-              for (int j = 0; j < kBlock; ++j) o[j * ROW] = __uint_as_float(r[j]);
+              for (int j = 0; j < kBlock; ++j) o[j * ROW] = x[j];
             }
           }
           tc_fence_before();
@@ -691,15 +709,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int j = 0; j < 16; ++j) v[j] = u[j] = 0.f;
           if (!dry && S == 1) {
-            uint32_t r[16], r2[16];
-            tmem_ld16(tacc + r0, r);
-            if constexpr (WT == 2) tmem_ld16(tacc + acc_cols(nb) + r0, r2);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              v[j] = __uint_as_float(r[j]);
-              if constexpr (WT == 2) u[j] = __uint_as_float(r2[j]);
-            }
+            load_block(tacc + r0, p.row_pairs, v);
+            if constexpr (WT == 2) load_block(tacc + acc_cols(nb) + r0, p.row_pairs, u);
           } else if (!dry) {
 #pragma unroll 1
             for (int s = 0; s < S; ++s) {   // rank order
@@ -817,7 +828,7 @@ cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorM
 }  // namespace
 
 FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
-                 int sms) {
+                 int row_pairs, int sms) {
   const int wt = w_tiles(epi);
   FewPlan best{};
   best.n_tiles = n_tiles;
@@ -825,6 +836,7 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
   const int nk = ((K + BK - 1) / BK) * (a_split ? 2 : 1);
   const double hbm = (double)n_tiles * wt * BM * K * 2 / 3500.0;   // weight bytes at 6.7 TB/s, 1.9 GHz
   for (int nb = 16; nb <= kMaxRows / wt; nb *= 2) {
+    if (row_pairs && nb != 2 * row_pairs) continue;
     const double groups = (double)seqs * (double)((rows_per_seq + nb - 1) / nb);
     // k-block: the products (2 cycles per row) or their operands' way into
     // shared memory (measured on the Qwen2.5 projections: 266 cycles for 18 KB,

@@ -18,9 +18,10 @@ struct FewPlan {
 };
 
 constexpr int kFewTileCols = 128;   // output columns of a tile
-// The plan for `groups(nb)` row groups: seqs sequences of at most rows_per_seq rows each.
+// The plan for seqs sequences of at most rows_per_seq rows each.  row_pairs > 0:
+// one group of 2 * row_pairs rows (GemmParams::row_pairs).
 FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
-                 int sms);
+                 int row_pairs, int sms);
 // a: A rows x K, box 64 x plan.nb; b (b2, b3): weights N x K, box 64 x 128, and
 // for rotated projections (EPI_QROPE's b, EPI_QKV's b and b2) the 5-D view
 // [heads][head_dim / 32][2][16][K], box {64, 16, 2, head_dim / 32, 128 / head_dim}.

@@ -65,6 +65,9 @@ struct GemmParams {
   int pair;                // run as CTA pairs (256-column tiles): the B tensor
                            // maps' boxes are 128 rows (each CTA loads half of a tile);
                            // raster 1 groups count pairs of row tiles
+  int row_pairs;           // few-row launches: > 0: the A rows are bf16 pairs, lo of row r at row
+                           // r + row_pairs of the same group (products hi W^T + lo W^T), and so
+                           // are the activations written (norm_out; SwiGLU's and Q's out)
   int out_split;           // EPI_SWIGLU, EPI_QROPE (not into the cache): out rows are
                            // [hi | lo], lo at column offset N
   int ab_f16;              // A and W are fp16 (else bf16): the fp16 operand mode

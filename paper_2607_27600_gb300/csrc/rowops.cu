@@ -171,11 +171,13 @@ __global__ void __launch_bounds__(kWarps * 32)
 
 // The inference cycle's embedding with the first layer's RMSNorm begun, over
 // its packed rows r < *total (one block each): h (fp32) = e, xn (bf16) = e * gain
-// (unnormalised) and ss[r] = sum e^2, where e = embed[token of slot rowmap[r]].
+// (unnormalised; row_pairs > 0: also the remainder, at row r + row_pairs) and
+// ss[r] = sum e^2, where e = embed[token of slot rowmap[r]].
 __global__ void __launch_bounds__(256)
     append_embed_kernel(const __nv_bfloat16 *embed, const int32_t *tokens, const int32_t *rowmap,
                         const int32_t *total, const __nv_bfloat16 *gain, float *h,
-                        __nv_bfloat16 *xn, float *ss, int d, int vocab, unsigned *status) {
+                        __nv_bfloat16 *xn, float *ss, int d, int vocab, int row_pairs,
+                        unsigned *status) {
   __shared__ float part[8];
   const int row = blockIdx.x;
   if (row >= *total) return;
@@ -199,6 +201,14 @@ __global__ void __launch_bounds__(256)
     v.z = pack_bf16x2(f[4] * g[4], f[5] * g[5]);
     v.w = pack_bf16x2(f[6] * g[6], f[7] * g[7]);
     *reinterpret_cast<uint4 *>(xn + (size_t)row * d + e) = v;
+    if (row_pairs) {
+      uint4 lo;
+      lo.x = pack_bf16x2(f[0] * g[0] - bf16_lo(v.x), f[1] * g[1] - bf16_hi(v.x));
+      lo.y = pack_bf16x2(f[2] * g[2] - bf16_lo(v.y), f[3] * g[3] - bf16_hi(v.y));
+      lo.z = pack_bf16x2(f[4] * g[4] - bf16_lo(v.z), f[5] * g[5] - bf16_hi(v.z));
+      lo.w = pack_bf16x2(f[6] * g[6] - bf16_lo(v.w), f[7] * g[7] - bf16_hi(v.w));
+      *reinterpret_cast<uint4 *>(xn + (size_t)(row + row_pairs) * d + e) = lo;
+    }
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc = fmaf(f[k], f[k], acc);
   }
@@ -421,12 +431,13 @@ cudaError_t launch_embed(const void *embed, const int32_t *tokens, float *h, int
 
 cudaError_t launch_append_embed(const void *embed, const int32_t *tokens, const AppendRows &r,
                                 int max_rows, const void *gain, float *h, void *xn, float *ss,
-                                int d, int vocab, unsigned *status, cudaStream_t st) {
+                                int d, int vocab, int row_pairs, unsigned *status,
+                                cudaStream_t st) {
   if (max_rows <= 0) return cudaSuccess;
   append_embed_kernel<<<max_rows, 256, 0, st>>>(
       reinterpret_cast<const __nv_bfloat16 *>(embed), tokens, r.rowmap, r.total,
       reinterpret_cast<const __nv_bfloat16 *>(gain), h, reinterpret_cast<__nv_bfloat16 *>(xn), ss,
-      d, vocab, status);
+      d, vocab, row_pairs, status);
   return cudaGetLastError();
 }
 

@@ -34,10 +34,12 @@ cudaError_t launch_append_prepare(const int32_t *seq_len, const int32_t *count,
                                   int32_t *tokens, int32_t *pos, const AppendRows &r, int batch,
                                   int cap, unsigned *status, cudaStream_t st);
 // Packed rows: h fp32 = embed[token], xn bf16 = h * gain, ss = sum h^2 (the
-// first layer's RMSNorm, finished by the projections' row scale).
+// first layer's RMSNorm, finished by the projections' row scale); row_pairs > 0:
+// also xn's remainder, row r's at row r + row_pairs.
 cudaError_t launch_append_embed(const void *embed, const int32_t *tokens, const AppendRows &r,
                                 int max_rows, const void *gain, float *h, void *xn, float *ss,
-                                int d, int vocab, unsigned *status, cudaStream_t st);
+                                int d, int vocab, int row_pairs, unsigned *status,
+                                cudaStream_t st);
 // out bf16 [slot][d] = h fp32 [packed row] (H^(L-1) recorded by the inference cycle)
 cudaError_t launch_store_bf16(const float *h, void *out, int d, const AppendRows &r, int max_rows,
                               cudaStream_t st);
