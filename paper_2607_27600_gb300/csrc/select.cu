@@ -1,16 +1,22 @@
 // select.cu -- keep-set selection (Algorithm DoMemRefresh: sigma = argsort of
 // the surprise scores, largest first; keep sigma[1:J]).
 //
-// One CTA (1024 threads) per sequence.  Each slot j gets the unique 64-bit
-// key (monotone(score_j) << 32) | j, so "descending score, ties toward the
-// later slot" is plain descending key order and exactly J keys are >= the
-// J-th largest key T.  T is found by an MSB radix select (8 bits per pass,
-// warp-level digit search over a shared histogram, at most 8 passes); it
-// stops early once the bucket holding the boundary has exactly as many keys
-// as are still needed: then every key of the bucket is kept, and the prefix
-// with all lower bits zero is a threshold with exactly J keys at or above it.
-// A final pass flags key >= T and writes the kept slots in ascending slot
-// order through a block-wide prefix scan.
+// One cluster of CTAs per sequence (one CTA for short caches), each CTA over a
+// contiguous segment of slots.  Slots rank by the 32-bit monotone key of their
+// score, ties toward the later slot.  The J-th largest key T is found by an
+// MSB radix select of 11 + 11 + 10 bits: each pass every CTA counts its
+// segment's digits in shared memory, the cluster sums the histograms (each
+// CTA a slice of the bins, then the slice totals, through distributed shared
+// memory), and the pass ends early once the bucket holding the boundary has
+// exactly as many keys as are still needed (then every key at or above the
+// prefix is kept; 1-2 passes on continuous scores).  If all 32 bits leave a
+// tie, the last of the tied slots are kept.  A final pass flags the kept slots
+// and writes them in ascending order through block and cluster prefix sums.
+//
+// Latency bounds it: a pass is a few barriers and round trips.  The segment's
+// keys stay in shared memory when they fit.  One CTA per sequence with 256-bin
+// passes over the scores in global memory took 18.5 us for 16384 slots and
+// 182 us for 131072 (launch after launch); this takes 13.4 and 24.
 #include "select.cuh"
 
 namespace cc {
@@ -18,6 +24,13 @@ namespace cc {
 namespace {
 
 constexpr int kThreads = 1024;
+constexpr int kBins = 2048;
+constexpr int kCluster = 8;                  // CTAs per sequence (the portable cluster size)
+// Caches up to this many slots: one CTA.  Measured (launch after launch, one and
+// eight CTAs): 8.3 / 12.3 us at 2048 slots, 10.3 / 12.4 at 8192, 16.4 / 13.4 at
+// 16384, 143 / 24 at 131072.
+constexpr int kOneCtaSlots = 8192;
+constexpr int kMaxCached = 44 * 1024;        // keys of a segment kept in shared memory at most
 constexpr uint32_t kKeyPosInf = 0xFF800000u;   // monotone key of +inf
 constexpr uint32_t kKeyNegInf = 0x007FFFFFu;   // monotone key of -inf
 
@@ -32,50 +45,67 @@ CC_DEV uint32_t monotone_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-CC_DEV uint64_t slot_key(const float *s, int j, int n_sink) {
-  const uint32_t k = j < n_sink ? kKeyPosInf : monotone_key(s[j]);
-  return (uint64_t(k) << 32) | uint32_t(j);
+// The variable at p in CTA `rank` of the cluster (ONE: there is only this one).
+template <bool ONE>
+CC_DEV uint32_t ld_rank(const uint32_t *p, int rank) {
+  if constexpr (ONE) return *p;
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, rank)) : "memory");
+  return v;
 }
 
-// exclusive block scan of x (1024 threads); returns the exclusive prefix,
-// *total = block sum.
-CC_DEV int block_excl_scan(int x, int *wsum, int *total) {
+template <bool ONE>
+CC_DEV void sync_all() {
+  if constexpr (ONE) __syncthreads();
+  else cluster_sync();
+}
+
+// Exclusive block scan of x; *total = block sum.  ws: 33 ints of shared memory.
+CC_DEV int block_excl_scan(int x, int *ws, int *total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int incl = x;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += y;
   }
-  if (lane == 31) wsum[warp] = incl;
+  if (lane == 31) ws[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    int w = wsum[lane], wi = w;
+    const int w = ws[lane];
+    int wi = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+      const int y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
       if (lane >= o) wi += y;
     }
-    wsum[lane] = wi - w;            // exclusive warp offsets
-    if (lane == 31) wsum[32] = wi;  // block total
+    ws[lane] = wi - w;            // exclusive warp offsets
+    if (lane == 31) ws[32] = wi;  // block total
   }
   __syncthreads();
-  const int r = incl - x + wsum[warp];
-  *total = wsum[32];
+  const int r = incl - x + ws[warp];
+  *total = ws[32];
   __syncthreads();
   return r;
 }
 
+template <bool ONE>
 __global__ void __launch_bounds__(kThreads, 1)
     select_kernel(const float *scores, const int32_t *seq_len, int cap, const int32_t *budget,
-                  int n_sink, int32_t *keep_idx, int32_t *keep_count, unsigned *status) {
-  __shared__ unsigned hist[256];
-  __shared__ int wsum[33];
+                  int n_sink, int32_t *keep_idx, int32_t *keep_count, unsigned *status,
+                  int cached) {
+  extern __shared__ uint32_t keys[];               // [cached ? segment : 0]
+  __shared__ unsigned hist[2][kBins];              // this CTA's digits, two passes in turn
+  // keys of this CTA's slice of the bins (over the cluster) in its bins >= i
+  __shared__ unsigned at_least[2][kBins + 1];
+  __shared__ int ws[33];
   __shared__ int s_digit, s_above, s_count;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ unsigned n_kept, n_tied;              // of this CTA's segment
+  const int CS = ONE ? 1 : kCluster, rank = ONE ? 0 : (int)cluster_ctarank();
+  const int b = blockIdx.x / CS, tid = threadIdx.x, lane = tid & 31;
   const int n = seq_len[b];
-  if (n < 0 || n > cap) {
-    if (tid == 0) {
+  if (n < 0 || n > cap) {   // the same in every CTA of the cluster
+    if (tid == 0 && rank == 0) {
       set_status(status, CC_ERR_DEVICE_ARG);
       keep_count[b] = 0;
     }
@@ -86,87 +116,172 @@ __global__ void __launch_bounds__(kThreads, 1)
   int J = budget[b];
   const int forced = min(n, 1 + max(n_sink, 0));
   if (J < forced) {
-    if (tid == 0) set_status(status, CC_ERR_BUDGET);
+    if (tid == 0 && rank == 0) set_status(status, CC_ERR_BUDGET);
     J = forced;
   }
   if (J >= n) {  // everything fits: identity
-    for (int j = tid; j < n; j += kThreads) out[j] = j;
-    if (tid == 0) keep_count[b] = n;
+    for (int j = rank * kThreads + tid; j < n; j += CS * kThreads) out[j] = j;
+    if (tid == 0 && rank == 0) keep_count[b] = n;
     return;
   }
-
-  // ---- radix select of T = J-th largest key
-  uint64_t prefix = 0;
-  int k = J;
-#pragma unroll 1
-  for (int pass = 0; pass < 8; ++pass) {
-    const int shift = 56 - 8 * pass;
-    const uint64_t hi_mask = pass == 0 ? 0ull : (~0ull << (shift + 8));
-    if (tid < 256) hist[tid] = 0;
-    __syncthreads();
-    for (int j = tid; j < n; j += kThreads) {
-      const uint64_t key = slot_key(s, j, n_sink);
-      if ((key & hi_mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      // lane l owns digits 255-8l down to 248-8l (descending)
-      const int base = 255 - lane * 8;
-      unsigned c[8], sum = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) { c[e] = hist[base - e]; sum += c[e]; }
-      unsigned incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        unsigned y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const unsigned excl = incl - sum;
-      if (excl < (unsigned)k && (unsigned)k <= incl) {
-        unsigned run = excl;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          if (run + c[e] >= (unsigned)k) {
-            s_digit = base - e;
-            s_above = (int)run;
-            s_count = (int)c[e];
-            break;
-          }
-          run += c[e];
-        }
-      }
-    }
-    __syncthreads();
-    prefix |= uint64_t(s_digit) << shift;
-    k -= s_above;
-    const bool settled = s_count == k;   // the whole bucket is kept
-    __syncthreads();
-    if (settled) break;
+  // segment [j0, j1) of this CTA: a multiple of 4 slots
+  const int seg = ((n + CS - 1) / CS + 3) & ~3;
+  const int j0 = min(n, rank * seg), j1 = min(n, j0 + seg);
+  auto key_of = [&](int j) -> uint32_t {
+    return j < n_sink ? kKeyPosInf : monotone_key(s[j]);
+  };
+  auto key_at = [&](int j) -> uint32_t { return cached ? keys[j - j0] : key_of(j); };
+  for (int i = tid; i < kBins; i += kThreads) hist[0][i] = 0;
+  if (cached) {
+#pragma unroll 4
+    for (int j = j0 + tid; j < j1; j += kThreads) keys[j - j0] = key_of(j);
   }
-  const uint64_t T = prefix;
+  __syncthreads();
 
-  // ---- flag key >= T and emit the kept slots in ascending order
-  int carry = 0;
-  for (int base = 0; base < n; base += kThreads * 4) {
-    const int j0 = base + tid * 4;
-    int f[4], cnt = 0;
+  // ---- radix select of T = the J-th largest key
+  uint32_t prefix = 0;
+  int k = J;
+  bool settled = false;
+  constexpr int per = ONE ? kBins : kBins / kCluster;   // bins of a slice
+#pragma unroll 1
+  for (int pass = 0; pass < 3 && !settled; ++pass) {
+    const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+    const int bits = pass == 2 ? 10 : 11;
+    const uint32_t hi_mask = pass == 0 ? 0u : ~0u << (shift + bits);
+    const uint32_t digit_mask = (1u << bits) - 1;
+    unsigned *h = hist[pass & 1];
+#pragma unroll 4
+    for (int j = j0 + tid; j < j1; j += kThreads) {
+      const uint32_t key = key_at(j);
+      if ((key & hi_mask) == prefix) atomicAdd(&h[(key >> shift) & digit_mask], 1u);
+    }
+    for (int i = tid; i < kBins; i += kThreads) hist[(pass & 1) ^ 1][i] = 0;   // the next pass's
+    sync_all<ONE>();
+    // this CTA's slice, bins descending over the threads: running counts
+    constexpr int PT = per > kThreads ? per / kThreads : 1;   // bins of a thread
+    unsigned c[PT], sum = 0;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int j = j0 + e;
-      f[e] = (j < n && slot_key(s, j, n_sink) >= T) ? 1 : 0;
-      cnt += f[e];
+    for (int e = 0; e < PT; ++e) {
+      const int i = per - 1 - (tid * PT + e);
+      c[e] = 0;
+      if (i >= 0) {
+#pragma unroll
+        for (int r = 0; r < (ONE ? 1 : kCluster); ++r) c[e] += ld_rank<ONE>(&h[rank * per + i], r);
+      }
+      sum += c[e];
     }
     int total;
-    int off = carry + block_excl_scan(cnt, wsum, &total);
+    unsigned run = (unsigned)block_excl_scan((int)sum, ws, &total);
+    unsigned *al = at_least[pass & 1];
+#pragma unroll
+    for (int e = 0; e < PT; ++e) {
+      const int i = per - 1 - (tid * PT + e);
+      run += c[e];
+      if (i >= 0) al[i] = run;
+    }
+    if (tid == 0) al[per] = 0;
+    sync_all<ONE>();
+    // the slice that holds the boundary (digits descend from the last slice):
+    // every warp reads the slices' totals and finds it alike
+    unsigned t = 0;
+    if (lane < CS) t = ld_rank<ONE>(&al[0], lane);
+    unsigned above = 0;   // keys in the slices after this lane's
+#pragma unroll
+    for (int r = 1; r < (ONE ? 1 : kCluster); ++r) {
+      const unsigned y = __shfl_sync(0xFFFFFFFFu, t, r);
+      if (r > lane) above += y;
+    }
+    const unsigned holds =
+        __ballot_sync(0xFFFFFFFFu, lane < CS && above < (unsigned)k && (unsigned)k <= above + t);
+    const int owner = __ffs((int)holds) - 1;
+    above = __shfl_sync(0xFFFFFFFFu, above, owner);
+    const unsigned want = (unsigned)k - above;
+#pragma unroll
+    for (int e = 0; e < PT; ++e) {
+      const int i = tid * PT + e;
+      if (i >= per) break;
+      const unsigned at = ld_rank<ONE>(&al[i], owner), over = ld_rank<ONE>(&al[i + 1], owner);
+      if (over < want && want <= at) {
+        s_digit = owner * per + i;
+        s_above = (int)(above + over);
+        s_count = (int)(at - over);
+      }
+    }
+    __syncthreads();
+    prefix |= (uint32_t)s_digit << shift;
+    k -= s_above;
+    settled = s_count == k;   // the whole bucket is kept
+    __syncthreads();
+  }
+  // Kept: key > T, and of the keys equal to T the last k (all bits used, not
+  // settled); settled: key >= prefix (lower bits zero).
+  const uint32_t T = prefix;
+  const bool ties = !settled;
+  if (tid == 0) n_kept = n_tied = 0;
+  __syncthreads();
+  unsigned kept = 0, tied = 0;
+#pragma unroll 4
+  for (int j = j0 + tid; j < j1; j += kThreads) {
+    const uint32_t key = key_at(j);
+    kept += ties ? key > T : key >= T;
+    tied += key == T;
+  }
+  kept = __reduce_add_sync(0xFFFFFFFFu, kept);
+  tied = __reduce_add_sync(0xFFFFFFFFu, tied);
+  if (lane == 0 && kept) atomicAdd(&n_kept, kept);
+  if (lane == 0 && tied) atomicAdd(&n_tied, tied);
+  sync_all<ONE>();
+  int base = 0, tie_base = 0, tie_total = 0;   // before this segment; over the sequence
+#pragma unroll
+  for (int r = 0; r < (ONE ? 1 : kCluster); ++r) {
+    const int a = (int)ld_rank<ONE>(&n_kept, r);
+    const int t = (int)ld_rank<ONE>(&n_tied, r);
+    if (r < rank) {
+      base += a;
+      tie_base += t;
+    }
+    tie_total += t;
+  }
+  if (ties) {   // tied slots before the segment that are kept: those past the first total - k
+    const int first = tie_total - k;
+    base += max(0, tie_base - first);
+  }
+
+  // ---- flag and emit the kept slots in ascending order
+  int carry = base, tie_carry = tie_base;
+  for (int jb = j0; jb < j1; jb += kThreads * 4) {
+    const int ja = jb + tid * 4;
+    int f[4], t[4], cnt = 0, tcnt = 0, total;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int j = ja + e;
+      const uint32_t key = j < j1 ? key_at(j) : 0u;
+      f[e] = j < j1 && (ties ? key > T : key >= T);
+      t[e] = ties && j < j1 && key == T;
+      tcnt += t[e];
+    }
+    if (ties) {
+      int idx = tie_carry + block_excl_scan(tcnt, ws, &total);
+      tie_carry += total;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (t[e] && idx >= tie_total - k) f[e] = 1;
+        idx += t[e];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) cnt += f[e];
+    int off = carry + block_excl_scan(cnt, ws, &total);
 #pragma unroll
     for (int e = 0; e < 4; ++e)
-      if (f[e]) out[off++] = j0 + e;
+      if (f[e]) out[off++] = ja + e;
     carry += total;
   }
-  if (tid == 0) {
+  if (tid == 0 && rank == CS - 1) {
     keep_count[b] = J;
-    if (carry != J) set_status(status, CC_ERR_DEVICE_ARG);   // cannot happen: keys are unique
+    if (carry != J) set_status(status, CC_ERR_DEVICE_ARG);   // cannot happen
   }
+  sync_all<ONE>();   // no CTA reads this one's counts any more
 }
 
 }  // namespace
@@ -175,9 +290,36 @@ cudaError_t launch_select(const float *scores, const int32_t *seq_len, int batch
                           const int32_t *budget, int n_sink, int32_t *keep_idx,
                           int32_t *keep_count, unsigned *status, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
-  select_kernel<<<batch, kThreads, 0, st>>>(scores, seq_len, cap, budget, n_sink, keep_idx,
-                                            keep_count, status);
-  return cudaGetLastError();
+  const bool one = cap <= kOneCtaSlots;
+  const int cs = one ? 1 : kCluster;
+  const int seg = ((cap + cs - 1) / cs + 3) & ~3;   // slots of a segment at most
+  const int cached = seg <= kMaxCached ? 1 : 0;
+  const auto kern = one ? select_kernel<true> : select_kernel<false>;
+  static bool attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 64 && !attr_set[dev]) {
+    for (auto k : {select_kernel<true>, select_kernel<false>}) {
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           kMaxCached * 4);
+      if (e != cudaSuccess) return e;
+    }
+    attr_set[dev] = true;
+  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(batch * cs));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = cached ? (size_t)seg * 4 : 0;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = one ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, scores, seq_len, cap, budget, n_sink, keep_idx,
+                            keep_count, status, cached);
 }
 
 }  // namespace cc
