@@ -1098,7 +1098,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
 }
 
 // compaction plan: arrays and unit counts
-// Compaction workspace: unit_base table | flags (zeroed per call) | readers table (-1 per call)
+// Compaction workspace: unit_base table | flags | readers table (cleared per call)
 struct CompactPlan {
   CompactParams p;
   size_t base_bytes, flags_bytes, deps_bytes, ws_bytes;
@@ -1136,7 +1136,8 @@ cc_status compact_plan(const cc_model_cfg *c, const cc_kv_cache *kv, CompactPlan
     A.bulk = bulk ? 1 : 0;
     A.paged = paged ? 1 : 0;
     A.head_major = head_major ? 1 : 0;
-    A.rows_per_chunk = bulk ? (row_bytes <= p.stage_bytes ? p.stage_bytes / row_bytes : 0)
+    A.rows_per_chunk = bulk ? std::min(kCompactMaxRows, row_bytes <= p.stage_bytes
+                                                            ? p.stage_bytes / row_bytes : 0)
                             : std::min(kCompactSmallRows, p.stage_bytes / 4);
     if (A.rows_per_chunk < 1) return false;
     A.n_chunks = (kv->cap + A.rows_per_chunk - 1) / A.rows_per_chunk;
@@ -1177,15 +1178,14 @@ cc_status compact_plan(const cc_model_cfg *c, const cc_kv_cache *kv, CompactPlan
   return CC_OK;
 }
 
-// Points the plan at workspace `ws` and clears what must start cleared.
-cc_status compact_bind(CompactPlan &plan, void *ws, cudaStream_t st) {
+// Points the plan at workspace `ws`.
+void compact_bind(CompactPlan &plan, void *ws) {
   uint8_t *w = reinterpret_cast<uint8_t *>(ws);
   plan.p.unit_base = reinterpret_cast<int *>(w);
   plan.p.flags = reinterpret_cast<unsigned *>(w + plan.base_bytes);
   plan.p.deps = reinterpret_cast<int2 *>(w + plan.base_bytes + plan.flags_bytes);
-  CC_TRY(cudaMemsetAsync(plan.p.flags, 0, plan.flags_bytes, st));
-  CC_TRY(cudaMemsetAsync(plan.p.deps, 0xFF, plan.deps_bytes, st));
-  return CC_OK;
+  plan.p.flags_bytes = plan.flags_bytes;
+  plan.p.deps_bytes = plan.deps_bytes;
 }
 
 }  // namespace
@@ -1487,7 +1487,7 @@ cc_status cc_compact_kv(const cc_model_cfg *cfg, const cc_kv_cache *cache,
   DevState *dev;
   if (!dev_state(&dev)) return device_fail();
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if ((s = compact_bind(plan, ws, st)) != CC_OK) return s;
+  compact_bind(plan, ws);
   plan.p.keep_idx = keep_idx;
   plan.p.keep_count = keep_count;
   plan.p.seq_len = cache->seq_len;
@@ -1706,14 +1706,14 @@ cudaError_t wait_kv_ready(const cc_kv_cache *kv, int l0, int l1, cudaStream_t st
 
 
 cc_status compact_plan_bind(const cc_model_cfg *cfg, const cc_kv_cache *cache, CompactParams &p,
-                            void *scratch, size_t scratch_cap, cudaStream_t st) {
+                            void *scratch, size_t scratch_cap) {
   static CompactPlan plan;
   static std::mutex mu;
   std::lock_guard<std::mutex> lk(mu);
   cc_status s = compact_plan(cfg, cache, plan);
   if (s != CC_OK) return s;
   if (plan.ws_bytes > scratch_cap) return CC_ERR_WORKSPACE;
-  if ((s = compact_bind(plan, scratch, st)) != CC_OK) return s;
+  compact_bind(plan, scratch);
   p = plan.p;
   return CC_OK;
 }

@@ -21,14 +21,16 @@
 // pre-pass over keep_idx (deps_kernel): chunk u's readers are the chunks
 // holding the first and last k with keep_idx[k] in u.
 //
-// A planning pre-pass numbers only the units that hold kept slots.  The
-// kernel is launched cooperatively (every warp resident) and warp w takes
+// A planning pre-pass numbers only the units that hold kept slots (and clears
+// the tables that start cleared).  The kernel is launched cooperatively (every warp resident) and warp w takes
 // units w, w + W, w + 2W, ... in ascending order, no atomics.  A unit waits
 // only on lower units and publishing never waits: the lowest unpublished
 // unit's warp is never blocked, so nothing can deadlock.  Each warp runs its
 // own two-buffer pipeline: the loads of its next unit are in flight while
-// the current unit waits and stores.  Each element is read once and written
-// once; rows with keep_idx[k] == k are not moved.
+// the current unit waits and stores, and the lookups of the unit after that
+// (its rows, its readers, whether it publishes) run while those loads fly.
+// Each element is read once and written once; rows with keep_idx[k] == k are
+// not moved.
 #include "compact.cuh"
 
 namespace cc {
@@ -63,6 +65,7 @@ CC_DEV bool wait_flag(const unsigned *flag, unsigned *status) {
 // Pre-pass: for every chunk u of class cls (chunks of class_rows[cls] slots),
 // the first and last chunk whose destinations read sources inside u.
 __global__ void deps_kernel(const __grid_constant__ CompactParams p) {
+  pdl_wait();
   const int cls = blockIdx.z, b = blockIdx.y;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   int J = p.keep_count[b];
@@ -80,11 +83,25 @@ __global__ void deps_kernel(const __grid_constant__ CompactParams p) {
   if (k == J - 1 || src_of(k + 1) / C != u) deps[u].y = k / C;
 }
 
-// Pre-pass: unit_base[a*batch + b] = first unit of (array a, sequence b),
-// counting ceil(keep_count[b] / rows_per_chunk) units each; the last entry
-// is the number of units.  One block: an exclusive scan over the
-// (array, sequence) pairs, 1024 pairs per round.
+// Pre-pass.  Block 0: unit_base[a*batch + b] = first unit of (array a,
+// sequence b), counting ceil(keep_count[b] / rows_per_chunk) units each; the
+// last entry is the number of units (an exclusive scan over the (array,
+// sequence) pairs, 1024 pairs per round).  The other blocks clear the flags (0)
+// and the readers table (-1).
+constexpr int kPlanBlocks = 65;
+
 __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ CompactParams p) {
+  pdl_trigger();   // deps_kernel waits for this grid before it writes
+  if (blockIdx.x > 0) {
+    const size_t nf = p.flags_bytes / 16, nd = p.deps_bytes / 16;
+    uint4 *f = reinterpret_cast<uint4 *>(p.flags), *d = reinterpret_cast<uint4 *>(p.deps);
+    for (size_t i = (size_t)(blockIdx.x - 1) * 1024 + threadIdx.x; i < nf + nd;
+         i += (size_t)(kPlanBlocks - 1) * 1024) {
+      if (i < nf) f[i] = make_uint4(0u, 0u, 0u, 0u);
+      else d[i - nf] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    return;
+  }
   __shared__ int warp_sums[32];
   __shared__ int carry;
   const int n_pairs = p.n_arrays * p.batch;
@@ -132,10 +149,15 @@ __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ Comp
   if (threadIdx.x == 0) p.unit_base[n_pairs] = carry;
 }
 
+// A warp's unit and what was looked up for it before its loads are issued.
 struct Unit {
   int t;          // unit number (>= total: none)
   int a, b, c;    // array, sequence, chunk
   int k0, k1;     // destination slots [k0, k1)
+  int src;        // bulk arrays: this lane's row k0 + lane comes from slot src,
+  bool moves;     //   and moves (its source differs and both rows exist)
+  bool publish;   // a higher unit waits for this one's reads
+  int dep_lo, dep_hi;   // chunks below c that read from this one's destinations
   bool loaded;    // bulk loads issued into the buffer
 };
 
@@ -172,28 +194,6 @@ __global__ void __launch_bounds__(kThreads)
   const int total = unit_base[n_pairs];
   const int stride = gridDim.x * n_warps;
   int next_t = blockIdx.x * n_warps + warp;
-  auto take = [&]() -> Unit {
-    Unit u;
-    u.t = next_t;
-    next_t += stride;
-    u.loaded = false;
-    u.a = u.b = u.c = u.k0 = u.k1 = 0;
-    if (u.t >= total) return u;
-    int lo = 0, hi = n_pairs - 1;   // last pair whose first unit <= t
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (unit_base[mid] <= u.t) lo = mid; else hi = mid - 1;
-    }
-    u.a = lo / p.batch;
-    u.b = lo - u.a * p.batch;
-    u.c = u.t - unit_base[lo];
-    const CompactArray &A = p.arr[u.a];
-    int J = p.keep_count[u.b];
-    if (J < 0 || J > p.cap) J = 0;
-    u.k0 = u.c * A.rows_per_chunk;
-    u.k1 = min(u.k0 + A.rows_per_chunk, J);
-    return u;
-  };
 
   // Source row of destination k; entries that are not ascending or out of
   // range are copied onto themselves (and reported by `report`).
@@ -236,36 +236,76 @@ __global__ void __launch_bounds__(kThreads)
       bulk_store(base + (size_t)arow(A, b, k) * A.row_bytes, src, A.row_bytes);
     }
   };
-  // A bulk row moves when its source differs and both rows exist.
-  auto moves = [&](const CompactArray &A, int b, int k, int src) {
-    return src != k && (!A.paged || (arow(A, b, k) >= 0 && arow(A, b, src) >= 0));
+  // The warp's next unit, with its lookups.
+  auto take = [&]() -> Unit {
+    Unit u;
+    u.t = next_t;
+    next_t += stride;
+    u.loaded = u.moves = u.publish = false;
+    u.a = u.b = u.c = u.k0 = u.k1 = u.src = 0;
+    u.dep_lo = 0;
+    u.dep_hi = -1;
+    if (u.t >= total) return u;
+    int lo = 0, hi = n_pairs - 1;   // last pair whose first unit <= t
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (unit_base[mid] <= u.t) lo = mid; else hi = mid - 1;
+    }
+    u.a = lo / p.batch;
+    u.b = lo - u.a * p.batch;
+    u.c = u.t - unit_base[lo];
+    const CompactArray &A = p.arr[u.a];
+    const int C = A.rows_per_chunk;
+    const int32_t *kidx = p.keep_idx + (size_t)u.b * p.cap;
+    u.k0 = u.c * C;
+    // (a unit that exists has a row, so k0 < J; rows past J read harmlessly
+    // below cap and are dropped)
+    int J = p.keep_count[u.b];
+    const int k = min(u.k0 + lane, p.cap - 1);
+    const int first = kidx[u.k0], mine = A.bulk ? kidx[k] : 0;
+    int2 d = make_int2(-1, -1);
+    if (u.c > 0)
+      d = p.deps[p.class_offset[A.dep_class] + (size_t)u.b * p.class_chunks[A.dep_class] + u.c];
+    if (J < 0 || J > p.cap) J = 0;
+    u.k1 = min(u.k0 + C, J);
+    if (u.k0 >= u.k1) return u;
+    const int last = kidx[u.k1 - 1];
+    auto fix = [&](int kk, int s) { return s < kk || s >= p.cap ? kk : s; };
+    if (A.bulk && u.k0 + lane < u.k1) {
+      u.src = fix(k, mine);
+      if (u.src != mine) set_status(p.status, CC_ERR_DEVICE_ARG);
+      u.moves = u.src != k && (!A.paged || (arow(A, u.b, k) >= 0 && arow(A, u.b, u.src) >= 0));
+    }
+    // A unit is waited on exactly when one of its source chunks is an active
+    // destination chunk above its own (the readers table lists it there), so
+    // only such units publish (a release store costs a memory barrier).
+    const int active = (J + C - 1) / C;
+    const int lo_u = max(u.c + 1, fix(u.k0, first) / C);
+    const int hi_u = min(active - 1, fix(u.k1 - 1, last) / C);
+    u.publish = lo_u <= hi_u && u.t != p.withhold_unit;
+    u.dep_lo = max(d.x, 0);
+    u.dep_hi = min(d.y, u.c - 1);
+    return u;
   };
 
   // Issues the reads of unit u into buffer slot s.
   auto load = [&](Unit &u, int s) {
     if (u.t >= total || u.k0 >= u.k1) return;
     const CompactArray &A = p.arr[u.a];
-    const int32_t *kidx = p.keep_idx + (size_t)u.b * p.cap;
-    uint8_t *base = reinterpret_cast<uint8_t *>(A.base);
-    const size_t seq_off = (size_t)u.b * p.cap;
     if (A.bulk) {
-      int moving = 0;
-      for (int k = u.k0 + lane; k < u.k1; k += 32) moving += moves(A, u.b, k, source(kidx, k, false));
-      moving = __reduce_add_sync(0xFFFFFFFFu, moving);
+      const int moving = __popc(__ballot_sync(0xFFFFFFFFu, u.moves));
       if (moving == 0) return;
       if (lane == 0) mbar_arrive_expect_tx(&bars[warp][s], (uint32_t)(moving * A.row_bytes));
       __syncwarp();
-      for (int k = u.k0 + lane; k < u.k1; k += 32) {
-        const int src = source(kidx, k, true);
-        if (moves(A, u.b, k, src))
-          row_load(A, u.b, src, buf[s] + (size_t)(k - u.k0) * A.row_bytes, &bars[warp][s]);
-      }
+      if (u.moves)
+        row_load(A, u.b, u.src, buf[s] + (size_t)lane * A.row_bytes, &bars[warp][s]);
       u.loaded = true;
     } else {   // 4-byte rows: plain loads staged in shared memory
+      const int32_t *kidx = p.keep_idx + (size_t)u.b * p.cap;
+      const uint32_t *base = reinterpret_cast<const uint32_t *>(A.base) + (size_t)u.b * p.cap;
       uint32_t *st = reinterpret_cast<uint32_t *>(buf[s]);
 #pragma unroll 8
-      for (int k = u.k0 + lane; k < u.k1; k += 32)
-        st[k - u.k0] = reinterpret_cast<const uint32_t *>(base)[seq_off + source(kidx, k, true)];
+      for (int k = u.k0 + lane; k < u.k1; k += 32) st[k - u.k0] = base[source(kidx, k, true)];
     }
   };
 
@@ -273,6 +313,7 @@ __global__ void __launch_bounds__(kThreads)
   load(cur, 0);
   Unit nxt = take();
   load(nxt, 1);
+  Unit nn = take();
   for (int i = 0; cur.t < total; ++i) {
     const int s = i & 1;
     const CompactArray &A = p.arr[cur.a];
@@ -283,58 +324,34 @@ __global__ void __launch_bounds__(kThreads)
     }
     __syncwarp();
     // ---- 2. publish; 3. wait for the lower units that read our destinations
-    // A unit is waited on exactly when one of its source chunks is an active
-    // destination chunk above its own (the readers table lists it there), so
-    // only such units publish (a release store costs a memory barrier).
     bool go = true;
     if (lane == 0) {
-      if (cur.k0 < cur.k1) {
-        const int32_t *kidx = p.keep_idx + (size_t)cur.b * p.cap;
-        const int C = A.rows_per_chunk;
-        int J = p.keep_count[cur.b];
-        J = (J < 0 || J > p.cap) ? 0 : J;
-        const int active = (J + C - 1) / C;
-        const int lo_u = max(cur.c + 1, source(kidx, cur.k0, false) / C);
-        const int hi_u = min(active - 1, source(kidx, cur.k1 - 1, false) / C);
-        if (lo_u <= hi_u && cur.t != p.withhold_unit) st_release(&p.flags[cur.t], 1u);
-      }
-      bool waited = false;
-      if (cur.k0 < cur.k1 && cur.c > 0) {
-        const int2 d = p.deps[p.class_offset[A.dep_class] +
-                              (size_t)cur.b * p.class_chunks[A.dep_class] + cur.c];
-        const int hi = min(d.y, cur.c - 1);
-        for (int c2 = max(d.x, 0); c2 <= hi && go; ++c2) {
-          go = wait_flag(&p.flags[unit_base[cur.a * p.batch + cur.b] + c2], p.status);
-          waited = true;
-        }
-      }
-      if (waited) fence_proxy_async_global();
+      if (cur.publish) st_release(&p.flags[cur.t], 1u);
+      for (int c2 = cur.dep_lo; c2 <= cur.dep_hi && go; ++c2)
+        go = wait_flag(&p.flags[cur.t - cur.c + c2], p.status);
+      if (cur.dep_lo <= cur.dep_hi) fence_proxy_async_global();
     }
     go = __shfl_sync(0xFFFFFFFFu, go ? 1 : 0, 0) != 0;
     // ---- 4. write the destinations
     if (go && cur.k0 < cur.k1) {
-      const int32_t *kidx = p.keep_idx + (size_t)cur.b * p.cap;
-      uint8_t *base = reinterpret_cast<uint8_t *>(A.base);
-      const size_t seq_off = (size_t)cur.b * p.cap;
       if (A.bulk) {
         if (cur.loaded) {
-          for (int k = cur.k0 + lane; k < cur.k1; k += 32)
-            if (moves(A, cur.b, k, source(kidx, k, false)))
-              row_store(A, cur.b, k, buf[s] + (size_t)(k - cur.k0) * A.row_bytes);
+          if (cur.moves)
+            row_store(A, cur.b, cur.k0 + lane, buf[s] + (size_t)lane * A.row_bytes);
           bulk_commit();
         }
       } else {
+        uint32_t *base = reinterpret_cast<uint32_t *>(A.base) + (size_t)cur.b * p.cap;
         const uint32_t *st = reinterpret_cast<const uint32_t *>(buf[s]);
-        for (int k = cur.k0 + lane; k < cur.k1; k += 32)
-          reinterpret_cast<uint32_t *>(base)[seq_off + k] = st[k - cur.k0];
+        for (int k = cur.k0 + lane; k < cur.k1; k += 32) base[k] = st[k - cur.k0];
       }
     }
     bulk_wait_all_read();   // buffer s may be refilled
     __syncwarp();
-    Unit nn = take();
     load(nn, s);
     cur = nxt;
     nxt = nn;
+    nn = take();   // its lookups run while the loads just issued are in flight
   }
   bulk_wait_all();
 }
@@ -390,12 +407,11 @@ cudaError_t launch_compact(const CompactParams &p, int sms, cudaStream_t st) {
   for (int cls = 0; cls < p.n_classes; ++cls) {
     if (p.class_rows[cls] <= 0) return cudaErrorInvalidValue;
   }
-  plan_kernel<<<1, 1024, 0, st>>>(p);
+  plan_kernel<<<kPlanBlocks, 1024, 0, st>>>(p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const dim3 dgrid((p.cap + 255) / 256, p.batch, p.n_classes);
-  deps_kernel<<<dgrid, 256, 0, st>>>(p);
-  e = cudaGetLastError();
+  e = launch_pdl(deps_kernel, dgrid, dim3(256), 0, st, p);
   if (e != cudaSuccess) return e;
   // cooperative: every warp resident, so the static unit order cannot deadlock
   void *args[] = {const_cast<CompactParams *>(&p)};

@@ -19,6 +19,8 @@ constexpr int kMaxCompactArrays = 2 * 128 + 3;
 // gathers per lane, so a sequence's few units spread over many warps
 // instead of one warp walking all of them.
 constexpr int kCompactSmallRows = 256;
+// Rows of a bulk unit at most: one per lane.
+constexpr int kCompactMaxRows = 32;
 constexpr int kMaxDepClasses = 3;        // distinct chunk sizes (K/V rows, H rows, 4-byte rows)
 
 struct CompactArray {
@@ -41,10 +43,11 @@ struct CompactParams {
   int32_t *seq_len;           // [batch], set to keep_count
   int *unit_base;             // [n_arrays*batch + 1] first unit of each (array, sequence),
                               // written by the planning pre-pass (units past keep_count skipped)
-  unsigned *flags;            // [total_units], zeroed before launch
-  int2 *deps;                 // readers table, (-1,-1)-filled before launch: per class c,
+  unsigned *flags;            // [total_units], zeroed by the planning pre-pass
+  int2 *deps;                 // readers table, (-1,-1)-filled by it: per class c,
                               // [batch][class_chunks[c]] at class_offset[c]: first and
                               // last chunk reading sources inside each chunk
+  size_t flags_bytes, deps_bytes;   // multiples of 16
   int n_classes;
   int class_rows[kMaxDepClasses];
   int class_chunks[kMaxDepClasses];
@@ -66,7 +69,7 @@ bool compact_shape(int max_row_bytes, int &stage_bytes, int &warps);
 // Sets p.ub_cached when the unit table fits beside the staging buffers.
 void compact_cache_units(CompactParams &p);
 size_t compact_smem_bytes(const CompactParams &p);
-// Launches the pre-passes and the (cooperative) compaction; `sms` = SM count.
+// Launches the pre-passes (which clear flags and deps) and the (cooperative) compaction; `sms` = SM count.
 cudaError_t launch_compact(const CompactParams &p, int sms, cudaStream_t st);
 
 }  // namespace cc

@@ -57,10 +57,9 @@ extern "C" cc_status cc_compact_kv_static(const cc_model_cfg *cfg, const cc_kv_c
   if (!cc::current_device_info(&status, &sms)) return CC_ERR_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // one plan build: rejected (CC_ERR_WORKSPACE, nothing enqueued) when its
-  // scratch exceeds the array; else the flags start at zero and the readers
-  // table at -1 (cleared on `st`), since the array keeps the last call's contents
-  if ((s = cc::compact_plan_bind(cfg, cache, p, scratch, kStaticScratchBytes, st)) != CC_OK)
-    return s;
+  // scratch exceeds the array (the launch clears the flags and the readers
+  // table, since the array keeps the last call's contents)
+  if ((s = cc::compact_plan_bind(cfg, cache, p, scratch, kStaticScratchBytes)) != CC_OK) return s;
   p.keep_idx = keep_idx;
   p.keep_count = keep_count;
   p.seq_len = cache->seq_len;

@@ -7,10 +7,9 @@ namespace cc {
 
 // Builds the compaction plan of `cache` (arrays, work units; the same checks
 // as cc_compact_kv) once, rejects it with CC_ERR_WORKSPACE when its scratch
-// exceeds `scratch_cap` bytes, else places the scratch at `scratch` and
-// enqueues on `st` the clearing of what must start cleared.
+// exceeds `scratch_cap` bytes, else places the scratch at `scratch`.
 cc_status compact_plan_bind(const cc_model_cfg *cfg, const cc_kv_cache *cache, CompactParams &p,
-                            void *scratch, size_t scratch_cap, cudaStream_t st);
+                            void *scratch, size_t scratch_cap);
 // launch_compact inside the same launch-timing scope as cc_compact_kv's
 // (cc_profile.h, kind CC_KERNEL_COMPACT).
 cudaError_t launch_compact_timed(const CompactParams &p, int sms, cudaStream_t st);
