@@ -166,17 +166,22 @@ CC_DEV uint64_t make_policy_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-// Barrier among `threads` threads (a multiple of 32) of the CTA, id 1..15.
 // Programmatic dependent launch: a kernel launched with the programmatic
 // stream-serialization attribute may start before its predecessor in the
 // stream has finished.  pdl_trigger: this CTA lets the next such kernel
 // launch (it launches once every CTA of this grid has triggered or exited);
 // pdl_wait: blocks until the predecessor grid has completed and its writes
-// are visible (a no-op for a kernel launched without the attribute).  A
-// kernel touches nothing its predecessors write before pdl_wait.
+// are visible (a no-op for a kernel launched without the attribute).
+// Rules that keep a chain of such kernels ordered as a stream is:
+//   - every CTA executes pdl_wait before it exits, so a grid completes only
+//     after all grids before it have;
+//   - a kernel touches nothing before pdl_wait but weights (the few-row GEMM's
+//     first tiles), which no kernel of a call writes; each API call with such
+//     a kernel begins with a plain launch, which waits for whatever wrote them.
 CC_DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 CC_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Barrier among `threads` threads (a multiple of 32) of the CTA, id 1..15.
 CC_DEV void named_barrier_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }

@@ -92,6 +92,7 @@ constexpr int kPlanBlocks = 65;
 
 __global__ void __launch_bounds__(1024) plan_kernel(const __grid_constant__ CompactParams p) {
   pdl_trigger();   // deps_kernel waits for this grid before it writes
+  pdl_wait();      // the keep-set comes from the kernel before
   if (blockIdx.x > 0) {
     const size_t nf = p.flags_bytes / 16, nd = p.deps_bytes / 16;
     uint4 *f = reinterpret_cast<uint4 *>(p.flags), *d = reinterpret_cast<uint4 *>(p.deps);
@@ -407,8 +408,7 @@ cudaError_t launch_compact(const CompactParams &p, int sms, cudaStream_t st) {
   for (int cls = 0; cls < p.n_classes; ++cls) {
     if (p.class_rows[cls] <= 0) return cudaErrorInvalidValue;
   }
-  plan_kernel<<<kPlanBlocks, 1024, 0, st>>>(p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(plan_kernel, dim3(kPlanBlocks), dim3(1024), 0, st, p);
   if (e != cudaSuccess) return e;
   const dim3 dgrid((p.cap + 255) / 256, p.batch, p.n_classes);
   e = launch_pdl(deps_kernel, dgrid, dim3(256), 0, st, p);

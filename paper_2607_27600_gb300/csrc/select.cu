@@ -103,6 +103,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ unsigned n_kept, n_tied;              // of this CTA's segment
   const int CS = ONE ? 1 : kCluster, rank = ONE ? 0 : (int)cluster_ctarank();
   const int b = blockIdx.x / CS, tid = threadIdx.x, lane = tid & 31;
+  pdl_trigger();
+  pdl_wait();   // the scores come from the kernel before
   const int n = seq_len[b];
   if (n < 0 || n > cap) {   // the same in every CTA of the cluster
     if (tid == 0 && rank == 0) {
@@ -306,18 +308,20 @@ cudaError_t launch_select(const float *scores, const int32_t *seq_len, int batch
     }
     attr_set[dev] = true;
   }
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cs;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(batch * cs));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = cached ? (size_t)seg * 4 : 0;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = one ? 0 : 1;
+  cfg.numAttrs = one ? 1 : 2;
   return cudaLaunchKernelEx(&cfg, kern, scores, seq_len, cap, budget, n_sink, keep_idx,
                             keep_count, status, cached);
 }
