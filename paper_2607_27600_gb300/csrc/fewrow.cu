@@ -38,14 +38,15 @@
 // operands' way into shared memory (about 630 cycles per 48 KB k-block) and the
 // tiles' ends.  Measured against the 128 x 256-tile kernel with K splits
 // chained through global memory, per launch (CUDA events): Qwen2.5-7B layer,
-// a 256-row chunk: q/k/v 43 -> 29 us, O 33 -> 26 us, down 71 -> 57 us; a
-// 512-slot cache: down 84 -> 75 us; the 512-slot tiny model's pass 78 -> 66 us.
+// a 256-row chunk: q/k/v 43 -> 28 us, O 33 -> 27 us, down 71 -> 50 us (four
+// CTAs, partials in two rounds), gate/up 86 -> 66 us; a 512-slot cache: down 84
+// -> 76 us; the 512-slot tiny model's pass 78 -> 60 us.
 // Decode steps (Qwen2.5-7B layer, one row) against CUDA-core GEMVs streaming
-// the weights: gate/up 57 -> 50 us (271 MB), LM head 186 -> 160 us (1.09 GB,
-// 6.8 TB/s), down 34 -> 34 us, q/k/v 15 -> 21 and O 14.5 -> 18 us when timed
+// the weights: gate/up 57 -> 50 us (271 MB), LM head 186 -> 159 us (1.09 GB,
+// 6.8 TB/s), down 34 -> 34 us, q/k/v 15 -> 20 and O 14.5 -> 19 us when timed
 // alone (each waits out its own prologue there; a step of four layers took
-// 680 us before and takes 649 us); 16 Llama-3-8B rows against one 128-row tile
-// per sequence: 4.25 -> 1.19 ms.
+// 680 us before and takes 618 us); 16 Llama-3-8B rows against one 128-row tile
+// per sequence: 4.25 -> 0.71 ms.
 #include "fewrow.cuh"
 
 #include <algorithm>
@@ -87,12 +88,17 @@ __host__ __device__ constexpr int stage_bytes(int wt, int nb) { return wt * W_BY
 __host__ __device__ constexpr int stage_count(int wt, int nb) {
   return kRingBytes / stage_bytes(wt, nb) < kMaxStages ? kRingBytes / stage_bytes(wt, nb) : kMaxStages;
 }
-// A split's exchange in the ring's memory: this CTA's partial tile (nb rows of
-// wt * 128 floats) and the share it finishes from each of the others.
-__host__ __device__ constexpr bool split_fits(int wt, int nb, int S) {
-  return (nb + (S - 1) * ((nb + S - 1) / S)) * wt * BM * 4 <= kRingBytes;
+// A split's exchange in the ring's memory: this CTA's partial rows (of wt * 128
+// floats) and the share it finishes from each of the others; in one round of
+// the group's nb rows, or in two of half of them.
+__host__ __device__ constexpr bool round_fits(int wt, int rows, int S) {
+  return (rows + (S - 1) * ((rows + S - 1) / S)) * wt * BM * 4 <= kRingBytes;
 }
-static_assert(split_fits(1, 256, 2) && split_fits(1, 128, 8) && split_fits(2, 128, 2),
+__host__ __device__ constexpr int split_rounds(int wt, int nb, int S) {   // 0: does not fit
+  return round_fits(wt, nb, S) ? 1 : round_fits(wt, nb / 2, S) ? 2 : 0;
+}
+static_assert(split_rounds(1, 256, 8) == 2 && split_rounds(2, 128, 8) == 2 &&
+                  split_rounds(2, 256, 2) == 2 && split_rounds(2, 256, 4) == 0,
               "partial tiles of a split");
 // Tensor-memory columns of one accumulator.
 __host__ __device__ constexpr int acc_cols(int nb) { return nb < 32 ? 32 : nb; }
@@ -218,20 +224,38 @@ CC_DEV LaneCol lane_col(const GemmParams &p, const ProjTile &d, int nt, int q, i
   return lc;
 }
 
-// One value as the next product's operand: bf16 (with lo > 0 also the
-// remainder at that offset) or fp16, a finite overflow reported.
-CC_DEV void store_act(uint16_t *o, float y, bool f16, long long lo, bool live, unsigned *status) {
-  uint16_t bits;
+// One value as the next product's operand, bf16 or fp16, without a branch: the
+// batches of rows below keep their arithmetic free of control flow, so that
+// rows overlap.
+CC_DEV uint16_t act_bits(float y, bool f16) {
+  const uint16_t h = __half_as_ushort(__float2half_rn(y));
+  const uint16_t b = __bfloat16_as_ushort(__float2bfloat16_rn(y));
+  return f16 ? h : b;
+}
+// N values y[k] to out + at[k] where live[k]: one branch each for the fp16
+// range report and (lo > 0) the remainders bf16(y - hi) at that offset.
+template <int N>
+CC_DEV void store_acts(uint16_t *out, const size_t (&at)[N], const float (&y)[N],
+                       const bool (&live)[N], bool f16, int lo, unsigned *status) {
+  uint16_t bits[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) bits[k] = act_bits(y[k], f16);
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (live[k]) out[at[k]] = bits[k];
   if (f16) {
-    if (live && f16_overflow(y)) set_status(status, CC_ERR_RANGE);
-    bits = __half_as_ushort(__float2half_rn(y));
-  } else {
-    bits = __bfloat16_as_ushort(__float2bfloat16_rn(y));
+    bool over = false;
+#pragma unroll
+    for (int k = 0; k < N; ++k) over |= live[k] && f16_overflow(y[k]);
+    if (over) set_status(status, CC_ERR_RANGE);
   }
-  if (live) *o = bits;
-  if (lo > 0 && live)
-    o[lo] = __bfloat16_as_ushort(
-        __float2bfloat16_rn(y - __bfloat162float(__ushort_as_bfloat16(bits))));
+  if (lo > 0) {
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if (live[k])
+        out[at[k] + lo] = __bfloat16_as_ushort(
+            __float2bfloat16_rn(y[k] - __bfloat162float(__ushort_as_bfloat16(bits[k]))));
+  }
 }
 
 // Sums of 16 rows over the warp's 32 lanes: lane l returns the sum of row
@@ -253,65 +277,67 @@ CC_DEV int row16_of(int lane) { return (lane >> 1) & 15; }   // bit 4 of the lan
 
 // Rows J .. J + 8 of finish_block for the projections and SwiGLU: no branch
 // between the rows, so that their arithmetic overlaps.
-template <int EPI, int J>
+template <int EPI, bool RP, int J>
 CC_DEV void finish_rows8(const GemmParams &p, const ProjTile &d, const LaneCol &lc,
                          const RowTab &tab, const float (&v)[16], const float (&u)[16], int r0,
                          int n, size_t row0, int lane, bool dry) {
   const bool f16 = p.out_f16 && !(is_proj<EPI> && d.kv);
-  const long long lo = is_proj<EPI> && d.kv ? 0 : p.row_pairs ? (long long)p.row_pairs * p.ldo
-                                                : p.out_split ? p.N : 0;
+  const int lo = is_proj<EPI> && d.kv ? 0 : RP ? p.row_pairs * p.ldo : p.out_split ? p.N : 0;
+  size_t at[8];
+  float y[8];
+  bool live[8];
   if constexpr (EPI == EPI_SWIGLU) {   // v: gate, u: up
 #pragma unroll
-    for (int j = J; j < J + 8; ++j) {
-      const float rs = tab.rs[r0 + j];
-      store_act(reinterpret_cast<uint16_t *>(p.out) + (row0 + r0 + j) * p.ldo + lc.c0,
-                silu(v[j] * rs) * (u[j] * rs), f16, lo, !dry && lc.ok && j < n, p.status);
+    for (int j = 0; j < 8; ++j) {
+      const float rs = tab.rs[r0 + J + j];
+      y[j] = silu(v[J + j] * rs) * (u[J + j] * rs);
+      at[j] = (row0 + r0 + J + j) * p.ldo + lc.c0;
+      live[j] = !dry && lc.ok && J + j < n;
     }
+    store_acts<8>(reinterpret_cast<uint16_t *>(p.out), at, y, live, f16, lo, p.status);
   } else {
     const int hf = lane >> 4;
 #pragma unroll
-    for (int j = J; j < J + 8; j += 2) {
+    for (int j = 0; j < 8; j += 2) {
       // rotated: lanes 0-15 take row j, lanes 16-31 row j + 1, each both
       // columns of its pair; else every lane its column of both rows
-      float x0 = v[j], x1 = v[j + 1];
-      int ra = r0 + j, rb = ra + 1;
-      bool la = !dry && lc.ok && j < n, lb = la && j + 1 < n;
-      float b1 = lc.b0;
-      size_t o1 = lc.e0;
-      if (d.rope) {
-        const float got = __shfl_xor_sync(0xFFFFFFFFu, hf ? x0 : x1, 16);
-        x0 = hf ? got : x0;
-        x1 = hf ? x1 : got;
-        la = lb = hf ? lb : la;
-        ra = rb = ra + hf;
-        b1 = lc.b1;
-        o1 = lc.e1;
-      }
+      float x0 = v[J + j], x1 = v[J + j + 1];
+      int ra = r0 + J + j, rb = ra + 1;
+      bool la = !dry && lc.ok && J + j < n, lb = la && J + j + 1 < n;
+      const float got = __shfl_xor_sync(0xFFFFFFFFu, hf ? x0 : x1, 16);
+      const float z0 = hf ? got : x0, z1 = hf ? x1 : got;
+      x0 = d.rope ? z0 : x0;
+      x1 = d.rope ? z1 : x1;
+      la = d.rope && hf ? lb : la;
+      lb = d.rope ? la : lb;
+      ra += d.rope ? hf : 0;
+      rb = d.rope ? ra : rb;
       x0 = fmaf(x0, tab.rs[ra], lc.b0);
-      x1 = fmaf(x1, tab.rs[rb], b1);
-      if (d.rope) {
-        float c, s;
-        rope_cs(tab.pos[ra], lc.turn, c, s);
-        const float y0 = x0 * c - x1 * s;
-        x1 = x1 * c + x0 * s;
-        x0 = y0;
-      }
+      x1 = fmaf(x1, tab.rs[rb], d.rope ? lc.b1 : lc.b0);
+      float c, s;
+      rope_cs(tab.pos[ra], lc.turn, c, s);
+      c = d.rope ? c : 1.f;
+      s = d.rope ? s : 0.f;
+      y[j] = d.rope ? x0 * c - x1 * s : x0;
+      y[j + 1] = d.rope ? x1 * c + x0 * s : x1;
       const long long ta = tab.dst[ra], tb = tab.dst[rb];
       const long long da = d.kv ? ta : (long long)(row0 + ra);
       const long long db = d.kv ? tb : (long long)(row0 + rb);
-      const size_t ea = (size_t)da * lc.row_mul + lc.e0, eb = (size_t)db * lc.row_mul + o1;
-      la = la && (ta >= 0 || !d.kv);   // a bad page has no cache row
-      lb = lb && (tb >= 0 || !d.kv);
-      if (d.fp8) {
-        uint8_t *o = reinterpret_cast<uint8_t *>(d.out);
-        const uint32_t e = pack_e4m3x2(x0 * d.qscale, x1 * d.qscale);
-        if (la) o[ea] = (uint8_t)e;
-        if (lb) o[eb] = (uint8_t)(e >> 8);
-      } else {
-        uint16_t *o = reinterpret_cast<uint16_t *>(d.out);
-        store_act(o + ea, x0, f16, lo, la, p.status);
-        store_act(o + eb, x1, f16, lo, lb, p.status);
+      at[j] = (size_t)da * lc.row_mul + lc.e0;
+      at[j + 1] = (size_t)db * lc.row_mul + (d.rope ? lc.e1 : lc.e0);
+      live[j] = la && (ta >= 0 || !d.kv);   // a bad page has no cache row
+      live[j + 1] = lb && (tb >= 0 || !d.kv);
+    }
+    if (d.fp8) {
+      uint8_t *o = reinterpret_cast<uint8_t *>(d.out);
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        const uint32_t e = pack_e4m3x2(y[j] * d.qscale, y[j + 1] * d.qscale);
+        if (live[j]) o[at[j]] = (uint8_t)e;
+        if (live[j + 1]) o[at[j + 1]] = (uint8_t)(e >> 8);
       }
+    } else {
+      store_acts<8>(reinterpret_cast<uint16_t *>(d.out), at, y, live, f16, lo, p.status);
     }
   }
 }
@@ -334,13 +360,13 @@ CC_DEV void prefetch_block(const GemmParams &p, const RowTab &tab, int r0, int e
 // v[j] is row r0 + j (SwiGLU: the gate, u the up projection).  row0: workspace
 // row of the group's first row.  red: per-quarter row sums.  dry: nothing is
 // stored (the code alone runs).
-template <int EPI>
+template <int EPI, bool RP>
 CC_DEV void finish_block(const GemmParams &p, const ProjTile &d, const LaneCol &lc,
                          const RowTab &tab, float (&v)[16], const float (&u)[16], int r0, int n,
                          size_t row0, int q, int lane, float2 *red, bool dry) {
   if constexpr (is_proj<EPI> || EPI == EPI_SWIGLU) {
-    finish_rows8<EPI, 0>(p, d, lc, tab, v, u, r0, n, row0, lane, dry);
-    if (n > 8 || dry) finish_rows8<EPI, 8>(p, d, lc, tab, v, u, r0, n, row0, lane, dry);
+    finish_rows8<EPI, RP, 0>(p, d, lc, tab, v, u, r0, n, row0, lane, dry);
+    if (n > 8 || dry) finish_rows8<EPI, RP, 8>(p, d, lc, tab, v, u, r0, n, row0, lane, dry);
   } else if constexpr (EPI == EPI_ARGMAX) {   // the quarter's largest logit and its first column
 #pragma unroll 1
     for (int j = 0; j < n; ++j) {
@@ -383,9 +409,7 @@ CC_DEV void finish_block(const GemmParams &p, const ProjTile &d, const LaneCol &
       if constexpr (EPI == EPI_RESID_LOGIT)
         w[j] = reinterpret_cast<const uint16_t *>(p.head_w)[(size_t)tab.tok[r] * p.N + cc];
     }
-    [[maybe_unused]] float z[16];
-    const long long norm_lo = p.row_pairs ? (long long)p.row_pairs * p.ld_norm
-                                          : p.norm_split ? p.N : 0;
+    float z[16];   // RESID_LOGIT: the products with the LM-head row; else the next norm's input
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const bool live = j < n && lc.ok;
@@ -396,11 +420,23 @@ CC_DEV void finish_block(const GemmParams &p, const ProjTile &d, const LaneCol &
       } else {
         const size_t row = row0 + r0 + j;
         if (live && !dry) reinterpret_cast<float *>(p.out)[row * p.ldo + lc.c0] = x;
-        if (p.norm_out)
-          store_act(reinterpret_cast<uint16_t *>(p.norm_out) + row * p.ld_norm + lc.c0, x * lc.gain,
-                    p.out_f16 != 0, norm_lo, live && !dry, p.status);
+        z[j] = x * lc.gain;
       }
       h[j] = live ? x * x : 0.f;
+    }
+    if constexpr (EPI != EPI_RESID_LOGIT) {
+      if (p.norm_out) {
+        const int norm_lo = RP ? p.row_pairs * p.ld_norm : p.norm_split ? p.N : 0;
+        size_t at[16];
+        bool live[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          at[j] = (row0 + r0 + j) * p.ld_norm + lc.c0;
+          live[j] = !dry && lc.ok && j < n;
+        }
+        store_acts<16>(reinterpret_cast<uint16_t *>(p.norm_out), at, z, live, p.out_f16 != 0,
+                       norm_lo, p.status);
+      }
     }
     if (EPI == EPI_RESID_LOGIT || p.norm_out) {
       const float ss = rows_sum(h, lane);
@@ -422,14 +458,17 @@ CC_DEV void bulk_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t ba
       : "memory");
 }
 // 16 rows of an accumulator (a row pair's two products added).
+template <bool RP>
 CC_DEV void load_block(uint32_t taddr, int row_pairs, float (&v)[16]) {
   uint32_t r[16], lo[16];
   tmem_ld16(taddr, r);
-  if (row_pairs) tmem_ld16(taddr + row_pairs, lo);
+  if constexpr (RP) tmem_ld16(taddr + row_pairs, lo);
   tmem_ld_wait();
 #pragma unroll
-  for (int j = 0; j < 16; ++j)
-    v[j] = __uint_as_float(r[j]) + (row_pairs ? __uint_as_float(lo[j]) : 0.f);
+  for (int j = 0; j < 16; ++j) {
+    v[j] = __uint_as_float(r[j]);
+    if constexpr (RP) v[j] += __uint_as_float(lo[j]);
+  }
 }
 CC_DEV uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t a;
@@ -437,7 +476,7 @@ CC_DEV uint32_t map_rank(uint32_t addr, uint32_t rank) {
   return a;
 }
 
-template <int EPI>
+template <int EPI, bool RP, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmB3,
@@ -462,14 +501,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   int *prefix = reinterpret_cast<int *>(smem + kOffPrefix);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int S = (int)cluster_nctarank();
-  const int rank = (int)cluster_ctarank();
+  const int S = SPLIT ? (int)cluster_nctarank() : 1;   // K splits: CTAs of the cluster
+  const int rank = SPLIT ? (int)cluster_ctarank() : 0;
   const int unit0 = (int)blockIdx.x / S, n_units = (int)gridDim.x / S;
   constexpr int WT = w_tiles(EPI);
   const int sb = stage_bytes(WT, nb), n_stages = stage_count(WT, nb);
   const int acc_stride = WT * acc_cols(nb);
+  const int n_rounds = SPLIT ? split_rounds(WT, nb, S) : 1;   // of a split's exchange
+  const int n_acc = 2 * acc_stride <= 512 ? 2 : 1;   // (one: SwiGLU groups of 256 rows)
   uint32_t tmem_cols = 64;
-  while ((int)tmem_cols < 2 * acc_stride) tmem_cols *= 2;
+  while ((int)tmem_cols < n_acc * acc_stride) tmem_cols *= 2;
 
   pdl_trigger();
   if (threadIdx.x == 0) {
@@ -496,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) tmem_alloc(tmem_slot, tmem_cols);
   tc_fence_before();
   __syncthreads();
-  if (S > 1) cluster_sync();   // every CTA's barriers exist before any remote arrival
+  if constexpr (SPLIT) cluster_sync();   // every CTA's barriers exist before any remote arrival
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -559,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           row0 = b * p.cap + (p.row_lo ? p.row_lo[b] : 0) + (g - prefix[b]) * nb;
         }
         // the ring holds the last tile's partials until they are summed
-        if (S > 1 && it > 0 && !(ok = mbar_wait(ring_free, (it - 1) & 1, abort_flag, p.status))) break;
+        if (SPLIT && it > 0 && !(ok = mbar_wait(ring_free, (it - 1) & 1, abort_flag, p.status))) break;
         for (int kb = kb0; kb < kb1; ++kb) {
           uint8_t *dst = ring + (size_t)stage * sb;
           if (it == 0 && kb - kb0 < prefetched) {
@@ -601,7 +642,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
         umma_commit(&tfull[acc]);
-        if (++acc == 2) { acc = 0; acc_phase ^= 1; }
+        if (++acc == n_acc) { acc = 0; acc_phase ^= 1; }
       }
     mma_done:;
     }
@@ -621,6 +662,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       bar_phase ^= 1;
       return r;
     };
+    // A split's round: rows [round * per_round, + nr) of a group of nv, CTA r
+    // finishing share r of them, rows [base, base + rows)
+    const int per_round = nb / n_rounds;
+    auto round_rows = [&](int round, int nv, int &nr, int &base, int &rows) {
+      const int first = round * per_round;
+      nr = !SPLIT ? nv : max(0, min(per_round, nv - first));
+      const int share = (nr + S - 1) / S;
+      base = first + min(nr, rank * share);
+      rows = first + min(nr, (rank + 1) * share) - base;
+    };
     uint32_t it = 0;
     for (int item = unit0; ok && item < total; item += n_units, ++it) {
       const int nt = item / num_g, g = item - nt * num_g;
@@ -630,7 +681,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int i0 = lo + (g - (one_group ? 0 : prefix[b])) * nb;
       const bool bad = lo < 0 || hi > p.cap;   // reported when the prefix was built
       // valid rows of the group
-      const int nv = bad ? 0 : max(0, min(p.row_pairs ? p.row_pairs : nb, hi - i0));
+      const int nv = bad ? 0 : max(0, min(RP ? p.row_pairs : nb, hi - i0));
       const size_t row0 = (size_t)b * p.cap + i0;
       // two tables in turn: warps are at most one item apart
       const int par = num_g == 1 ? 0 : (int)(it & 1);
@@ -647,88 +698,109 @@ __global__ void __launch_bounds__(kThreads, 1)
       // A CTA's first tile is preceded by a dry pass over one block: the
       // code's instruction fetches (measured several microseconds from a
       // cold instruction cache) then overlap the products
+      int fin_base0 = 0, fin_rows0 = 0, fin_base1 = 0, fin_rows1 = 0;   // rows finished (per round)
       for (int pass = it == 0 && nv > 0 ? 0 : 1; ok && pass < 2; ++pass) {
         const bool dry = pass == 0;
-        int base = 0, rows = dry ? 1 : nv;     // rows of the group this CTA finishes
-        const float *own = reinterpret_cast<const float *>(ring);
-        const int share = (nv + S - 1) / S;
-        constexpr int ROW = WT * BM;                  // floats of a partial row
-        const float *recv = own + (size_t)nb * ROW;   // [S - 1][share][ROW], peers in rank order
         if (!dry) {
           if constexpr (EPI == EPI_RESID_BF16 || EPI == EPI_RESID_LOGIT) {
-            const int r_lo = S == 1 ? 0 : min(nv, rank * share);
-            const int r_hi = S == 1 ? nv : min(nv, r_lo + share);
-            for (int r0 = r_lo + grp * kBlock; r0 < r_hi; r0 += 2 * kBlock)
-              prefetch_block<EPI>(p, tab, r0, r_hi, row0, nt, q, lane);
+            for (int round = 0; round < n_rounds; ++round) {
+              int nr, base, rows;
+              round_rows(round, nv, nr, base, rows);
+              for (int r0 = base + grp * kBlock; r0 < base + rows; r0 += 2 * kBlock)
+                prefetch_block<EPI>(p, tab, r0, base + rows, row0, nt, q, lane);
+            }
           }
           if (!(ok = mbar_wait(&tfull[acc], acc_phase, abort_flag, p.status))) break;
           tc_fence_after();
         }
-        if (!dry && S > 1) {
-          // every CTA's products are done: no ring of the cluster is read any more
-          if (ew == 0 && lane < S) mbar_arrive_cluster(map_rank(smem_u32(peers_done), lane));
-          if (!(ok = mbar_wait<true>(peers_done, it & 1, abort_flag, p.status))) break;
-          // this CTA's partial rows into its own ring: CTA r finishes rows
-          // [r share, (r + 1) share) of the group
-          base = min(nv, rank * share);
-          rows = min(nv, base + share) - base;
-          if (ew == 0 && lane == 0)
-            mbar_arrive_expect_tx(parts_in, (uint32_t)((S - 1) * rows * ROW * 4));
-          for (int r0 = grp * kBlock; r0 < nv; r0 += 2 * kBlock) {
-#pragma unroll
-            for (int w = 0; w < WT; ++w) {
-              float x[16];
-              load_block(tacc + w * acc_cols(nb) + r0, p.row_pairs, x);
-              float *o = reinterpret_cast<float *>(ring) + r0 * ROW + w * BM + c;
-#pragma unroll
-              for (int j = 0; j < kBlock; ++j) o[j * ROW] = x[j];
-            }
-          }
-          tc_fence_before();
-          fence_proxy_async_smem();   // the bulk copies read what was just written
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(&tempty[acc]);
-            mbar_arrive(own_in);
-          }
-          if (!(ok = mbar_wait(own_in, it & 1, abort_flag, p.status))) break;
-          if (ew == 0 && lane < S && lane != rank) {
-            const int d0 = min(nv, lane * share), dn = min(nv, d0 + share) - d0;
-            const int slot = rank < lane ? rank : rank - 1;   // this CTA's place among lane's peers
-            if (dn > 0)
-              bulk_to_peer(map_rank(smem_u32(recv + (size_t)slot * share * ROW), lane),
-                           smem_u32(own + (size_t)d0 * ROW), (uint32_t)(dn * ROW * 4),
-                           map_rank(smem_u32(parts_in), lane));
-          }
-          if (!(ok = mbar_wait<true>(parts_in, it & 1, abort_flag, p.status))) break;
-        }
+        constexpr int ROW = WT * BM;                  // floats of a partial row
+        const int rounds = dry ? 1 : n_rounds;
 #pragma unroll 1
-        for (int r0 = dry ? 0 : grp * kBlock; r0 < rows; r0 += 2 * kBlock) {
-          const int n = min(kBlock, rows - r0);
-          float v[16], u[16];   // u: the up projection (SwiGLU)
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = u[j] = 0.f;
-          if (!dry && S == 1) {
-            load_block(tacc + r0, p.row_pairs, v);
-            if constexpr (WT == 2) load_block(tacc + acc_cols(nb) + r0, p.row_pairs, u);
-          } else if (!dry) {
-#pragma unroll 1
-            for (int s = 0; s < S; ++s) {   // rank order
-              const float *src = (s == rank ? own + (size_t)base * ROW
-                                            : recv + (size_t)(s < rank ? s : s - 1) * share * ROW) +
-                                 r0 * ROW + c;
-#pragma unroll
-              for (int j = 0; j < 16; ++j)
-                if (j < n) {
-                  v[j] += src[j * ROW];
-                  if constexpr (WT == 2) u[j] += src[j * ROW + BM];
-                }
+        for (int round = 0; ok && round < rounds; ++round) {
+          const int lo_r = round * per_round;
+          int nr = 1, base = 0, rows = 1;
+          if (!dry) round_rows(round, nv, nr, base, rows);
+          const int share = (nr + S - 1) / S;
+          const float *own = reinterpret_cast<const float *>(ring);   // row lo_r first
+          const float *recv = own + (size_t)per_round * ROW;   // [S - 1][share][ROW], peers in rank order
+          if (SPLIT && !dry) {
+            const uint32_t ph = (it * n_rounds + round) & 1;
+            // every CTA's products are done (round 0) or its last round is summed:
+            // no ring of the cluster is read any more
+            if (round > 0) {
+              fence_proxy_async_smem();   // generic reads before the peers' next copies
+              if (!(ok = epi_sync())) break;
             }
+            if (ew == 0 && lane < S) mbar_arrive_cluster(map_rank(smem_u32(peers_done), lane));
+            if (!(ok = mbar_wait<true>(peers_done, ph, abort_flag, p.status))) break;
+            // this CTA's partial rows of the round into its own ring
+            if (ew == 0 && lane == 0)
+              mbar_arrive_expect_tx(parts_in, (uint32_t)((S - 1) * rows * ROW * 4));
+            for (int r0 = grp * kBlock; r0 < nr; r0 += 2 * kBlock) {
+#pragma unroll
+              for (int w = 0; w < WT; ++w) {
+                float x[16];
+                load_block<RP>(tacc + w * acc_cols(nb) + lo_r + r0, p.row_pairs, x);
+                float *o = reinterpret_cast<float *>(ring) + r0 * ROW + w * BM + c;
+#pragma unroll
+                for (int j = 0; j < kBlock; ++j) o[j * ROW] = x[j];
+              }
+            }
+            tc_fence_before();
+            fence_proxy_async_smem();   // the bulk copies read what was just written
+            __syncwarp();
+            if (lane == 0) {
+              if (round == n_rounds - 1) mbar_arrive(&tempty[acc]);
+              mbar_arrive(own_in);
+            }
+            if (!(ok = mbar_wait(own_in, ph, abort_flag, p.status))) break;
+            if (ew == 0 && lane < S && lane != rank) {
+              const int d0 = min(nr, lane * share), dn = min(nr, d0 + share) - d0;
+              const int slot = rank < lane ? rank : rank - 1;   // this CTA's place among lane's peers
+              if (dn > 0)
+                bulk_to_peer(map_rank(smem_u32(recv + (size_t)slot * share * ROW), lane),
+                             smem_u32(own + (size_t)d0 * ROW), (uint32_t)(dn * ROW * 4),
+                             map_rank(smem_u32(parts_in), lane));
+            }
+            if (!(ok = mbar_wait<true>(parts_in, ph, abort_flag, p.status))) break;
           }
-          finish_block<EPI>(p, d, lc, tab, v, u, base + r0, n, row0, q, lane, red, dry);
+#pragma unroll 1
+          for (int r0 = dry ? 0 : grp * kBlock; r0 < rows; r0 += 2 * kBlock) {
+            const int n = min(kBlock, rows - r0);
+            float v[16], u[16];   // u: the up projection (SwiGLU)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = u[j] = 0.f;
+            if (!SPLIT && !dry) {
+              load_block<RP>(tacc + r0, p.row_pairs, v);
+              if constexpr (WT == 2) load_block<RP>(tacc + acc_cols(nb) + r0, p.row_pairs, u);
+            } else if (!dry) {
+#pragma unroll 1
+              for (int s = 0; s < S; ++s) {   // rank order
+                const float *src = (s == rank ? own + (size_t)(base - lo_r) * ROW
+                                              : recv + (size_t)(s < rank ? s : s - 1) * share * ROW) +
+                                   r0 * ROW + c;
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  if (j < n) {
+                    v[j] += src[j * ROW];
+                    if constexpr (WT == 2) u[j] += src[j * ROW + BM];
+                  }
+              }
+            }
+            finish_block<EPI, RP>(p, d, lc, tab, v, u, base + r0, n, row0, q, lane, red, dry);
+          }
+          if (dry) continue;
+          if (round == 0) {   // the rows this CTA finished, for the sums below
+            fin_base0 = base;
+            fin_rows0 = rows;
+          } else {
+            fin_base1 = base;
+            fin_rows1 = rows;
+          }
         }
+        if (!ok) break;
         if (dry) continue;
-        if (S == 1) {
+        if constexpr (!SPLIT) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -746,8 +818,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           const bool wanted = EPI == EPI_RESID_LOGIT || EPI == EPI_ARGMAX || p.norm_out;
           if (wanted && !(ok = epi_sync())) break;
           const int t = (int)threadIdx.x - 64;
-          if (wanted && t < rows) {
-            const int r = base + t;
+          if (wanted && t < fin_rows0 + fin_rows1) {
+            const int r = t < fin_rows0 ? fin_base0 + t : fin_base1 + t - fin_rows0;
             const float2 x0 = red[r], x1 = red[kMaxRows + r], x2 = red[2 * kMaxRows + r],
                          x3 = red[3 * kMaxRows + r];
             const size_t row = row0 + r;
@@ -769,13 +841,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      if (++acc == 2) { acc = 0; acc_phase ^= 1; }
+      if (++acc == n_acc) { acc = 0; acc_phase ^= 1; }
     }
   }
 
   tc_fence_before();
   __syncthreads();
-  if (S > 1) cluster_sync();   // no CTA of the cluster still writes to this one
+  if constexpr (SPLIT) cluster_sync();   // no CTA of the cluster still writes to this one
   if (*abort_flag) __nanosleep(1000000);   // let copies still in flight land
   if (warp == 1) {
     tc_fence_after();
@@ -783,11 +855,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-template <int EPI>
+template <int EPI, bool RP, bool SPLIT>
 cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                      const CUtensorMap &b3, const GemmParams &p, const FewPlan &plan,
                      bool one_group, int sms, cudaStream_t stream) {
-  auto kern = few_kernel<EPI>;
+  auto kern = few_kernel<EPI, RP, SPLIT>;
   static int max_clusters[64][4] = {};   // co-resident clusters of 1, 2, 4 and 8 CTAs (0: unknown)
   int dev = 0;
   cudaGetDevice(&dev);
@@ -835,7 +907,7 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
   best.cycles = 1e300;
   const int nk = ((K + BK - 1) / BK) * (a_split ? 2 : 1);
   const double hbm = (double)n_tiles * wt * BM * K * 2 / 3500.0;   // weight bytes at 6.7 TB/s, 1.9 GHz
-  for (int nb = 16; nb <= kMaxRows / wt; nb *= 2) {
+  for (int nb = 16; nb <= kMaxRows; nb *= 2) {
     if (row_pairs && nb != 2 * row_pairs) continue;
     const double groups = (double)seqs * (double)((rows_per_seq + nb - 1) / nb);
     // k-block: the products (2 cycles per row) or their operands' way into
@@ -843,16 +915,22 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
     // 570 for 32 KB, 630 to 670 for 48 KB)
     const double tk = std::max(2.0 * nb * wt, 180.0 + stage_bytes(wt, nb) / 105.0);
     for (int S = 1; S <= kFewMaxSplit; S *= 2) {
-      if (S > 1 && (nk < 4 * S || !split_fits(wt, nb, S))) break;
+      const int rounds = S > 1 ? split_rounds(wt, nb, S) : 1;
+      if (S > 1 && (nk < 4 * S || rounds == 0)) break;
       const double units = floor(sms / S * (S >= 4 ? 0.95 : 1.0));
       const double waves = std::ceil(groups * n_tiles / std::max(1.0, units));
-      // a tile's end: about 3600 cycles per 16-row block of a warp, for a split
-      // the exchange before it; without a split it overlaps the next tile's
-      // products
-      const double fin = 1500.0 + 112.0 * std::min<double>(nb, (double)rows_per_seq) * wt / S;
-      const double fix = S > 1 ? 2000.0 + 20.0 * wt * nb + fin : 300.0;
-      const double sm = waves * (std::ceil((double)nk / S) * tk + fix) + (S > 1 ? 0.0 : fin);
-      const double t = std::max(sm, hbm * 1.1) + 0.05 * sm;
+      // a tile's end: about 3600 cycles per 16-row block of a warp (SwiGLU 2600),
+      // for a split the exchange before it; without a split it overlaps the
+      // next tile's products while two accumulators fit
+      const double fin = 1500.0 + (wt == 2 ? 80.0 : 112.0) * std::min<double>(nb, (double)rows_per_seq) / S;
+      const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
+      const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
+      const double main = waves * std::ceil((double)nk / S) * tk;
+      const double ends = waves * fix + (overlapped ? fin : 0.0);
+      // several groups read the same weight tiles at the same time, which holds
+      // the SMs' requests longer (gate/up of 256 rows, 271 MB: 128-row groups
+      // 70 us at 4.9 TB/s, one of 256 rows 66 us)
+      const double t = std::max(main, hbm * (groups > 1 ? 1.5 : 1.1)) + ends + 0.05 * (main + ends);
       if (t < best.cycles * 0.98) {
         best.nb = nb;
         best.split = S;
@@ -866,17 +944,27 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
 cudaError_t launch_few(int epi, const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                        const CUtensorMap &b3, const GemmParams &p, const FewPlan &plan,
                        bool one_group, int sms, cudaStream_t st) {
+  // (row pairs: the products of a decode step)
+#define CC_FEW_T(E, R)                                                                   \
+  (plan.split > 1 ? launch_t<E, R, true>(a, b, b2, b3, p, plan, one_group, sms, st)      \
+                  : launch_t<E, R, false>(a, b, b2, b3, p, plan, one_group, sms, st))
+#define CC_FEW(E) CC_FEW_T(E, false)
+#define CC_FEW_DECODE(E) (p.row_pairs ? CC_FEW_T(E, true) : CC_FEW_T(E, false))
+  if (p.row_pairs && (epi == EPI_RESID_BF16 || epi == EPI_RESID_LOGIT)) return cudaErrorInvalidValue;
   switch (epi) {
-    case EPI_QROPE: return launch_t<EPI_QROPE>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_RESID_BF16: return launch_t<EPI_RESID_BF16>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_RESID_F32: return launch_t<EPI_RESID_F32>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_SWIGLU: return launch_t<EPI_SWIGLU>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_BF16: return launch_t<EPI_BF16>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_QKV: return launch_t<EPI_QKV>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_ARGMAX: return launch_t<EPI_ARGMAX>(a, b, b2, b3, p, plan, one_group, sms, st);
-    case EPI_RESID_LOGIT: return launch_t<EPI_RESID_LOGIT>(a, b, b2, b3, p, plan, one_group, sms, st);
+    case EPI_QROPE: return CC_FEW_DECODE(EPI_QROPE);
+    case EPI_RESID_BF16: return CC_FEW(EPI_RESID_BF16);
+    case EPI_RESID_F32: return CC_FEW_DECODE(EPI_RESID_F32);
+    case EPI_SWIGLU: return CC_FEW_DECODE(EPI_SWIGLU);
+    case EPI_BF16: return CC_FEW_DECODE(EPI_BF16);
+    case EPI_QKV: return CC_FEW_DECODE(EPI_QKV);
+    case EPI_ARGMAX: return CC_FEW_DECODE(EPI_ARGMAX);
+    case EPI_RESID_LOGIT: return CC_FEW(EPI_RESID_LOGIT);
     default: return cudaErrorInvalidValue;
   }
+#undef CC_FEW_DECODE
+#undef CC_FEW
+#undef CC_FEW_T
 }
 
 }  // namespace cc

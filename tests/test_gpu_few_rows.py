@@ -83,6 +83,25 @@ def test_scores_equal_the_tile_kernel(pkg, monkeypatch, dh, mode, full):
         assert rel_err(got[b, :n], ref[b, :n]) < tol, b
 
 
+@pytest.mark.parametrize("n", [129, 250, 256])
+def test_wide_layer_equals_the_tile_kernel(pkg, monkeypatch, n):
+    """d_ff 16384 at d_model 2048: one gate/up group of up to 256 rows over a
+    single accumulator pair, and a down projection over 8 CTAs whose partial
+    rows are exchanged in two rounds.  Summation order differs (1e-6 relative
+    per sum, and roundings of 16-bit activations that fall the other way: the
+    bound of the test above)."""
+    from paper_2607_27600_gb300 import cc
+    shape = ModelShape(1, 2048, 4, 2, 128, 16384, 700, 1e4, 1e-5)
+    w = synth.model_weights(shape, 5, device="cuda", with_kv_proj=True)
+    c = synth.synthetic_cache(shape, [n], 260, 6, device="cuda")
+    got = _score(pkg, shape, w, c, cc.SCORE_LOGIT, False)
+    monkeypatch.setenv("CC_GEMM_PAIRS", "0")
+    ref = _score(pkg, shape, w, c, cc.SCORE_LOGIT, False)
+    f = np.isfinite(ref[0])
+    assert np.array_equal(f, np.isfinite(got[0])) and f.sum() == n - 1
+    assert rel_err(got[0, :n], ref[0, :n]) < 5e-3
+
+
 @pytest.mark.parametrize("dh", [64, 128])
 @pytest.mark.parametrize("layout", ["slot", "head", "paged", "e4m3"])
 @pytest.mark.parametrize("counts", [[1, 0, 1], [37, 128, 5]])
