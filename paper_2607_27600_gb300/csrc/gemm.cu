@@ -17,7 +17,9 @@
 // Large launches run as CTA pairs (clusters of two, cta_group::2): one
 // M = 256, N = 256 product per pair, each CTA staging its own 128 A rows and
 // half of the B tile, so a CTA moves 32 KB instead of 48 KB through L2 and
-// shared memory per 128 x 256 x 64 block of its output.
+// shared memory per 128 x 256 x 64 block of its output.  Where their last wave
+// would leave half of the pairs or more without a tile, its tiles are cut along
+// K over those pairs (split_wave below).
 #include "gemm.cuh"
 
 #include <algorithm>
@@ -565,6 +567,81 @@ CC_DEV void tile_coords(const GemmParams &p, int t, int num_m, int &m, int &n) {
   }
 }
 
+// K splits of each of the rem tiles of a CTA-pair launch's last wave.  A pair
+// takes one part: part i of tile j is pair j S + i's.  Every epilogue warp
+// writes its 32 rows' partial sums to scratch and counts itself; the last of a
+// tile's S parts sums all of them in part order (a fixed order) back into
+// tensor memory and finishes the rows, so no CTA waits for another.
+// A part keeps at least kSplitStages barrier stages (two k-blocks each, about
+// 15 us): the exchange and the sums cost 15 to 20 us.  Measured on the down
+// projection of 2313 Llama-3-8B rows (160 tiles on 76 pairs): 229 us whole,
+// 201 us in eight parts, 194 us in four; the O projection (K = 4096) 78 us
+// whole, 92 us in four.  Its own kernel variant, of the residual products
+// alone (the others are shorter): the code costs the plain epilogues registers.
+constexpr int kSplitStages = 28, kMaxSplit = 8;
+CC_DEV int split_wave(int rem, int n_units, int n_stages) {
+  if (rem == 0) return 1;
+  return max(1, min(min(n_units, kGemmSplitSlots) / rem, min(n_stages / kSplitStages, kMaxSplit)));
+}
+// This warp's 32 x 256 partial sums in slot `slot`: chunk c's column k of row
+// `lane` at [c][k][lane].
+CC_DEV float *split_rows(const GemmParams &p, int slot, int rank, int q) {
+  return p.split_part + (size_t)slot * kGemmSplitFloats + (rank * 4 + q) * (32 * 256);
+}
+// Publishes this part's sums; true in the warp that comes last, with the sums
+// of all parts in its accumulator rows.
+CC_DEV bool split_join(const GemmParams &p, uint32_t tacc, int tile, int part, int S, int rank, int q) {
+  const int lane = threadIdx.x & 31;
+  float *mine = split_rows(p, tile * S + part, rank, q);
+#pragma unroll 1
+  for (int c = 0; c < 8; ++c) {
+    uint32_t r[32];
+    tmem_ld32(tacc + c * 32, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < 32; ++k) __stcg(mine + (c * 32 + k) * 32 + lane, __uint_as_float(r[k]));
+  }
+  __threadfence();
+  __syncwarp();
+  unsigned *count = p.split_count + (tile * 2 + rank) * 4 + q;
+  unsigned before = 0;
+  if (lane == 0) before = atomicAdd(count, 1u);
+  before = __shfl_sync(0xFFFFFFFFu, before, 0);
+  if (before != (unsigned)(S - 1)) return false;
+  __threadfence();
+  if (lane == 0) *count = 0;   // for the next launch
+  const float *from = split_rows(p, tile * S, rank, q) + lane;
+#pragma unroll 1
+  for (int c = 0; c < 8; ++c) {
+    float a[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) a[k] = 0.f;
+#pragma unroll 1
+    for (int s0 = 0; s0 < S; s0 += 4) {   // four parts' loads in flight
+      float x[4][32];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (s0 + j < S) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            x[j][k] = __ldcg(from + (size_t)(s0 + j) * kGemmSplitFloats + (c * 32 + k) * 32);
+        }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (s0 + j < S) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) a[k] += x[j][k];
+        }
+    }
+    uint32_t r[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) r[k] = __float_as_uint(a[k]);
+    tmem_st32(tacc + c * 32, r);
+  }
+  tmem_st_wait();
+  return true;
+}
+
 // One CTA per SM (PAIR false) or a CTA pair per two SMs (PAIR true, a
 // cluster of two), persistent over the output tiles.  A pair computes
 // 256-row tiles: CTA r holds row tile 2 mu + r of row unit mu (two
@@ -577,7 +654,7 @@ CC_DEV void tile_coords(const GemmParams &p, int t, int num_m, int &m, int &n) {
 // (A relay thread in CTA 1 that waited for its own stage barrier and then
 // arrived on CTA 0's measured 3.4x slower on the gate/up shape: the
 // hand-over latency sat on every stage.)
-template <int EPI, int TBN, bool PAIR>
+template <int EPI, int TBN, bool PAIR, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmB3,
@@ -651,6 +728,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int nk_total = p.a_split ? 2 * nk : nk;  // split A: the hi pass, then the lo pass
   const int unit0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int n_units = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+  // the i-th item of this unit: a tile and its barrier stages [s0, s1); the last
+  // wave's tiles in `splits` parts each
+  const int n_stages = (nk_total + KB2 - 1) / KB2;
+  const int whole = total / n_units * n_units;
+  const int splits = SPLIT ? split_wave(total - whole, n_units, n_stages) : 1;
+  struct Item {
+    int tile, s0, s1, part;   // part: -1 for a whole tile
+  };
+  auto item_at = [&](int i, Item &it) {
+    it = {unit0 + i * n_units, 0, n_stages, -1};
+    if (!SPLIT || it.tile < whole || splits == 1) return it.tile < total;
+    if (it.tile - unit0 != whole || unit0 >= (total - whole) * splits) return false;
+    const int j = unit0 / splits;
+    it.part = unit0 - j * splits;
+    it.tile = whole + j;
+    it.s0 = it.part * n_stages / splits;
+    it.s1 = (it.part + 1) * n_stages / splits;
+    return true;
+  };
   // row tile of this CTA in row unit u (-1: past the last tile, the second
   // CTA of an odd pair: it loads its B share only and stores nothing)
   auto row_tile = [&](int u) { const int mt = PAIR ? 2 * u + (int)rank : u; return mt < num_m ? mt : -1; };
@@ -668,9 +764,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = unit0; ok && tile < total; tile += n_units) {
+      Item it;
+      for (int i = 0; ok && item_at(i, it); ++i) {
         int mu, nt;
-        tile_coords(p, tile, num_mu, mu, nt);
+        tile_coords(p, it.tile, num_mu, mu, nt);
         const int mt = row_tile(mu);
         int row0 = 0;
         if (mt >= 0) {
@@ -679,8 +776,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         // a pair's second row tile exists (CTA 0 counts its A bytes)
         const bool a1 = PAIR && 2 * mu + 1 < num_m;
-        for (int kbs = 0; kbs < nk_total; kbs += KB2) {
-          const int nb = min(KB2, nk_total - kbs);
+        for (int ks = it.s0; ks < it.s1; ++ks) {
+          const int kbs = ks * KB2, nb = min(KB2, nk_total - kbs);
           if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status))) break;
           if (!PAIR) mbar_arrive_expect_tx(&full[stage], nb * (A_BYTES + TB_BYTES));
           else if (rank == 0) mbar_arrive_expect_tx(&full[stage], nb * ((a1 ? 2 : 1) * A_BYTES + TB_BYTES));
@@ -728,23 +825,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t b_desc0 = make_sdesc_sw128(smem_u32(sB), 16, 1024);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
-      for (int tile = unit0; tile < total; tile += n_units) {
+      Item it;
+      for (int i = 0; item_at(i, it); ++i) {
         if (!mbar_wait<PAIR>(&tempty[acc], acc_phase ^ 1, abort_flag, p.status)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * TBN;
-        for (int kbs = 0; kbs < nk_total; kbs += KB2) {
-          const int nb = min(KB2, nk_total - kbs);
+        for (int ks = it.s0; ks < it.s1; ++ks) {
+          const int kbs = ks * KB2, nb = min(KB2, nk_total - kbs);
           if (!mbar_wait<PAIR>(&full[stage], phase, abort_flag, p.status)) goto mma_done;
           tc_fence_after();
           for (int j = 0; j < nb; ++j) {
-            const int kb = kbs + j, slot = stage * KB2 + j;
+            const int slot = stage * KB2 + j;
             // descriptors of this stage; a K step of 16 columns advances the
             // start-address field by 32 bytes (+2 in 16-byte units)
             const uint64_t ad = a_desc0 + (uint64_t)(slot * (A_BYTES >> 4));
             const uint64_t bd = b_desc0 + (uint64_t)(slot * (SB >> 4));
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k) {
-              const uint32_t accum = (kb != 0 || k != 0) ? 1u : 0u;
+              const uint32_t accum = (ks != it.s0 || j != 0 || k != 0) ? 1u : 0u;
               if constexpr (PAIR) umma_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, accum);
               else umma_ss(d_tmem, ad + 2 * k, bd + 2 * k, idesc, accum);
             }
@@ -764,9 +862,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = q * 32 + lane;   // accumulator row of this thread
     int acc = 0;
     uint32_t acc_phase = 0;
-    for (int tile = unit0; tile < total; tile += n_units) {
+    Item it;
+    for (int n = 0; item_at(n, it); ++n) {
       int mu, nt;
-      tile_coords(p, tile, num_mu, mu, nt);
+      tile_coords(p, it.tile, num_mu, mu, nt);
       const int mt = row_tile(mu);
       bool valid = false;
       int grow = 0;
@@ -779,7 +878,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, p.status)) break;
       tc_fence_after();
       const uint32_t tacc = tmem_base + acc * TBN + (uint32_t(q * 32) << 16);
-      if (mt >= 0)
+      bool finish = mt >= 0;
+      if constexpr (SPLIT) {
+        if (finish && it.part >= 0)   // a warp without a row joins nothing, in no part
+          finish = __any_sync(0xFFFFFFFFu, valid) &&
+                   split_join(p, tacc, it.tile - whole, it.part, splits, (int)rank, q);
+      }
+      if (finish)
         epilogue_tile<EPI, TBN>(p, tacc, grow, valid, nt, nt * TBN, stage_all + q * 32 * kStageLd);
       tc_fence_before();
       __syncwarp();
@@ -802,10 +907,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-template <int EPI, int TBN, bool PAIR>
+template <int EPI, int TBN, bool PAIR, bool SPLIT = false>
 cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                      const CUtensorMap &b3, const GemmParams &p, int grid, cudaStream_t stream) {
-  auto kern = gemm_kernel<EPI, TBN, PAIR>;
+  auto kern = gemm_kernel<EPI, TBN, PAIR, SPLIT>;
   static bool attr_set[64] = {};
   static int max_pairs[64] = {};   // co-resident CTA pairs (cluster occupancy)
   int dev = 0;
@@ -854,6 +959,10 @@ template <int EPI>
 cudaError_t launch(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                    const CUtensorMap &b3, const GemmParams &p, int grid, cudaStream_t stream) {
   constexpr bool kWide = EPI == EPI_SWIGLU || EPI == EPI_LSE || EPI == EPI_QKV;
+  if constexpr (EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32 || EPI == EPI_RESID_LOGIT) {
+    if (p.split_part && gemm_may_split(EPI, p, grid))
+      return launch_t<EPI, BN, true, true>(a, b, b2, b3, p, grid, stream);
+  }
   if constexpr (EPI != EPI_ARGMAX) {
     if (p.pair && (kWide || p.block_n == BN)) return launch_t<EPI, BN, true>(a, b, b2, b3, p, grid, stream);
   }
@@ -867,6 +976,16 @@ cudaError_t launch(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap
 }
 
 }  // namespace
+
+// (up to six waves at the row bound: the variant's epilogue is 1 % slower, 532
+// -> 538 us on the down projection of 8192 rows in seven waves)
+bool gemm_may_split(int epi, const GemmParams &p, int sms) {
+  const long long tiles = ((long long)p.batch * p.cap + 255) / 256 * p.n_tiles;
+  if (tiles > 6LL * (sms / 2)) return false;
+  const int stages = ((p.K + BK - 1) / BK * (p.a_split ? 2 : 1) + 1) / 2;
+  return (epi == EPI_RESID_BF16 || epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT) && p.pair &&
+         p.block_n == BN && stages >= 2 * kSplitStages;
+}
 
 int gemm_block_n(int epi) { return epi == EPI_SWIGLU ? 128 : BN; }
 int gemm_max_batch() { return kMaxBatch; }

@@ -65,6 +65,11 @@ struct GemmParams {
   int pair;                // run as CTA pairs (256-column tiles): the B tensor
                            // maps' boxes are 128 rows (each CTA loads half of a tile);
                            // raster 1 groups count pairs of row tiles
+  // CTA pairs, both or neither: partial tiles of the last, incomplete wave
+  // (kGemmSplitSlots of kGemmSplitFloats) and their counters
+  // (kGemmSplitCounters, zero; left zero)
+  float *split_part;
+  unsigned *split_count;
   int row_pairs;           // few-row launches: > 0: the A rows are bf16 pairs, lo of row r at row
                            // r + row_pairs of the same group (products hi W^T + lo W^T), and so
                            // are the activations written (norm_out; SwiGLU's and Q's out)
@@ -90,7 +95,15 @@ struct GemmParams {
   unsigned long long turns[64];  // EPI_QROPE: inv_freq_k / (2 pi) in 0.64 fixed point
 };
 
+// Scratch of the K split of a CTA-pair launch's last wave: a slot is one
+// pair's fp32 tile (256 x 256).
+constexpr int kGemmSplitSlots = 80;
+constexpr size_t kGemmSplitFloats = 256 * 256;
+constexpr int kGemmSplitCounters = kGemmSplitSlots / 2 * 8;   // tiles x (CTA, epilogue warp)
+
 int gemm_block_n(int epi);
+// Whether a launch with scratch for it may split its last wave.
+bool gemm_may_split(int epi, const GemmParams &p, int sms);
 int gemm_max_batch();
 // a: A rows x K (box 64 x 128); b (and b2 for SwiGLU, b2 and b3 for the fused
 // projections): weights N x K (box 64 x 256, or 64 x 128 for SwiGLU and for CTA pairs).
