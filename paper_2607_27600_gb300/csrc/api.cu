@@ -379,7 +379,9 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   const bool few = g.few.nb > 0;
   const uint32_t b_box = few || epi == EPI_SWIGLU || pair ? 128 : (uint32_t)bn;
   // row pairs: lo rows row_pairs past the hi ones
-  if (!tmap_rows(&g.a, A, row_pairs ? 2 * (uint64_t)row_pairs : R, a_split ? 2 * K : K, few ? (uint32_t)g.few.nb : 128)) return tmap_fail();
+  if (!tmap_rows(&g.a, A, row_pairs ? 2 * (uint64_t)row_pairs : R, a_split ? 2 * K : K,
+                 few ? (uint32_t)(g.few.pair ? g.few.nb / 2 : g.few.nb) : 128))
+    return tmap_fail();
   if (!tmap_rows(&g.b, W, N, K, b_box)) return tmap_fail();
   if (epi == EPI_SWIGLU) {
     if (!tmap_rows(&g.b2, W2, N, K, b_box)) return tmap_fail();

@@ -28,6 +28,11 @@
 // launch, so the second half of the N side costs nothing and the activations
 // carry 16 significant bits instead of 8 (Qwen2.5-7B and Llama-3-8B, 4 layers:
 // the largest logit's error against 64 bits 2e-3 with single bf16 rows).
+// Where a residual product's splits take whole 256-row groups, the CTAs of two
+// column tiles form a pair (cta_group::2): one M = 256 product, each CTA with
+// its own weight rows and half of the activation rows, 32 KB instead of 48 KB a
+// k-block into its shared memory (down projection of 512 rows 76 -> 67 us, of 256
+// rows 50 -> 47 us).  A pair's CTA 0 issues the products; all else stays per CTA.
 // Without a split two TMEM accumulators let the epilogue of one tile overlap
 // the main loop of the next; with a split the partials take the ring's
 // memory, so the next tile's loads begin when the sums are done.
@@ -84,9 +89,10 @@ static_assert(kSmemBytes <= 232448, "shared memory");
 
 // Weight tiles of a stage and accumulators of an output tile.
 __host__ __device__ constexpr int w_tiles(int epi) { return epi == EPI_SWIGLU ? 2 : 1; }
-__host__ __device__ constexpr int stage_bytes(int wt, int nb) { return wt * W_BYTES + nb * BK * 2; }
-__host__ __device__ constexpr int stage_count(int wt, int nb) {
-  return kRingBytes / stage_bytes(wt, nb) < kMaxStages ? kRingBytes / stage_bytes(wt, nb) : kMaxStages;
+// (rows: activation rows that a CTA stages)
+__host__ __device__ constexpr int stage_bytes(int wt, int rows) { return wt * W_BYTES + rows * BK * 2; }
+__host__ __device__ constexpr int stage_count(int wt, int rows) {
+  return kRingBytes / stage_bytes(wt, rows) < kMaxStages ? kRingBytes / stage_bytes(wt, rows) : kMaxStages;
 }
 // A split's exchange in the ring's memory: this CTA's partial rows (of wt * 128
 // floats) and the share it finishes from each of the others; in one round of
@@ -476,7 +482,7 @@ CC_DEV uint32_t map_rank(uint32_t addr, uint32_t rank) {
   return a;
 }
 
-template <int EPI, bool RP, bool SPLIT>
+template <int EPI, bool RP, bool SPLIT, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
     few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmB3,
@@ -501,11 +507,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   int *prefix = reinterpret_cast<int *>(smem + kOffPrefix);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int S = SPLIT ? (int)cluster_nctarank() : 1;   // K splits: CTAs of the cluster
-  const int rank = SPLIT ? (int)cluster_ctarank() : 0;
-  const int unit0 = (int)blockIdx.x / S, n_units = (int)gridDim.x / S;
+  // the cluster: S K splits (rank: this CTA's) of a column tile, or of two
+  // (tile_of: this CTA's), whose CTAs of one split are a pair
+  constexpr int PT = PAIR ? 2 : 1;
+  const int cta = SPLIT || PAIR ? (int)cluster_ctarank() : 0;
+  const int S = SPLIT ? (int)cluster_nctarank() / PT : 1;
+  const int rank = cta / PT, tile_of = cta % PT;
+  const int lead = cta - tile_of;                     // the pair's CTA 0
+  auto peer = [&](int r) { return (uint32_t)(r * PT + tile_of); };   // this tile's CTA of split r
+  const int unit0 = (int)blockIdx.x / (S * PT), n_units = (int)gridDim.x / (S * PT);
   constexpr int WT = w_tiles(EPI);
-  const int sb = stage_bytes(WT, nb), n_stages = stage_count(WT, nb);
+  const int a_rows = nb / PT;   // activation rows of a group that this CTA stages
+  const int sb = stage_bytes(WT, a_rows), n_stages = stage_count(WT, a_rows);
   const int acc_stride = WT * acc_cols(nb);
   const int n_rounds = SPLIT ? split_rounds(WT, nb, S) : 1;   // of a split's exchange
   const int n_acc = 2 * acc_stride <= 512 ? 2 : 1;   // (one: SwiGLU groups of 256 rows)
@@ -520,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull[a], 1);
-      mbar_init(&tempty[a], kEpiWarps);
+      mbar_init(&tempty[a], PT * kEpiWarps);
     }
     mbar_init(peers_done, S);
     mbar_init(own_in, kEpiWarps);
@@ -534,10 +547,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (EPI == EPI_SWIGLU || EPI == EPI_QKV) tma_prefetch_desc(&tmB2);
     if (EPI == EPI_QKV) tma_prefetch_desc(&tmB3);
   }
-  if (warp == 1) tmem_alloc(tmem_slot, tmem_cols);
+  if (warp == 1) {
+    if constexpr (PAIR) tmem_alloc_pair(tmem_slot, tmem_cols);
+    else tmem_alloc(tmem_slot, tmem_cols);
+  }
   tc_fence_before();
   __syncthreads();
-  if constexpr (SPLIT) cluster_sync();   // every CTA's barriers exist before any remote arrival
+  if constexpr (SPLIT || PAIR) cluster_sync();   // every CTA's barriers exist before any remote arrival
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -545,11 +561,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int nk_total = p.a_split ? 2 * nk : nk;   // split A: the hi pass, then the lo pass
   const int kb0 = rank * nk_total / S, kb1 = (rank + 1) * nk_total / S;
 
-  // weight rows of tile nt, k-block column kw, into ring slot `dst`
+  // weight rows of tile nt, k-block column kw, into ring slot `dst`; a pair's
+  // loads complete on the barrier of its CTA 0
+  auto load2 = [&](uint8_t *dst, const CUtensorMap *m, uint64_t *bar, int c0, int c1, uint64_t pol) {
+    if constexpr (PAIR) tma_load_2d_pair_hint(dst, m, cluster_addr(bar, lead), c0, c1, pol);
+    else tma_load_2d_hint(dst, m, bar, c0, c1, pol);
+  };
   auto load_w = [&](uint8_t *dst, uint64_t *bar, int nt, int kw, uint64_t pol) {
     if constexpr (EPI == EPI_SWIGLU) {
-      tma_load_2d_hint(dst, &tmB, bar, kw, nt * BM, pol);
-      tma_load_2d_hint(dst + W_BYTES, &tmB2, bar, kw, nt * BM, pol);
+      load2(dst, &tmB, bar, kw, nt * BM, pol);
+      load2(dst + W_BYTES, &tmB2, bar, kw, nt * BM, pol);
     } else if constexpr (EPI == EPI_QROPE || EPI == EPI_QKV) {
       // whole heads of a rotated projection: rows in the order of pair_base
       const int heads = BM / p.head_dim;
@@ -559,9 +580,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       else if (nt < nq + nkt)
         tma_load_5d_hint(dst, &tmB2, bar, kw, 0, 0, 0, (nt - nq) * heads, pol);
       else
-        tma_load_2d_hint(dst, &tmB3, bar, kw, (nt - nq - nkt) * BM, pol);
+        load2(dst, &tmB3, bar, kw, (nt - nq - nkt) * BM, pol);
     } else {
-      tma_load_2d_hint(dst, &tmB, bar, kw, nt * BM, pol);
+      load2(dst, &tmB, bar, kw, nt * BM, pol);
     }
   };
   auto w_col = [&](int kb) { return (kb < nk ? kb : kb - nk) * BK; };
@@ -569,11 +590,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   // weights first: they depend on no earlier kernel
   int prefetched = 0;
   const uint64_t keep = make_policy_evict_last(), stream_pol = make_policy_evict_first();
-  if (one_group && warp == 0 && lane == 0 && unit0 < p.n_tiles) {
+  const int n_tiles_u = (p.n_tiles + PT - 1) / PT;   // tiles of a unit: PT each, the last maybe one short
+  if (one_group && warp == 0 && lane == 0 && unit0 < n_tiles_u) {
     prefetched = min(n_stages, kb1 - kb0);
     for (int i = 0; i < prefetched; ++i) {
-      mbar_arrive_expect_tx(&full[i], sb);
-      load_w(ring + (size_t)i * sb, &full[i], unit0, w_col(kb0 + i), stream_pol);
+      if (tile_of == 0) mbar_arrive_expect_tx(&full[i], PT * sb);
+      load_w(ring + (size_t)i * sb, &full[i], unit0 * PT + tile_of, w_col(kb0 + i), stream_pol);
     }
   }
   pdl_wait();   // the rows, their ranges and every output belong to earlier kernels until here
@@ -583,7 +605,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // walked even when it turns out to have no row (prefix only reports its range)
   if (!one_group) __syncthreads();
   const int num_g = one_group ? 1 : prefix[p.batch];
-  const int total = num_g * p.n_tiles;
+  const int total = num_g * n_tiles_u;
 
   if (warp == 0) {
     if (lane == 0) {  // ---------------- TMA producer
@@ -593,7 +615,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       int it = 0;
       for (int item = unit0; ok && item < total; item += n_units, ++it) {
-        const int nt = item / num_g, g = item - nt * num_g;
+        const int ntu = item / num_g, g = item - ntu * num_g, nt = ntu * PT + tile_of;
         int row0 = p.row_lo ? p.row_lo[0] : 0;
         if (!one_group) {
           const int b = find_seq(prefix, p.batch, g);
@@ -607,41 +629,56 @@ __global__ void __launch_bounds__(kThreads, 1)
             ;   // armed, its weights on their way
           } else {
             if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status))) break;
-            mbar_arrive_expect_tx(&full[stage], sb);
+            if (tile_of == 0) mbar_arrive_expect_tx(&full[stage], PT * sb);
             load_w(dst, &full[stage], nt, w_col(kb), pol_w);
           }
           // A column block kb of [hi | lo] (hi and lo halves are K apart)
           const int ka = kb < nk ? kb * BK : p.K + (kb - nk) * BK;
-          tma_load_2d_hint(dst + WT * W_BYTES, &tmA, &full[stage], ka, row0, keep);
+          load2(dst + WT * W_BYTES, &tmA, &full[stage], ka, row0 + tile_of * a_rows, keep);
+          if (++stage == n_stages) { stage = 0; phase ^= 1; }
+        }
+      }
+      if (PAIR && ok) {
+        // every stage's last release (a commit of the pair's CTA 0) has landed
+        // before the CTA may leave
+        for (int i = 0; i < n_stages; ++i) {
+          if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status)) break;
           if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------- MMA issuer
-      const uint32_t idesc = p.ab_f16 ? make_idesc_f16(BM, nb, 0, 0) : make_idesc_bf16(BM, nb, 0, 0);
+    if (lane == 0 && tile_of == 0) {  // ---------------- MMA issuer (a pair's CTA 0, for both)
+      const uint32_t idesc =
+          p.ab_f16 ? make_idesc_f16(PT * BM, nb, 0, 0) : make_idesc_bf16(PT * BM, nb, 0, 0);
+      const uint16_t both = (uint16_t)(3u << lead);
       const uint64_t w_desc0 = make_sdesc_sw128(smem_u32(ring), 16, 1024);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       for (int item = unit0; item < total; item += n_units) {
-        if (!mbar_wait(&tempty[acc], acc_phase ^ 1, abort_flag, p.status)) break;
+        if (!mbar_wait<PAIR>(&tempty[acc], acc_phase ^ 1, abort_flag, p.status)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem + acc * acc_stride;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(&full[stage], phase, abort_flag, p.status)) goto mma_done;
+          if (!mbar_wait<PAIR>(&full[stage], phase, abort_flag, p.status)) goto mma_done;
           tc_fence_after();
           const uint64_t wd = w_desc0 + (uint64_t)((stage * sb) >> 4);
           const uint64_t ad = wd + ((WT * W_BYTES) >> 4);
 #pragma unroll
           for (int w = 0; w < WT; ++w)
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_ss(d_tmem + w * acc_cols(nb), wd + w * (W_BYTES >> 4) + 2 * k, ad + 2 * k, idesc,
-                      (kb != kb0 || k != 0) ? 1u : 0u);
-          umma_commit(&empty[stage]);
+            for (int k = 0; k < BK / 16; ++k) {
+              const uint32_t dt = d_tmem + w * acc_cols(nb), accum = kb != kb0 || k != 0;
+              const uint64_t wk = wd + w * (W_BYTES >> 4) + 2 * k, ak = ad + 2 * k;
+              if constexpr (PAIR) umma_ss_pair(dt, wk, ak, idesc, accum);
+              else umma_ss(dt, wk, ak, idesc, accum);
+            }
+          if constexpr (PAIR) umma_commit_pair(&empty[stage], both);
+          else umma_commit(&empty[stage]);
           if (++stage == n_stages) { stage = 0; phase ^= 1; }
         }
-        umma_commit(&tfull[acc]);
+        if constexpr (PAIR) umma_commit_pair(&tfull[acc], both);
+        else umma_commit(&tfull[acc]);
         if (++acc == n_acc) { acc = 0; acc_phase ^= 1; }
       }
     mma_done:;
@@ -662,6 +699,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       bar_phase ^= 1;
       return r;
     };
+    auto acc_free = [&]() {   // to the issuer of this accumulator's products
+      if (PAIR && tile_of) mbar_arrive_cluster(cluster_addr(&tempty[acc], lead));
+      else mbar_arrive(&tempty[acc]);
+    };
     // A split's round: rows [round * per_round, + nr) of a group of nv, CTA r
     // finishing share r of them, rows [base, base + rows)
     const int per_round = nb / n_rounds;
@@ -674,12 +715,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     uint32_t it = 0;
     for (int item = unit0; ok && item < total; item += n_units, ++it) {
-      const int nt = item / num_g, g = item - nt * num_g;
+      const int ntu = item / num_g, g = item - ntu * num_g, nt = ntu * PT + tile_of;
       const int b = one_group ? 0 : find_seq(prefix, p.batch, g);
       const int lo = p.row_lo ? p.row_lo[b] : 0;
       const int hi = p.seq_len ? p.seq_len[b] : p.cap;
       const int i0 = lo + (g - (one_group ? 0 : prefix[b])) * nb;
-      const bool bad = lo < 0 || hi > p.cap;   // reported when the prefix was built
+      // (bad ranges were reported when the prefix was built)
+      const bool bad = lo < 0 || hi > p.cap || (PAIR && nt >= p.n_tiles);
       // valid rows of the group
       const int nv = bad ? 0 : max(0, min(RP ? p.row_pairs : nb, hi - i0));
       const size_t row0 = (size_t)b * p.cap + i0;
@@ -731,7 +773,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               fence_proxy_async_smem();   // generic reads before the peers' next copies
               if (!(ok = epi_sync())) break;
             }
-            if (ew == 0 && lane < S) mbar_arrive_cluster(map_rank(smem_u32(peers_done), lane));
+            if (ew == 0 && lane < S) mbar_arrive_cluster(map_rank(smem_u32(peers_done), peer(lane)));
             if (!(ok = mbar_wait<true>(peers_done, ph, abort_flag, p.status))) break;
             // this CTA's partial rows of the round into its own ring
             if (ew == 0 && lane == 0)
@@ -750,7 +792,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             fence_proxy_async_smem();   // the bulk copies read what was just written
             __syncwarp();
             if (lane == 0) {
-              if (round == n_rounds - 1) mbar_arrive(&tempty[acc]);
+              if (round == n_rounds - 1) acc_free();
               mbar_arrive(own_in);
             }
             if (!(ok = mbar_wait(own_in, ph, abort_flag, p.status))) break;
@@ -758,9 +800,9 @@ __global__ void __launch_bounds__(kThreads, 1)
               const int d0 = min(nr, lane * share), dn = min(nr, d0 + share) - d0;
               const int slot = rank < lane ? rank : rank - 1;   // this CTA's place among lane's peers
               if (dn > 0)
-                bulk_to_peer(map_rank(smem_u32(recv + (size_t)slot * share * ROW), lane),
+                bulk_to_peer(map_rank(smem_u32(recv + (size_t)slot * share * ROW), peer(lane)),
                              smem_u32(own + (size_t)d0 * ROW), (uint32_t)(dn * ROW * 4),
-                             map_rank(smem_u32(parts_in), lane));
+                             map_rank(smem_u32(parts_in), peer(lane)));
             }
             if (!(ok = mbar_wait<true>(parts_in, ph, abort_flag, p.status))) break;
           }
@@ -803,7 +845,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if constexpr (!SPLIT) {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&tempty[acc]);
+          if (lane == 0) acc_free();
         } else {
           // generic reads of the ring before the next tile's bulk writes to it;
           // the peers' copies into this CTA are done, so their sources may go
@@ -811,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(ring_free);
           if (ew == 0 && lane < S && lane != rank)
-            mbar_arrive_cluster(map_rank(smem_u32(ring_free), lane));
+            mbar_arrive_cluster(map_rank(smem_u32(ring_free), peer(lane)));
         }
         if constexpr (is_resid<EPI> || EPI == EPI_ARGMAX) {
           // the four quarters' row sums (or maxima) of the tile
@@ -847,26 +889,27 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   tc_fence_before();
   __syncthreads();
-  if constexpr (SPLIT) cluster_sync();   // no CTA of the cluster still writes to this one
+  if constexpr (SPLIT || PAIR) cluster_sync();   // no CTA of the cluster still writes to this one
   if (*abort_flag) __nanosleep(1000000);   // let copies still in flight land
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, tmem_cols);
+    if constexpr (PAIR) tmem_dealloc_pair(tmem, tmem_cols);
+    else tmem_dealloc(tmem, tmem_cols);
   }
 }
 
-template <int EPI, bool RP, bool SPLIT>
+template <int EPI, bool RP, bool SPLIT, bool PAIR = false>
 cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                      const CUtensorMap &b3, const GemmParams &p, const FewPlan &plan,
                      bool one_group, int sms, cudaStream_t stream) {
-  auto kern = few_kernel<EPI, RP, SPLIT>;
+  auto kern = few_kernel<EPI, RP, SPLIT, PAIR>;
   static int max_clusters[64][4] = {};   // co-resident clusters of 1, 2, 4 and 8 CTAs (0: unknown)
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  const int S = plan.split;
+  const int S = plan.split * (PAIR ? 2 : 1);   // CTAs of a cluster
   const int si = S == 1 ? 0 : S == 2 ? 1 : S == 4 ? 2 : 3;
-  if (S != 1 << si || plan.nb < 16 || plan.nb > 256 || plan.nb % 16) return cudaErrorInvalidValue;
+  if (S != 1 << si || S > kFewMaxSplit || plan.nb < 16 || plan.nb > 256 || plan.nb % 16) return cudaErrorInvalidValue;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -906,35 +949,45 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
   best.n_tiles = n_tiles;
   best.cycles = 1e300;
   const int nk = ((K + BK - 1) / BK) * (a_split ? 2 : 1);
+  const bool resid = epi == EPI_RESID_BF16 || epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT;
   const double hbm = (double)n_tiles * wt * BM * K * 2 / 3500.0;   // weight bytes at 6.7 TB/s, 1.9 GHz
   for (int nb = 16; nb <= kMaxRows; nb *= 2) {
     if (row_pairs && nb != 2 * row_pairs) continue;
     const double groups = (double)seqs * (double)((rows_per_seq + nb - 1) / nb);
-    // k-block: the products (2 cycles per row) or their operands' way into
-    // shared memory (measured on the Qwen2.5 projections: 266 cycles for 18 KB,
-    // 570 for 32 KB, 630 to 670 for 48 KB)
-    const double tk = std::max(2.0 * nb * wt, 180.0 + stage_bytes(wt, nb) / 105.0);
     for (int S = 1; S <= kFewMaxSplit; S *= 2) {
       const int rounds = S > 1 ? split_rounds(wt, nb, S) : 1;
       if (S > 1 && (nk < 4 * S || rounds == 0)) break;
-      const double units = floor(sms / S * (S >= 4 ? 0.95 : 1.0));
-      const double waves = std::ceil(groups * n_tiles / std::max(1.0, units));
-      // a tile's end: about 3600 cycles per 16-row block of a warp (SwiGLU 2600),
-      // for a split the exchange before it; without a split it overlaps the
-      // next tile's products while two accumulators fit
-      const double fin = 1500.0 + (wt == 2 ? 80.0 : 112.0) * std::min<double>(nb, (double)rows_per_seq) / S;
-      const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
-      const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
-      const double main = waves * std::ceil((double)nk / S) * tk;
-      const double ends = waves * fix + (overlapped ? fin : 0.0);
-      // several groups read the same weight tiles at the same time, which holds
-      // the SMs' requests longer (gate/up of 256 rows, 271 MB: 128-row groups
-      // 70 us at 4.9 TB/s, one of 256 rows 66 us)
-      const double t = std::max(main, hbm * (groups > 1 ? 1.5 : 1.1)) + ends + 0.05 * (main + ends);
-      if (t < best.cycles * 0.98) {
-        best.nb = nb;
-        best.split = S;
-        best.cycles = t;
+      for (int pt = 1; pt <= 2; ++pt) {   // 2: CTA pairs
+        // whole groups of the residual products, split (128-row groups measured
+        // 62 us against 59, the projections the same, gate/up 64 against 65)
+        if (pt == 2 && (!resid || nb != kMaxRows || S == 1 || 2 * S > kFewMaxSplit || row_pairs))
+          break;
+        // k-block: the products (2 cycles per row) or their operands' way into
+        // shared memory (measured on the Qwen2.5 projections: 266 cycles for 18 KB,
+        // 570 for 32 KB, 630 to 670 for 48 KB)
+        const double tk = std::max(2.0 * nb * wt, 180.0 + stage_bytes(wt, nb / pt) / 105.0);
+        const int ctas = S * pt;
+        const double units = floor(sms / ctas * (ctas >= 4 ? 0.95 : 1.0));
+        const double waves = std::ceil(groups * ((n_tiles + pt - 1) / pt) / std::max(1.0, units));
+        // a tile's end: about 3600 cycles per 16-row block of a warp (SwiGLU 2600),
+        // for a split the exchange before it; without a split it overlaps the
+        // next tile's products while two accumulators fit
+        const double fin = 1500.0 + (wt == 2 ? 80.0 : 112.0) * std::min<double>(nb, (double)rows_per_seq) / S;
+        const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
+        const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
+        const double main = waves * std::ceil((double)nk / S) * tk;
+        // (a pair's set-up and hand-overs: about 2 us a launch)
+        const double ends = waves * fix + (overlapped ? fin : 0.0) + (pt == 2 ? 3500.0 : 0.0);
+        // several groups read the same weight tiles at the same time, which holds
+        // the SMs' requests longer (gate/up of 256 rows, 271 MB: 128-row groups
+        // 70 us at 4.9 TB/s, one of 256 rows 66 us)
+        const double t = std::max(main, hbm * (groups > 1 ? 1.5 : 1.1)) + ends + 0.05 * (main + ends);
+        if (t < best.cycles * 0.98) {
+          best.nb = nb;
+          best.split = S;
+          best.pair = pt == 2;
+          best.cycles = t;
+        }
       }
     }
   }
@@ -948,22 +1001,25 @@ cudaError_t launch_few(int epi, const CUtensorMap &a, const CUtensorMap &b, cons
 #define CC_FEW_T(E, R)                                                                   \
   (plan.split > 1 ? launch_t<E, R, true>(a, b, b2, b3, p, plan, one_group, sms, st)      \
                   : launch_t<E, R, false>(a, b, b2, b3, p, plan, one_group, sms, st))
-#define CC_FEW(E) CC_FEW_T(E, false)
+#define CC_FEW_RESID(E)                                                                  \
+  (plan.pair ? launch_t<E, false, true, true>(a, b, b2, b3, p, plan, one_group, sms, st) \
+             : CC_FEW_T(E, false))
 #define CC_FEW_DECODE(E) (p.row_pairs ? CC_FEW_T(E, true) : CC_FEW_T(E, false))
   if (p.row_pairs && (epi == EPI_RESID_BF16 || epi == EPI_RESID_LOGIT)) return cudaErrorInvalidValue;
   switch (epi) {
     case EPI_QROPE: return CC_FEW_DECODE(EPI_QROPE);
-    case EPI_RESID_BF16: return CC_FEW(EPI_RESID_BF16);
-    case EPI_RESID_F32: return CC_FEW_DECODE(EPI_RESID_F32);
+    case EPI_RESID_BF16: return CC_FEW_RESID(EPI_RESID_BF16);
+    case EPI_RESID_F32:
+      return p.row_pairs ? CC_FEW_T(EPI_RESID_F32, true) : CC_FEW_RESID(EPI_RESID_F32);
     case EPI_SWIGLU: return CC_FEW_DECODE(EPI_SWIGLU);
     case EPI_BF16: return CC_FEW_DECODE(EPI_BF16);
     case EPI_QKV: return CC_FEW_DECODE(EPI_QKV);
     case EPI_ARGMAX: return CC_FEW_DECODE(EPI_ARGMAX);
-    case EPI_RESID_LOGIT: return CC_FEW(EPI_RESID_LOGIT);
+    case EPI_RESID_LOGIT: return CC_FEW_RESID(EPI_RESID_LOGIT);
     default: return cudaErrorInvalidValue;
   }
 #undef CC_FEW_DECODE
-#undef CC_FEW
+#undef CC_FEW_RESID
 #undef CC_FEW_T
 }
 

@@ -13,6 +13,7 @@ constexpr int kFewMaxSplit = 8;   // K splits = CTAs of a cluster (the portable 
 // of a cluster.
 struct FewPlan {
   int nb, split;
+  bool pair;       // two column tiles to a pair of CTAs, which share the activation rows
   int n_tiles;     // column tiles (EPI_QKV: those of Q, K and V, each rounded up)
   double cycles;   // estimated SM cycles
 };
@@ -22,7 +23,7 @@ constexpr int kFewTileCols = 128;   // output columns of a tile
 // one group of 2 * row_pairs rows (GemmParams::row_pairs).
 FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
                  int row_pairs, int sms);
-// a: A rows x K, box 64 x plan.nb; b (b2, b3): weights N x K, box 64 x 128, and
+// a: A rows x K, box 64 x plan.nb (half of it with pair); b (b2, b3): weights N x K, box 64 x 128, and
 // for rotated projections (EPI_QROPE's b, EPI_QKV's b and b2) the 5-D view
 // [heads][head_dim / 32][2][16][K], box {64, 16, 2, head_dim / 32, 128 / head_dim}.
 // one_group: the launch has one row group (known on the host), so the first
