@@ -976,8 +976,10 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
         const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
         const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
         const double main = waves * std::ceil((double)nk / S) * tk;
-        // (a pair's set-up and hand-overs: about 2 us a launch)
-        const double ends = waves * fix + (overlapped ? fin : 0.0) + (pt == 2 ? 3500.0 : 0.0);
+        // (a pair's set-up and hand-overs: about 2 us for a launch alone, less
+        // behind another kernel: the O projection of 512 Qwen2.5-7B rows is 35 us
+        // alone either way, and all 28 layers take 6860 us without, 6710 with)
+        const double ends = waves * fix + (overlapped ? fin : 0.0) + (pt == 2 ? 1500.0 : 0.0);
         // several groups read the same weight tiles at the same time, which holds
         // the SMs' requests longer (gate/up of 256 rows, 271 MB: 128-row groups
         // 70 us at 4.9 TB/s, one of 256 rows 66 us)
