@@ -243,12 +243,8 @@ bool kv_format_ok(const cc_model_cfg *c, const cc_kv_cache *kv) {
   return true;
 }
 
-// Up to so many rows a CTA-pair launch has too few row tiles for a last wave
-// worth splitting, and gets no scratch for it.
-constexpr size_t kSplitMinRows = 512;
-
 struct ScoreWs {
-  size_t xn, q, o, h, act, part, ztgt, hpart, sspart, split_count, split_part, total;
+  size_t xn, q, o, h, act, part, ztgt, hpart, sspart, total;
   int n_vtiles;
   int n_htiles;   // column tiles of a d-column projection (at most d / 128): partials of
                   // the fused logit head (logit mode) and of the post-attention RMSNorm
@@ -278,10 +274,6 @@ ScoreWs score_layout(const cc_model_cfg *c, int batch, int cap, cc_score_mode mo
     w.hpart = take(R * w.n_htiles * 8);
   }
   w.sspart = take(R * w.n_htiles * 4);
-  if (R > kSplitMinRows) {
-    w.split_count = take(kGemmSplitCounters * 4);
-    w.split_part = take(kGemmSplitSlots * kGemmSplitFloats * 4);
-  }
   w.total = off;
   return w;
 }
@@ -477,19 +469,14 @@ cc_status rope_weights(Gemm &g, const void *w, int n, int k, int head_dim) {
   return CC_OK;
 }
 
-// Scratch of a pass's CTA-pair launches (GemmParams::split_part), the counters
-// cleared before the pass's first.
+// Scratch of an append's CTA-pair launches (GemmParams::split_part), the counters
+// cleared before its first.  (A scored row's bits must not depend on the range
+// of rows it is scored with, so scoring passes leave their last waves whole.)
 struct GemmSplit {
   float *part = nullptr;
   unsigned *count = nullptr;
   bool clear = false;
 };
-GemmSplit gemm_split(const ScoreWs &L, uint8_t *ws) {
-  if (!L.split_part) return {};
-  return {reinterpret_cast<float *>(ws + L.split_part),
-          reinterpret_cast<unsigned *>(ws + L.split_count), false};
-}
-
 cc_status run_gemm(Gemm &g, int epi, int kind, int sms, cudaStream_t st, GemmSplit *split = nullptr) {
   TimedScope t(kind, st);
   if (split && split->part && gemm_may_split(epi, g.p, sms)) {
@@ -665,8 +652,12 @@ cc_status run_attention(const cc_model_cfg *c, const void *q, const void *k, con
 struct AppendWs {
   ScoreWs s;          // xn, q, o, h, act: the appended slots as packed rows
   size_t lo, hi, pbase, ptotal, rowmap;   // AppendRows
-  size_t part_o, part_ml, total;          // part_*: key-split partials of the attention
+  size_t part_o, part_ml;                 // key-split partials of the attention
+  size_t split_count, split_part, total;  // GemmSplit (0: none)
 };
+// Up to so many rows a CTA-pair launch has too few row tiles for a last wave
+// worth splitting, and gets no scratch for it.
+constexpr size_t kSplitMinRows = 512;
 
 AppendWs append_layout(const cc_model_cfg *c, int batch, int cap) {
   AppendWs w{};
@@ -680,6 +671,10 @@ AppendWs append_layout(const cc_model_cfg *c, int batch, int cap) {
   w.rowmap = take((size_t)batch * cap * 4);
   w.part_o = take((size_t)kAttnMaxSplitSlots * 256 * c->head_dim * 4);
   w.part_ml = take((size_t)kAttnMaxSplitSlots * 256 * 8);
+  if ((size_t)batch * cap > kSplitMinRows) {
+    w.split_count = take(kGemmSplitCounters * 4);
+    w.split_part = take(kGemmSplitSlots * kGemmSplitFloats * 4);
+  }
   w.total = off;
   return w;
 }
@@ -766,7 +761,11 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   const AppendRows rows = append_rows(L, wsb);
   const int32_t *total = rows.total;
   unsigned *status = dev->status;
-  GemmSplit ksplit = gemm_split(L.s, wsb);
+  GemmSplit ksplit;
+  if (L.split_part) {
+    ksplit.part = reinterpret_cast<float *>(wsb + L.split_part);
+    ksplit.count = reinterpret_cast<unsigned *>(wsb + L.split_count);
+  }
   const int max_rows = (int)std::min((uint64_t)batch * max_count, (uint64_t)batch * cap);
   // (the decode attention, which reads and writes the pairs, takes groups of 8 at most)
   const int rp = max_count == 1 && c->n_q_heads / c->n_kv_heads <= kDecMaxG
@@ -836,7 +835,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
       g.p.k_qscale = 1.f / kvf.k_scale;
       g.p.v_qscale = 1.f / kvf.v_scale;
       g.p.pg = kvf.pg;
-      if ((s = run_gemm(g, EPI_QKV, CC_KERNEL_GEMM_QKV, dev->sms, st, &ksplit)) != CC_OK) return s;
+      if ((s = run_gemm(g, EPI_QKV, CC_KERNEL_GEMM_QKV, dev->sms, st)) != CC_OK) return s;
     } else {
       struct Proj { const void *w, *bias; void *out; int n, epi, kind; };
       const Proj projs[3] = {{lw.wq, lw.bq, q, qd, EPI_QROPE, CC_KERNEL_GEMM_QROPE},
@@ -866,7 +865,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
           rope_turns(c, g.p.turns);
           if ((s = rope_weights(g, pj.w, pj.n, d, c->head_dim)) != CC_OK) return s;
         }
-        if ((s = run_gemm(g, pj.epi, pj.kind, dev->sms, st, &ksplit)) != CC_OK) return s;
+        if ((s = run_gemm(g, pj.epi, pj.kind, dev->sms, st)) != CC_OK) return s;
       }
     }
     // o = attention of the chunk rows over the memory and the chunk (causal)
@@ -884,7 +883,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     scaled(gu);
     gu.p.out = act;
     gu.p.ldo = f;
-    if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st, &ksplit)) != CC_OK) return s;
+    if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
     const void *next_gain = l + 1 < c->n_layers ? w->layers[l + 1].attn_norm : final_gain;
     if ((s = resid(act, f, lw.w_down, next_gain, CC_KERNEL_GEMM_DOWN)) != CC_OK) return s;
   }
@@ -968,7 +967,6 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
   const bool logit = (mode & 0xFF) == CC_SCORE_LOGIT;
   const bool keep_outside = (mode & CC_SCORE_RANGE_ONLY) != 0;   // other entries untouched
   uint8_t *wsb = reinterpret_cast<uint8_t *>(ws);
-  GemmSplit ksplit = gemm_split(L, wsb);
   void *xn = wsb + L.xn, *q = wsb + L.q, *o = wsb + L.o, *act = wsb + L.act;
   float *h = reinterpret_cast<float *>(wsb + L.h);
   // the row kernels' row ends (the range's, or the sequence ends); attention
@@ -1021,7 +1019,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     gq.p.head_dim = c->head_dim;
     rope_turns(c, gq.p.turns);
     if ((s = rope_weights(gq, lw.wq, qd, d, c->head_dim)) != CC_OK) return s;
-    if ((s = run_gemm(gq, EPI_QROPE, CC_KERNEL_GEMM_QROPE, dev->sms, st, &ksplit)) != CC_OK) return s;
+    if ((s = run_gemm(gq, EPI_QROPE, CC_KERNEL_GEMM_QROPE, dev->sms, st)) != CC_OK) return s;
     // O = counter-causal attention
     CC_TRY(wait_kv_ready(kv, l, l + 1, st));
     // (act is free until the MLP: the layer's bf16 copy of an e4m3 cache, or its
@@ -1051,7 +1049,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     go.p.norm_split = split ? 1 : 0;
     go.p.ss_part = ss_part;
     go.p.ab_f16 = go.p.out_f16 = f16 ? 1 : 0;
-    if ((s = run_gemm(go, epi_o, CC_KERNEL_GEMM_OPROJ, dev->sms, st, &ksplit)) != CC_OK) return s;
+    if ((s = run_gemm(go, epi_o, CC_KERNEL_GEMM_OPROJ, dev->sms, st)) != CC_OK) return s;
     // act = silu(xn Wg^T / rms(h)) * (xn Wu^T / rms(h))
     Gemm gu;
     if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, batch, cap, sl, status,
@@ -1066,7 +1064,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     gu.p.ss_d = d;
     gu.p.eps = c->rms_eps;
     gu.p.ab_f16 = gu.p.out_f16 = f16 ? 1 : 0;
-    if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st, &ksplit)) != CC_OK) return s;
+    if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
     // h = h + act Wd^T; in logit mode the last layer's add is fused with the
     // head: per column tile, partial sums of h^2 and of h * g . W_U[x_i]
     const int epi_d = logit && l == c->n_layers - 1 ? EPI_RESID_LOGIT : EPI_RESID_F32;
@@ -1095,7 +1093,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
       gd.p.ss_part = ss_part;
       ss_tiles = gd.p.n_tiles;
     }
-    if ((s = run_gemm(gd, epi_d, CC_KERNEL_GEMM_DOWN, dev->sms, st, &ksplit)) != CC_OK) return s;
+    if ((s = run_gemm(gd, epi_d, CC_KERNEL_GEMM_DOWN, dev->sms, st)) != CC_OK) return s;
   }
   // head
   if (logit) {
@@ -1120,7 +1118,7 @@ cc_status run_score(const cc_model_cfg *c, const cc_model_weights *w, const cc_k
     gl.p.ldo = L.n_vtiles;
     gl.p.tokens = kv->tokens;
     gl.p.z_target = zt;
-    if ((s = run_gemm(gl, EPI_LSE, CC_KERNEL_GEMM_LMHEAD, dev->sms, st, &ksplit)) != CC_OK) return s;
+    if ((s = run_gemm(gl, EPI_LSE, CC_KERNEL_GEMM_LMHEAD, dev->sms, st)) != CC_OK) return s;
     TimedScope t(CC_KERNEL_LSE_COMBINE, st);
     CC_TRY(launch_lse_combine(part, L.n_vtiles, zt, scores, kv->seq_len, cap, rows, st, rng_lo,
                               rng_hi, keep_outside));

@@ -43,9 +43,9 @@
 // operands' way into shared memory (about 630 cycles per 48 KB k-block) and the
 // tiles' ends.  Measured against the 128 x 256-tile kernel with K splits
 // chained through global memory, per launch (CUDA events): Qwen2.5-7B layer,
-// a 256-row chunk: q/k/v 43 -> 28 us, O 33 -> 27 us, down 71 -> 50 us (four
-// CTAs, partials in two rounds), gate/up 86 -> 66 us; a 512-slot cache: down 84
-// -> 76 us; the 512-slot tiny model's pass 78 -> 60 us.
+// a 256-row chunk: q/k/v 43 -> 28 us, O 33 -> 27 us, down 71 -> 48 us (pairs,
+// four splits, partials in two rounds), gate/up 75 -> 66 us; a 512-slot cache:
+// down 84 -> 67 us; the 512-slot tiny model's pass 78 -> 60 us.
 // Decode steps (Qwen2.5-7B layer, one row) against CUDA-core GEMVs streaming
 // the weights: gate/up 57 -> 50 us (271 MB), LM head 186 -> 159 us (1.09 GB,
 // 6.8 TB/s), down 34 -> 34 us, q/k/v 15 -> 20 and O 14.5 -> 19 us when timed

@@ -6,7 +6,7 @@
 
 namespace cc {
 
-constexpr int kFewMaxSplit = 8;   // K splits = CTAs of a cluster (the portable cluster size)
+constexpr int kFewMaxSplit = 8;   // CTAs of a cluster: K splits, or half as many of pairs (the portable size)
 
 // How a launch is cut: row groups of nb activation rows (the N of a product),
 // column tiles of 128 columns, and the K range of each tile over `split` CTAs

@@ -18,8 +18,8 @@
 // M = 256, N = 256 product per pair, each CTA staging its own 128 A rows and
 // half of the B tile, so a CTA moves 32 KB instead of 48 KB through L2 and
 // shared memory per 128 x 256 x 64 block of its output.  Where their last wave
-// would leave half of the pairs or more without a tile, its tiles are cut along
-// K over those pairs (split_wave below).
+// would leave half of the pairs or more without a tile, an append's long products
+// are cut along K there (split_wave below).
 #include "gemm.cuh"
 
 #include <algorithm>
@@ -576,8 +576,10 @@ CC_DEV void tile_coords(const GemmParams &p, int t, int num_m, int &m, int &n) {
 // 15 us): the exchange and the sums cost 15 to 20 us.  Measured on the down
 // projection of 2313 Llama-3-8B rows (160 tiles on 76 pairs): 229 us whole,
 // 201 us in eight parts, 194 us in four; the O projection (K = 4096) 78 us
-// whole, 92 us in four.  Its own kernel variant, of the residual products
-// alone (the others are shorter): the code costs the plain epilogues registers.
+// whole, 92 us in four.  Its own kernel variant, of the residual add alone (an
+// append's other products are shorter): the code costs a plain epilogue
+// registers.  A row's bits then depend on how many rows the launch has, which a
+// scored row's may not (row ranges): appends only.
 constexpr int kSplitStages = 28, kMaxSplit = 8;
 CC_DEV int split_wave(int rem, int n_units, int n_stages) {
   if (rem == 0) return 1;
@@ -959,7 +961,7 @@ template <int EPI>
 cudaError_t launch(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                    const CUtensorMap &b3, const GemmParams &p, int grid, cudaStream_t stream) {
   constexpr bool kWide = EPI == EPI_SWIGLU || EPI == EPI_LSE || EPI == EPI_QKV;
-  if constexpr (EPI == EPI_RESID_BF16 || EPI == EPI_RESID_F32 || EPI == EPI_RESID_LOGIT) {
+  if constexpr (EPI == EPI_RESID_F32) {
     if (p.split_part && gemm_may_split(EPI, p, grid))
       return launch_t<EPI, BN, true, true>(a, b, b2, b3, p, grid, stream);
   }
@@ -977,14 +979,13 @@ cudaError_t launch(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap
 
 }  // namespace
 
-// (up to six waves at the row bound: the variant's epilogue is 1 % slower, 532
-// -> 538 us on the down projection of 8192 rows in seven waves)
+// (up to six waves at the row bound: the variant's epilogue was 1 % slower, 532
+// -> 538 us, on a down projection of 8192 rows in seven waves)
 bool gemm_may_split(int epi, const GemmParams &p, int sms) {
   const long long tiles = ((long long)p.batch * p.cap + 255) / 256 * p.n_tiles;
   if (tiles > 6LL * (sms / 2)) return false;
   const int stages = ((p.K + BK - 1) / BK * (p.a_split ? 2 : 1) + 1) / 2;
-  return (epi == EPI_RESID_BF16 || epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT) && p.pair &&
-         p.block_n == BN && stages >= 2 * kSplitStages;
+  return epi == EPI_RESID_F32 && p.pair && p.block_n == BN && stages >= 2 * kSplitStages;
 }
 
 int gemm_block_n(int epi) { return epi == EPI_SWIGLU ? 128 : BN; }
