@@ -1357,7 +1357,6 @@ def run_append(args, dist):
                 "h2d_bytes_per_step": int(host_tok.numel() * 4 + 4), "d2h_bytes_per_step": 4,
                 "ms_per_step": round(e2e_ms, 4)},
         "gpu_launches": int(sum(c for c, _ in kernels.values())),
-        "dtype": "f16" if f16 else "bf16",
         "roofline": {"kernel": dom, "bound": d.get("bound"), "achieved": d.get("achieved"),
                      "peak": peaks["bf16_tflops"] if d.get("bound") == "tensor" else peaks["hbm_gbs"],
                      "unit": d.get("unit"), "frac": d.get("frac"), "traffic": None,
@@ -1484,7 +1483,6 @@ def run_decode(args, dist):
                 "h2d_bytes_per_step": 4 * B, "d2h_bytes_per_step": 4 * B,
                 "ms_per_step": round(e2e_ms, 4)},
         "gpu_launches": int(sum(c for c, _ in kernels.values())),
-        "dtype": "f16" if f16 else "bf16",
         "roofline": {"kernel": dom, "bound": dd.get("bound"), "achieved": dd.get("achieved"),
                      "peak": peaks["hbm_gbs"], "unit": dd.get("unit"), "frac": dd.get("frac"),
                      "traffic": None, "peak_source": f"{peak_src} (HBM copy)"},
