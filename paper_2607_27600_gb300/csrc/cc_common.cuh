@@ -499,6 +499,8 @@ CC_DEV float silu(float x) {
   const float c = fmaf(fmaf(-q, y, x), r, q);
   return y > 0x1.fffffep127f || x > 64.0f ? q : c;
 }
+// The same with a full division (the same bits for |x| < 80).
+CC_DEV float silu_div(float x) { return x / (1.0f + __expf(-x)); }
 
 // cos/sin of pos * inv_freq, with the angle reduced exactly: turns is
 // inv_freq / (2 pi) in 0.64 fixed point, so pos * turns mod 2^64 is the
