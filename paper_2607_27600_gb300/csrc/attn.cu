@@ -834,13 +834,19 @@ __global__ void __launch_bounds__(kDecWarps * 32, 3)
   const int vstep = p.pg.head_major ? 1 : p.n_kv_heads;
   constexpr int EB = FP8 ? 1 : 2;
 
-  // vector index of a chunk's first key (-1: bad page, its keys are skipped)
+  // vector index of a chunk's first key (-1: bad page, its keys are skipped;
+  // the chunk's loads report it)
   auto chunk_base = [&](int c) -> long long {
     return kv_vec(p.pg, p.cap, u.b, u.g, k0 + c * kDecChunk);
   };
+  auto load_base = [&](int c) -> long long {
+    const long long base = chunk_base(c);
+    if (base < 0 && tid == 0) set_status(p.status, CC_ERR_DEVICE_ARG);
+    return base;
+  };
   auto issue = [&](int c, int st) {   // bf16: chunk c into stage st; past the end: zeros
     if (c < chunks) {
-      const long long base = chunk_base(c);
+      const long long base = load_base(c);
       const int n = base < 0 ? 0 : min(kDecChunk, k1 - (k0 + c * kDecChunk));
       const uint32_t kd = sbase + st * 2 * L::TILE, vd = kd + L::TILE;
 #pragma unroll
@@ -859,7 +865,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, 3)
   uint4 kc[FPER], vc[FPER];
   auto fetch8 = [&](int c) {
     if (c >= chunks) return;
-    const long long base = chunk_base(c);
+    const long long base = load_base(c);
     const int n = base < 0 ? 0 : min(kDecChunk, k1 - (k0 + c * kDecChunk));
 #pragma unroll
     for (int x = 0; x < FPER; ++x) {
@@ -898,7 +904,6 @@ __global__ void __launch_bounds__(kDecWarps * 32, 3)
   } else {
     for (int c = 0; c < kDecStages - 1; ++c) issue(c, c);
   }
-  if (chunk_base(0) < 0 && tid == 0) set_status(p.status, CC_ERR_DEVICE_ARG);
 
   // Q as the first operand: row lane / 4 = the head's hi part, + 8 its lo part
   const int head = lane >> 2, quad = lane & 3;

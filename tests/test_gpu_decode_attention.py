@@ -61,3 +61,56 @@ def test_step_matches_oracle(pkg, dh, hkv, g, lens, cap, layout):
     for i, n in enumerate(lens):
         want = cn["h_last"][i, n]
         assert np.abs(got[i, n] - want).max() <= tol * np.abs(want).max(), (i, n)
+
+
+def keys_per_split(shape, lens, cap):
+    """Keys of a split as the kernel plans them (csrc/attn.cu, dec_split_keys)
+    for the longest of sequences of `lens` keys."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    units = len(lens) * shape.n_kv_heads
+    ctas = max(sms, 3 * sms - units // 2)
+    splits = max(1, min(128, -(-cap // 64), 160 * 256 // 8 // units, 4 * ctas // units))
+    even = int(sum(lens) * shape.n_kv_heads / ctas)
+    return -(-max(even, -(-max(lens) // splits)) // 64) * 64
+
+
+def decode(pkg, shape, w, c):
+    from paper_2607_27600_gb300 import cc
+    b, cap = c["tokens"].shape
+    nxt = torch.empty(b, dtype=torch.int32, device="cuda")
+    best = torch.empty(b, dtype=torch.float32, device="cuda")
+    ws = cc.alloc_workspace(cc.cc_decode_workspace_size(shape, b, cap))
+    tok = np.random.default_rng(5).integers(0, shape.vocab, size=b)
+    cc.cc_decode_step(shape, pkg.Weights(w), pkg.Cache(c),
+                      torch.from_numpy(tok.astype(np.int32)).cuda(), nxt, best, ws)
+    return cc.cc_get_status(), tok, nxt.cpu().numpy(), best.cpu().numpy()
+
+
+@pytest.mark.parametrize("kv", ["bf16", "e4m3"])
+@pytest.mark.parametrize("entry", [1 << 20, -1])
+def test_bad_page_inside_a_split_is_reported(pkg, kv, entry):
+    """A block-table entry outside the pool whose slots start no split: its
+    keys are skipped and CC_ERR_DEVICE_ARG recorded; the other sequences'
+    tokens and logits keep their bits and the context stays usable."""
+    import bench
+    from paper_2607_27600_gb300 import cc
+    from tests.test_gpu_fp8 import fp8_views
+    shape = ModelShape(2, 128, 4, 1, 64, 256, 300, 1e4, 1e-5)
+    lens, cap = [3900 + i for i in range(32)], 4096
+    per = keys_per_split(shape, [n + 1 for n in lens], cap)
+    page = next(i for i in range(1, 20) if (128 * i) % per >= 64 and (128 * i) // per == (128 * i + 127) // per)
+    w = to_device(to_np(synth.model_weights(shape, 3, with_kv_proj=True)))
+    c_np = to_np(synth.synthetic_cache(shape, lens, cap, 4))
+    good = bench.to_paged_cache(fp8_views(c_np)[1] if kv == "e4m3" else to_device(c_np), 128, 11)
+    bad = {k: v.clone() if isinstance(v, torch.Tensor) else v for k, v in good.items()}
+    bad.update({k: [x.clone() for x in good[k]] for k in ("k", "v")})
+    bad["block_table"][7, page] = entry
+    status, _, nxt, best = decode(pkg, shape, w, good)
+    assert status == cc.CC_OK
+    bad_status, _, bad_nxt, bad_best = decode(pkg, shape, w, bad)
+    assert bad_status == cc.CC_ERR_DEVICE_ARG
+    others = np.arange(len(lens)) != 7
+    np.testing.assert_array_equal(bad_nxt[others], nxt[others])
+    np.testing.assert_array_equal(bad_best[others], best[others])
+    assert np.isfinite(bad_best[7])
+    assert cc.cc_get_status() == cc.CC_OK
