@@ -652,9 +652,10 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
     for (int e = 0; e < DPL; ++e) o[e] *= f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      // a split without keys holds no O row (its memory may hold any bits)
-      if (!(ml[k].y > 0.f)) continue;
-      const float w = fast_exp2((ml[k].x - mx) * c);
+      // a split without keys holds no O row (its memory may hold any bits); one
+      // with a NaN sum makes the row's sum NaN, and the row 0
+      if (ml[k].y == 0.f) continue;
+      const float w = ml[k].y > 0.f ? fast_exp2((ml[k].x - mx) * c) : 0.f;
       l = fmaf(w, ml[k].y, l);
 #pragma unroll
       for (int e = 0; e < DPL; ++e) o[e] = fmaf(w, reinterpret_cast<const float *>(&v[k])[e], o[e]);
@@ -666,7 +667,8 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
                        (size_t)(u.g * G + hl) * DH + lane * DPL;
 #pragma unroll
   for (int e = 0; e < DPL; e += 2)
-    *reinterpret_cast<uint32_t *>(dst + e) = pack_bf16x2(o[e] * inv, o[e + 1] * inv);
+    *reinterpret_cast<uint32_t *>(dst + e) =
+        l > 0.f ? pack_bf16x2(o[e] * inv, o[e + 1] * inv) : 0u;
 }
 
 template <int DH, bool CAUSAL, bool SPLIT = false, bool F16 = false>
@@ -1075,8 +1077,8 @@ __global__ void __launch_bounds__(kDecGroups * DH)
   part[grp][d] = acc;
   __syncthreads();
   if (grp > 0) return;
-  const float v = ((part[0][d] + part[1][d]) + (part[2][d] + part[3][d])) *
-                  (l > 0.f ? p.v_scale / l : 0.f);
+  const float sum = (part[0][d] + part[1][d]) + (part[2][d] + part[3][d]);
+  const float v = l > 0.f ? sum * (p.v_scale / l) : 0.f;   // (a NaN sum of weights: 0)
   store_decode(p, (size_t)(slot0_row<true>(p, u) + u.p0) * p.out_ld + (size_t)(u.g * p.group + h) * DH + d, v);
 }
 

@@ -114,3 +114,37 @@ def test_bad_page_inside_a_split_is_reported(pkg, kv, entry):
     np.testing.assert_array_equal(bad_best[others], best[others])
     assert np.isfinite(bad_best[7])
     assert cc.cc_get_status() == cc.CC_OK
+
+
+@pytest.mark.parametrize("slot", [0, 1400, 2999])
+@pytest.mark.parametrize("rows", [1, 40])
+def test_nan_key_gives_zero_rows(pkg, rows, slot):
+    """A row that attends a NaN key comes out 0, whichever key split holds the
+    key: a decode step (rows 1) and a chunk append, both with their keys split,
+    against the same call over zero values.  (Zero new values too: Wv = 0.)"""
+    from paper_2607_27600_gb300 import cc
+    shape = ModelShape(2, 128, 4, 1, 64, 256, 300, 1e4, 1e-5)
+    n, cap = 3000, 3200
+    w_np = to_np(synth.model_weights(shape, 3, with_kv_proj=True))
+    w_np["layers"][0]["wv"] = np.zeros_like(w_np["layers"][0]["wv"])
+    out = []
+    for nan in (True, False):
+        c = to_device(to_np(synth.synthetic_cache(shape, [n], cap, 4)))
+        if nan:
+            c["k"][0][0, slot] = float("nan")
+        else:
+            c["v"][0].zero_()
+        weights, cache = pkg.Weights(to_device(w_np)), pkg.Cache(c)
+        tok = torch.arange(rows, dtype=torch.int32, device="cuda").reshape(1, rows)
+        if rows == 1:
+            ws = cc.alloc_workspace(cc.cc_decode_workspace_size(shape, 1, cap))
+            nxt = torch.empty(1, dtype=torch.int32, device="cuda")
+            cc.cc_decode_step(shape, weights, cache, tok[0], nxt, None, ws)
+        else:
+            ws = cc.alloc_workspace(cc.cc_append_workspace_size(shape, 1, cap))
+            count = torch.tensor([rows], dtype=torch.int32, device="cuda")
+            cc.cc_append_chunk(shape, weights, cache, tok, None, count, rows, ws)
+        assert cc.cc_get_status() == cc.CC_OK
+        out.append(c["h_last"][0, n:n + rows].float().cpu().numpy())
+    np.testing.assert_array_equal(out[0], out[1])
+    assert np.isfinite(out[0]).all()
