@@ -788,7 +788,7 @@ CC_DEV float add_parts(float hi, float lo) { return fabsf(hi) == INFINITY ? hi :
 CC_DEV void store_decode(const AttnParams &p, size_t el, float v) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(v);
   p.out[el] = hi;
-  if (p.out_lo_off > 0) p.out[el + p.out_lo_off] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  if (p.out_lo_off > 0) p.out[el + p.out_lo_off] = __float2bfloat16_rn(pair_rest(v, __bfloat162float(hi)));
 }
 
 // Keys of one split of a unit with n_keys keys: the batch's keys over about

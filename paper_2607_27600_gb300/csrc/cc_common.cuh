@@ -476,6 +476,10 @@ CC_DEV long long kv_vec(const KvLayout &L, int cap, int b, int g, int i) {
   return r < 0 ? -1 : r * L.hkv + g;
 }
 
+// What bf16 `hi` leaves out of x in a pair hi + lo; an infinite hi stands alone
+// (x - hi would be NaN there, or an infinity of the other sign).
+CC_DEV float pair_rest(float x, float hi) { return fabsf(hi) == INFINITY ? 0.f : x - hi; }
+
 // Two e4m3 codes (lo in the low byte): round to nearest even, saturating to
 // +-448 (the e4m3 K/V cache's element encoding).
 CC_DEV uint32_t pack_e4m3x2(float lo, float hi) {

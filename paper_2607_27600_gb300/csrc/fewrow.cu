@@ -260,7 +260,7 @@ CC_DEV void store_acts(uint16_t *out, const size_t (&at)[N], const float (&y)[N]
     for (int k = 0; k < N; ++k)
       if (live[k])
         out[at[k] + lo] = __bfloat16_as_ushort(
-            __float2bfloat16_rn(y[k] - __bfloat162float(__ushort_as_bfloat16(bits[k]))));
+            __float2bfloat16_rn(pair_rest(y[k], __bfloat162float(__ushort_as_bfloat16(bits[k])))));
   }
 }
 

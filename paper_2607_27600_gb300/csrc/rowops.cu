@@ -203,10 +203,10 @@ __global__ void __launch_bounds__(256)
     *reinterpret_cast<uint4 *>(xn + (size_t)row * d + e) = v;
     if (row_pairs) {
       uint4 lo;
-      lo.x = pack_bf16x2(f[0] * g[0] - bf16_lo(v.x), f[1] * g[1] - bf16_hi(v.x));
-      lo.y = pack_bf16x2(f[2] * g[2] - bf16_lo(v.y), f[3] * g[3] - bf16_hi(v.y));
-      lo.z = pack_bf16x2(f[4] * g[4] - bf16_lo(v.z), f[5] * g[5] - bf16_hi(v.z));
-      lo.w = pack_bf16x2(f[6] * g[6] - bf16_lo(v.w), f[7] * g[7] - bf16_hi(v.w));
+      lo.x = pack_bf16x2(pair_rest(f[0] * g[0], bf16_lo(v.x)), pair_rest(f[1] * g[1], bf16_hi(v.x)));
+      lo.y = pack_bf16x2(pair_rest(f[2] * g[2], bf16_lo(v.y)), pair_rest(f[3] * g[3], bf16_hi(v.y)));
+      lo.z = pack_bf16x2(pair_rest(f[4] * g[4], bf16_lo(v.z)), pair_rest(f[5] * g[5], bf16_hi(v.z)));
+      lo.w = pack_bf16x2(pair_rest(f[6] * g[6], bf16_lo(v.w)), pair_rest(f[7] * g[7], bf16_hi(v.w)));
       *reinterpret_cast<uint4 *>(xn + (size_t)(row + row_pairs) * d + e) = lo;
     }
 #pragma unroll

@@ -148,3 +148,25 @@ def test_nan_key_gives_zero_rows(pkg, rows, slot):
         out.append(c["h_last"][0, n:n + rows].float().cpu().numpy())
     np.testing.assert_array_equal(out[0], out[1])
     assert np.isfinite(out[0]).all()
+
+
+@pytest.mark.parametrize("batch", [1, 20])
+def test_infinite_activation_stays_infinite(pkg, batch):
+    """One SwiGLU activation past fp32's range: the residual stream takes the
+    sign of its down weights, as with single bf16 activations; the remainder of
+    an infinite value in a bf16 pair is 0, not a NaN."""
+    shape = ModelShape(2, 128, 4, 1, 64, 256, 300, 1e4, 1e-5)
+    w_np = to_np(synth.model_weights(shape, 3, with_kv_proj=True))
+    w_np["embed"][:, 0] = 1.0
+    for key in ("w_gate", "w_up"):
+        w_np["layers"][0][key][0] = 0.0
+        w_np["layers"][0][key][0, 0] = 3e19
+    down = w_np["layers"][0]["w_down"][:, 0]
+    down[down == 0.0] = 0.01
+    lens = [3 + i for i in range(batch)]
+    c = to_device(to_np(synth.synthetic_cache(shape, lens, 64, 4)))
+    status = decode(pkg, shape, to_device(w_np), c)[0]
+    assert status == 0
+    got = c["h_last"].float().cpu().numpy()
+    for i, n in enumerate(lens):
+        np.testing.assert_array_equal(got[i, n], np.sign(down) * np.float32(np.inf))
