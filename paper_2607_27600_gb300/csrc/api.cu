@@ -1478,7 +1478,7 @@ cc_status cc_partition_rows(const cc_model_cfg *cfg, int32_t full, const int32_t
 size_t cc_select_workspace_size(int32_t batch, int32_t cap) {
   (void)batch;
   (void)cap;
-  return 0;   // one CTA per sequence keeps its histograms in shared memory
+  return 0;   // the histograms live in shared memory
 }
 
 cc_status cc_select_keep(const float *scores, const int32_t *seq_len, int32_t batch, int32_t cap,

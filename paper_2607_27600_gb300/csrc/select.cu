@@ -1,7 +1,7 @@
 // select.cu -- keep-set selection (Algorithm DoMemRefresh: sigma = argsort of
 // the surprise scores, largest first; keep sigma[1:J]).
 //
-// One cluster of CTAs per sequence (one CTA for short caches), each CTA over a
+// One cluster of 1, 2, 4 or 8 CTAs per sequence (cluster_size), each CTA over a
 // contiguous segment of slots.  Slots rank by the 32-bit monotone key of their
 // score, ties toward the later slot.  The J-th largest key T is found by an
 // MSB radix select of 11 + 11 + 10 bits: each pass every CTA counts its
@@ -15,9 +15,11 @@
 //
 // Latency bounds it: a pass is a few barriers and round trips.  The segment's
 // keys stay in shared memory when they fit.  One CTA per sequence with 256-bin
-// passes over the scores in global memory took 18.5 us for 16384 slots and
-// 182 us for 131072 (launch after launch); this takes 13.4 and 24.
+// passes over the scores in global memory took 18.8 us for 16384 slots and
+// 151 us for 131072 (launch after launch); a cluster of eight takes 11.5 and 23.
 #include "select.cuh"
+
+#include <atomic>
 
 namespace cc {
 
@@ -25,11 +27,6 @@ namespace {
 
 constexpr int kThreads = 1024;
 constexpr int kBins = 2048;
-constexpr int kCluster = 8;                  // CTAs per sequence (the portable cluster size)
-// Caches up to this many slots: one CTA.  Measured (launch after launch, one and
-// eight CTAs): 8.3 / 12.3 us at 2048 slots, 10.3 / 12.4 at 8192, 16.4 / 13.4 at
-// 16384, 143 / 24 at 131072.
-constexpr int kOneCtaSlots = 8192;
 constexpr int kMaxCached = 44 * 1024;        // keys of a segment kept in shared memory at most
 constexpr uint32_t kKeyPosInf = 0xFF800000u;   // monotone key of +inf
 constexpr uint32_t kKeyNegInf = 0x007FFFFFu;   // monotone key of -inf
@@ -45,18 +42,18 @@ CC_DEV uint32_t monotone_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// The variable at p in CTA `rank` of the cluster (ONE: there is only this one).
-template <bool ONE>
+// The variable at p in CTA `rank` of the cluster of CS.
+template <int CS>
 CC_DEV uint32_t ld_rank(const uint32_t *p, int rank) {
-  if constexpr (ONE) return *p;
+  if constexpr (CS == 1) return *p;
   uint32_t v;
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(p, rank)) : "memory");
   return v;
 }
 
-template <bool ONE>
+template <int CS>
 CC_DEV void sync_all() {
-  if constexpr (ONE) __syncthreads();
+  if constexpr (CS == 1) __syncthreads();
   else cluster_sync();
 }
 
@@ -89,7 +86,7 @@ CC_DEV int block_excl_scan(int x, int *ws, int *total) {
   return r;
 }
 
-template <bool ONE>
+template <int CS>
 __global__ void __launch_bounds__(kThreads, 1)
     select_kernel(const float *scores, const int32_t *seq_len, int cap, const int32_t *budget,
                   int n_sink, int32_t *keep_idx, int32_t *keep_count, unsigned *status,
@@ -101,7 +98,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int ws[33];
   __shared__ int s_digit, s_above, s_count;
   __shared__ unsigned n_kept, n_tied;              // of this CTA's segment
-  const int CS = ONE ? 1 : kCluster, rank = ONE ? 0 : (int)cluster_ctarank();
+  const int rank = CS == 1 ? 0 : (int)cluster_ctarank();
   const int b = blockIdx.x / CS, tid = threadIdx.x, lane = tid & 31;
   pdl_trigger();
   pdl_wait();   // the scores come from the kernel before
@@ -144,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t prefix = 0;
   int k = J;
   bool settled = false;
-  constexpr int per = ONE ? kBins : kBins / kCluster;   // bins of a slice
+  constexpr int per = kBins / CS;   // bins of a slice
 #pragma unroll 1
   for (int pass = 0; pass < 3 && !settled; ++pass) {
     const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
@@ -158,7 +155,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if ((key & hi_mask) == prefix) atomicAdd(&h[(key >> shift) & digit_mask], 1u);
     }
     for (int i = tid; i < kBins; i += kThreads) hist[(pass & 1) ^ 1][i] = 0;   // the next pass's
-    sync_all<ONE>();
+    sync_all<CS>();
     // this CTA's slice, bins descending over the threads: running counts
     constexpr int PT = per > kThreads ? per / kThreads : 1;   // bins of a thread
     unsigned c[PT], sum = 0;
@@ -168,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       c[e] = 0;
       if (i >= 0) {
 #pragma unroll
-        for (int r = 0; r < (ONE ? 1 : kCluster); ++r) c[e] += ld_rank<ONE>(&h[rank * per + i], r);
+        for (int r = 0; r < CS; ++r) c[e] += ld_rank<CS>(&h[rank * per + i], r);
       }
       sum += c[e];
     }
@@ -182,14 +179,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (i >= 0) al[i] = run;
     }
     if (tid == 0) al[per] = 0;
-    sync_all<ONE>();
+    sync_all<CS>();
     // the slice that holds the boundary (digits descend from the last slice):
     // every warp reads the slices' totals and finds it alike
     unsigned t = 0;
-    if (lane < CS) t = ld_rank<ONE>(&al[0], lane);
+    if (lane < CS) t = ld_rank<CS>(&al[0], lane);
     unsigned above = 0;   // keys in the slices after this lane's
 #pragma unroll
-    for (int r = 1; r < (ONE ? 1 : kCluster); ++r) {
+    for (int r = 1; r < CS; ++r) {
       const unsigned y = __shfl_sync(0xFFFFFFFFu, t, r);
       if (r > lane) above += y;
     }
@@ -202,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int e = 0; e < PT; ++e) {
       const int i = tid * PT + e;
       if (i >= per) break;
-      const unsigned at = ld_rank<ONE>(&al[i], owner), over = ld_rank<ONE>(&al[i + 1], owner);
+      const unsigned at = ld_rank<CS>(&al[i], owner), over = ld_rank<CS>(&al[i + 1], owner);
       if (over < want && want <= at) {
         s_digit = owner * per + i;
         s_above = (int)(above + over);
@@ -232,12 +229,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   tied = __reduce_add_sync(0xFFFFFFFFu, tied);
   if (lane == 0 && kept) atomicAdd(&n_kept, kept);
   if (lane == 0 && tied) atomicAdd(&n_tied, tied);
-  sync_all<ONE>();
+  sync_all<CS>();
   int base = 0, tie_base = 0, tie_total = 0;   // before this segment; over the sequence
 #pragma unroll
-  for (int r = 0; r < (ONE ? 1 : kCluster); ++r) {
-    const int a = (int)ld_rank<ONE>(&n_kept, r);
-    const int t = (int)ld_rank<ONE>(&n_tied, r);
+  for (int r = 0; r < CS; ++r) {
+    const int a = (int)ld_rank<CS>(&n_kept, r);
+    const int t = (int)ld_rank<CS>(&n_tied, r);
     if (r < rank) {
       base += a;
       tie_base += t;
@@ -283,7 +280,30 @@ __global__ void __launch_bounds__(kThreads, 1)
     keep_count[b] = J;
     if (carry != J) set_status(status, CC_ERR_DEVICE_ARG);   // cannot happen
   }
-  sync_all<ONE>();   // no CTA reads this one's counts any more
+  sync_all<CS>();   // no CTA reads this one's counts any more
+}
+
+// CTAs per sequence of a launch: the least estimated time over the sizes, all
+// the batch's clusters in as many waves as the device's resident ones need.
+// Fitted to every size at batches of 1 to 256 and caps of 4096 to 131072 (launch
+// after launch): a lone CTA 5.5 us + 0.65 ns a slot, 1.24 ns past the slots whose
+// keys it holds; a cluster 12 us + 0.8 ns a slot of a CTA.  Eight CTAs whatever
+// the batch took 103 us for 128 sequences of 16384 slots, one CTA each 16 us.
+int cluster_size(int batch, int cap, uint64_t resident) {   // (16 bits per size)
+  int best = 1;
+  double least = 1e300;
+  for (int i = 0; i < 4; ++i) {
+    const int cs = 1 << i;
+    const double seg = (double)cap / cs;
+    const double one = (i == 0 ? 5.5e3 : 12e3) +
+                       seg * (seg > kMaxCached ? 1.24 : i == 0 ? 0.65 : 0.8);
+    const double t = ceil((double)batch / (double)(resident >> (16 * i) & 0xFFFF)) * one;
+    if (t < least) {
+      least = t;
+      best = cs;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -292,36 +312,48 @@ cudaError_t launch_select(const float *scores, const int32_t *seq_len, int batch
                           const int32_t *budget, int n_sink, int32_t *keep_idx,
                           int32_t *keep_count, unsigned *status, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
-  const bool one = cap <= kOneCtaSlots;
-  const int cs = one ? 1 : kCluster;
-  const int seg = ((cap + cs - 1) / cs + 3) & ~3;   // slots of a segment at most
-  const int cached = seg <= kMaxCached ? 1 : 0;
-  const auto kern = one ? select_kernel<true> : select_kernel<false>;
-  static bool attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 64 && !attr_set[dev]) {
-    for (auto k : {select_kernel<true>, select_kernel<false>}) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kMaxCached * 4);
-      if (e != cudaSuccess) return e;
-    }
-    attr_set[dev] = true;
-  }
+  using Kernel = decltype(&select_kernel<1>);
+  const Kernel kerns[4] = {select_kernel<1>, select_kernel<2>, select_kernel<4>, select_kernel<8>};
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)cs;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(batch * cs));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = cached ? (size_t)seg * 4 : 0;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = one ? 1 : 2;
+  static std::atomic<uint64_t> resident[64];   // clusters resident with full segments (0: unknown)
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  uint64_t fit = resident[dev].load();
+  if (fit == 0) {
+    for (int i = 0; i < 4; ++i) {
+      cudaError_t e = cudaFuncSetAttribute(kerns[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           kMaxCached * 4);
+      if (e != cudaSuccess) return e;
+      attr[0].val.clusterDim.x = 1u << i;
+      cfg.gridDim = dim3(1u << i);
+      cfg.dynamicSmemBytes = kMaxCached * 4;
+      cfg.numAttrs = 1;
+      int n = 0;
+      e = cudaOccupancyMaxActiveClusters(&n, kerns[i], &cfg);
+      if (e != cudaSuccess) return e;
+      fit |= (uint64_t)(n < 1 ? 1 : n > 0xFFFF ? 0xFFFF : n) << (16 * i);
+    }
+    resident[dev].store(fit);
+  }
+  const int cs = cluster_size(batch, cap, fit);
+  const int seg = ((cap + cs - 1) / cs + 3) & ~3;   // slots of a segment at most
+  const int cached = seg <= kMaxCached ? 1 : 0;
+  attr[0].val.clusterDim.x = (unsigned)cs;
+  cfg.gridDim = dim3((unsigned)(batch * cs));
+  cfg.dynamicSmemBytes = cached ? (size_t)seg * 4 : 0;
+  cfg.numAttrs = 2;
+  const Kernel kern = cs == 1 ? kerns[0] : cs == 2 ? kerns[1] : cs == 4 ? kerns[2] : kerns[3];
   return cudaLaunchKernelEx(&cfg, kern, scores, seq_len, cap, budget, n_sink, keep_idx,
                             keep_count, status, cached);
 }

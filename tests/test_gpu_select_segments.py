@@ -1,5 +1,5 @@
-"""The keep-set select's segments (csrc/select.cu): one CTA up to 8192 slots,
-a cluster of eight above, keys kept in shared memory up to 45056 slots of a
+"""The keep-set select's segments (csrc/select.cu): a sequence over 1, 2, 4 or
+8 CTAs by cap and batch, keys kept in shared memory up to 45056 slots of a
 segment and re-read above.  Lengths around those lines and around segment
 ends, ties that straddle segments, sinks, and batches whose sequences end in
 different segments: exact against the oracle's select."""
@@ -19,6 +19,22 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("kind", ["normal", "ties", "special", "one value"])
 @pytest.mark.parametrize("n_sink", [0, 5])
 def test_select_matches_the_oracle(cap, lens, kind, n_sink):
+    _check(cap, lens, kind, n_sink, (0.003, 0.5, 0.97))
+
+
+@pytest.mark.parametrize("cap", [9001, 16384, 50000])
+@pytest.mark.parametrize("batch", [12, 17, 40, 80, 160])
+@pytest.mark.parametrize("kind", ["normal", "ties"])
+def test_select_of_a_batch(cap, batch, kind):
+    """Batches whose clusters of eight would queue for the SMs take fewer CTAs
+    per sequence, down to one, with keys held and re-read."""
+    r = np.random.default_rng(batch)
+    lens = r.integers(1, cap + 1, batch).tolist()
+    lens[:3] = [cap, cap - 1, 1]
+    _check(cap, lens, kind, 2, (0.3,))
+
+
+def _check(cap, lens, kind, n_sink, parts):
     from paper_2607_27600_gb300 import cc
     cc.load_library()
     r = np.random.default_rng(cap + len(kind) + n_sink)
@@ -31,7 +47,7 @@ def test_select_matches_the_oracle(cap, lens, kind, n_sink):
             s[r.random((b, cap)) < 0.15] = v
     elif kind == "one value":
         s[:] = -1.5
-    for part in (0.003, 0.5, 0.97):
+    for part in parts:
         budget = [max(int(n * part), min(n, 1 + n_sink)) for n in lens]
         idx = torch.full((b, cap), -7, dtype=torch.int32, device="cuda")
         cnt = torch.zeros(b, dtype=torch.int32, device="cuda")
