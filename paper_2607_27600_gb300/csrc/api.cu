@@ -1165,8 +1165,7 @@ cc_status compact_plan(const cc_model_cfg *c, const cc_kv_cache *kv, CompactPlan
     A.bulk = bulk ? 1 : 0;
     A.paged = paged ? 1 : 0;
     A.head_major = head_major ? 1 : 0;
-    A.rows_per_chunk = bulk ? std::min(kCompactMaxRows, row_bytes <= p.stage_bytes
-                                                            ? p.stage_bytes / row_bytes : 0)
+    A.rows_per_chunk = bulk ? (row_bytes <= p.stage_bytes ? p.stage_bytes / row_bytes : 0)
                             : std::min(kCompactSmallRows, p.stage_bytes / 4);
     if (A.rows_per_chunk < 1) return false;
     A.n_chunks = (kv->cap + A.rows_per_chunk - 1) / A.rows_per_chunk;

@@ -155,13 +155,17 @@ struct Unit {
   int t;          // unit number (>= total: none)
   int a, b, c;    // array, sequence, chunk
   int k0, k1;     // destination slots [k0, k1)
-  int src;        // bulk arrays: this lane's row k0 + lane comes from slot src,
-  bool moves;     //   and moves (its source differs and both rows exist)
+  int src;        // bulk arrays: this lane's first row, k0 + lane, comes from slot src,
+  bool moves;     //   and moves (its source differs and both rows exist); its further
+                  //   rows (units of rows below 1/32 of the buffer) are looked up as moved
   bool publish;   // a higher unit waits for this one's reads
   int dep_lo, dep_hi;   // chunks below c that read from this one's destinations
   bool loaded;    // bulk loads issued into the buffer
 };
 
+// MANY: some bulk units have more rows than lanes (rows below 1/32 of the buffer;
+// their loops cost the others 1.5 %: 16384 Llama-3-8B slots 217 -> 221 us).
+template <bool MANY>
 __global__ void __launch_bounds__(kThreads)
     compact_kernel(const __grid_constant__ CompactParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -237,6 +241,17 @@ __global__ void __launch_bounds__(kThreads)
       bulk_store(base + (size_t)arow(A, b, k) * A.row_bytes, src, A.row_bytes);
     }
   };
+  // Calls f(k, src) for each of this lane's rows of bulk unit u that moves
+  // (report: bad entries of the further rows).
+  auto each_row = [&](const CompactArray &A, const Unit &u, bool report, auto f) {
+    if (u.moves) f(u.k0 + lane, u.src);
+    if constexpr (!MANY) return;
+    const int32_t *kidx = p.keep_idx + (size_t)u.b * p.cap;
+    for (int k = u.k0 + 32 + lane; k < u.k1; k += 32) {
+      const int src = source(kidx, k, report);
+      if (src != k && (!A.paged || (arow(A, u.b, k) >= 0 && arow(A, u.b, src) >= 0))) f(k, src);
+    }
+  };
   // The warp's next unit, with its lookups.
   auto take = [&]() -> Unit {
     Unit u;
@@ -294,12 +309,20 @@ __global__ void __launch_bounds__(kThreads)
     if (u.t >= total || u.k0 >= u.k1) return;
     const CompactArray &A = p.arr[u.a];
     if (A.bulk) {
-      const int moving = __popc(__ballot_sync(0xFFFFFFFFu, u.moves));
+      int moving;
+      if (!MANY || u.k1 - u.k0 <= 32) {
+        moving = __popc(__ballot_sync(0xFFFFFFFFu, u.moves));
+      } else {
+        int mine = 0;
+        each_row(A, u, true, [&](int, int) { ++mine; });
+        moving = __reduce_add_sync(0xFFFFFFFFu, mine);
+      }
       if (moving == 0) return;
       if (lane == 0) mbar_arrive_expect_tx(&bars[warp][s], (uint32_t)(moving * A.row_bytes));
       __syncwarp();
-      if (u.moves)
-        row_load(A, u.b, u.src, buf[s] + (size_t)lane * A.row_bytes, &bars[warp][s]);
+      each_row(A, u, false, [&](int k, int src) {
+        row_load(A, u.b, src, buf[s] + (size_t)(k - u.k0) * A.row_bytes, &bars[warp][s]);
+      });
       u.loaded = true;
     } else {   // 4-byte rows: plain loads staged in shared memory
       const int32_t *kidx = p.keep_idx + (size_t)u.b * p.cap;
@@ -337,8 +360,9 @@ __global__ void __launch_bounds__(kThreads)
     if (go && cur.k0 < cur.k1) {
       if (A.bulk) {
         if (cur.loaded) {
-          if (cur.moves)
-            row_store(A, cur.b, cur.k0 + lane, buf[s] + (size_t)lane * A.row_bytes);
+          each_row(A, cur, false, [&](int k, int) {
+            row_store(A, cur.b, k, buf[s] + (size_t)(k - cur.k0) * A.row_bytes);
+          });
           bulk_commit();
         }
       } else {
@@ -380,30 +404,32 @@ size_t compact_smem_bytes(const CompactParams &p) {
 
 cudaError_t launch_compact(const CompactParams &p, int sms, cudaStream_t st) {
   // resident CTAs per SM for this shape (the cooperative launch needs all of them)
-  static bool attr_set[64] = {};
-  static int occ_cache[64][kCompactMaxWarps + 1] = {};
-  static int occ_smem[64][kCompactMaxWarps + 1] = {};
+  static bool attr_set[2][64] = {};
+  static int occ_cache[2][64][kCompactMaxWarps + 1] = {};
+  static int occ_smem[2][64][kCompactMaxWarps + 1] = {};
+  int many = 0;
+  for (int a = 0; a < p.n_arrays; ++a) many |= p.arr[a].bulk && p.arr[a].rows_per_chunk > 32;
+  const auto kern = many ? compact_kernel<true> : compact_kernel<false>;
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (p.warps < 1 || p.warps > kCompactMaxWarps || p.stage_bytes < 16) return cudaErrorInvalidValue;
   const size_t smem = compact_smem_bytes(p);
-  if (!attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (!attr_set[many][dev]) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kCompactSmemBytes);
     if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
+    attr_set[many][dev] = true;
   }
-  if (occ_smem[dev][p.warps] != (int)smem) {
+  if (occ_smem[many][dev][p.warps] != (int)smem) {
     int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compact_kernel, p.warps * 32,
-                                                                  smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, p.warps * 32, smem);
     if (e != cudaSuccess) return e;
     if (n < 1) return cudaErrorLaunchOutOfResources;
-    occ_cache[dev][p.warps] = n;
-    occ_smem[dev][p.warps] = (int)smem;
+    occ_cache[many][dev][p.warps] = n;
+    occ_smem[many][dev][p.warps] = (int)smem;
   }
-  const int blocks_per_sm = occ_cache[dev][p.warps];
+  const int blocks_per_sm = occ_cache[many][dev][p.warps];
   if (p.total_units <= 0) return cudaSuccess;
   for (int cls = 0; cls < p.n_classes; ++cls) {
     if (p.class_rows[cls] <= 0) return cudaErrorInvalidValue;
@@ -415,7 +441,7 @@ cudaError_t launch_compact(const CompactParams &p, int sms, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   // cooperative: every warp resident, so the static unit order cannot deadlock
   void *args[] = {const_cast<CompactParams *>(&p)};
-  return cudaLaunchCooperativeKernel((const void *)compact_kernel, dim3(sms * blocks_per_sm),
+  return cudaLaunchCooperativeKernel((const void *)kern, dim3(sms * blocks_per_sm),
                                      dim3(p.warps * 32), args, smem, st);
 }
 

@@ -19,8 +19,6 @@ constexpr int kMaxCompactArrays = 2 * 128 + 3;
 // gathers per lane, so a sequence's few units spread over many warps
 // instead of one warp walking all of them.
 constexpr int kCompactSmallRows = 256;
-// Rows of a bulk unit at most: one per lane.
-constexpr int kCompactMaxRows = 32;
 constexpr int kMaxDepClasses = 3;        // distinct chunk sizes (K/V rows, H rows, 4-byte rows)
 
 struct CompactArray {

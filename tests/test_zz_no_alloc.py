@@ -74,3 +74,69 @@ def test_static_scratch_rejects_caches_beyond_its_size():
     with pytest.raises(cc.CCError) as e:
         cc.cc_compact_kv_static(big, cache, idx, idx)
     assert e.value.code == cc.CC_ERR_WORKSPACE
+
+
+@pytest.mark.parametrize("layout", ["slot", "paged", "head"])
+@pytest.mark.parametrize("d_model", [256, 4096])
+def test_units_of_more_rows_than_lanes(layout, d_model):
+    """64-byte K/V rows (one head of 64 e4m3 values): units of 64 rows, or 128
+    beside 8 KB H rows.  Exact against a gather; an entry below its slot in a
+    unit's second half is reported and its row left alone."""
+    import bench
+    import paper_2607_27600_gb300 as pkg
+    from paper_2607_27600_gb300 import cc
+    pkg.load_library()
+    shape = ModelShape(2, d_model, 8, 1, 64, 384, 1000, 1e4, 1e-5)
+    seq, cap = [2000, 777], 2048
+    c = synth.synthetic_cache(shape, seq, cap, seed=7, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(3)
+    for key in ("k", "v"):
+        c[key] = [torch.randint(0, 120, x.shape, dtype=torch.uint8, device="cuda", generator=g)
+                  for x in c[key]]
+    c["kv_scale"] = [(1.0, 1.0)] * 2
+    before = {k: [x.clone() for x in c[k]] for k in ("k", "v")}
+    if layout == "paged":
+        bench.to_paged_cache(c, 128, 5)
+    elif layout == "head":
+        for key in ("k", "v"):
+            c[key] = [x.permute(0, 2, 1, 3).contiguous() for x in c[key]]
+        c["kv_layout"] = 1
+    idx, cnt = _keep(seq, cap, 9)
+    bad = 50                               # the second half of the first unit
+    idx[0, bad] = bad - 1
+    cache = pkg.Cache(c)
+    ws = cc.alloc_workspace(cc.cc_compact_workspace_size(shape, cache))
+    cc.cc_compact_kv(shape, cache, idx, cnt, ws)
+    assert cc.cc_get_status() == cc.CC_ERR_DEVICE_ARG
+    idx[0, bad] = bad
+    for key in ("k", "v"):
+        for l in range(2):
+            got = bench.logical_kv(c, key, l)
+            for b in range(2):
+                n = int(cnt[b])
+                assert torch.equal(got[b, :n], before[key][l][b, idx[b, :n].long()])
+
+
+def test_static_scratch_takes_short_rows():
+    """64-byte rows move in units of 64 slots: 128 (array, sequence) pairs of
+    98304 slots need 0.8 MiB of scratch, within the fixed array."""
+    import paper_2607_27600_gb300 as pkg
+    from paper_2607_27600_gb300 import cc
+    pkg.load_library()
+    shape = ModelShape(8, 256, 8, 1, 64, 384, 1000, 1e4, 1e-5)
+    b, cap = 8, 98304
+    c = {k: [torch.randint(0, 120, (b, cap, 1, 64), dtype=torch.uint8, device="cuda")
+             for _ in range(8)] for k in ("k", "v")}
+    c.update(h_last=None, kv_scale=[(1.0, 1.0)] * 8,
+             tokens=torch.arange(b * cap, dtype=torch.int32, device="cuda").reshape(b, cap),
+             pos=torch.zeros((b, cap), dtype=torch.int32, device="cuda"),
+             seq_len=torch.full((b,), cap, dtype=torch.int32, device="cuda"))
+    cache = pkg.Cache(c)
+    assert cc.cc_compact_workspace_size(shape, cache) <= 1 << 20
+    idx, cnt = _keep([cap] * b, cap, 4)
+    want = {k: [x[1, idx[1, :int(cnt[1])].long()] for x in c[k]] for k in ("k", "v")}
+    cc.cc_compact_kv_static(shape, cache, idx, cnt)
+    assert cc.cc_get_status() == cc.CC_OK
+    for key in ("k", "v"):
+        for x, y in zip(c[key], want[key]):
+            assert torch.equal(x[1, :int(cnt[1])], y)
