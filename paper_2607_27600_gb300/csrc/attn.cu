@@ -629,6 +629,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
   const float c = p.scale_log2;
   const size_t base = (size_t)unit_id * S * 256 + R;   // split s's row: base + s * 256
   float m = -INFINITY, l = 0.f, o[DPL];
+  bool nan = false;   // a split's row sum
 #pragma unroll
   for (int e = 0; e < DPL; ++e) o[e] = 0.f;
 #pragma unroll 1
@@ -644,8 +645,10 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
     }
     float mx = m;   // reference max over the splits that saw keys
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
+    for (int k = 0; k < 8; ++k) {
       if (ml[k].y > 0.f) mx = fmaxf(mx, ml[k].x);
+      nan |= isnan(ml[k].y);
+    }
     const float f = l > 0.f ? fast_exp2((m - mx) * c) : 0.f;
     l *= f;
 #pragma unroll
@@ -653,9 +656,9 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       // a split without keys holds no O row (its memory may hold any bits); one
-      // with a NaN sum makes the row's sum NaN, and the row 0
-      if (ml[k].y == 0.f) continue;
-      const float w = ml[k].y > 0.f ? fast_exp2((ml[k].x - mx) * c) : 0.f;
+      // with a NaN sum makes the row 0
+      if (!(ml[k].y > 0.f)) continue;
+      const float w = fast_exp2((ml[k].x - mx) * c);
       l = fmaf(w, ml[k].y, l);
 #pragma unroll
       for (int e = 0; e < DPL; ++e) o[e] = fmaf(w, reinterpret_cast<const float *>(&v[k])[e], o[e]);
@@ -668,7 +671,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
 #pragma unroll
   for (int e = 0; e < DPL; e += 2)
     *reinterpret_cast<uint32_t *>(dst + e) =
-        l > 0.f ? pack_bf16x2(o[e] * inv, o[e + 1] * inv) : 0u;
+        l > 0.f && !nan ? pack_bf16x2(o[e] * inv, o[e + 1] * inv) : 0u;
 }
 
 template <int DH, bool CAUSAL, bool SPLIT = false, bool F16 = false>

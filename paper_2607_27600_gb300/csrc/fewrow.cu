@@ -240,7 +240,7 @@ CC_DEV uint16_t act_bits(float y, bool f16) {
 }
 // N values y[k] to out + at[k] where live[k]: one branch each for the fp16
 // range report and (lo > 0) the remainders bf16(y - hi) at that offset.
-template <int N>
+template <bool RP, int N>
 CC_DEV void store_acts(uint16_t *out, const size_t (&at)[N], const float (&y)[N],
                        const bool (&live)[N], bool f16, int lo, unsigned *status) {
   uint16_t bits[N];
@@ -258,9 +258,11 @@ CC_DEV void store_acts(uint16_t *out, const size_t (&at)[N], const float (&y)[N]
   if (lo > 0) {
 #pragma unroll
     for (int k = 0; k < N; ++k)
-      if (live[k])
+      if (live[k]) {
+        const float hi = __bfloat162float(__ushort_as_bfloat16(bits[k]));
         out[at[k] + lo] = __bfloat16_as_ushort(
-            __float2bfloat16_rn(pair_rest(y[k], __bfloat162float(__ushort_as_bfloat16(bits[k])))));
+            __float2bfloat16_rn(RP ? pair_rest(y[k], hi) : y[k] - hi));
+      }
   }
 }
 
@@ -300,7 +302,7 @@ CC_DEV void finish_rows8(const GemmParams &p, const ProjTile &d, const LaneCol &
       at[j] = (row0 + r0 + J + j) * p.ldo + lc.c0;
       live[j] = !dry && lc.ok && J + j < n;
     }
-    store_acts<8>(reinterpret_cast<uint16_t *>(p.out), at, y, live, f16, lo, p.status);
+    store_acts<RP, 8>(reinterpret_cast<uint16_t *>(p.out), at, y, live, f16, lo, p.status);
   } else {
     const int hf = lane >> 4;
 #pragma unroll
@@ -343,7 +345,7 @@ CC_DEV void finish_rows8(const GemmParams &p, const ProjTile &d, const LaneCol &
         if (live[j + 1]) o[at[j + 1]] = (uint8_t)(e >> 8);
       }
     } else {
-      store_acts<8>(reinterpret_cast<uint16_t *>(d.out), at, y, live, f16, lo, p.status);
+      store_acts<RP, 8>(reinterpret_cast<uint16_t *>(d.out), at, y, live, f16, lo, p.status);
     }
   }
 }
@@ -440,7 +442,7 @@ CC_DEV void finish_block(const GemmParams &p, const ProjTile &d, const LaneCol &
           at[j] = (row0 + r0 + j) * p.ld_norm + lc.c0;
           live[j] = !dry && lc.ok && j < n;
         }
-        store_acts<16>(reinterpret_cast<uint16_t *>(p.norm_out), at, z, live, p.out_f16 != 0,
+        store_acts<RP, 16>(reinterpret_cast<uint16_t *>(p.norm_out), at, z, live, p.out_f16 != 0,
                        norm_lo, p.status);
       }
     }
