@@ -43,11 +43,12 @@ using namespace cc;
 constexpr int kMaxDevices = 64;
 
 // ---------------------------------------------------------------------------
-// per-device state: status-word address, SM count
+// per-device state: status-word address, SM count, resident clusters
 // ---------------------------------------------------------------------------
 struct DevState {
   unsigned *status = nullptr;
   int sms = 0;
+  cc::FewClusters fit = {};
   bool ready = false;
 };
 DevState g_dev[kMaxDevices];
@@ -64,6 +65,7 @@ bool dev_state(DevState **out) {
     if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return false;
     d.status = reinterpret_cast<unsigned *>(p);
+    d.fit = cc::few_clusters(d.sms);
     d.ready = true;
   }
   *out = &d;
@@ -333,40 +335,106 @@ struct Gemm {
   bool one_group;      // few: one row group
 };
 
+// CC_GEMM_PAIRS (tests): '0' or '2' keeps every product on the tile kernel, on
+// single CTAs or on pairs wherever the tiles are 256 columns wide.  0: unset.
+char gemm_pairs_env() {
+  const char *e = getenv("CC_GEMM_PAIRS");
+  return e && (e[0] == '0' || e[0] == '2') ? e[0] : 0;
+}
+
+// Estimated microseconds of a launch below two waves of 128 x 256 tiles, m row
+// tiles of N columns and nk k-blocks, on the tile kernel with bn-column tiles, or
+// on CTA pairs.  Fitted to the q, q/k/v, O and down projections of Llama-3-8B and
+// Qwen2.5-7B at 128 to 2816 rows, bf16 and split operands (rms 2 to 4 %).
+double tile_us(int epi, int bn, bool pair, double m, int N, int K, int nk, int sms) {
+  const double n = (N + bn - 1) / bn;
+  const double waves = pair ? ceil(ceil(m / 2) * n / (sms / 2)) : ceil(m * n / sms);
+  const double t = pair ? 24.1 + 0.283 * nk * waves
+                        : bn == 128 ? 15.7 + 0.297 * nk * waves : 22.0 + 0.343 * nk * waves;
+  const double hbm = 12.0 + 1.1 * 2.0 * N * K / 6.8e6;   // the weights once
+  return std::max(t, hbm) + (epi == EPI_QKV ? 3.0 : 0.0);
+}
+// The same of the few-row kernel from its plan's cycles: what measured launches took
+// beyond them, less what its prologue, which runs under the kernel before, saves.
+double few_us(int epi, const FewPlan &plan, double cycles) {
+  double beyond = 9.3;
+  if (plan.split == 1 && plan.nb == 256) beyond = epi == EPI_QROPE || epi == EPI_BF16 ? 0.0 : 6.5;
+  else if (plan.split == 1 && epi == EPI_QKV) beyond = 14.5;
+  else if (plan.split == 4 && plan.pair) beyond = 16.0;
+  return cycles / 1900.0 + beyond - 2.0;
+}
+
 // One GEMM over the cache rows: A [R][K] (bf16 workspace) x W [N][K]^T.
 // a_split: A rows are [hi | lo] (2K values) and the product is hi W^T + lo W^T.
+// rows_least: rows there will be at least (appends; 0: unknown), for the choice of
+// a kernel.
 cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, const void *W2, int N,
                      int batch, int cap, const int32_t *seq_len, unsigned *status,
-                     bool a_split = false, int few_tiles = 0, int row_pairs = 0) {
+                     bool a_split = false, int few_tiles = 0, int row_pairs = 0,
+                     uint64_t rows_least = 0) {
   const uint64_t R = (uint64_t)batch * cap;
   int bn = gemm_block_n(epi);
-  // narrow problems (less than one wave of 256-column tiles) that stay on this
-  // kernel: 128-column tiles double the tiles that share the SMs
+  // narrow problems (less than one wave of 256-column tiles) on the tile kernel:
+  // 128-column tiles double the tiles that share the SMs
   const bool narrowable = epi == EPI_F32 || epi == EPI_QROPE || epi == EPI_RESID_BF16 ||
                           epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT || epi == EPI_BF16;
   DevState *dev_info = nullptr;
   const bool have_dev = dev_state(&dev_info);
   // CTA pairs: for launches of two waves or more of 128 x 256 tiles (a pair
-  // takes two of them at once).  CC_GEMM_PAIRS=0: never; =2: whenever the
-  // tiles are 256 columns wide (narrow problems keep wide tiles then)
-  const char *pairs_env = getenv("CC_GEMM_PAIRS");
-  const int pair_mode = !pairs_env ? 1 : pairs_env[0] == '0' ? 0 : pairs_env[0] == '2' ? 2 : 1;
-  if (narrowable && have_dev && pair_mode != 2 &&
+  // takes two of them at once)
+  const char env = gemm_pairs_env();
+  if (narrowable && have_dev && env != '2' &&
       ((R + 127) / 128) * (uint64_t)((N + 255) / 256) < (uint64_t)dev_info->sms)
     bn = 128;
-  const bool pair = have_dev && epi != EPI_ARGMAX && row_pairs == 0 && (epi == EPI_SWIGLU || bn == 256) &&
-                    (pair_mode == 2 ||
-                     (pair_mode == 1 && ((R + 127) / 128) * (uint64_t)((N + bn - 1) / bn) >=
-                                            2 * (uint64_t)dev_info->sms));
-  // launches below two waves of tiles: few.nb rows per group on the N side,
-  // the K range over a cluster's CTAs (CC_GEMM_PAIRS keeps them on this kernel)
+  bool pair = have_dev && epi != EPI_ARGMAX && row_pairs == 0 && (epi == EPI_SWIGLU || bn == 256) &&
+              (env == '2' ||
+               (!env && ((R + 127) / 128) * (uint64_t)((N + bn - 1) / bn) >= 2 * (uint64_t)dev_info->sms));
+  // launches below two waves of tiles: the few-row kernel (few.nb rows per group
+  // on the N side, the K range over a cluster's CTAs), or the tile form that the
+  // estimates above put below it.  (SwiGLU: the few-row kernel up
+  // to two waves, pairs above; within 5 % of the best form at every size measured.)
+  // Against the few-row kernel for all of them: appends of 640 and 1280 rows to two
+  // Llama-3-8B layers 815 -> 748 and 1298 -> 1175 us, three Qwen2.5-7B sequences of
+  // 700, 300 and 64 slots scored 529 -> 437 us.
   g.few = FewPlan{};
   g.one_group = false;
-  if (have_dev && !pair && !pairs_env && epi != EPI_F32 && epi != EPI_LSE) {
+  if (have_dev && !pair && !env && epi != EPI_F32 && epi != EPI_LSE) {
     g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
-                     batch, cap, row_pairs, dev_info->sms);
-    g.one_group = batch == 1 && cap <= g.few.nb;
-    bn = kFewTileCols;
+                     batch, cap, row_pairs, dev_info->fit);
+    // (up to 256 rows the few-row kernel was the faster throughout, 1.2 to 3 times)
+    if (R > 256 && row_pairs == 0 && epi != EPI_SWIGLU && epi != EPI_ARGMAX) {
+      // R bounds the rows: one sequence's end somewhere in the last 128 slots of its
+      // cache, several sequences' anywhere between one cache and all of them (an
+      // append of one sequence brings its bound's rows): the mean over the bound, the
+      // least and their middle
+      const uint64_t least_rows = rows_least ? std::min(rows_least, R)
+                                             : batch > 1 ? cap : R - std::min<uint64_t>(R - 1, 128);
+      const uint64_t rows[3] = {R, (R + least_rows) / 2, least_rows};
+      const int nk = ((K + 63) / 64) * (a_split ? 2 : 1), sms = dev_info->sms;
+      auto tiles = [&](int cols, bool on_pairs) {
+        double t = 0;
+        for (uint64_t r : rows) t += tile_us(epi, cols, on_pairs, (double)((r + 127) / 128), N, K, nk, sms);
+        return t;
+      };
+      double least = 0;
+      for (uint64_t r : rows)
+        least += few_us(epi, g.few, r == R ? g.few.cycles : few_cycles(g.few, epi, K, a_split, (long long)r, cap, dev_info->fit));
+      auto consider = [&](int cols, bool on_pairs) {
+        const double t = tiles(cols, on_pairs);
+        if (t >= least) return;
+        least = t;
+        g.few = FewPlan{};
+        bn = cols;
+        pair = on_pairs;
+      };
+      if (narrowable) consider(128, false);
+      consider(256, false);
+      consider(256, true);
+    }
+    if (g.few.nb) {
+      g.one_group = batch == 1 && cap <= g.few.nb;
+      bn = kFewTileCols;
+    }
   }
   const bool few = g.few.nb > 0;
   const uint32_t b_box = few || epi == EPI_SWIGLU || pair ? 128 : (uint32_t)bn;
@@ -439,11 +507,11 @@ bool qkv_fusable(const cc_model_cfg *c) {
 
 cc_status gemm_setup_qkv(Gemm &g, const void *xn, const cc_model_cfg *c,
                          const cc_layer_weights &lw, int batch, int cap, const int32_t *seq_len,
-                         unsigned *status, int row_pairs) {
+                         unsigned *status, int row_pairs, uint64_t rows_least) {
   const int d = c->d_model, qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
   const int fq = (qd + 127) / 128, fk = (kvd + 127) / 128;   // column tiles of a few-row launch
   cc_status s = gemm_setup(g, EPI_QKV, xn, d, lw.wq, nullptr, qd + 2 * kvd, batch, cap, seq_len,
-                           status, false, fq + 2 * fk, row_pairs);
+                           status, false, fq + 2 * fk, row_pairs, rows_least);
   if (s != CC_OK) return s;
   const bool few = g.few.nb > 0;
   const uint32_t box = few || g.p.pair ? 128 : 256;   // a pair's CTAs load half a tile each
@@ -486,7 +554,7 @@ cc_status run_gemm(Gemm &g, int epi, int kind, int sms, cudaStream_t st, GemmSpl
     g.p.split_count = split->count;
   }
   if (g.few.nb)
-    CC_TRY(launch_few(epi, g.a, g.b, g.b2, g.b3, g.p, g.few, g.one_group, sms, st));
+    CC_TRY(launch_few(epi, g.a, g.b, g.b2, g.b3, g.p, g.few, g.one_group, st));
   else
     CC_TRY(launch_gemm(epi, g.a, g.b, g.b2, g.b3, g.p, sms, st));
   return CC_OK;
@@ -729,7 +797,7 @@ cc_status check_append_args(const cc_model_cfg *c, const cc_model_weights *w,
 // GEMM (GemmParams::row_pairs; 0: single rows): up to 64 sequences, where the
 // weights bound every product, and buffers that hold the lo rows.
 int decode_row_pairs(int batch, int cap) {
-  if (getenv("CC_GEMM_PAIRS")) return 0;   // keeps every product on the tile kernel
+  if (gemm_pairs_env()) return 0;   // keeps every product on the tile kernel
   for (int half = 16; half <= 64; half *= 2)
     if (batch <= half) return 2LL * half <= (long long)batch * cap ? half : 0;
   return 0;
@@ -798,7 +866,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   auto resid = [&](const void *a, int k, const void *wm, const void *gain, int kind) -> cc_status {
     Gemm g;
     cc_status r = gemm_setup(g, EPI_RESID_F32, a, k, wm, nullptr, d, 1, max_rows, total, status,
-                             false, 0, rp);
+                             false, 0, rp, max_count);
     if (r != CC_OK) return r;
     g.p.out = h;
     g.p.ldo = d;
@@ -823,7 +891,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     // v = xn Wv^T + bv straight into the cache slots of the chunk
     if (qkv_fusable(c)) {   // one GEMM over [Wq; Wk; Wv]
       Gemm g;
-      if ((s = gemm_setup_qkv(g, xn, c, lw, 1, max_rows, total, status, rp)) != CC_OK) return s;
+      if ((s = gemm_setup_qkv(g, xn, c, lw, 1, max_rows, total, status, rp, max_count)) != CC_OK) return s;
       scaled(g);
       g.p.out = q;
       g.p.out_k = kv->k[l];
@@ -844,7 +912,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
       for (const Proj &pj : projs) {
         Gemm g;
         if ((s = gemm_setup(g, pj.epi, xn, d, pj.w, nullptr, pj.n, 1, max_rows, total, status,
-                            false, 0, rp)) != CC_OK)
+                            false, 0, rp, max_count)) != CC_OK)
           return s;
         scaled(g);
         g.p.out = pj.out;
@@ -878,7 +946,7 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     if ((s = resid(o, qd, lw.wo, lw.mlp_norm, CC_KERNEL_GEMM_OPROJ)) != CC_OK) return s;
     Gemm gu;
     if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, 1, max_rows, total, status,
-                        false, 0, rp)) != CC_OK)
+                        false, 0, rp, max_count)) != CC_OK)
       return s;
     scaled(gu);
     gu.p.out = act;

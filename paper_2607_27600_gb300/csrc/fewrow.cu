@@ -55,6 +55,7 @@
 #include "fewrow.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 namespace cc {
@@ -903,15 +904,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int EPI, bool RP, bool SPLIT, bool PAIR = false>
 cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                      const CUtensorMap &b3, const GemmParams &p, const FewPlan &plan,
-                     bool one_group, int sms, cudaStream_t stream) {
+                     bool one_group, cudaStream_t stream) {
   auto kern = few_kernel<EPI, RP, SPLIT, PAIR>;
-  static int max_clusters[64][4] = {};   // co-resident clusters of 1, 2, 4 and 8 CTAs (0: unknown)
+  static std::atomic<bool> attr_set[64];
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   const int S = plan.split * (PAIR ? 2 : 1);   // CTAs of a cluster
   const int si = S == 1 ? 0 : S == 2 ? 1 : S == 4 ? 2 : 3;
-  if (S != 1 << si || S > kFewMaxSplit || plan.nb < 16 || plan.nb > 256 || plan.nb % 16) return cudaErrorInvalidValue;
+  if (S != 1 << si || S > kFewMaxSplit || plan.clusters < 1 || plan.nb < 16 || plan.nb > 256 || plan.nb % 16) return cudaErrorInvalidValue;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -926,70 +927,102 @@ cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorM
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (max_clusters[dev][si] == 0) {
+  if (!attr_set[dev].load()) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    int n = 0;
-    cudaLaunchConfig_t q = cfg;
-    q.attrs = &attr[1];
-    q.numAttrs = 1;
-    e = cudaOccupancyMaxActiveClusters(&n, kern, &q);
-    if (e != cudaSuccess) return e;
-    max_clusters[dev][si] = std::max(n, 1);
+    attr_set[dev].store(true);
   }
-  const int units = std::max(1, std::min(max_clusters[dev][si], sms / S));
-  cfg.gridDim = dim3((unsigned)(units * S));
+  cfg.gridDim = dim3((unsigned)(plan.clusters * S));
   return cudaLaunchKernelEx(&cfg, kern, a, b, b2, b3, p, plan.nb, one_group ? 1 : 0);
 }
 
 }  // namespace
 
+// Every form of the kernel holds an SM's shared memory, so one form's count is all
+// forms'.
+FewClusters few_clusters(int sms) {
+  FewClusters r = {{sms, sms / 2, sms / 4, sms / 8}};
+  auto kern = few_kernel<EPI_RESID_F32, false, true, true>;
+  bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) ==
+            cudaSuccess;
+  for (int i = 0; ok && i < 4; ++i) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << i;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << i);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    ok = cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess;
+    if (ok) r.n[i] = std::max(1, std::min(n, r.n[i]));
+  }
+  if (!ok) (void)cudaGetLastError();   // the counts are a plan's: a launch reports its own errors
+  return r;
+}
+
+static int cluster_log2(int ctas) { return ctas == 1 ? 0 : ctas == 2 ? 1 : ctas == 4 ? 2 : 3; }
+// Estimated SM cycles of a plan over `groups` row groups of at most rows_per_seq rows.
+static double plan_cycles(int epi, int n_tiles, int K, bool a_split, double groups,
+                          long long rows_per_seq, int nb, int S, int pt, const FewClusters &fit) {
+  const int wt = w_tiles(epi);
+  const int nk = ((K + BK - 1) / BK) * (a_split ? 2 : 1);
+  const double hbm = (double)n_tiles * wt * BM * K * 2 / 3500.0;   // weight bytes at 6.7 TB/s, 1.9 GHz
+  const int rounds = S > 1 ? split_rounds(wt, nb, S) : 1;
+  // k-block: the products (2 cycles per row) or their operands' way into
+  // shared memory (measured on the Qwen2.5 projections: 266 cycles for 18 KB,
+  // 570 for 32 KB, 630 to 670 for 48 KB)
+  const double tk = std::max(2.0 * nb * wt, 180.0 + stage_bytes(wt, nb / pt) / 105.0);
+  const double waves = std::ceil(groups * ((n_tiles + pt - 1) / pt) / fit.n[cluster_log2(S * pt)]);
+  // a tile's end: about 3600 cycles per 16-row block of a warp (SwiGLU 2600),
+  // for a split the exchange before it; without a split it overlaps the
+  // next tile's products while two accumulators fit
+  const double fin = 1500.0 + (wt == 2 ? 80.0 : 112.0) * std::min<double>(nb, (double)rows_per_seq) / S;
+  const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
+  const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
+  const double per = std::ceil((double)nk / S) * tk;
+  // (an end longer than the next tile's products is what a wave takes: 8192
+  // rows of a 512-wide model, eight k-blocks)
+  const double main = overlapped ? per + (waves - 1) * std::max(per, fin) : waves * per;
+  // (a pair's set-up and hand-overs: about 2 us for a launch alone, less
+  // behind another kernel: the O projection of 512 Qwen2.5-7B rows is 35 us
+  // alone either way, and all 28 layers take 6860 us without, 6710 with)
+  const double ends = waves * fix + (overlapped ? fin : 0.0) + (pt == 2 ? 1500.0 : 0.0);
+  // several groups read the same weight tiles at the same time, which holds
+  // the SMs' requests longer (gate/up of 256 rows, 271 MB: 128-row groups
+  // 70 us at 4.9 TB/s, one of 256 rows 66 us)
+  return std::max(main, hbm * (groups > 1 ? 1.5 : 1.1)) + ends + 0.05 * (main + ends);
+}
+
 FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
-                 int row_pairs, int sms) {
+                 int row_pairs, const FewClusters &fit) {
   const int wt = w_tiles(epi);
   FewPlan best{};
   best.n_tiles = n_tiles;
   best.cycles = 1e300;
   const int nk = ((K + BK - 1) / BK) * (a_split ? 2 : 1);
   const bool resid = epi == EPI_RESID_BF16 || epi == EPI_RESID_F32 || epi == EPI_RESID_LOGIT;
-  const double hbm = (double)n_tiles * wt * BM * K * 2 / 3500.0;   // weight bytes at 6.7 TB/s, 1.9 GHz
   for (int nb = 16; nb <= kMaxRows; nb *= 2) {
     if (row_pairs && nb != 2 * row_pairs) continue;
+    if (!row_pairs && nb > 16 && nb / 2 >= rows_per_seq) break;   // half of it holds every row
     const double groups = (double)seqs * (double)((rows_per_seq + nb - 1) / nb);
     for (int S = 1; S <= kFewMaxSplit; S *= 2) {
-      const int rounds = S > 1 ? split_rounds(wt, nb, S) : 1;
-      if (S > 1 && (nk < 4 * S || rounds == 0)) break;
+      if (S > 1 && (nk < 4 * S || split_rounds(wt, nb, S) == 0)) break;
       for (int pt = 1; pt <= 2; ++pt) {   // 2: CTA pairs
         // whole groups of the residual products, split (128-row groups measured
         // 62 us against 59, the projections the same, gate/up 64 against 65)
         if (pt == 2 && (!resid || nb != kMaxRows || S == 1 || 2 * S > kFewMaxSplit || row_pairs))
           break;
-        // k-block: the products (2 cycles per row) or their operands' way into
-        // shared memory (measured on the Qwen2.5 projections: 266 cycles for 18 KB,
-        // 570 for 32 KB, 630 to 670 for 48 KB)
-        const double tk = std::max(2.0 * nb * wt, 180.0 + stage_bytes(wt, nb / pt) / 105.0);
-        const int ctas = S * pt;
-        const double units = floor(sms / ctas * (ctas >= 4 ? 0.95 : 1.0));
-        const double waves = std::ceil(groups * ((n_tiles + pt - 1) / pt) / std::max(1.0, units));
-        // a tile's end: about 3600 cycles per 16-row block of a warp (SwiGLU 2600),
-        // for a split the exchange before it; without a split it overlaps the
-        // next tile's products while two accumulators fit
-        const double fin = 1500.0 + (wt == 2 ? 80.0 : 112.0) * std::min<double>(nb, (double)rows_per_seq) / S;
-        const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
-        const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
-        const double main = waves * std::ceil((double)nk / S) * tk;
-        // (a pair's set-up and hand-overs: about 2 us for a launch alone, less
-        // behind another kernel: the O projection of 512 Qwen2.5-7B rows is 35 us
-        // alone either way, and all 28 layers take 6860 us without, 6710 with)
-        const double ends = waves * fix + (overlapped ? fin : 0.0) + (pt == 2 ? 1500.0 : 0.0);
-        // several groups read the same weight tiles at the same time, which holds
-        // the SMs' requests longer (gate/up of 256 rows, 271 MB: 128-row groups
-        // 70 us at 4.9 TB/s, one of 256 rows 66 us)
-        const double t = std::max(main, hbm * (groups > 1 ? 1.5 : 1.1)) + ends + 0.05 * (main + ends);
+        const double t = plan_cycles(epi, n_tiles, K, a_split, groups, rows_per_seq, nb, S, pt, fit);
         if (t < best.cycles * 0.98) {
           best.nb = nb;
           best.split = S;
           best.pair = pt == 2;
+          best.clusters = fit.n[cluster_log2(S * pt)];
           best.cycles = t;
         }
       }
@@ -998,15 +1031,21 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
   return best;
 }
 
+double few_cycles(const FewPlan &plan, int epi, int K, bool a_split, long long rows,
+                  long long rows_per_seq, const FewClusters &fit) {
+  return plan_cycles(epi, plan.n_tiles, K, a_split, (double)((rows + plan.nb - 1) / plan.nb),
+                     rows_per_seq, plan.nb, plan.split, plan.pair ? 2 : 1, fit);
+}
+
 cudaError_t launch_few(int epi, const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                        const CUtensorMap &b3, const GemmParams &p, const FewPlan &plan,
-                       bool one_group, int sms, cudaStream_t st) {
+                       bool one_group, cudaStream_t st) {
   // (row pairs: the products of a decode step)
 #define CC_FEW_T(E, R)                                                                   \
-  (plan.split > 1 ? launch_t<E, R, true>(a, b, b2, b3, p, plan, one_group, sms, st)      \
-                  : launch_t<E, R, false>(a, b, b2, b3, p, plan, one_group, sms, st))
+  (plan.split > 1 ? launch_t<E, R, true>(a, b, b2, b3, p, plan, one_group, st)      \
+                  : launch_t<E, R, false>(a, b, b2, b3, p, plan, one_group, st))
 #define CC_FEW_RESID(E)                                                                  \
-  (plan.pair ? launch_t<E, false, true, true>(a, b, b2, b3, p, plan, one_group, sms, st) \
+  (plan.pair ? launch_t<E, false, true, true>(a, b, b2, b3, p, plan, one_group, st) \
              : CC_FEW_T(E, false))
 #define CC_FEW_DECODE(E) (p.row_pairs ? CC_FEW_T(E, true) : CC_FEW_T(E, false))
   if (p.row_pairs && (epi == EPI_RESID_BF16 || epi == EPI_RESID_LOGIT)) return cudaErrorInvalidValue;

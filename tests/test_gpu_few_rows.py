@@ -157,3 +157,31 @@ def test_appends_equal_the_tile_kernel(pkg, monkeypatch, dh, layout, counts):
         tol = 0.13 if layout == "e4m3" else 4e-2
         assert (val(x) - val(y)).abs().max() <= tol * val(y)[rows].abs().max()
     assert (c0["h_last"].float() - c1["h_last"].float()).abs().max() <= 4e-2 * c1["h_last"].float().abs().max()
+
+
+@pytest.mark.parametrize("lens,counts", [([0], [257]), ([64], [520]), ([0], [600]), ([300], [1100]),
+                                         ([0, 5, 100], [700, 40, 1]), ([0, 0], [640, 639])])
+def test_appends_of_every_form_equal_the_tile_kernel(pkg, monkeypatch, lens, counts):
+    """Row counts past one group, where a product goes to the few-row kernel, to
+    single CTAs of 128 or 256 columns or to CTA pairs: against single CTAs for
+    all of them.  bf16 rows through two layers: 4e-2 of the largest, as above."""
+    from paper_2607_27600_gb300 import cc
+    shape, cap = ModelShape(2, 2048, 16, 8, 128, 6144, 700, 1e4, 1e-5), 1408
+    w = synth.model_weights(shape, 9, device="cuda", with_kv_proj=True)
+    toks = synth.tokens((len(lens), max(counts)), shape.vocab, 3).cuda()
+    cnt = torch.tensor(counts, dtype=torch.int32, device="cuda")
+    ws = cc.alloc_workspace(cc.cc_append_workspace_size(shape, len(lens), cap))
+    out = []
+    for env in (None, None, "0"):
+        if env:
+            monkeypatch.setenv("CC_GEMM_PAIRS", env)
+        c = synth.synthetic_cache(shape, lens, cap, 10, device="cuda")
+        cc.cc_append_chunk(shape, pkg.Weights(w), pkg.Cache(c), toks, None, cnt, max(counts), ws)
+        assert cc.cc_get_status() == cc.CC_OK
+        out.append(c["k"] + c["v"] + [c["h_last"]])
+    for x, again, y in zip(*out):
+        assert torch.equal(x, again)
+        for b, (n, m) in enumerate(zip(lens, counts)):
+            assert torch.equal(x[b, :n], y[b, :n]) and torch.equal(x[b, n + m:], y[b, n + m:])
+            a, r = x[b, n:n + m].float(), y[b, n:n + m].float()
+            assert (a - r).abs().max() <= 4e-2 * r.abs().max(), b

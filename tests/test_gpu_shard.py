@@ -9,6 +9,7 @@ import pytest
 import torch
 
 import synth
+from synth.configs import ModelShape
 from tests._util import causal_cache, to_device, to_np
 from tests.test_gpu_score import SMALL_GPU
 
@@ -62,6 +63,22 @@ def test_llama_layer_8k_rows_in_blocks_equal_the_single_call(pkg, world):
     c = synth.synthetic_cache(wl.shape, wl.seq_lens, wl.cap, wl.seed, device="cuda", layers=[last])
     single, merged, parts = _single_and_sharded(pkg, wl.shape, w, c, cc.SCORE_LOGIT, False, world)
     _check(single, merged, parts, wl.seq_lens)
+
+
+@pytest.mark.parametrize("name,lens,cap", [("llama8b-layer-8k", [650], 768), ("llama8b-layer-8k", [1200], 1280),
+                                           ("qwen7b-layer-128k", [600], 640), ("qwen7b-layer-128k", [700, 300, 64], 768),
+                                           ("qwen7b-layer-128k", [2200], 2304)])
+@pytest.mark.parametrize("precise", [False, True])
+def test_rows_in_blocks_below_two_waves(pkg, name, lens, cap, precise):
+    """Sizes at which a layer's products go to the few-row kernel, to single CTAs
+    and to CTA pairs: the choice is the whole cache's, never a block's."""
+    from paper_2607_27600_gb300 import cc
+    shape = ModelShape(**{**synth.WORKLOADS[name].shape.__dict__, "n_layers": 1})
+    w = synth.model_weights(shape, 3, device="cuda", with_embed=False)
+    c = synth.synthetic_cache(shape, lens, cap, 4, device="cuda")
+    mode = cc.SCORE_LOGIT | (cc.SCORE_PRECISE if precise else 0)
+    single, merged, parts = _single_and_sharded(pkg, shape, w, c, mode, False, 3)
+    _check(single, merged, parts, lens)
 
 
 @pytest.mark.parametrize("mode_name", ["logit", "logprob", "precise"])
