@@ -401,8 +401,11 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   if (have_dev && !pair && !env && epi != EPI_F32 && epi != EPI_LSE) {
     g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
                      batch, cap, row_pairs, dev_info->fit);
-    // (up to 256 rows the few-row kernel was the faster throughout, 1.2 to 3 times)
-    if (R > 256 && row_pairs == 0 && epi != EPI_SWIGLU && epi != EPI_ARGMAX) {
+    // (up to 256 rows the few-row kernel was the faster throughout, 1.2 to 3 times; a
+    // short K, d_model 512, is its launches' ends and overlapped starts, which the
+    // estimates leave out: with them scores of three such sequences took 10 % longer)
+    const int nk = ((K + 63) / 64) * (a_split ? 2 : 1);
+    if (R > 256 && nk >= 32 && row_pairs == 0 && epi != EPI_SWIGLU && epi != EPI_ARGMAX) {
       // R bounds the rows: one sequence's end somewhere in the last 128 slots of its
       // cache, several sequences' anywhere between one cache and all of them (an
       // append of one sequence brings its bound's rows): the mean over the bound, the
@@ -410,7 +413,7 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
       const uint64_t least_rows = rows_least ? std::min(rows_least, R)
                                              : batch > 1 ? cap : R - std::min<uint64_t>(R - 1, 128);
       const uint64_t rows[3] = {R, (R + least_rows) / 2, least_rows};
-      const int nk = ((K + 63) / 64) * (a_split ? 2 : 1), sms = dev_info->sms;
+      const int sms = dev_info->sms;
       auto tiles = [&](int cols, bool on_pairs) {
         double t = 0;
         for (uint64_t r : rows) t += tile_us(epi, cols, on_pairs, (double)((r + 127) / 128), N, K, nk, sms);

@@ -984,10 +984,7 @@ static double plan_cycles(int epi, int n_tiles, int K, bool a_split, double grou
   const double fin = 1500.0 + (wt == 2 ? 80.0 : 112.0) * std::min<double>(nb, (double)rows_per_seq) / S;
   const bool overlapped = S == 1 && 2 * wt * acc_cols(nb) <= 512;
   const double fix = S > 1 ? 2500.0 * rounds + 20.0 * wt * nb + fin : overlapped ? 300.0 : fin;
-  const double per = std::ceil((double)nk / S) * tk;
-  // (an end longer than the next tile's products is what a wave takes: 8192
-  // rows of a 512-wide model, eight k-blocks)
-  const double main = overlapped ? per + (waves - 1) * std::max(per, fin) : waves * per;
+  const double main = waves * std::ceil((double)nk / S) * tk;
   // (a pair's set-up and hand-overs: about 2 us for a launch alone, less
   // behind another kernel: the O projection of 512 Qwen2.5-7B rows is 35 us
   // alone either way, and all 28 layers take 6860 us without, 6710 with)
