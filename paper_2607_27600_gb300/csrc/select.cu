@@ -283,13 +283,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   sync_all<CS>();   // no CTA reads this one's counts any more
 }
 
-// CTAs per sequence of a launch: the least estimated time over the sizes, all
-// the batch's clusters in as many waves as the device's resident ones need.
-// Fitted to every size at batches of 1 to 256 and caps of 4096 to 131072 (launch
-// after launch): a lone CTA 5.5 us + 0.65 ns a slot, 1.24 ns past the slots whose
-// keys it holds; a cluster 12 us + 0.8 ns a slot of a CTA.  Eight CTAs whatever
-// the batch took 103 us for 128 sequences of 16384 slots, one CTA each 16 us.
+// CTAs per sequence of a launch: one up to 8192 slots (launch after launch, one and
+// eight CTAs: 9.2 / 10.8 us there, 14.3 / 11.5 at 16384), eight above while every
+// sequence's cluster is resident; else the least estimated time over the sizes, the
+// clusters in as many waves as they need.  Fitted to every size at batches of 1 to
+// 256 and caps of 4096 to 131072: a lone CTA 5.5 us + 0.65 ns a slot, 1.24 ns past
+// the slots whose keys it holds; a cluster 12 us + 0.8 ns a slot of a CTA.  Eight
+// CTAs whatever the batch took 103 us for 128 sequences of 16384 slots, one CTA each
+// 16 us.
 int cluster_size(int batch, int cap, uint64_t resident) {   // (16 bits per size)
+  if (cap <= 8192) return 1;
+  if (batch <= (int)(resident >> 48)) return 8;
   int best = 1;
   double least = 1e300;
   for (int i = 0; i < 4; ++i) {
