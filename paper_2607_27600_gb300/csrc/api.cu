@@ -23,6 +23,7 @@
 #include "compact.cuh"
 #include "fewrow.cuh"
 #include "gemm.cuh"
+#include "gemv.cuh"
 #include "keyattn.cuh"
 #include "rowops.cuh"
 #include "select.cuh"
@@ -806,6 +807,75 @@ int decode_row_pairs(int batch, int cap) {
   return 0;
 }
 
+// One GEMV launch: up to three weight matrices (segments) over the same rows.
+struct GemvCall {
+  GemvLaunch l{};
+  const void *w[kGemvMaxSegs][2] = {};
+  GemvSeg &add(const void *w0, const void *w1, const void *bias, void *out, int ldo, int n, int epi) {
+    GemvSeg &sg = l.p.seg[l.p.n_seg];
+    sg = GemvSeg{};
+    sg.bias = reinterpret_cast<const __nv_bfloat16 *>(bias);
+    sg.out = out;
+    sg.ldo = ldo;
+    sg.N = n;
+    sg.epi = epi;
+    w[l.p.n_seg][0] = w0;
+    w[l.p.n_seg][1] = w1;
+    ++l.p.n_seg;
+    return sg;
+  }
+};
+
+cc_status run_gemv(GemvCall &g, int kind, int sms, cudaStream_t st) {
+  GemvParams &p = g.l.p;
+  if (!gemv_plan(p, sms)) return CC_ERR_UNSUPPORTED;
+  for (int s = 0; s < p.n_seg; ++s) {
+    const uint64_t dims[2] = {(uint64_t)p.K, (uint64_t)p.seg[s].N};
+    const uint64_t strides[1] = {(uint64_t)p.K * 2};
+    const uint32_t box[2] = {(uint32_t)kGemvBoxK, 8};
+    for (int j = 0; j < 2; ++j)
+      if (g.w[s][j] && !make_tmap(&g.l.w[s][j], g.w[s][j], 2, dims, strides, box,
+                                  CU_TENSOR_MAP_SWIZZLE_NONE))
+        return tmap_fail();
+  }
+  TimedScope t(kind, st);
+  CC_TRY(launch_gemv(g.l, st));
+  return CC_OK;
+}
+
+// Which products of an append run as GEMVs: one row per sequence, one to four
+// sequences, and shapes that the kernel takes.
+struct GemvUse {
+  bool qkv = false, o = false, gateup = false, down = false;
+};
+GemvUse gemv_use(const cc_model_cfg *c, int batch, int max_count, int cap, int sms) {
+  GemvUse u;
+  const int d = c->d_model, qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
+  const int f = c->d_ff;
+  if (max_count != 1 || batch > kGemvMaxRows || gemm_pairs_env()) return u;
+  if (kvd < 16 || f < 16) return u;   // a box of weight rows, and 16 outputs of a group
+  auto fits = [&](int K) {   // boxes no wider than the weights, room for the rows and a ring
+    GemvParams p{};
+    p.batch = batch;
+    p.K = K;
+    return K >= kGemvBoxK && K % 8 == 0 && gemv_plan(p, 1);
+  };
+  // a sum of squares per CTA and row where the tile kernels keep one per column tile
+  const bool sums = (size_t)batch * sms <= (size_t)batch * cap * ((d + 127) / 128);
+  // The few-row GEMM costs a launch a few microseconds more, the GEMV 30 to 40 ns per
+  // weight megabyte for each row past the first.  Decode steps in us, few-row GEMM
+  // for all / GEMVs: one sequence, Llama-3-8B, 16 layers 1845 / 1668, Qwen2.5-7B 1910 /
+  // 1763 (all but gate/up: 235 and 272 MB, few-row 538 and 569 against 540 and 607
+  // in four layers), six layers of d_model 2048 450 / 309, of 1024 355 / 200; four
+  // sequences of 1024 366 / 303, of 2048 450 / 429, of 3072 517 / 598.
+  const double row = 2.0 * d * (batch - 1);   // weight bytes of a column, times the rows past the first
+  u.qkv = fits(d) && row * (qd + 2.0 * kvd) <= 48e6;
+  u.o = fits(qd) && sums && row * qd <= 48e6;
+  u.gateup = fits(d) && (batch == 1 ? 4.0 * d * f <= 150e6 : row * 2.0 * f <= 32e6);
+  u.down = fits(f) && sums && row * f <= 48e6;
+  return u;
+}
+
 // Appends a chunk (or a decode step's token) per sequence through every layer.
 // The workspace rows are the appended slots packed (AppendRows), so a batch
 // of sequences with a few rows each reads every weight once.  final_gain
@@ -841,6 +911,26 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
   // (the decode attention, which reads and writes the pairs, takes groups of 8 at most)
   const int rp = max_count == 1 && c->n_q_heads / c->n_kv_heads <= kDecMaxG
                      ? decode_row_pairs(batch, cap) : 0;
+  const GemvUse gemv = gemv_use(c, batch, max_count, cap, dev->sms);
+  auto gemv_call = [&](const void *x, int ldx, int K, const void *norm_gain, long long x_lo) {
+    GemvCall g;
+    GemvParams &p = g.l.p;
+    p.batch = max_rows;
+    p.total = total;
+    p.rowmap = rows.rowmap;
+    p.cap = cap;
+    p.pos = kv->pos;
+    p.head_dim = c->head_dim;
+    p.eps = c->rms_eps;
+    p.status = status;
+    p.x = x;
+    p.ldx = ldx;
+    p.K = K;
+    p.norm_gain = reinterpret_cast<const __nv_bfloat16 *>(norm_gain);
+    p.x_lo = x_lo;
+    rope_turns(c, p.turns);
+    return g;
+  };
   AttnPartials parts;
   parts.o = reinterpret_cast<float *>(wsb + L.part_o);
   parts.ml = reinterpret_cast<float2 *>(wsb + L.part_ml);
@@ -866,7 +956,21 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     g.p.eps = c->rms_eps;
   };
   // residual add, with the next norm's gain (or null) fused as in the scoring pass
-  auto resid = [&](const void *a, int k, const void *wm, const void *gain, int kind) -> cc_status {
+  auto resid = [&](const void *a, int k, const void *wm, const void *gain, int kind,
+                   bool as_gemv) -> cc_status {
+    if (as_gemv) {
+      GemvCall g = gemv_call(a, k, k, nullptr, (long long)rp * k);
+      g.add(wm, nullptr, nullptr, h, d, d, GEMV_RESID_F32);
+      GemvParams &p = g.l.p;
+      p.next_gain = reinterpret_cast<const __nv_bfloat16 *>(gain);
+      p.xn = reinterpret_cast<__nv_bfloat16 *>(xn);
+      p.ld_xn = d;
+      p.xn_lo = (long long)rp * d;
+      p.ss_part = ss_part;
+      const cc_status r = run_gemv(g, kind, dev->sms, st);
+      if (gain) ss_tiles = p.ctas;
+      return r;
+    }
     Gemm g;
     cc_status r = gemm_setup(g, EPI_RESID_F32, a, k, wm, nullptr, d, 1, max_rows, total, status,
                              false, 0, rp, max_count);
@@ -892,7 +996,20 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
     }
     // q = RoPE(xn Wq^T + bq) into the workspace; k = RoPE(xn Wk^T + bk) and
     // v = xn Wv^T + bv straight into the cache slots of the chunk
-    if (qkv_fusable(c)) {   // one GEMM over [Wq; Wk; Wv]
+    if (gemv.qkv) {   // RMSNorm fused
+      GemvCall g = gemv_call(h, d, d, lw.attn_norm, 0);
+      g.add(lw.wq, nullptr, lw.bq, q, qd, qd, GEMV_ROPE).out_lo = (long long)rp * qd;
+      g.add(lw.wk, nullptr, lw.bk, kv->k[l], kvd, kvd, GEMV_ROPE);
+      g.add(lw.wv, nullptr, lw.bv, kv->v[l], kvd, kvd, GEMV_BF16);
+      for (int j = 1; j < 3; ++j) {   // K and V into the cache (e4m3 codes; paged rows)
+        GemvSeg &sg = g.l.p.seg[j];
+        sg.fp8 = kvf.fp8 ? 1 : 0;
+        sg.qscale = 1.f / (j == 1 ? kvf.k_scale : kvf.v_scale);
+        sg.kv_dest = 1;
+      }
+      g.l.p.pg = kvf.pg;
+      if ((s = run_gemv(g, CC_KERNEL_GEMM_QKV, dev->sms, st)) != CC_OK) return s;
+    } else if (qkv_fusable(c)) {   // one GEMM over [Wq; Wk; Wv]
       Gemm g;
       if ((s = gemm_setup_qkv(g, xn, c, lw, 1, max_rows, total, status, rp, max_count)) != CC_OK) return s;
       scaled(g);
@@ -946,17 +1063,28 @@ cc_status run_append(const cc_model_cfg *c, const cc_model_weights *w, const cc_
                            (size_t)batch * cap * c->d_ff * 2, false, rows.pbase, max_rows, rp)) != CC_OK)
       return s;
     // h += o Wo^T; act = SwiGLU(RMSNorm(h)); h += act Wd^T
-    if ((s = resid(o, qd, lw.wo, lw.mlp_norm, CC_KERNEL_GEMM_OPROJ)) != CC_OK) return s;
-    Gemm gu;
-    if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, 1, max_rows, total, status,
-                        false, 0, rp, max_count)) != CC_OK)
+    // (a GEMV norms the rows itself: no gain then)
+    if ((s = resid(o, qd, lw.wo, gemv.gateup ? nullptr : lw.mlp_norm, CC_KERNEL_GEMM_OPROJ,
+                   gemv.o)) != CC_OK)
       return s;
-    scaled(gu);
-    gu.p.out = act;
-    gu.p.ldo = f;
-    if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
-    const void *next_gain = l + 1 < c->n_layers ? w->layers[l + 1].attn_norm : final_gain;
-    if ((s = resid(act, f, lw.w_down, next_gain, CC_KERNEL_GEMM_DOWN)) != CC_OK) return s;
+    if (gemv.gateup) {
+      GemvCall g = gemv_call(h, d, d, lw.mlp_norm, 0);
+      g.add(lw.w_gate, lw.w_up, nullptr, act, f, f, GEMV_SWIGLU).out_lo = (long long)rp * f;
+      if ((s = run_gemv(g, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
+    } else {
+      Gemm gu;
+      if ((s = gemm_setup(gu, EPI_SWIGLU, xn, d, lw.w_gate, lw.w_up, f, 1, max_rows, total, status,
+                          false, 0, rp, max_count)) != CC_OK)
+        return s;
+      scaled(gu);
+      gu.p.out = act;
+      gu.p.ldo = f;
+      if ((s = run_gemm(gu, EPI_SWIGLU, CC_KERNEL_GEMM_GATEUP, dev->sms, st)) != CC_OK) return s;
+    }
+    const void *next_gain = l + 1 == c->n_layers ? final_gain
+                            : gemv.qkv           ? nullptr
+                                                 : w->layers[l + 1].attn_norm;
+    if ((s = resid(act, f, lw.w_down, next_gain, CC_KERNEL_GEMM_DOWN, gemv.down)) != CC_OK) return s;
   }
   if (final_gain) {
     *ss_tiles_out = ss_tiles;

@@ -46,12 +46,11 @@
 // a 256-row chunk: q/k/v 43 -> 28 us, O 33 -> 27 us, down 71 -> 48 us (pairs,
 // four splits, partials in two rounds), gate/up 75 -> 66 us; a 512-slot cache:
 // down 84 -> 67 us; the 512-slot tiny model's pass 78 -> 60 us.
-// Decode steps (Qwen2.5-7B layer, one row) against CUDA-core GEMVs streaming
-// the weights: gate/up 57 -> 50 us (271 MB), LM head 186 -> 159 us (1.09 GB,
-// 6.8 TB/s), down 34 -> 34 us, q/k/v 15 -> 20 and O 14.5 -> 19 us when timed
-// alone (each waits out its own prologue there; a step of four layers took
-// 680 us before and takes 618 us); 16 Llama-3-8B rows against one 128-row tile
-// per sequence: 4.25 -> 0.71 ms.
+// Decode steps: of one to four sequences the smaller products run as GEMVs
+// (gemv.cuh; a launch here waits out its cluster's set-up and exchange: one
+// Qwen2.5-7B row q/k/v 20 us against 15, O 19 against 14.5); gate/up 57 -> 50 us
+// (271 MB) and the LM head 186 -> 159 us (1.09 GB, 6.8 TB/s) against such GEMVs.
+// 16 Llama-3-8B rows against one 128-row tile per sequence: 4.25 -> 0.71 ms.
 #include "fewrow.cuh"
 
 #include <algorithm>
