@@ -1,9 +1,10 @@
 """The decode attention kernel (csrc/attn.cu, attn_decode_kernel and its
-combine) at the edges of its 64-key chunks, splits and pages: key counts 1 to
-700, one split and many, 1 to 8 query heads per KV head, both head dims, the
-K/V layouts, and a batch past the 64 sequences whose activations travel as
-bf16 pairs.  Checked on H^(L-1), the residual stream after the first layer,
-against the oracle."""
+combine): key counts 1 to 700 at the edges of 64-key chunks and pages, one split
+and many of one chunk, splits of several chunks, 1 to 8 query heads per KV head,
+both head dims, the K/V layouts and types, what it reports and what NaN and
+infinity do; and decode batches around the sizes at which the activations'
+bf16 pairs change layout (16, 32) and end (64).  Checked on H^(L-1), the residual
+stream after the first layer, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -170,3 +171,76 @@ def test_infinite_activation_stays_infinite(pkg, batch):
     got = c["h_last"].float().cpu().numpy()
     for i, n in enumerate(lens):
         np.testing.assert_array_equal(got[i, n], np.sign(down) * np.float32(np.inf))
+
+
+@pytest.mark.parametrize("dh,hkv,g,layout", [(64, 1, 4, "slot"), (128, 1, 8, "head"), (128, 2, 3, "paged"),
+                                             (64, 1, 8, "e4m3"), (128, 1, 2, "e4m3")])
+def test_splits_of_several_chunks(pkg, dh, hkv, g, layout):
+    """Splits of three chunks and more: stages refilled, pages changing inside a
+    split, and a reference max that later chunks raise (keys grow sixtyfold along
+    the cache).  The tolerance of test_step_matches_oracle (e4m3: the new row's
+    codes may round the other way, one key of thousands: 2^-6)."""
+    import bench
+    from tests.test_gpu_fp8 import fp8_views
+    from tests._util import bf16_round
+    shape = ModelShape(2, 256, hkv * g, hkv, dh, 512, 300, 1e4, 1e-5)
+    lens, cap = [3900 - 27 * i for i in range(32 // hkv)], 4096
+    lens += [2500 + i for i in range(16)] if hkv > 1 else []
+    assert keys_per_split(shape, [n + 1 for n in lens], cap) >= 3 * 64
+    w_np = to_np(synth.model_weights(shape, 3, with_kv_proj=True))
+    c_np = to_np(synth.synthetic_cache(shape, lens, cap, 4))
+    ramp = np.linspace(1.0, 60.0, cap, dtype=np.float32)[None, :, None, None]
+    c_np["k"] = [bf16_round(x * ramp) for x in c_np["k"]]
+    on, c = fp8_views(c_np) if layout == "e4m3" else (c_np, to_device(c_np))
+    on = {k: ([np.asarray(x, np.float64).copy() for x in v] if k in ("k", "v") else
+              v if isinstance(v, list) else np.asarray(v).copy()) for k, v in on.items()}
+    if layout == "paged":
+        bench.to_paged_cache(c, 128, 11)
+    elif layout == "head":
+        for key in ("k", "v"):
+            c[key] = [x.permute(0, 2, 1, 3).contiguous() for x in c[key]]
+        c["kv_layout"] = 1
+    status, tok, _, _ = decode(pkg, shape, to_device(w_np), c)
+    assert status == 0
+    oracle.decode_step(shape, w_np, on, tok)
+    got, tol = c["h_last"].float().cpu().numpy(), 2.0 ** (-6 if layout == "e4m3" else -7)
+    for i, n in enumerate(lens):
+        want = on["h_last"][i, n]
+        assert np.abs(got[i, n] - want).max() <= tol * np.abs(want).max(), (i, n)
+
+
+@pytest.mark.parametrize("batch", [5, 16, 17, 32, 33, 64, 65])
+def test_batches_around_the_pair_layouts(pkg, batch):
+    """Every sequence's appended K/V rows, H^(L-1), next token and logit, over a
+    vocabulary that ends inside a column tile; the third sequence has no room, so
+    the packed rows after it move up.  Pairs: 2^-7 of a row's largest; 65
+    sequences travel as single bf16 rows: 2^-6."""
+    shape = ModelShape(2, 256, 8, 2, 64, 512, 300, 1e4, 1e-5)
+    cap = 160
+    lens = [(37 * i) % 150 for i in range(batch)]
+    lens[2] = cap
+    w_np = to_np(synth.model_weights(shape, 3, with_kv_proj=True))
+    c_np = to_np(synth.synthetic_cache(shape, lens, cap, 4))
+    c = to_device(c_np)
+    status, tok, nxt, best = decode(pkg, shape, to_device(w_np), c)
+    assert status == 7 and nxt[2] == -1   # CC_ERR_DEVICE_ARG: the full sequence
+    assert c["seq_len"].tolist() == [n + (i != 2) for i, n in enumerate(lens)]
+    tol = 2.0 ** (-6 if batch > 64 else -7)
+    cn = {k: ([np.asarray(x, np.float64).copy() for x in v] if isinstance(v, list) else
+              np.asarray(v).copy()) for k, v in c_np.items()}
+    for i, n in enumerate(lens):
+        if i == 2:
+            for key in ("k", "v"):
+                for l in range(2):
+                    assert np.array_equal(c[key][l][i].float().cpu().numpy(), c_np[key][l][i])
+            continue
+        one = {k: [x[i:i + 1] for x in v] if isinstance(v, list) else v[i:i + 1] for k, v in cn.items()}
+        _, _, logits = oracle.decode_step(shape, w_np, one, tok[i:i + 1])
+        rows = [(c["h_last"][i, n], one["h_last"][0, n])]
+        rows += [(c[key][l][i, n], one[key][l][0, n]) for key in ("k", "v") for l in range(2)]
+        for got, want in rows:
+            want = np.asarray(want, np.float64)
+            assert np.abs(got.float().cpu().numpy() - want).max() <= tol * np.abs(want).max(), i
+        top = logits[0].max()
+        assert logits[0][nxt[i]] >= top - tol * np.abs(logits[0]).max(), i
+        assert abs(best[i] - top) <= tol * np.abs(logits[0]).max(), i

@@ -30,6 +30,8 @@ def _launches(cc):
 SHAPES = {
     "small": ModelShape(3, 288, 8, 2, 64, 608, 300, 1e4, 1e-5, qkv_bias=True),
     "head128": ModelShape(2, 512, 5, 1, 128, 2592, 300, 1e4, 1e-6),
+    # more query heads per KV head than the decode attention takes: single bf16 rows
+    "g12": ModelShape(2, 256, 12, 1, 64, 320, 300, 1e4, 1e-5),
     "g1": ModelShape(2, 256, 4, 4, 64, 256, 300, 1e4, 1e-5, qkv_bias=True),
 }
 
