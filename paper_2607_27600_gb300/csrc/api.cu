@@ -336,8 +336,9 @@ struct Gemm {
   bool one_group;      // few: one row group
 };
 
-// CC_GEMM_PAIRS (tests): '0' or '2' keeps every product on the tile kernel, on
-// single CTAs or on pairs wherever the tiles are 256 columns wide.  0: unset.
+// CC_GEMM_PAIRS (tests, whose reference the tile kernel is): '0' or '2' keeps every
+// product but the greedy LM head on it, on single CTAs or on pairs wherever the tiles
+// are 256 columns wide.  0: unset.
 char gemm_pairs_env() {
   const char *e = getenv("CC_GEMM_PAIRS");
   return e && (e[0] == '0' || e[0] == '2') ? e[0] : 0;
@@ -399,7 +400,7 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   // 700, 300 and 64 slots scored 529 -> 437 us.
   g.few = FewPlan{};
   g.one_group = false;
-  if (have_dev && !pair && !env && epi != EPI_F32 && epi != EPI_LSE) {
+  if (have_dev && !pair && (!env || epi == EPI_ARGMAX) && epi != EPI_F32 && epi != EPI_LSE) {
     g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
                      batch, cap, row_pairs, dev_info->fit);
     // (up to 256 rows the few-row kernel was the faster throughout, 1.2 to 3 times; a

@@ -532,28 +532,6 @@ CC_DEV void epilogue_tile(const GemmParams &p, uint32_t tacc, int grow, bool val
       reinterpret_cast<float2 *>(p.out)[(size_t)grow * p.ldo + nt] = make_float2(m, s);
       if (has_t) p.z_target[grow] = zt;
     }
-  } else if constexpr (EPI == EPI_ARGMAX) {
-    // the tile's largest logit and its first column (NaN never wins)
-    float m = -INFINITY;
-    int mi = -1;
-#pragma unroll 1
-    for (int c = 0; c < TBN / 32; ++c) {
-      uint32_t r[32];
-      tmem_ld32(tacc + c * 32, r);
-      tmem_ld_wait();
-      const int col = tile_n0 + c * 32;
-#pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const float v = __uint_as_float(r[k]);
-        if (col + k < p.N && v > m) {
-          m = v;
-          mi = col + k;
-        }
-      }
-    }
-    if (valid)
-      reinterpret_cast<float2 *>(p.out)[(size_t)grow * p.ldo + nt] =
-          make_float2(m * row_rms_scale(p, grow, valid), __int_as_float(mi));
   }
 }
 
@@ -967,7 +945,7 @@ cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorM
 
 // SwiGLU (gate and up halves), LSE and the fused q/k/v projections always
 // use 256-wide tiles; the others take p.block_n (128 or 256).  p.pair: CTA
-// pairs (256-wide tiles only; greedy decoding's argmax never pairs).
+// pairs (256-wide tiles only).
 template <int EPI>
 cudaError_t launch(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,
                    const CUtensorMap &b3, const GemmParams &p, int grid, cudaStream_t stream) {
@@ -976,9 +954,7 @@ cudaError_t launch(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap
     if (p.split_part && gemm_may_split(EPI, p, grid))
       return launch_t<EPI, BN, true, true>(a, b, b2, b3, p, grid, stream);
   }
-  if constexpr (EPI != EPI_ARGMAX) {
-    if (p.pair && (kWide || p.block_n == BN)) return launch_t<EPI, BN, true>(a, b, b2, b3, p, grid, stream);
-  }
+  if (p.pair && (kWide || p.block_n == BN)) return launch_t<EPI, BN, true>(a, b, b2, b3, p, grid, stream);
   if (p.pair) return cudaErrorInvalidValue;
   if constexpr (kWide) {
     return launch_t<EPI, BN, false>(a, b, b2, b3, p, grid, stream);
@@ -1013,7 +989,6 @@ cudaError_t launch_gemm(int epi, const CUtensorMap &a, const CUtensorMap &b, con
     case EPI_LSE: return launch<EPI_LSE>(a, b, b2, b3, p, grid, stream);
     case EPI_BF16: return launch<EPI_BF16>(a, b, b2, b3, p, grid, stream);
     case EPI_QKV: return launch<EPI_QKV>(a, b, b2, b3, p, grid, stream);
-    case EPI_ARGMAX: return launch<EPI_ARGMAX>(a, b, b2, b3, p, grid, stream);
     case EPI_RESID_LOGIT: return launch<EPI_RESID_LOGIT>(a, b, b2, b3, p, grid, stream);
     default: return cudaErrorInvalidValue;
   }

@@ -15,7 +15,8 @@ enum GemmEpi : int {
   EPI_BF16 = 6,       // out bf16 [rows][ldo] = acc (+ bias[col] if bias)
   EPI_QKV = 7,        // fused q/k/v projections (B = Wq, B2 = Wk, B3 = Wv, stacked by column
                       // tiles): Q RoPE'd to out, K RoPE'd to out_k, V to out_v
-  EPI_ARGMAX = 8,     // greedy decoding: out float2 [rows][ldo = n_tiles] = (max, first column of the max) per column tile
+  EPI_ARGMAX = 8,     // greedy decoding (the few-row kernel alone): out float2 [rows][ldo = n_tiles] =
+                      // (max, first column of the max) per column tile
   EPI_RESID_LOGIT = 9 // the last residual add fused with the logit head: x = out + acc
                       // (fp32 [rows][ldo], not stored back); head_part float2 [rows][n_tiles]
                       // = per column tile (sum x^2, sum x * head_gain * head_w[tokens[row]])
