@@ -44,12 +44,11 @@ using namespace cc;
 constexpr int kMaxDevices = 64;
 
 // ---------------------------------------------------------------------------
-// per-device state: status-word address, SM count, resident clusters
+// per-device state: status-word address, SM count
 // ---------------------------------------------------------------------------
 struct DevState {
   unsigned *status = nullptr;
   int sms = 0;
-  cc::FewClusters fit = {};
   bool ready = false;
 };
 DevState g_dev[kMaxDevices];
@@ -66,7 +65,6 @@ bool dev_state(DevState **out) {
     if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return false;
     d.status = reinterpret_cast<unsigned *>(p);
-    d.fit = cc::few_clusters(d.sms);
     d.ready = true;
   }
   *out = &d;
@@ -402,7 +400,7 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
   g.one_group = false;
   if (have_dev && !pair && (!env || epi == EPI_ARGMAX) && epi != EPI_F32 && epi != EPI_LSE) {
     g.few = few_plan(epi, few_tiles ? few_tiles : (N + kFewTileCols - 1) / kFewTileCols, K, a_split,
-                     batch, cap, row_pairs, dev_info->fit);
+                     batch, cap, row_pairs, few_clusters(dev_info->sms));
     // (up to 256 rows the few-row kernel was the faster throughout, 1.2 to 3 times; a
     // short K, d_model 512, is its launches' ends and overlapped starts, which the
     // estimates leave out: with them scores of three such sequences took 10 % longer)
@@ -423,7 +421,7 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
       };
       double least = 0;
       for (uint64_t r : rows)
-        least += few_us(epi, g.few, r == R ? g.few.cycles : few_cycles(g.few, epi, K, a_split, (long long)r, cap, dev_info->fit));
+        least += few_us(epi, g.few, r == R ? g.few.cycles : few_cycles(g.few, epi, K, a_split, (long long)r, cap, few_clusters(sms)));
       auto consider = [&](int cols, bool on_pairs) {
         const double t = tiles(cols, on_pairs);
         if (t >= least) return;

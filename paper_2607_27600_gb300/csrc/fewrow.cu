@@ -937,31 +937,8 @@ cudaError_t launch_t(const CUtensorMap &a, const CUtensorMap &b, const CUtensorM
 
 }  // namespace
 
-// Every form of the kernel holds an SM's shared memory, so one form's count is all
-// forms'.
 FewClusters few_clusters(int sms) {
-  FewClusters r = {{sms, sms / 2, sms / 4, sms / 8}};
-  auto kern = few_kernel<EPI_RESID_F32, false, true, true>;
-  bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) ==
-            cudaSuccess;
-  for (int i = 0; ok && i < 4; ++i) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 1u << i;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1u << i);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    ok = cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess;
-    if (ok) r.n[i] = std::max(1, std::min(n, r.n[i]));
-  }
-  if (!ok) (void)cudaGetLastError();   // the counts are a plan's: a launch reports its own errors
-  return r;
+  return {{sms, std::max(1, sms / 2), std::max(1, sms / 4 * 19 / 20), std::max(1, sms / 10)}};
 }
 
 static int cluster_log2(int ctas) { return ctas == 1 ? 0 : ctas == 2 ? 1 : ctas == 4 ? 2 : 3; }

@@ -20,12 +20,14 @@ struct FewPlan {
 };
 
 constexpr int kFewTileCols = 128;   // output columns of a tile
-// Clusters of 2^i CTAs that the device holds at once (clusters of eight leave SMs of a
-// GPC over: 15 of them on 152 SMs, 36 of four, 76 of two).
+// Clusters of 2^i CTAs that a device holds at once, one CTA per SM: those of four and
+// eight leave SMs of a GPC over (152 SMs: 76 of two, 36 of four and 15 of eight by the
+// occupancy query).  From the SM count alone, not the query: which SMs are missing
+// differs between devices, and a row's K split, so its bits, would with it.
 struct FewClusters {
   int n[4];
 };
-FewClusters few_clusters(int sms);   // of the current device
+FewClusters few_clusters(int sms);
 // The plan for seqs sequences of at most rows_per_seq rows each.  row_pairs > 0:
 // one group of 2 * row_pairs rows (GemmParams::row_pairs).
 FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
