@@ -490,22 +490,25 @@ CC_DEV uint32_t pack_e4m3x2(float lo, float hi) {
 
 // x / (1 + e^-x) without the branches of a full division, so that the rows of
 // an epilogue overlap (a 128 x 128 SwiGLU tile's end: 7.2 -> 5.8 us): the fast
-// reciprocal, one Newton step on it and one residual correction of the quotient
-// (Markstein, 1990), which round as the division does.  Compared over every
-// float: the bits of silu_div (without the Newton step one float, 0.1608038,
-// came out a last place off).
-CC_DEV float silu(float x) {
+// reciprocal and one residual correction of the quotient (Markstein, 1990).
+// EXACT: with one Newton step on the reciprocal first, which rounds as the division
+// does: the bits of silu_div for every float (without it one float, 0.1608038, comes
+// out a last place off, and -0 as +0).  The few-row kernel, whose rows all take this
+// form, leaves the step out (gate/up of 256 rows 67.0 -> 66.5 us).
+template <bool EXACT>
+CC_DEV float silu_as(float x) {
   const float y = 1.0f + __expf(-x);
   // the reciprocal of a y near 2^128 would be flushed; that of infinity is 0, and
-  // a residual with it no number; past 64 and at 0 (of either sign) the quotient
-  // is x times the reciprocal
+  // a residual with it no number; past 64 (and at 0) the quotient is x times the
+  // reciprocal
   const float s = y > 0x1p100f ? 0x1p-64f : 1.0f;
   const float r0 = __fdividef(1.0f, y * s) * s;
-  const float r = fmaf(fmaf(-y, r0, 1.0f), r0, r0);
-  const float q = x * (y > 0x1.fffffep127f ? r0 : r);
+  const float r = EXACT ? fmaf(fmaf(-y, r0, 1.0f), r0, r0) : r0;
+  const float q = x * (EXACT && y > 0x1.fffffep127f ? r0 : r);
   const float c = fmaf(fmaf(-q, y, x), r, q);
-  return y > 0x1.fffffep127f || x > 64.0f || x == 0.0f ? q : c;
+  return y > 0x1.fffffep127f || x > 64.0f || (EXACT && x == 0.0f) ? q : c;
 }
+CC_DEV float silu(float x) { return silu_as<true>(x); }
 // The same with a full division (the same bits).
 CC_DEV float silu_div(float x) { return x / (1.0f + __expf(-x)); }
 

@@ -298,7 +298,7 @@ CC_DEV void finish_rows8(const GemmParams &p, const ProjTile &d, const LaneCol &
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const float rs = tab.rs[r0 + J + j];
-      y[j] = silu(v[J + j] * rs) * (u[J + j] * rs);
+      y[j] = silu_as<false>(v[J + j] * rs) * (u[J + j] * rs);
       at[j] = (row0 + r0 + J + j) * p.ldo + lc.c0;
       live[j] = !dry && lc.ok && J + j < n;
     }
