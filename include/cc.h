@@ -354,7 +354,11 @@ size_t cc_append_workspace_size(const cc_model_cfg *cfg, int32_t batch, int32_t 
  * sequence that could not append: full cache, reported on the device) and,
  * if next_logit is non-NULL, its logit.  Needs everything cc_append_chunk
  * needs plus final_norm and lm_head.  The sequences' rows are packed into one
- * product: every weight is read once per step. */
+ * product: every weight is read once per step.  Up to 64 sequences (of at most
+ * eight query heads per KV head, and where batch * cap is at least 2 * 16, 2 * 32
+ * or 2 * 64 rows for up to 16, 32 or 64 of them) the activations pass between the
+ * products as bf16 pairs, 16 significant bits; past that as single bf16 values,
+ * as in cc_append_chunk. */
 size_t cc_decode_workspace_size(const cc_model_cfg *cfg, int32_t batch, int32_t cap);
 cc_status cc_decode_step(const cc_model_cfg *cfg, const cc_model_weights *w,
                          const cc_kv_cache *cache, const int32_t *tokens_in,
@@ -410,7 +414,7 @@ cc_status cc_score_h2o(const cc_kv_cache *cache, int32_t recent, float *scores, 
  *   - The first call on a device looks up the array's device address (with
  *     that device current); make that first call before any stream capture.
  *   - All calls on a device share the array and each call clears it first
- *     (an asynchronous memset on `stream`): calls whose work overlaps on the
+ *     (in a kernel on `stream`): calls whose work overlaps on the
  *     GPU (different streams, no ordering between them) race on it and must
  *     not be issued. */
 cc_status cc_compact_kv_static(const cc_model_cfg *cfg, const cc_kv_cache *cache,

@@ -728,8 +728,13 @@ cudaError_t launch_dh(const CUtensorMap &q, const CUtensorMap &k, const CUtensor
 // cores.  The 16 rows of a product are the group's heads twice: the hi and
 // the lo parts of fp32 values (hi = bf16(x), lo = bf16(x - hi)), for the
 // queries and for the probabilities alike, so both products carry 16
-// significant bits of them against exact bf16 keys and values.  A thread then
-// holds both parts of its head's scores, which are the operand layout of the
+// significant bits of them against exact bf16 keys and values.  (Errors of a step
+// against 64 bits, batches of 1 to 96, 64 to 16000 slots, against the fp32
+// probabilities of the CUDA-core kernel: no larger anywhere; K/V rows of up to 64
+// sequences 6e-3 -> 1.7e-3 and the largest logit 2e-3 -> 5e-5, since the queries are
+// pairs too, past 64 sequences 6.3e-3 -> 5.9e-3.  A third part with the last 8
+// bits changed no error and cost 16 sequences 707 -> 784 us a step.)  A thread
+// then holds both parts of its head's scores, which are the operand layout of the
 // second product: no exchange between the two.
 // CTA = 4 warps over one (unit, key split), 16 keys of each chunk per warp, the
 // splits of a batch equally long whatever the sequences' lengths; warps keep

@@ -62,7 +62,7 @@ constexpr int kAttnPartRowFloats = 256;   // rows of a unit (times head_dim + 2 
 cudaError_t launch_attention(const CUtensorMap &q, const CUtensorMap &k, const CUtensorMap &v,
                              const AttnParams &p, cudaStream_t stream);
 // Causal attention of one query row per sequence (q_span == 1, group <=
-// kDecMaxG): CUDA-core kernel over kv_splits (1 .. kDecMaxSplits) key ranges
+// kDecMaxG): warp-level tensor products over kv_splits (1 .. kDecMaxSplits) key ranges
 // per unit, then (kv_splits > 1) the combine; needs q, k, v, part_o and part_ml.
 cudaError_t launch_attention_decode(const AttnParams &p, cudaStream_t stream);
 

@@ -220,7 +220,7 @@ def test_fp8_append_llama_fused_projection(cc):
 @pytest.mark.parametrize("case", ["small", "small-long"])
 def test_fp8_decode_steps(cc, case):
     """Greedy decode over an e4m3 cache (weight-streaming GEMVs write the
-    codes; the CUDA-core decode attention reads them, key splits in the long
+    codes; the decode attention reads them, key splits in the long
     case), teacher-forced with the oracle's tokens."""
     import paper_2607_27600_gb300 as pkg
     seq, cap = ([50, 20, 33], 64) if case == "small" else ([1500, 300, 1999], 2048)
