@@ -1,5 +1,5 @@
-"""The few-row GEMM (csrc/fewrow.cu): every launch below two waves of 128 x 256
-tiles.  Row counts at the edges of its row groups (16 to 256) and 16-row
+"""The few-row GEMM (csrc/fewrow.cu), and the choice between it and the tile kernel
+below two waves of 128 x 256 tiles.  Row counts at the edges of its row groups (16 to 256) and 16-row
 blocks, K ranges cut over 1 to 8 CTAs of a cluster, head dims 64 and 128 and
 column counts that end inside a 128-column tile, against the oracle; and the
 general tile kernel (CC_GEMM_PAIRS=0) over every form both take."""
