@@ -406,22 +406,25 @@ cc_status gemm_setup(Gemm &g, int epi, const void *A, int K, const void *W, cons
     // estimates leave out: with them scores of three such sequences took 10 % longer)
     const int nk = ((K + 63) / 64) * (a_split ? 2 : 1);
     if (R > 256 && nk >= 32 && row_pairs == 0 && epi != EPI_SWIGLU && epi != EPI_ARGMAX) {
-      // R bounds the rows: one sequence's end somewhere in the last 128 slots of its
-      // cache, several sequences' anywhere between one cache and all of them (an
-      // append of one sequence brings its bound's rows): the mean over the bound, the
-      // least and their middle
+      // R bounds the rows: one sequence's end lies somewhere in the last 128 slots of
+      // its cache, several sequences hold between one cache and all of them (an append
+      // of one sequence brings its bound's rows): the mean over the bound, twice since
+      // buffers are sized for what they hold, the least and their middle, the
+      // sequences (an append's are packed as one) alike
       const uint64_t least_rows = rows_least ? std::min(rows_least, R)
                                              : batch > 1 ? cap : R - std::min<uint64_t>(R - 1, 128);
-      const uint64_t rows[3] = {R, (R + least_rows) / 2, least_rows};
+      const uint64_t rows[4] = {R, R, (R + least_rows) / 2, least_rows};
       const int sms = dev_info->sms;
+      auto each = [&](uint64_t r) { return (long long)((r + batch - 1) / batch); };   // of a sequence
       auto tiles = [&](int cols, bool on_pairs) {
         double t = 0;
-        for (uint64_t r : rows) t += tile_us(epi, cols, on_pairs, (double)((r + 127) / 128), N, K, nk, sms);
+        for (uint64_t r : rows)
+          t += tile_us(epi, cols, on_pairs, (double)batch * ((each(r) + 127) / 128), N, K, nk, sms);
         return t;
       };
       double least = 0;
       for (uint64_t r : rows)
-        least += few_us(epi, g.few, r == R ? g.few.cycles : few_cycles(g.few, epi, K, a_split, (long long)r, cap, few_clusters(sms)));
+        least += few_us(epi, g.few, few_cycles(g.few, epi, K, a_split, batch, each(r), few_clusters(sms)));
       auto consider = [&](int cols, bool on_pairs) {
         const double t = tiles(cols, on_pairs);
         if (t >= least) return;

@@ -1004,10 +1004,11 @@ FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long 
   return best;
 }
 
-double few_cycles(const FewPlan &plan, int epi, int K, bool a_split, long long rows,
-                  long long rows_per_seq, const FewClusters &fit) {
-  return plan_cycles(epi, plan.n_tiles, K, a_split, (double)((rows + plan.nb - 1) / plan.nb),
-                     rows_per_seq, plan.nb, plan.split, plan.pair ? 2 : 1, fit);
+double few_cycles(const FewPlan &plan, int epi, int K, bool a_split, int seqs, long long rows_per_seq,
+                  const FewClusters &fit) {
+  const double groups = (double)seqs * (double)((rows_per_seq + plan.nb - 1) / plan.nb);
+  return plan_cycles(epi, plan.n_tiles, K, a_split, groups, rows_per_seq, plan.nb, plan.split,
+                     plan.pair ? 2 : 1, fit);
 }
 
 cudaError_t launch_few(int epi, const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &b2,

@@ -32,10 +32,9 @@ FewClusters few_clusters(int sms);
 // one group of 2 * row_pairs rows (GemmParams::row_pairs).
 FewPlan few_plan(int epi, int n_tiles, int K, bool a_split, int seqs, long long rows_per_seq,
                  int row_pairs, const FewClusters &fit);
-// The plan's estimated SM cycles where only `rows` rows, in groups that follow one
-// another, turn out to be there.
-double few_cycles(const FewPlan &plan, int epi, int K, bool a_split, long long rows,
-                  long long rows_per_seq, const FewClusters &fit);
+// The plan's estimated SM cycles where each sequence turns out to have rows_per_seq rows.
+double few_cycles(const FewPlan &plan, int epi, int K, bool a_split, int seqs, long long rows_per_seq,
+                  const FewClusters &fit);
 // a: A rows x K, box 64 x plan.nb (half of it with pair); b (b2, b3): weights N x K, box 64 x 128, and
 // for rotated projections (EPI_QROPE's b, EPI_QKV's b and b2) the 5-D view
 // [heads][head_dim / 32][2][16][K], box {64, 16, 2, head_dim / 32, 128 / head_dim}.
