@@ -18,7 +18,9 @@
 // What bounds it: the weights' bytes, and for the smaller matrices the latency of
 // what follows the kernel before: the rows' way into shared memory (no tensor
 // memory, cluster or exchange to set up) and what of the weights did not fit the
-// ring.
+// ring.  Alone, one Qwen2.5-7B row: q/k/v 15.6 us (33 MB, 2.1 TB/s), O 12.9 (26 MB),
+// down 34.3 (136 MB, 4.0 TB/s); in a step of 28 layers, with gate/up and the LM head on
+// the few-row GEMM, 2.98 ms against 3.24 with every product there.
 #include "gemv.cuh"
 
 #include <algorithm>
